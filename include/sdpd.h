@@ -185,13 +185,14 @@ int sdpd_reset_counters(sdpd_t* s);
 /* Number of CUDA kernels the handle has launched so far (a VV step launches
  * 8, a sweep 9 plus 5 when its schedule is rebuilt -- it is reused while the
  * positions do not change, as in FD-only runs -- sdpd_set_state 8,
- * sdpd_observables 2). */
+ * sdpd_observables 2).  The nine of a sweep are the random numbers of all its
+ * pairs and the eight colours. */
 int64_t sdpd_kernel_launches(const sdpd_t* s);
 
 /* Per-stage timing with CUDA events recorded on the handle's stream around
  * every stage that sdpd_step launches.  Stages: 0 first kick + drift +
  * binning, 1 sort, 2 density + EOS, 3 second kick, 4 sweep schedule,
- * 5 sweep colours (8 launches per sweep); and of sdpd_vv_adjoint: 6 loading
+ * 5 the sweep's random numbers and colours (9 launches per sweep); and of sdpd_vv_adjoint: 6 loading
  * a stored position (bin, sort, density), 7 pair pass A, 8 pair pass B,
  * 9 the elementwise steps between them.  sdpd_stage_times synchronises and
  * returns, per stage, the summed milliseconds and the number of kernel
@@ -311,8 +312,10 @@ void sdpd_ensemble_destroy(sdpd_ens_t* e);
 typedef struct {
   int fd_variant;   /* blocks per warp x warps per thread block of the colour
                        launches: 0 (2 x 2), 1 (2 x 1), 2 (1 x 1), 3 (1 x 2),
-                       4 (1 x 4); -1 = the precision's default (0 mixed,
-                       1 float64).  Float64 handles take 1, 2 and 3 only (the
+                       4 (1 x 4); -1 = chosen at launch by the blocks per
+                       colour (3 up to 2432 of them, else the precision's
+                       default: 0 mixed, 1 float64, which sdpd_get_tuning
+                       then reports); a new handle starts with -1.  Float64 handles take 1, 2 and 3 only (the
                        others need more than 48 KB of shared memory) */
   int pair_threads; /* threads per block of the density and force passes:
                        32, 64 or 128; 0 = 128 */

@@ -183,9 +183,17 @@ size_t layout(sdpd_handle* s, Workspace* w, char* base) {
   w->rcoord = (uint32_t*)at(nc * 4);
   for (int d = 0; d < 3; ++d) w->xmin[d] = (uint32_t*)at((size_t)c.nc[d] * 4);
   w->sched_hdr = (uint32_t*)at(nc * 4);
-  w->sched_lvl = (uint16_t*)at(nc * (kMaxLevels + 1) * 2);
-  w->sched_pair = (uint16_t*)at(2 * nc * kMaxPairs * 2);
-  w->level_of = (uint8_t*)at(nc * kMaxPairs);
+  // the sweep's pair lists and staged pair data (none without a sweep)
+  const size_t sweep = s->prm.scheme == SDPD_SCHEME_NONE ? 0 : 1;
+  const size_t cap = sweep * sched_pair_capacity(c.N, c.nbr_cap, c.ncell);
+  const size_t rec = P::mixed || s->prm.sweep_f32 ? sizeof(F4) : sizeof(D4);
+  w->sched_canon = (uint16_t*)at(sweep * nc * kMaxPairs * 2);
+  w->sched_rsize = (uint8_t*)at(sweep * nc * kRoundStride);
+  w->sched_off = (unsigned long long*)at(nc * 8);
+  w->sched_total = (unsigned long long*)at(8);
+  w->sched_pair = (uint16_t*)at(cap * 2);
+  w->st_geom = at(cap * rec);
+  w->st_rnd = at(cap * rec);
   w->io_q = (double*)at(3 * N * 8);
   w->io_p = (double*)at(3 * N * 8);
   w->io_e = (double*)at(N * 8);
@@ -346,12 +354,18 @@ void fd_sweep_step(sdpd_handle* s, double dt_fd, uint64_t seed) {
   if (rec) cudaMemsetAsync(s->w.pair_rec_count, 0, 8, s->stream);
   if (!s->sched_valid) {  // positions unchanged since the last sweep: reuse it
     StageTimer t(s, 4, 5);
-    launch_fd_schedule<P>(c, s->w, s->cur, s->stream);
+    launch_fd_schedule<P>(c, s->w, s->cur, fd_round_width(fd_launch_variant(c, sweep_float(s))), s->stream);
+    if constexpr (std::is_same<P, Fp64>::value) {
+      if (s->prm.sweep_f32) launch_stage_geometry<Fp64, Mixed>(c, s->w, s->cur, s->stream);
+      else launch_stage_geometry<Fp64, Fp64>(c, s->w, s->cur, s->stream);
+    } else {
+      launch_stage_geometry<P, P>(c, s->w, s->cur, s->stream);
+    }
     s->launches += 5;
     s->sched_valid = true;
   }
   {
-    StageTimer t(s, 5, 8);
+    StageTimer t(s, 5, 9);
     if constexpr (std::is_same<P, Fp64>::value) {
       if (s->prm.sweep_f32) launch_fd_colours<Fp64, Mixed>(c, s->w, s->cur, dt_fd, seed, rec, s->stream);
       else launch_fd_colours<Fp64, Fp64>(c, s->w, s->cur, dt_fd, seed, rec, s->stream);
@@ -359,7 +373,6 @@ void fd_sweep_step(sdpd_handle* s, double dt_fd, uint64_t seed) {
       launch_fd_colours<P, P>(c, s->w, s->cur, dt_fd, seed, rec, s->stream);
     }
   }
-  launch_advance_sweep(s->w, s->stream);
   s->launches += 9;
   s->fd_step++;
 }
@@ -493,6 +506,7 @@ int sdpd_create(int64_t N, const double box[3], double m, double h, const sdpd_p
   c.kernel = prm->kernel;
   c.fd_variant = fd_default_variant(prm->precision == SDPD_MIXED || prm->sweep_f32 != 0);
   c.pair_threads = 128;
+  c.fd_auto = true;
   c.scheme = prm->scheme;
   s->prm = *prm;
   s->K = K;
@@ -809,6 +823,7 @@ int sdpd_set_tuning(sdpd_t* s, const sdpd_tuning* t) {
   if (v >= kFdVariants || !fd_variant_fits(sweep_float(s), v) || !pair_threads_ok(pt))
     return SDPD_ERR_INVALID_ARG;
   s->c.fd_variant = v;
+  s->c.fd_auto = t->fd_variant < 0;
   s->c.pair_threads = pt;
   return SDPD_OK;
 }
@@ -833,6 +848,7 @@ int sdpd_autotune(sdpd_t* s, double dt, int64_t steps, uint64_t seed, sdpd_tunin
   // time per step of one candidate; infinity when it failed
   auto trial = [&](int v, int pt) -> double {
     s->c.fd_variant = v;
+    s->c.fd_auto = false;
     s->c.pair_threads = pt;
     reload_handle(s, sv);
     if (mixed) do_steps<Mixed>(s, dt, 1, seed);
@@ -850,6 +866,7 @@ int sdpd_autotune(sdpd_t* s, double dt, int64_t steps, uint64_t seed, sdpd_tunin
     return (double)ms / (double)steps;
   };
   const int v0 = s->c.fd_variant, t0 = s->c.pair_threads;
+  const bool auto0 = s->c.fd_auto;
   int bv = v0, bt = 128;
   double bms = INFINITY;
   for (int v = 0; v < kFdVariants; ++v) {
@@ -865,6 +882,7 @@ int sdpd_autotune(sdpd_t* s, double dt, int64_t steps, uint64_t seed, sdpd_tunin
   cudaEventDestroy(ev[1]);
   if (!isfinite(bms)) { bv = v0; bt = t0; }
   s->c.fd_variant = bv;
+  s->c.fd_auto = !isfinite(bms) && auto0;
   s->c.pair_threads = bt;
   reload_handle(s, sv);  // back to the state and counters the call started from
   e = finish_restore(s, sv);
@@ -1457,7 +1475,7 @@ int sdpd_ensemble_step(sdpd_ens_t* e, double dt, int64_t nsteps, const uint64_t*
     phase.push_back(h->vv_step % std::max(1, h->prm.theta));
     // the graph holds the buffer pointers and launch shapes of its capture
     shape.push_back(h->cur);
-    shape.push_back(h->c.fd_variant);
+    shape.push_back(h->c.fd_auto ? -1 : h->c.fd_variant);
     shape.push_back(h->c.pair_threads);
   }
   if (units > 0) {
@@ -1558,6 +1576,7 @@ int sdpd_ensemble_autotune(sdpd_ens_t* e, double dt, int64_t steps, const uint64
   for (size_t c = 0; c < cand.size() && !err; ++c) {
     for (size_t i = 0; i < n; ++i) {
       e->m[i]->c.fd_variant = cand[c][i].fd_variant;
+      e->m[i]->c.fd_auto = false;
       e->m[i]->c.pair_threads = cand[c][i].pair_threads;
       reload_handle(e->m[i], sv[i]);
     }
@@ -1584,6 +1603,7 @@ int sdpd_ensemble_autotune(sdpd_ens_t* e, double dt, int64_t steps, const uint64
   // the chosen shapes, and every member back where the call found it
   for (size_t i = 0; i < n; ++i) {
     e->m[i]->c.fd_variant = cand[best][i].fd_variant;
+    e->m[i]->c.fd_auto = false;
     e->m[i]->c.pair_threads = cand[best][i].pair_threads;
     reload_handle(e->m[i], sv[i]);
   }

@@ -20,18 +20,20 @@
 // position of the id among the block's particles, i the lower id.  Any
 // schedule that keeps, for every particle, its pairs in that order gives the
 // same result as the sequential sweep; the schedule used here runs the pairs
-// in dependency levels (level = length of the longest chain of earlier pairs
-// sharing a particle), so the pairs of a level touch disjoint particles.
+// in rounds of at most `width` pairs of disjoint particles, each pair in the
+// first round that has room after the rounds of its particles' earlier pairs.
 //
-// Three kernels prepare the schedule of every block (it depends on the
+// Five launches prepare the schedule of every block (it depends on the
 // positions only, which are fixed during the sweep): k_sched_enum (one
 // thread block per block: owned pairs in canonical order, from the
-// neighbour lists of the density pass), k_sched_walk (one thread per
-// block: the dependency level of every pair) and k_sched_bucket (one warp per
-// block: pairs bucketed by level); two more order each colour's blocks by
-// depth (k_sched_order_scan, k_sched_order_scatter); then k_fd_colour (sdpd_fd_colour.cuh)
-// runs once per colour: the pair updates level by level in shared memory,
-// one or two blocks per warp as the launch's block schedule says.
+// neighbour lists of the density pass), k_sched_rounds (one warp per block:
+// the round of every pair, and the pairs written round by round), two that
+// order each colour's blocks by their number of rounds (k_sched_order_scan,
+// k_sched_order_scatter) and k_stage_geometry (the pairs' unit vectors and
+// friction factors).  A sweep is then k_stage_random (the pairs' random
+// numbers) and k_fd_colour once per colour (sdpd_fd_colour.cuh): the pair
+// updates round by round in shared memory, one or two blocks per warp as the
+// launch's block schedule says.
 #include "sdpd_fd_common.cuh"
 
 namespace sdpd {
@@ -104,10 +106,12 @@ __global__ void __launch_bounds__(kEnumThreads)
     k_sched_enum(Consts c, const int32_t* __restrict__ pid, const int32_t* __restrict__ cell_start,
                  const int32_t* __restrict__ mrank, const uint32_t* __restrict__ nlist,
                  const int32_t* __restrict__ nn, const uint32_t* __restrict__ cend, uint32_t* __restrict__ hdr,
-                 uint16_t* __restrict__ canon, uint32_t* __restrict__ blk_hist, uint32_t* __restrict__ big_count) {
+                 uint16_t* __restrict__ canon, uint32_t* __restrict__ blk_hist, uint32_t* __restrict__ big_count,
+                 unsigned long long* __restrict__ sched_total) {
   __shared__ EnumSmem sm;
   const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
-  if (blockIdx.x == 0) {  // the depth histogram and the lists of blocks beyond capacity that k_sched_walk fills
+  if (blockIdx.x == 0) {  // what k_sched_rounds counts in: the depth histogram, the lists of blocks beyond capacity
+    if (t == 0) *sched_total = 0ull;
     for (int k = t; k < 8 * 256; k += kEnumThreads) blk_hist[k] = 0u;
     if (t < 16) big_count[t] = 0u;
   }
@@ -381,76 +385,100 @@ __global__ void __launch_bounds__(kEnumThreads)
   if (t == 0) hdr[o] = (uint32_t)npairs;
 }
 
-// Levels, step 1: one thread per block walks that block's canonical list and
-// records the level of every pair (the longest chain of earlier pairs sharing
-// a particle).  A warp handles 32 consecutive blocks and moves their lists
-// and levels through shared memory 32 entries at a time, so every global
-// access is coalesced.
-constexpr int kLevelThreads = 32;
-constexpr int kTile = 32;
+// Rounds: one warp per block takes the block's canonical list 32 pairs at a
+// time.  A pair may go after all earlier pairs of its two particles, so the
+// lanes of a chunk first claim their particles (smallest lane wins, in
+// shared memory); a lane that holds both of its claims has no earlier pair
+// of the chunk left in its way and takes the first round >= the ones its
+// particles are free from that still has room, by an atomic count.  The
+// others try again; a chunk takes as many passes as its longest chain of
+// pairs sharing particles (mostly one or two: a row of the canonical order
+// shares particles only between pairs one row distance apart).
+// Round width: the lanes that a colour launch gives a block.  Limiting the
+// rounds here instead of splitting wide dependency levels there fills the
+// lanes better (16 lanes, 32^3 lattice: 53 rounds per block instead of 68).
+// One thread per block walking the list sequentially, with the bucketing by
+// level in a second launch, took 109 + 14 us at 32^3 (800 pairs in a chain
+// of ~190 cycles each).
+constexpr int kRoundWarps = 4;
 
-__global__ void __launch_bounds__(kLevelThreads) k_sched_walk(int64_t ncell, int nc0, int nc1, int nc2,
-                                                            uint32_t* __restrict__ hdr,
-                                                            const uint16_t* __restrict__ canon,
-                                                            uint8_t* __restrict__ level_of,
-                                                            uint32_t* __restrict__ blk_hist,
-                                                            const int32_t* __restrict__ cell_start,
-                                                            const int32_t* __restrict__ mrank,
-                                                            uint32_t* __restrict__ big_count,
-                                                            int2* __restrict__ big_list) {
-  __shared__ uint8_t last_s[kMaxBlock][kLevelThreads];  // level after which a particle is free
-  __shared__ uint16_t tile[kLevelThreads][kTile + 1];
-  __shared__ uint8_t ltile[kLevelThreads][kTile + 4];
-  const int t = threadIdx.x;
-  const int64_t o0 = (int64_t)blockIdx.x * kLevelThreads;
-  const int64_t o = o0 + t;
-  const bool live = o < ncell;
-  const bool big = live && hdr[o] == kHdrBig;
-  const int np = live && !big ? (int)(hdr[o] & 0xffffu) : 0;
-  int npmax = np;
-  for (int s = 16; s > 0; s >>= 1) npmax = max(npmax, __shfl_xor_sync(0xffffffffu, npmax, s));
-  for (int k = 0; k < kMaxBlock; ++k) last_s[k][t] = 0;
-  int nlev = 0;
+struct RoundSmem {
+  uint32_t claim[kMaxBlock];
+  uint32_t cnt[kMaxLevels + 1];
+  uint16_t place[kMaxPairs];  // round << 5 | place in the round
+  uint8_t last[kMaxBlock];    // first round in which a particle is free
+};
+
+__global__ void __launch_bounds__(kRoundWarps * 32)
+    k_sched_rounds(int64_t ncell, int nc0, int nc1, int nc2, int width, uint32_t* __restrict__ hdr,
+                   const uint16_t* __restrict__ canon, uint8_t* __restrict__ rsize,
+                   unsigned long long* __restrict__ off, unsigned long long* __restrict__ total,
+                   unsigned long long cap, uint16_t* __restrict__ pairs, uint32_t* __restrict__ blk_hist,
+                   const int32_t* __restrict__ cell_start, const int32_t* __restrict__ mrank,
+                   uint32_t* __restrict__ big_count, int2* __restrict__ big_list) {
+  __shared__ RoundSmem sm_all[kRoundWarps];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t o = (int64_t)blockIdx.x * kRoundWarps + warp;
+  if (o >= ncell) return;
+  RoundSmem& sm = sm_all[warp];
+  const uint32_t hd = hdr[o];
+  bool big = hd == kHdrBig;
+  const int np = big ? 0 : (int)(hd & 0xffffu);
+  for (int k = lane; k < kMaxBlock; k += 32) sm.claim[k] = 0xffffffffu;
+  for (int k = lane; k <= kMaxLevels; k += 32) sm.cnt[k] = 0u;
+  for (int k = lane; k < kMaxBlock / 4; k += 32) reinterpret_cast<uint32_t*>(sm.last)[k] = 0u;
+  __syncwarp();
+  const uint16_t* in = canon + o * kMaxPairs;
+  int full = 0;  // rounds below are full
   bool overflow = false;
-  for (int k0 = 0; k0 < npmax; k0 += kTile) {
-    // the next 32 entries of the 32 blocks' lists: all loads issued before
-    // the first is used
-    uint16_t v[kLevelThreads];
-#pragma unroll
-    for (int j = 0; j < kLevelThreads; ++j) {
-      const int64_t oj = o0 + j;
-      v[j] = oj < ncell ? canon[oj * kMaxPairs + k0 + t] : (uint16_t)0;
+  uint16_t nxt = lane < np ? in[lane] : (uint16_t)0;
+  for (int k0 = 0; k0 < np; k0 += 32) {
+    const uint16_t pr = nxt;
+    if (k0 + 32 + lane < np) nxt = in[k0 + 32 + lane];
+    const int u = pr & 255, v = pr >> 8;
+    bool pending = k0 + lane < np;
+    while (__any_sync(0xffffffffu, pending)) {
+      if (pending) {
+        atomicMin(&sm.claim[u], (uint32_t)lane);
+        atomicMin(&sm.claim[v], (uint32_t)lane);
+      }
+      __syncwarp();
+      const bool ready = pending && sm.claim[u] == (uint32_t)lane && sm.claim[v] == (uint32_t)lane;
+      __syncwarp();
+      if (pending) sm.claim[u] = sm.claim[v] = 0xffffffffu;
+      if (ready) {
+        int L = max(full, max((int)sm.last[u], (int)sm.last[v]));
+        uint32_t s = 0;
+        while (L < kMaxLevels && (s = atomicAdd(&sm.cnt[L], 1u)) >= (uint32_t)width) ++L;
+        if (L >= kMaxLevels) {
+          overflow = true;
+        } else {
+          sm.last[u] = sm.last[v] = (uint8_t)(L + 1);
+          sm.place[k0 + lane] = (uint16_t)(L << 5 | (int)s);
+        }
+        pending = false;
+      }
+      __syncwarp();
     }
-    __syncwarp();
-#pragma unroll
-    for (int j = 0; j < kLevelThreads; ++j) tile[j][t] = v[j];
-    __syncwarp();
-    const int kn = min(kTile, np - k0);
-    for (int k = 0; k < kn; ++k) {
-      const uint16_t pr = tile[t][k];
-      const int u = pr & 255, v = pr >> 8;
-      const int L = max(last_s[u][t], last_s[v][t]);
-      if (L >= kMaxLevels) { overflow = true; ltile[t][k] = 0; continue; }
-      last_s[u][t] = last_s[v][t] = (uint8_t)(L + 1);
-      ltile[t][k] = (uint8_t)L;
-      nlev = max(nlev, L + 1);
-    }
-    __syncwarp();
-#pragma unroll
-    for (int j = 0; j < kLevelThreads; ++j) {
-      const int64_t oj = o0 + j;
-      if (oj < ncell) level_of[oj * kMaxPairs + k0 + t] = ltile[j][t];
-    }
+    if (__any_sync(0xffffffffu, overflow)) break;
+    while (full < kMaxLevels && sm.cnt[full] >= (uint32_t)width) ++full;
   }
-  if (live) {
-    // the block's colour is the parity pattern of its owner cell
-    const int ox = (int)(o % nc0), oy = (int)((o / nc0) % nc1), oz = (int)(o / ((int64_t)nc0 * nc1));
-    const int colour = (ox & 1) | ((oy & 1) << 1) | ((oz & 1) << 2);
-    if (overflow || big) {
-      // swept pair by pair after the colour's other blocks: listed with the
-      // place of its particles in big_perm (blocks of a colour are disjoint)
+  big = big || __any_sync(0xffffffffu, overflow);
+  __syncwarp();
+  // the block's place in the dense pair arrays (their capacity covers every
+  // schedule; a block past it would be swept pair by pair)
+  unsigned long long at = 0ull;
+  if (!big && lane == 0) at = atomicAdd(total, (unsigned long long)((np + 7) & ~7));
+  at = __shfl_sync(0xffffffffu, at, 0);
+  big = big || at + (unsigned long long)np > cap;
+  // the block's colour is the parity pattern of its owner cell
+  const int ox = (int)(o % nc0), oy = (int)((o / nc0) % nc1), oz = (int)(o / ((int64_t)nc0 * nc1));
+  const int colour = (ox & 1) | ((oy & 1) << 1) | ((oz & 1) << 2);
+  if (big) {
+    // swept pair by pair after the colour's other blocks: listed with the
+    // place of its particles in big_perm (blocks of a colour are disjoint)
+    if (lane == 0) {
       hdr[o] = kHdrBig;
-      nlev = kMaxLevels;
       int nb = 0;
       for (int d = 0; d < 8; ++d) {
         int cx = ox + (d & 1), cy = oy + ((d >> 1) & 1), cz = oz + ((d >> 2) & 1);
@@ -460,13 +488,50 @@ __global__ void __launch_bounds__(kLevelThreads) k_sched_walk(int64_t ncell, int
         const int r = mrank[cx + nc0 * (cy + nc1 * cz)];
         nb += cell_start[r + 1] - cell_start[r];
       }
-      const uint32_t off = atomicAdd(&big_count[8 + colour], (uint32_t)nb);
+      const uint32_t first = atomicAdd(&big_count[8 + colour], (uint32_t)nb);
       const uint32_t slot = atomicAdd(&big_count[colour], 1u);
-      big_list[colour * (ncell >> 3) + slot] = make_int2((int)o, (int)off);
-    } else {
-      hdr[o] = (uint32_t)np | ((uint32_t)nlev << 16);
+      big_list[colour * (ncell >> 3) + slot] = make_int2((int)o, (int)first);
+      atomicAdd(&blk_hist[colour * 256 + kMaxLevels], 1u);
     }
-    atomicAdd(&blk_hist[colour * 256 + nlev], 1u);
+    return;
+  }
+  // round sizes and their first positions: 8 consecutive rounds per lane
+  // (rounds are contiguous: a pair enters round L > 0 only after a pair in
+  // round L - 1 or because that round is full)
+  int v[8], sum = 0, nr = 0;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int L = lane * 8 + q;
+    v[q] = L < kMaxLevels ? min((int)sm.cnt[L], width) : 0;
+    sum += v[q];
+    nr += v[q] > 0;
+  }
+  int incl = sum;
+#pragma unroll
+  for (int sh = 1; sh < 32; sh <<= 1) {
+    const int x = __shfl_up_sync(0xffffffffu, incl, sh);
+    if (lane >= sh) incl += x;
+  }
+  nr = __reduce_add_sync(0xffffffffu, nr);
+  if (lane == 0) {
+    off[o] = at;
+    hdr[o] = (uint32_t)np | ((uint32_t)nr << 16);
+    atomicAdd(&blk_hist[colour * 256 + nr], 1u);
+  }
+  int run = incl - sum;
+  uint32_t packed[2] = {0u, 0u};
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    packed[q >> 2] |= (uint32_t)v[q] << (8 * (q & 3));
+    sm.cnt[lane * 8 + q] = (uint32_t)run;
+    run += v[q];
+  }
+  if (lane * 8 < nr) reinterpret_cast<uint2*>(rsize + o * kRoundStride)[lane] = make_uint2(packed[0], packed[1]);
+  __syncwarp();
+#pragma unroll 4
+  for (int k = lane; k < np; k += 32) {
+    const int pl = sm.place[k];
+    pairs[at + sm.cnt[pl >> 5] + (pl & 31)] = in[k];
   }
 }
 
@@ -514,75 +579,16 @@ __global__ void k_sched_order_scatter(int64_t ncell, int nc0, int nc1, const uin
   blk_order[colour * (ncell >> 3) + pos] = w;
 }
 
-// Levels, step 2: one warp per block buckets the canonical list by level
-// (order inside a level is free: its pairs touch disjoint particles) and
-// writes the level offsets.
-constexpr int kBucketWarps = 4;
-
-__global__ void __launch_bounds__(kBucketWarps * 32) k_sched_bucket(int64_t ncell, const uint32_t* __restrict__ hdr,
-                                                                  const uint16_t* __restrict__ canon,
-                                                                  const uint8_t* __restrict__ level_of,
-                                                                  uint16_t* __restrict__ lvl,
-                                                                  uint16_t* __restrict__ pairs) {
-  __shared__ int32_t cnt_s[kBucketWarps][kMaxLevels + 1];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t o = (int64_t)blockIdx.x * kBucketWarps + warp;
-  if (o >= ncell) return;
-  const uint32_t hd = hdr[o];
-  if (hd == kHdrBig) return;
-  const int np = (int)(hd & 0xffffu), nlev = (int)(hd >> 16);
-  int32_t* cnt = cnt_s[warp];
-  for (int L = lane; L <= kMaxLevels; L += 32) cnt[L] = 0;
-  __syncwarp();
-  const uint16_t* in = canon + o * kMaxPairs;
-  const uint8_t* lv = level_of + o * kMaxPairs;
-#pragma unroll 4
-  for (int k = lane; k < np; k += 32) atomicAdd(&cnt[lv[k]], 1);
-  __syncwarp();
-  // exclusive scan over nlev (<= 255) levels: 8 per lane
-  int v[8], sum = 0;
-#pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    const int L = lane * 8 + q;
-    v[q] = L < nlev ? cnt[L] : 0;
-    sum += v[q];
-  }
-  int incl = sum;
-  for (int s = 1; s < 32; s <<= 1) {
-    const int t = __shfl_up_sync(0xffffffffu, incl, s);
-    if (lane >= s) incl += t;
-  }
-  int run = incl - sum;
-  uint16_t* off = lvl + o * (kMaxLevels + 1);
-#pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    const int L = lane * 8 + q;
-    if (L < nlev) {
-      off[L] = (uint16_t)run;
-      cnt[L] = run;
-    }
-    run += v[q];
-  }
-  if (lane == 31) off[nlev] = (uint16_t)run;
-  __syncwarp();
-  uint16_t* out = pairs + o * kMaxPairs;
-#pragma unroll 4
-  for (int k = lane; k < np; k += 32) out[atomicAdd(&cnt[lv[k]], 1)] = in[k];
-}
-
-
 template <class P>
-void launch_fd_schedule(const Consts& c, const Workspace& w, int cur, cudaStream_t s) {
+void launch_fd_schedule(const Consts& c, const Workspace& w, int cur, int width, cudaStream_t s) {
   if (c.N == 0) return;
   Arrays<P> a = view<P>(w, cur);
-  uint16_t* canon = w.sched_pair + (size_t)c.ncell * kMaxPairs;
   k_sched_enum<<<(unsigned)c.ncell, kEnumThreads, 0, s>>>(c, a.id, w.cell_start, w.mrank, w.nlist, w.nn, w.cend,
-                                                          w.sched_hdr, canon, w.blk_hist, w.big_count);
-  k_sched_walk<<<(unsigned)((c.ncell + kLevelThreads - 1) / kLevelThreads), kLevelThreads, 0, s>>>(
-      c.ncell, c.nc[0], c.nc[1], c.nc[2], w.sched_hdr, canon, w.level_of, w.blk_hist, w.cell_start, w.mrank,
-      w.big_count, w.big_list);
-  k_sched_bucket<<<(unsigned)((c.ncell + kBucketWarps - 1) / kBucketWarps), kBucketWarps * 32, 0, s>>>(
-      c.ncell, w.sched_hdr, canon, w.level_of, w.sched_lvl, w.sched_pair);
+                                                          w.sched_hdr, w.sched_canon, w.blk_hist, w.big_count,
+                                                          w.sched_total);
+  k_sched_rounds<<<(unsigned)((c.ncell + kRoundWarps - 1) / kRoundWarps), kRoundWarps * 32, 0, s>>>(
+      c.ncell, c.nc[0], c.nc[1], c.nc[2], width, w.sched_hdr, w.sched_canon, w.sched_rsize, w.sched_off,
+      w.sched_total, (unsigned long long)sched_pair_capacity(c.N, c.nbr_cap, c.ncell), w.sched_pair, w.blk_hist, w.cell_start, w.mrank, w.big_count, w.big_list);
   k_sched_order_scan<<<8, 256, 0, s>>>(w.blk_hist);
   k_sched_order_scatter<<<(unsigned)((c.ncell + 255) / 256), 256, 0, s>>>(c.ncell, c.nc[0], c.nc[1], w.sched_hdr,
                                                                          w.blk_hist, w.blk_order);
@@ -596,7 +602,7 @@ void launch_set_sweep(const Workspace& w, unsigned long long value, cudaStream_t
 }
 void launch_advance_sweep(const Workspace& w, cudaStream_t s) { k_sweep_advance<<<1, 1, 0, s>>>(w.sweep); }
 
-template void launch_fd_schedule<Fp64>(const Consts&, const Workspace&, int, cudaStream_t);
-template void launch_fd_schedule<Mixed>(const Consts&, const Workspace&, int, cudaStream_t);
+template void launch_fd_schedule<Fp64>(const Consts&, const Workspace&, int, int, cudaStream_t);
+template void launch_fd_schedule<Mixed>(const Consts&, const Workspace&, int, int, cudaStream_t);
 
 }  // namespace sdpd

@@ -293,7 +293,7 @@ static __device__ __noinline__ double mixed_margin_fp64(const MixedRatioIn& r, d
 // evaluated (always when `exact` is set).  exact_e(ei, ej) gives the two
 // current energies in float64 and uniform() the pair's uniform U (both for
 // the rare float64 evaluations).
-template <class ExactE, class Uniform>
+template <bool SEQ, class ExactE, class Uniform>
 __device__ __forceinline__ int fd_pair_mixed(const FDConst<float>& k, float ex, float ey, float ez, float base,
                                              const float G[3], Uniform uniform, float lnU, float* pi, float* pj,
                                              float eif, float ejf, ExactE exact_e, float& dh, float& dl,
@@ -311,8 +311,11 @@ __device__ __forceinline__ int fd_pair_mixed(const FDConst<float>& k, float ex, 
   pair_coeffs(k, kpar, kperp, eif, ejf, mpar, mperp, zpar, zperp);
   // proposal, Eq. (proposal), as the velocity change
   // v' - v = m_perp v + zt_perp G + [(m_par - m_perp) v_par + (zt_par - zt_perp) G_par] e
-  const float vpar = ex * vx + ey * vy + ez * vz;
-  const float gpar = ex * G[0] + ey * G[1] + ez * G[2];
+  // (the rounding order is written out so that it does not depend on the code
+  // around it; SEQ: the order of the pair-by-pair sweep)
+  const float vpar = __fmaf_rn(ez, vz, __fmaf_rn(ex, vx, __fmul_rn(ey, vy)));
+  const float gpar = __fmaf_rn(ez, G[2], SEQ ? __fmaf_rn(ey, G[1], __fmul_rn(ex, G[0]))
+                                             : __fmaf_rn(ex, G[0], __fmul_rn(ey, G[1])));
   const float cpar = (mpar - mperp) * vpar + (zpar - zperp) * gpar;
   const float dvx = mperp * vx + zperp * G[0] + cpar * ex;
   const float dvy = mperp * vy + zperp * G[1] + cpar * ey;
@@ -433,21 +436,6 @@ __device__ __forceinline__ int fd_pair_mixed(const FDConst<float>& k, float ex, 
   return decision;
 }
 
-// ---------------------------------------------------------------------------
-// One colour of the sweep.  A warp runs OPW blocks of the colour
-// side by side, each on its own group of lanes, in lockstep over the blocks'
-// dependency levels.
-//
-// A block's particles (momenta and energies) live in shared memory.  The
-// block's pairs are consumed in chunks of kChunk consecutive pairs of its
-// level-ordered list: first every lane of the group stages the chunk's
-// state-independent data (unit vector, F(r)/(rho_i rho_j), random numbers),
-// then the chunk's levels (or parts of a level: pairs of one level are
-// independent) run one after the other, the lanes of the group sharing a
-// level's pairs.
-// ---------------------------------------------------------------------------
-constexpr int kChunk = 32;
-
 // Cell code inside the block of owner (ox, oy, oz) of a particle whose cell
 // bits are w: bit k set iff the particle sits in the upper cell along axis k.
 template <class T>
@@ -457,31 +445,183 @@ __device__ __forceinline__ int block_code(T w, int ox, int oy, int oz) {
   return (cx != ox) | ((cy != oy) << 1) | ((cz != oz) << 2);
 }
 
-template <class R>
-struct FdSmemBase {
-  R px[kMaxBlock], py[kMaxBlock], pz[kMaxBlock];
+// Shared memory of one block in a colour launch: momenta and energy of each
+// particle in one record (so a pair reads two records with wide loads).
+// float64 pair arithmetic: (p, eps).  float32: (p, es) with es the energy at
+// load rounded to float32 plus the visit's changes, and its compensation ec
+// (the rounding errors of that sum and the low parts of the changes), so
+// that the energy is eps(load) + (es - (float)eps(load)) + ec.
+struct FdCells {
   int32_t cst[8], cbs[8];  // the block's cells: first storage index, offset in the block
-  // staged pair data of the current chunk
-  R G0[kChunk], G1[kChunk], G2[kChunk], lnU[kChunk];
-  R ex[kChunk], ey[kChunk], ez[kChunk], base[kChunk];
-  uint16_t pr[kChunk];
-  uint16_t off[kMaxLevels + 1];  // level offsets of the block's pair list
 };
 template <class R>
 struct FdSmem;
-// float64 pair arithmetic: the energies themselves
 template <>
-struct FdSmem<double> : FdSmemBase<double> {
-  double e[kMaxBlock];
+struct FdSmem<double> {
+  D4 s[kMaxBlock];
+  FdCells cells;
 };
-// float32 pair arithmetic: each particle's energy as a running float32 sum
-// es (the energy at load rounded to float32, plus the visit's changes) and
-// its compensation ec (the rounding errors of that sum and the low parts of
-// the changes), so that the energy is eps(load) + (es - (float)eps(load)) + ec
 template <>
-struct FdSmem<float> : FdSmemBase<float> {
-  float es[kMaxBlock], ec[kMaxBlock];
+struct FdSmem<float> {
+  F4 s[kMaxBlock];
+  float ec[kMaxBlock];
+  FdCells cells;
 };
+__device__ __forceinline__ D4 lds4(const D4* p) {
+  const double2* q = reinterpret_cast<const double2*>(p);
+  const double2 a = q[0], b = q[1];
+  return D4{a.x, a.y, b.x, b.y};
+}
+__device__ __forceinline__ F4 lds4(const F4* p) {
+  const float4 a = *reinterpret_cast<const float4*>(p);
+  return F4{a.x, a.y, a.z, a.w};
+}
+
+// Storage index of block particle q; d receives its cell in the block.
+__device__ __forceinline__ int block_gidx(const FdCells& c, int q, int& d) {
+  d = 0;
+#pragma unroll
+  for (int t = 1; t < 8; ++t) d += (q >= c.cbs[t]);
+  return c.cst[d] + (q - c.cbs[d]);
+}
+__device__ __forceinline__ int block_gidx(const FdCells& c, int q) {
+  int d;
+  return block_gidx(c, q, d);
+}
+
+// ---------------------------------------------------------------------------
+// Staged pair data.  What a pair update needs besides the momenta and
+// energies is computed ahead of the colour launches by kernels that run one
+// warp per block over all 8 colours at once, in the order of the blocks'
+// scheduled pair lists (dense arrays indexed by sched_off[block] + position):
+// the geometry (unit vector, F(r)/(rho_i rho_j)) with the schedule, since it
+// depends on positions and densities only, and the random numbers once per
+// sweep.  Outside the colour launches this work has full warps and the whole
+// GPU, also when a colour has few blocks; inside them it sat on the path of
+// every block's dependency chain.
+// ---------------------------------------------------------------------------
+constexpr int kStageWarps = 4;
+
+// F at distance r (see kernel_F); the rounding of 1 - r/h in Lucy's kernel is
+// written out so that it does not depend on the code around it.
+__device__ __forceinline__ float one_minus(float r, float inv_h) { return __fmaf_rn(-r, inv_h, 1.0f); }
+__device__ __forceinline__ double one_minus(double r, double inv_h) { return __fma_rn(-r, inv_h, 1.0); }
+template <int KIND, class S>
+__device__ __forceinline__ S stage_F(S r, S inv_h, S cF) {
+  if (KIND == SDPD_KERNEL_LUCY) {
+    const S y = one_minus(r, inv_h);
+    return cF * (y * y);
+  }
+  return kernel_F<KIND>(r * inv_h, cF);
+}
+
+// The block's cells into shared memory, by the whole warp.
+__device__ __forceinline__ void stage_cells(const Consts& c, int64_t o, const int32_t* __restrict__ mrank,
+                                            const int32_t* __restrict__ cell_start, int lane, FdCells& cells) {
+  int ox, oy, oz;
+  owner_coords(c, o, ox, oy, oz);
+  int cst = 0, cnt = 0;
+  if (lane < 8) {
+    int cx = ox + (lane & 1), cy = oy + ((lane >> 1) & 1), cz = oz + ((lane >> 2) & 1);
+    if (cx >= c.nc[0]) cx -= c.nc[0];
+    if (cy >= c.nc[1]) cy -= c.nc[1];
+    if (cz >= c.nc[2]) cz -= c.nc[2];
+    const int r = __ldg(&mrank[cx + c.nc[0] * (cy + c.nc[1] * cz)]);
+    cst = __ldg(&cell_start[r]);
+    cnt = __ldg(&cell_start[r + 1]) - cst;
+  }
+  int inc = cnt;
+#pragma unroll
+  for (int sh = 1; sh < 8; sh <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, inc, sh);
+    if (lane >= sh) inc += v;
+  }
+  if (lane < 8) {
+    cells.cst[lane] = cst;
+    cells.cbs[lane] = inc - cnt;
+  }
+  __syncwarp();
+}
+
+template <class P, class A, int KIND>
+__global__ void __launch_bounds__(kStageWarps * 32)
+    k_stage_geometry(Consts c, const typename P::V4* __restrict__ qr4, const int32_t* __restrict__ cell_start,
+                     const int32_t* __restrict__ mrank, const uint32_t* __restrict__ xmx,
+                     const uint32_t* __restrict__ xmy, const uint32_t* __restrict__ xmz,
+                     const uint32_t* __restrict__ hdr, const unsigned long long* __restrict__ sched_off,
+                     const uint16_t* __restrict__ pairs, typename A::V4* __restrict__ geom) {
+  using R = typename A::R;
+  using S = typename P::R;
+  __shared__ FdCells cells_s[kStageWarps];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t o = (int64_t)blockIdx.x * kStageWarps + warp;
+  if (o >= c.ncell) return;
+  const uint32_t hd = hdr[o];
+  const int np = hd == kHdrBig ? 0 : (int)(hd & 0xffffu);
+  if (np == 0) return;
+  FdCells& cells = cells_s[warp];
+  stage_cells(c, o, mrank, cell_start, lane, cells);
+  int ox, oy, oz;
+  owner_coords(c, o, ox, oy, oz);
+  BlockGeom<P> geo;
+  geo.init(c, ox, oy, oz, xmx, xmy, xmz);
+  const S inv_h = (S)(1.0 / c.h), cF = (S)c.cF;
+  const unsigned long long base = sched_off[o];
+  for (int t = lane; t < np; t += 32) {
+    const uint16_t pr = pairs[base + t];
+    int da, db;
+    const int ga = block_gidx(cells, pr & 255, da), gb = block_gidx(cells, pr >> 8, db);
+    S xa, ya, za, xb, yb, zb, rx, ry, rz;
+    // positions and densities of the latest density pass (one load each)
+    const typename P::V4 qa = ld4(&qr4[ga]), qb = ld4(&qr4[gb]);
+    geo.local(qa, da, xa, ya, za);
+    geo.local(qb, db, xb, yb, zb);
+    geo.disp(xa, ya, za, xb, yb, zb, rx, ry, rz);
+    const S r2 = r2_of(rx, ry, rz);
+    const S inv_r = fm::rsqrt(r2);
+    typename A::V4 v;
+    v.x = (R)(rx * inv_r);
+    v.y = (R)(ry * inv_r);
+    v.z = (R)(rz * inv_r);
+    v.w = (R)fm::div(stage_F<KIND>(r2 * inv_r, inv_h, cF), qa.w * qb.w);
+    st4(&geom[base + t], v);
+  }
+}
+
+// Three normals and the uniform (its logarithm for EMS, whose Metropolis
+// test needs only that) of every scheduled pair at the current sweep.
+template <class A>
+__global__ void __launch_bounds__(kStageWarps * 32)
+    k_stage_random(Consts c, const int32_t* __restrict__ id, const int32_t* __restrict__ cell_start,
+                   const int32_t* __restrict__ mrank, const uint32_t* __restrict__ hdr,
+                   const unsigned long long* __restrict__ sched_off, const uint16_t* __restrict__ pairs,
+                   uint64_t seed, const unsigned long long* __restrict__ sweep_ptr,
+                   typename A::V4* __restrict__ rnd) {
+  using R = typename A::R;
+  __shared__ FdCells cells_s[kStageWarps];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t o = (int64_t)blockIdx.x * kStageWarps + warp;
+  if (o >= c.ncell) return;
+  const uint32_t hd = hdr[o];
+  const int np = hd == kHdrBig ? 0 : (int)(hd & 0xffffu);
+  if (np == 0) return;
+  FdCells& cells = cells_s[warp];
+  stage_cells(c, o, mrank, cell_start, lane, cells);
+  const uint64_t sweep = *sweep_ptr;
+  const unsigned long long base = sched_off[o];
+  for (int t = lane; t < np; t += 32) {
+    const uint16_t pr = pairs[base + t];
+    const int ga = block_gidx(cells, pr & 255), gb = block_gidx(cells, pr >> 8);  // pr & 255 holds the lower id
+    R G[3], U;
+    pair_randoms_fast(seed, sweep, (uint64_t)id[ga], (uint64_t)id[gb], G, &U);
+    typename A::V4 v;
+    v.x = G[0];
+    v.y = G[1];
+    v.z = G[2];
+    v.w = c.scheme == SDPD_SCHEME_EMS ? fm::log(U) : U;
+    st4(&rnd[base + t], v);
+  }
+}
 
 // A block beyond the capacities of the shared-memory schedule (kHdrBig: more
 // than kMaxBlock particles, kMaxPairs owned pairs or kMaxLevels levels).
@@ -500,7 +640,7 @@ struct BigCounts {
   int negative, bad;
 };
 
-template <class P, class A, int KIND>
+template <class P, class A>
 __device__ __noinline__ BigCounts fd_big_block(const Consts& c, const FDConst<typename A::R>& k, const Arrays<P>& a,
                                           typename P::V4* __restrict__ qp4, const int32_t* __restrict__ cell_start,
                                           const int32_t* __restrict__ mrank, const uint32_t* xmx,
@@ -571,7 +711,9 @@ __device__ __noinline__ BigCounts fd_big_block(const Consts& c, const FDConst<ty
           const S r2 = r2_of(rx, ry, rz);
           const S inv_r = fm::rsqrt(r2);
           const R ex = (R)(rx * inv_r), ey = (R)(ry * inv_r), ez = (R)(rz * inv_r);
-          const R bs = (R)fm::div(kernel_F<KIND>(r2 * inv_r * inv_h, cF), a.rho[ga] * a.rho[gb]);
+          const S F = c.kernel == SDPD_KERNEL_LUCY ? stage_F<SDPD_KERNEL_LUCY>(r2 * inv_r, inv_h, cF)
+                                                   : stage_F<SDPD_KERNEL_CUBIC>(r2 * inv_r, inv_h, cF);
+          const R bs = (R)fm::div(F, a.rho[ga] * a.rho[gb]);
           R G[3], U;
           pair_randoms_fast(seed, sweep, (uint64_t)a.id[ga], (uint64_t)a.id[gb], G, &U);
           const R lnU = k.scheme == SDPD_SCHEME_EMS ? fm::log(U) : U;
@@ -585,7 +727,7 @@ __device__ __noinline__ BigCounts fd_big_block(const Consts& c, const FDConst<ty
             auto exact_e = [&](double& x, double& y) { x = a.eps[ga]; y = a.eps[gb]; };
             float dh, dl;
             auto uniform = [&]() { return U; };
-            dcs = fd_pair_mixed(k, ex, ey, ez, bs, G, uniform, lnU, pa, pb, (float)a.eps[ga], (float)a.eps[gb],
+            dcs = fd_pair_mixed<true>(k, ex, ey, ez, bs, G, uniform, lnU, pa, pb, (float)a.eps[ga], (float)a.eps[gb],
                                 exact_e, dh, dl, margin, m32, tol, recs != nullptr, negative);
             if (dcs == 0) {
               const double de = (double)dh + (double)dl;
@@ -646,42 +788,64 @@ __device__ __noinline__ BigCounts fd_big_block(const Consts& c, const FDConst<ty
   return BigCounts{n_tot, n_acc, n_rb, n_rm, (int)negative, (int)bad};
 }
 
-// Block schedule of a colour launch: OPW blocks per warp (each on 32 / OPW
-// lanes) and W warps per thread block.  Every variant runs the same pair
-// updates in the same per-particle order, so the results are identical; only
-// the mapping onto the GPU differs.  Register budget: 128 per thread for the
-// mixed path (16 warps per SM), none for float64.
-template <class P, int W>
-constexpr int fd_min_blocks() { return P::mixed ? 16 / W : (W >= 4 ? 1 : 4 / W); }
+// The float64 energies of a pair of the mixed path during a block visit: the
+// stored energies plus the visit's changes.  The pair's uniform drawn again.
+// Both serve the rare float64 decisions (near ties of the bound or the
+// ratio) and are kept out of the hot loop.
+static __device__ __noinline__ void fd_exact_energies(const double* eps, const FdSmem<float>& sm, int ia, int ib,
+                                                      float eaf, float ebf, double& ea, double& eb) {
+  const double ga = eps[block_gidx(sm.cells, ia)], gb = eps[block_gidx(sm.cells, ib)];
+  ea = ga + (((double)eaf - (double)(float)ga) + (double)sm.ec[ia]);
+  eb = gb + (((double)ebf - (double)(float)gb) + (double)sm.ec[ib]);
+}
+static __device__ __noinline__ float fd_uniform_again(uint64_t seed, uint64_t sweep, int32_t ida, int32_t idb) {
+  float G[3], U;
+  pair_randoms_fast(seed, sweep, (uint64_t)ida, (uint64_t)idb, G, &U);
+  return U;
+}
 
+// ---------------------------------------------------------------------------
+// One colour of the sweep.  A warp runs OPW blocks of the colour side by
+// side, each on its own group of 32 / OPW lanes, in lockstep over the blocks'
+// rounds (k_sched_rounds: at most 32 / OPW pairs of disjoint particles each).
+// A block's particles (momenta and energies) live in shared memory; the
+// pairs' staged data stream from global memory one round ahead of their use.
 // P is the storage policy of the state arrays, A the arithmetic policy of
 // the pair updates: A = P except for a float64 state swept with float32
 // pair arithmetic (P = Fp64, A = Mixed), where momenta and energies go back
 // as their float64 values plus the float32 increments of the visit.
-template <class P, class A, int KIND, int OPW, int W>
-__global__ void __launch_bounds__(W * 32, fd_min_blocks<A, W>())
+// REC: keep a record per pair (every Metropolis margin in float64).
+// Thread blocks of 1 to 4 warps; 128 registers per thread for float32
+// arithmetic (16 warps per SM), up to 168 for float64 (12 warps).
+// ---------------------------------------------------------------------------
+template <class A>
+constexpr int fd_min_blocks() { return A::mixed ? 4 : 3; }
+
+template <class P, class A, int OPW, bool REC>
+__global__ void __launch_bounds__(128, fd_min_blocks<A>())
     k_fd_colour(Consts c, FDConst<typename A::R> k, Arrays<P> a, typename P::V4* __restrict__ qp4,
-                const typename P::V4* __restrict__ qr4,
                 const int32_t* __restrict__ cell_start, const int32_t* __restrict__ mrank,
                 const uint32_t* __restrict__ xmx, const uint32_t* __restrict__ xmy,
                 const uint32_t* __restrict__ xmz, const uint32_t* __restrict__ hdr,
-                const uint16_t* __restrict__ lvl, const uint16_t* __restrict__ pairs, int colour, uint64_t seed,
-                const unsigned long long* __restrict__ sweep_ptr, unsigned long long* counters, int* status,
+                const uint8_t* __restrict__ rsize, const unsigned long long* __restrict__ sched_off,
+                const uint16_t* __restrict__ pairs, const typename A::V4* __restrict__ geom,
+                const typename A::V4* __restrict__ rnd, int colour, uint64_t seed,
+                unsigned long long* __restrict__ sweep_ptr, unsigned long long* counters, int* status,
                 sdpd_pair_rec* recs, unsigned long long* rec_count, int64_t rec_cap, unsigned* __restrict__ queue,
                 const int32_t* __restrict__ order, int32_t* __restrict__ big_perm,
                 const int2* __restrict__ big_list, const uint32_t* __restrict__ big_count) {
   using R = typename A::R;  // pair arithmetic
   using S = typename P::R;  // stored momenta, densities, geometry
+  using AV4 = typename A::V4;
   constexpr bool kSame = std::is_same<R, S>::value;
   constexpr int kGroupLanes = 32 / OPW;
-  __shared__ FdSmem<R> sm_all[W][OPW];
+  extern __shared__ __align__(32) unsigned char fd_smem_raw[];
   const uint64_t sweep = *sweep_ptr;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int grp = lane / kGroupLanes, gl = lane % kGroupLanes;
   const int hx = c.nc[0] >> 1, hy = c.nc[1] >> 1, hz = c.nc[2] >> 1;
   const int64_t nown = (int64_t)hx * hy * hz;
-  FdSmem<R>& sm = sm_all[warp][grp];
-  const S inv_h = (S)(1.0 / c.h), cF = (S)c.cF;
+  FdSmem<R>& sm = reinterpret_cast<FdSmem<R>*>(fd_smem_raw)[warp * OPW + grp];
   const S pi_coef = (S)(c.c_rho / (c.C_K * c.m));
   unsigned n_tot = 0, n_rb = 0, n_rm = 0;  // per lane (accepted = total - rejected)
   bool negative = false, bad = false;
@@ -709,199 +873,140 @@ __global__ void __launch_bounds__(W * 32, fd_min_blocks<A, W>())
       oz = 2 * (int)(w / ((int64_t)hx * hy)) + ((colour >> 2) & 1);
       o = ox + (int64_t)c.nc[0] * (oy + (int64_t)c.nc[1] * oz);
       const uint32_t hd = hdr[o];
-      if (hd != kHdrBig) {  // (a block beyond capacity was swept above)
+      if (hd != kHdrBig) {  // (a block beyond capacity is swept below)
         np = (int)(hd & 0xffffu);
         nlev = (int)(hd >> 16);
       }
     }
+    if (gl == 0) n_tot += (unsigned)np;
+    // the pairs' staged data: this lane's element of the next round, loaded
+    // one round ahead (`left` pairs of the current round not yet loaded)
+    const unsigned long long first = np > 0 ? sched_off[o] : 0ull;
+    const uint8_t* rs = rsize + o * kRoundStride;
+    int r = 0, sizes = gl < nlev ? (int)rs[gl] : 0;  // sizes of rounds [r - r % kGroupLanes, ...)
+    int left = __shfl_sync(0xffffffffu, sizes, 0, kGroupLanes);
+    int pos = 0, n = min(left, kGroupLanes);
+    uint16_t pr = 0;
+    AV4 ge{}, rn{};
+    auto fetch = [&]() {
+      if (gl < n) {
+        pr = __ldg(&pairs[first + pos + gl]);
+        ge = ld4(&geom[first + pos + gl]);
+        rn = ld4(&rnd[first + pos + gl]);
+      }
+    };
+    fetch();
     BlockCells b;
     b.base[8] = 0;
     if (np > 0) block_cells(c, ox, oy, oz, mrank, cell_start, b);
     const int nb = np > 0 ? b.base[8] : 0;
-    BlockGeom<P> geo;
-    geo.init(c, ox, oy, oz, xmx, xmy, xmz);
 #pragma unroll
     for (int t = 0; t < 8; ++t)
-      if (gl == t) {
-        sm.cst[t] = b.start[t];
-        sm.cbs[t] = b.base[t];
+      if (gl == t % kGroupLanes) {
+        sm.cells.cst[t] = b.start[t];
+        sm.cells.cbs[t] = b.base[t];
       }
     __syncwarp();
-    // storage index of block particle q (recomputed where needed, which keeps
-    // shared memory small enough for eight thread blocks per SM)
-    auto gidx = [&](int q) {
-      int d = 0;
-#pragma unroll
-      for (int t = 1; t < 8; ++t) d += (q >= sm.cbs[t]);
-      return sm.cst[d] + (q - sm.cbs[d]);
-    };
-    // the same, also giving the particle's cell in the block
-    auto gidx_code = [&](int q, int& d) {
-      d = 0;
-#pragma unroll
-      for (int t = 1; t < 8; ++t) d += (q >= sm.cbs[t]);
-      return sm.cst[d] + (q - sm.cbs[d]);
-    };
     for (int q = gl; q < nb; q += kGroupLanes) {
-      const int g = gidx(q);
-      sm.px[q] = a.px[g]; sm.py[q] = a.py[g]; sm.pz[q] = a.pz[g];
-      if constexpr (A::mixed) {
-        sm.es[q] = (float)a.eps[g];
-        sm.ec[q] = 0.0f;
-      } else {
-        sm.e[q] = a.eps[g];
-      }
+      const int g = block_gidx(sm.cells, q);
+      AV4 v;
+      v.x = (R)a.px[g];
+      v.y = (R)a.py[g];
+      v.z = (R)a.pz[g];
+      v.w = (R)a.eps[g];
+      sm.s[q] = v;
+      if constexpr (A::mixed) sm.ec[q] = 0.0f;
     }
-    for (int L = gl; L <= nlev; L += kGroupLanes) sm.off[L] = lvl[o * (kMaxLevels + 1) + L];
     __syncwarp();
-    const uint16_t* off = sm.off;
-    const uint16_t* pl = pairs + o * kMaxPairs;
-    int L = 0, pos = 0;
-    while (__any_sync(0xffffffffu, pos < np)) {
-      // stage pairs [cbeg, cend) of the level-ordered list; the chunk ends on
-      // a level boundary when at least one whole level fits, so that no level
-      // is split over two chunks (a split level costs an extra round)
-      const int cbeg = pos;
-      int cend = min(pos + kChunk, np);
-      if (pos < np && (int)off[L + 1] <= cend) {
-        int Le = L + 1;
-        while (Le < nlev && (int)off[Le + 1] <= cend) ++Le;
-        cend = off[Le];
+    while (__any_sync(0xffffffffu, n > 0)) {
+      const bool act = gl < n;
+      const int level = r;
+      const uint16_t cpr = pr;
+      const AV4 cg = ge, cr = rn;
+      // advance to the next round (or the rest of a wide one) and load it
+      pos += n;
+      left -= n;
+      if (left == 0 && r < nlev) {
+        ++r;
+        if (r % kGroupLanes == 0) sizes = r + gl < nlev ? (int)rs[r + gl] : 0;
       }
-      for (int t = cbeg + gl; t < cend; t += kGroupLanes) {
-        const uint16_t pr = pl[t];
-        const int ia = pr & 255, ib = pr >> 8;  // ia holds the lower id
-        int da, db;
-        const int ga = gidx_code(ia, da), gb = gidx_code(ib, db);
-        S xa, ya, za, xb, yb, zb, rx, ry, rz;
-        // positions and densities of the latest density pass (one load each)
-        const typename P::V4 qa = ld4(&qr4[ga]), qb = ld4(&qr4[gb]);
-        geo.local(qa, da, xa, ya, za);
-        geo.local(qb, db, xb, yb, zb);
-        geo.disp(xa, ya, za, xb, yb, zb, rx, ry, rz);
-        const S r2 = r2_of(rx, ry, rz);
-        const S inv_r = fm::rsqrt(r2);
-        const int slot = t - cbeg;
-        sm.pr[slot] = pr;
-        sm.ex[slot] = (R)(rx * inv_r);
-        sm.ey[slot] = (R)(ry * inv_r);
-        sm.ez[slot] = (R)(rz * inv_r);
-        sm.base[slot] = (R)fm::div(kernel_F<KIND>(r2 * inv_r * inv_h, cF), qa.w * qb.w);
-        R G[3], U;
-        pair_randoms_fast(seed, sweep, (uint64_t)a.id[ga], (uint64_t)a.id[gb], G, &U);
-        sm.G0[slot] = G[0]; sm.G1[slot] = G[1]; sm.G2[slot] = G[2];
-        sm.lnU[slot] = k.scheme == SDPD_SCHEME_EMS ? fm::log(U) : U;  // off the pairs' dependency chain
-      }
-      __syncwarp();
-      // the chunk's levels, or parts of them
-      bool more = cbeg < cend;
-      while (__any_sync(0xffffffffu, more)) {
-        int lb = 0, le = 0;
-        if (more) {
-          lb = max((int)off[L], cbeg);
-          le = min((int)off[L + 1], cend);
-        }
-        for (int t = lb + gl; t < le; t += kGroupLanes) {
-          const int slot = t - cbeg;
-          const uint16_t pr = sm.pr[slot];
-          const int ia = pr & 255, ib = pr >> 8;
-          R pa[3] = {sm.px[ia], sm.py[ia], sm.pz[ia]};
-          R pb[3] = {sm.px[ib], sm.py[ib], sm.pz[ib]};
-          const R G[3] = {sm.G0[slot], sm.G1[slot], sm.G2[slot]};
-          double margin;
-          float m32 = 0.0f, tol = 0.0f;
-          int dcs;
-          if constexpr (A::mixed) {
-            const float eaf = sm.es[ia], ebf = sm.es[ib];
-            // rare (near ties of the bound or the ratio): the two energies in
-            // float64, and the pair's uniform drawn again
-            auto exact_e = [&](double& ea, double& eb) {
-              const double ga = a.eps[gidx(ia)], gb = a.eps[gidx(ib)];
-              ea = ga + (((double)eaf - (double)(float)ga) + (double)sm.ec[ia]);
-              eb = gb + (((double)ebf - (double)(float)gb) + (double)sm.ec[ib]);
-            };
-            auto uniform = [&]() {
-              R Gr[3], U;
-              pair_randoms_fast(seed, sweep, (uint64_t)a.id[gidx(ia)], (uint64_t)a.id[gidx(ib)], Gr, &U);
-              return U;
-            };
-            float dh, dl;
-            dcs = fd_pair_mixed(k, sm.ex[slot], sm.ey[slot], sm.ez[slot], sm.base[slot], G, uniform,
-                                sm.lnU[slot], pa, pb, eaf, ebf, exact_e, dh, dl, margin, m32, tol,
-                                recs != nullptr, negative);
-            if (dcs == 0) {
-              sm.px[ia] = pa[0]; sm.py[ia] = pa[1]; sm.pz[ia] = pa[2];
-              sm.px[ib] = pb[0]; sm.py[ib] = pb[1]; sm.pz[ib] = pb[2];
-              float s, e;
-              eft::two_sum(eaf, dh, s, e);
-              sm.ec[ia] = __fadd_rn(sm.ec[ia], __fadd_rn(e, dl));
-              sm.es[ia] = s;
-              eft::two_sum(ebf, dh, s, e);
-              sm.ec[ib] = __fadd_rn(sm.ec[ib], __fadd_rn(e, dl));
-              sm.es[ib] = s;
-              bad |= !isfinite(sm.es[ia]) || !isfinite(sm.es[ib]);
-            }
-          } else {
-            const double ea = sm.e[ia], eb = sm.e[ib];
-            double deps;
-            dcs = fd_pair(k, sm.ex[slot], sm.ey[slot], sm.ez[slot], sm.base[slot], G, sm.lnU[slot], pa, pb, ea,
-                          eb, deps, margin, negative);
-            if (dcs == 0) {
-              sm.px[ia] = pa[0]; sm.py[ia] = pa[1]; sm.pz[ia] = pa[2];
-              sm.px[ib] = pb[0]; sm.py[ib] = pb[1]; sm.pz[ib] = pb[2];
-              sm.e[ia] = ea + deps;
-              sm.e[ib] = eb + deps;
-              bad |= !isfinite(sm.e[ia]) || !isfinite(sm.e[ib]);
-            }
+      const int nx = __shfl_sync(0xffffffffu, sizes, r % kGroupLanes, kGroupLanes);
+      if (left == 0) left = r < nlev ? nx : 0;
+      n = min(left, kGroupLanes);
+      fetch();
+      if (act) {
+        const int ia = cpr & 255, ib = cpr >> 8;
+        const AV4 sa = lds4(&sm.s[ia]), sb = lds4(&sm.s[ib]);
+        R pa[3] = {sa.x, sa.y, sa.z};
+        R pb[3] = {sb.x, sb.y, sb.z};
+        const R G[3] = {cr.x, cr.y, cr.z};
+        double margin;
+        float m32 = 0.0f, tol = 0.0f;
+        int dcs;
+        if constexpr (A::mixed) {
+          const float eaf = sa.w, ebf = sb.w;
+          auto exact_e = [&](double& ea, double& eb) { fd_exact_energies(a.eps, sm, ia, ib, eaf, ebf, ea, eb); };
+          auto uniform = [&]() {
+            return fd_uniform_again(seed, sweep, a.id[block_gidx(sm.cells, ia)], a.id[block_gidx(sm.cells, ib)]);
+          };
+          float dh, dl;
+          dcs = fd_pair_mixed<false>(k, cg.x, cg.y, cg.z, cg.w, G, uniform, cr.w, pa, pb, eaf, ebf, exact_e, dh, dl, margin,
+                              m32, tol, REC, negative);
+          if (dcs == 0) {
+            float s, e;
+            eft::two_sum(eaf, dh, s, e);
+            sm.ec[ia] = __fadd_rn(sm.ec[ia], __fadd_rn(e, dl));
+            sm.s[ia] = F4{pa[0], pa[1], pa[2], s};
+            eft::two_sum(ebf, dh, s, e);
+            sm.ec[ib] = __fadd_rn(sm.ec[ib], __fadd_rn(e, dl));
+            sm.s[ib] = F4{pb[0], pb[1], pb[2], s};
           }
-          ++n_tot;
-          n_rb += dcs == 1;
-          n_rm += dcs == 2;
-          if (recs) {
-            const unsigned long long s = atomicAdd(rec_count, 1ull);
-            if ((int64_t)s < rec_cap) {
-              sdpd_pair_rec rc;
-              rc.id_i = a.id[gidx(ia)];
-              rc.id_j = a.id[gidx(ib)];
-              rc.colour = colour;
-              rc.owner = (int32_t)o;
-              rc.decision = dcs;
-              rc.level = L;
-              rc.margin = margin;
-              rc.margin_lo = A::mixed ? (double)m32 : margin;
-              rc.margin_tol = (double)tol;
-              recs[s] = rc;
-            }
+        } else {
+          double deps;
+          dcs = fd_pair(k, cg.x, cg.y, cg.z, cg.w, G, cr.w, pa, pb, sa.w, sb.w, deps, margin, negative);
+          if (dcs == 0) {
+            sm.s[ia] = D4{pa[0], pa[1], pa[2], sa.w + deps};
+            sm.s[ib] = D4{pb[0], pb[1], pb[2], sb.w + deps};
           }
         }
-        __syncwarp();
-        if (more) {
-          if ((int)off[L + 1] <= cend) {  // level L done
-            ++L;
-            more = L < nlev && (int)off[L] < cend;
-          } else {
-            more = false;  // level L continues in the next chunk
+        n_rb += dcs == 1;
+        n_rm += dcs == 2;
+        if constexpr (REC) {
+          const unsigned long long s = atomicAdd(rec_count, 1ull);
+          if ((int64_t)s < rec_cap) {
+            sdpd_pair_rec rc;
+            rc.id_i = a.id[block_gidx(sm.cells, ia)];
+            rc.id_j = a.id[block_gidx(sm.cells, ib)];
+            rc.colour = colour;
+            rc.owner = (int32_t)o;
+            rc.decision = dcs;
+            rc.level = level;
+            rc.margin = margin;
+            rc.margin_lo = A::mixed ? (double)m32 : margin;
+            rc.margin_tol = (double)tol;
+            recs[s] = rc;
           }
         }
       }
-      pos = cend;
       __syncwarp();
     }
     for (int q = gl; q < nb; q += kGroupLanes) {
-      const int g = gidx(q);
+      const int g = block_gidx(sm.cells, q);
+      const AV4 v = lds4(&sm.s[q]);
       if constexpr (kSame) {
-        a.px[g] = sm.px[q]; a.py[g] = sm.py[q]; a.pz[g] = sm.pz[q];
+        a.px[g] = v.x; a.py[g] = v.y; a.pz[g] = v.z;
       } else {  // the stored value plus this visit's increment
-        a.px[g] += (S)(sm.px[q] - (R)a.px[g]);
-        a.py[g] += (S)(sm.py[q] - (R)a.py[g]);
-        a.pz[g] += (S)(sm.pz[q] - (R)a.pz[g]);
+        a.px[g] += (S)(v.x - (R)a.px[g]);
+        a.py[g] += (S)(v.y - (R)a.py[g]);
+        a.pz[g] += (S)(v.z - (R)a.pz[g]);
       }
       double e;
       if constexpr (A::mixed) {  // once per visit: the load value plus the visit's exact change
         const double e0 = a.eps[g];
-        e = e0 + (((double)sm.es[q] - (double)(float)e0) + (double)sm.ec[q]);
+        e = e0 + (((double)v.w - (double)(float)e0) + (double)sm.ec[q]);
       }
-      else e = sm.e[q];
+      else e = v.w;
+      bad |= !isfinite(v.w);  // (a sum that was not finite once never is again)
       a.eps[g] = e;
       // pressure over rho^2 of the new energy, Eq. (pg-eos): pi = c_rho eps / (C_K m rho)
       // (from the stored float64 energy, as a restart recomputes it)
@@ -920,8 +1025,8 @@ __global__ void __launch_bounds__(W * 32, fd_min_blocks<A, W>())
     const int64_t ob = ent.x;
     int bx, by, bz;
     owner_coords(c, ob, bx, by, bz);
-    const BigCounts bc = fd_big_block<P, A, KIND>(c, k, a, qp4, cell_start, mrank, xmx, xmy, xmz, ob, bx, by, bz,
-                                                  colour, seed, sweep, recs, rec_count, rec_cap, big_perm + ent.y);
+    const BigCounts bc = fd_big_block<P, A>(c, k, a, qp4, cell_start, mrank, xmx, xmy, xmz, ob, bx, by, bz, colour,
+                                            seed, sweep, REC ? recs : nullptr, rec_count, rec_cap, big_perm + ent.y);
     unsigned long long bt = bc.tot, ba = bc.acc, bb = bc.rb, bm = bc.rm;  // (rare: counted at once)
     for (int s = 16; s > 0; s >>= 1) {
       bt += __shfl_xor_sync(0xffffffffu, bt, s);
@@ -939,19 +1044,19 @@ __global__ void __launch_bounds__(W * 32, fd_min_blocks<A, W>())
     bad |= bc.bad != 0;
   }
   if (lane == 0) {
-    const unsigned total = gridDim.x * (unsigned)W;
+    const unsigned total = gridDim.x * (blockDim.x >> 5);
     __threadfence();  // this warp's last take from queue[0] is performed before it counts as done
     if (atomicAdd(&queue[1], 1u) == total - 1u) {  // every warp has taken its last block
       queue[0] = 0u;
       queue[1] = 0u;
       queue[2] = 0u;
+      if (colour == 7) *sweep_ptr = sweep + 1ull;  // (every warp has read it) the sweep is done
     }
   }
   // counters
-  unsigned long long c_tot = n_tot, c_rb = n_rb, c_rm = n_rm, c_acc = n_tot - n_rb - n_rm;
+  unsigned long long c_tot = n_tot, c_rb = n_rb, c_rm = n_rm;
   for (int s = 16; s > 0; s >>= 1) {
     c_tot += __shfl_xor_sync(0xffffffffu, c_tot, s);
-    c_acc += __shfl_xor_sync(0xffffffffu, c_acc, s);
     c_rb += __shfl_xor_sync(0xffffffffu, c_rb, s);
     c_rm += __shfl_xor_sync(0xffffffffu, c_rm, s);
   }
@@ -959,7 +1064,7 @@ __global__ void __launch_bounds__(W * 32, fd_min_blocks<A, W>())
   if (lane == 0) {
     if (c_tot) {
       atomicAdd(&counters[0], c_tot);
-      atomicAdd(&counters[1], c_acc);
+      atomicAdd(&counters[1], c_tot - c_rb - c_rm);
       atomicAdd(&counters[2], c_rb);
       atomicAdd(&counters[3], c_rm);
     }
@@ -991,95 +1096,104 @@ static FDConst<R> fd_const(const Consts& c, double dt) {
   return k;
 }
 
+// Block schedules of the colour launches: blocks per warp and warps per
+// thread block of each variant (see sdpd_tuning).  The mapping onto the GPU
+// differs, the pair updates and their order per particle do not.
+constexpr int kFdOpw[kFdVariants] = {2, 2, 1, 1, 1};
+constexpr int kFdWarps[kFdVariants] = {2, 1, 1, 2, 4};
+
+// A block schedule fits when its groups' shared memory stays within 48 KB.
+template <class A>
+constexpr bool fd_fits(int v) { return sizeof(FdSmem<typename A::R>) * kFdOpw[v] * kFdWarps[v] <= 48 * 1024; }
+
 // Thread blocks of a colour kernel that the device holds at once (SMs x
 // blocks per SM, from the occupancy calculator; at least one), computed once
-// per kernel on the device current at the first launch.
-template <class P, class A, int KIND, int OPW, int W>
+// per kernel and warps per thread block on the device current at the first
+// launch.
+template <class P, class A, int OPW, bool REC, int W>
 int fd_resident_blocks() {
   static const int n = [] {
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fd_colour<P, A, KIND, OPW, W>, W * 32, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fd_colour<P, A, OPW, REC>, W * 32,
+                                                  sizeof(FdSmem<typename A::R>) * OPW * W);
     return std::max(1, sms) * std::max(1, per_sm);
   }();
   return n;
 }
-
-// A block schedule fits when its groups' shared memory stays within the 48 KB
-// a thread block may declare statically.
-template <class P, int OPW, int W>
-constexpr bool fd_fits() { return sizeof(FdSmem<typename P::R>) * OPW * W <= 48 * 1024; }
-
-constexpr int kFdOpw[kFdVariants] = {2, 2, 1, 1, 1};
-constexpr int kFdWarps[kFdVariants] = {2, 1, 1, 2, 4};
-
-// One colour launch with block-schedule variant (OPW, W); a schedule that
-// does not fit runs as variant 1.
-template <class P, class A, int KIND, int OPW, int W>
-void launch_colour(const Consts& c, const FDConst<typename A::R>& k, const Arrays<P>& a, const Workspace& w,
-                   int col, uint64_t seed, sdpd_pair_rec* recs, cudaStream_t s) {
-  if constexpr (!fd_fits<A, OPW, W>()) {
-    launch_colour<P, A, KIND, 2, 1>(c, k, a, w, col, seed, recs, s);
-  } else {
-    const int64_t nown = (int64_t)(c.nc[0] / 2) * (c.nc[1] / 2) * (c.nc[2] / 2);
-    const int64_t per_block = (int64_t)W * OPW;
-    const int64_t need = (nown + per_block - 1) / per_block;
-    const int64_t resident = (int64_t)fd_resident_blocks<P, A, KIND, OPW, W>();
-    const unsigned gf = (unsigned)std::max<int64_t>(1, std::min(need, resident));
-    k_fd_colour<P, A, KIND, OPW, W><<<gf, W * 32, 0, s>>>(
-        c, k, a, (typename P::V4*)w.qp4, (const typename P::V4*)w.qr4, w.cell_start, w.mrank, w.xmin[0], w.xmin[1], w.xmin[2], w.sched_hdr,
-        w.sched_lvl, w.sched_pair, col, seed, w.sweep, w.counters, w.status, recs, w.pair_rec_count,
-        w.pair_rec_cap, w.fd_queue + 3 * col, w.blk_order, w.big_perm, w.big_list, w.big_count);
+template <class P, class A, bool REC>
+int fd_resident(int variant) {
+  switch (variant) {
+    case 0: return fd_resident_blocks<P, A, 2, REC, 2>();
+    case 1: return fd_resident_blocks<P, A, 2, REC, 1>();
+    case 2: return fd_resident_blocks<P, A, 1, REC, 1>();
+    case 3: return fd_resident_blocks<P, A, 1, REC, 2>();
+    default: return fd_resident_blocks<P, A, 1, REC, 4>();
   }
 }
 
-// The eight colour launches of one sweep.  variant indexes the block
-// schedules (blocks per warp, warps per thread block):
-// 0 (2, 2), 1 (2, 1), 2 (1, 1), 3 (1, 2), 4 (1, 4).
-template <class P, class A, int KIND>
-void launch_colours_kind(const Consts& c, const Workspace& w, int cur, double dt, uint64_t seed, int record,
-                         int variant, cudaStream_t s) {
+// The eight colour launches of one sweep.
+template <class P, class A, bool REC>
+void launch_colours_rec(const Consts& c, const Workspace& w, int cur, double dt, uint64_t seed, int variant,
+                        cudaStream_t s) {
   const FDConst<typename A::R> k = fd_const<typename A::R>(c, dt);
   const Arrays<P> a = view<P>(w, cur);
-  sdpd_pair_rec* recs = record ? w.pair_recs : nullptr;
-  for (int col = 0; col < 8; ++col) {
-    switch (variant) {
-      case 0: launch_colour<P, A, KIND, 2, 2>(c, k, a, w, col, seed, recs, s); break;
-      case 1: launch_colour<P, A, KIND, 2, 1>(c, k, a, w, col, seed, recs, s); break;
-      case 2: launch_colour<P, A, KIND, 1, 1>(c, k, a, w, col, seed, recs, s); break;
-      case 3: launch_colour<P, A, KIND, 1, 2>(c, k, a, w, col, seed, recs, s); break;
-      default: launch_colour<P, A, KIND, 1, 4>(c, k, a, w, col, seed, recs, s); break;
-    }
-  }
+  const int64_t nown = (int64_t)(c.nc[0] / 2) * (c.nc[1] / 2) * (c.nc[2] / 2);
+  const int opw = kFdOpw[variant], W = kFdWarps[variant];
+  const int64_t need = (nown + W * opw - 1) / (W * opw);
+  const unsigned gf = (unsigned)std::max<int64_t>(1, std::min<int64_t>(need, fd_resident<P, A, REC>(variant)));
+  const size_t smem = sizeof(FdSmem<typename A::R>) * (size_t)(opw * W);
+  auto kern = opw == 2 ? k_fd_colour<P, A, 2, REC> : k_fd_colour<P, A, 1, REC>;
+  for (int col = 0; col < 8; ++col)
+    kern<<<gf, W * 32, smem, s>>>(c, k, a, (typename P::V4*)w.qp4, w.cell_start, w.mrank, w.xmin[0], w.xmin[1],
+                                  w.xmin[2], w.sched_hdr, w.sched_rsize, w.sched_off, w.sched_pair,
+                                  (const typename A::V4*)w.st_geom, (const typename A::V4*)w.st_rnd, col, seed,
+                                  w.sweep, w.counters, w.status, REC ? w.pair_recs : nullptr, w.pair_rec_count,
+                                  w.pair_rec_cap, w.fd_queue + 3 * col, w.blk_order, w.big_perm, w.big_list,
+                                  w.big_count);
 }
 
 // Fills the resident-block counts of every block schedule ahead of time (a
 // host query, kept out of stream captures).
 template <class P, class A>
 void fd_prepare() {
-  fd_resident_blocks<P, A, SDPD_KERNEL_LUCY, 2, 2>();
-  fd_resident_blocks<P, A, SDPD_KERNEL_LUCY, 2, 1>();
-  fd_resident_blocks<P, A, SDPD_KERNEL_LUCY, 1, 1>();
-  fd_resident_blocks<P, A, SDPD_KERNEL_LUCY, 1, 2>();
-  fd_resident_blocks<P, A, SDPD_KERNEL_LUCY, 1, 4>();
-  fd_resident_blocks<P, A, SDPD_KERNEL_CUBIC, 2, 2>();
-  fd_resident_blocks<P, A, SDPD_KERNEL_CUBIC, 2, 1>();
-  fd_resident_blocks<P, A, SDPD_KERNEL_CUBIC, 1, 1>();
-  fd_resident_blocks<P, A, SDPD_KERNEL_CUBIC, 1, 2>();
-  fd_resident_blocks<P, A, SDPD_KERNEL_CUBIC, 1, 4>();
+  for (int v = 0; v < kFdVariants; ++v)
+    if (fd_fits<A>(v)) {
+      fd_resident<P, A, false>(v);
+      fd_resident<P, A, true>(v);
+    }
 }
 
+static inline unsigned stage_blocks(const Consts& c) { return (unsigned)((c.ncell + kStageWarps - 1) / kStageWarps); }
+
+// The staged geometry of every scheduled pair (the last launch of a schedule).
+template <class P, class A>
+void launch_stage_geometry(const Consts& c, const Workspace& w, int cur, cudaStream_t s) {
+  if (c.N == 0) return;
+  (void)cur;
+  auto kern = c.kernel == SDPD_KERNEL_LUCY ? k_stage_geometry<P, A, SDPD_KERNEL_LUCY>
+                                           : k_stage_geometry<P, A, SDPD_KERNEL_CUBIC>;
+  kern<<<stage_blocks(c), kStageWarps * 32, 0, s>>>(c, (const typename P::V4*)w.qr4, w.cell_start, w.mrank, w.xmin[0],
+                                                   w.xmin[1], w.xmin[2], w.sched_hdr, w.sched_off, w.sched_pair,
+                                                   (typename A::V4*)w.st_geom);
+}
+
+// One sweep: the random numbers of every scheduled pair, then the colours;
+// the last colour launch advances the sweep counter.
 template <class P, class A>
 void launch_fd_colours(const Consts& c, const Workspace& w, int cur, double dt, uint64_t seed, int record,
                        cudaStream_t s) {
-  if (c.N == 0) return;
-  int variant = c.fd_variant;
-  if (variant < 0 || variant >= kFdVariants) variant = fd_default_variant(A::mixed);
-  if (c.kernel == SDPD_KERNEL_LUCY)
-    launch_colours_kind<P, A, SDPD_KERNEL_LUCY>(c, w, cur, dt, seed, record, variant, s);
-  else
-    launch_colours_kind<P, A, SDPD_KERNEL_CUBIC>(c, w, cur, dt, seed, record, variant, s);
+  if (c.N == 0) {
+    launch_advance_sweep(w, s);
+    return;
+  }
+  const int variant = fd_launch_variant(c, A::mixed);
+  k_stage_random<A><<<stage_blocks(c), kStageWarps * 32, 0, s>>>(c, w.id[cur], w.cell_start, w.mrank, w.sched_hdr,
+                                                                w.sched_off, w.sched_pair, seed, w.sweep,
+                                                                (typename A::V4*)w.st_rnd);
+  if (record) launch_colours_rec<P, A, true>(c, w, cur, dt, seed, variant, s);
+  else launch_colours_rec<P, A, false>(c, w, cur, dt, seed, variant, s);
 }
 
 }  // namespace sdpd

@@ -7,24 +7,18 @@ namespace sdpd {
 
 template void fd_prepare<Fp64, Fp64>();
 template void fd_prepare<Fp64, Mixed>();
+template void launch_stage_geometry<Fp64, Fp64>(const Consts&, const Workspace&, int, cudaStream_t);
+template void launch_stage_geometry<Fp64, Mixed>(const Consts&, const Workspace&, int, cudaStream_t);
 template void launch_fd_colours<Fp64, Fp64>(const Consts&, const Workspace&, int, double, uint64_t, int,
                                           cudaStream_t);
 // float64 state, float32 pair arithmetic
 template void launch_fd_colours<Fp64, Mixed>(const Consts&, const Workspace&, int, double, uint64_t, int,
                                            cudaStream_t);
 
-template <class P, int V>
-constexpr bool fits_v() { return fd_fits<P, kFdOpw[V], kFdWarps[V]>(); }
+int fd_round_width(int variant) { return 32 / kFdOpw[variant]; }
 
 bool fd_variant_fits(bool mixed, int v) {
-  switch (v) {
-    case 0: return mixed ? fits_v<Mixed, 0>() : fits_v<Fp64, 0>();
-    case 1: return mixed ? fits_v<Mixed, 1>() : fits_v<Fp64, 1>();
-    case 2: return mixed ? fits_v<Mixed, 2>() : fits_v<Fp64, 2>();
-    case 3: return mixed ? fits_v<Mixed, 3>() : fits_v<Fp64, 3>();
-    case 4: return mixed ? fits_v<Mixed, 4>() : fits_v<Fp64, 4>();
-    default: return false;
-  }
+  return v >= 0 && v < kFdVariants && (mixed ? fd_fits<Mixed>(v) : fd_fits<Fp64>(v));
 }
 
 }  // namespace sdpd

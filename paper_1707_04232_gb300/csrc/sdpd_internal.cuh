@@ -19,6 +19,13 @@ constexpr int kMaxLevels = 255;  // dependency levels of a block's pair schedule
 // in canonical order, one pair after the other, on the whole warp that takes
 // it (no shared-memory schedule), so any block size completes.
 constexpr uint32_t kHdrBig = 0xFFFFFFFFu;
+constexpr int kRoundStride = 256;  // bytes per block of the round sizes (>= kMaxLevels)
+// Entries of the dense pair arrays: the scheduled blocks own at most half the
+// neighbour-list entries (a member whose list overflowed leaves its block to
+// the pair-by-pair sweep), each block's run starting at a multiple of 8.
+inline size_t sched_pair_capacity(int64_t N, int nbr_cap, int64_t ncell) {
+  return (size_t)(N > 0 ? N : 1) * (size_t)(nbr_cap / 2) + 8 * (size_t)ncell + 32;
+}
 
 // Sticky device status bits, mapped to SDPD_ERR_* on the host.
 enum : int {
@@ -51,12 +58,24 @@ struct Consts {
   // launch shapes (results do not depend on them): the block schedule of the
   // sweep's colour launches and the threads per block of the pair passes
   int fd_variant, pair_threads;
+  bool fd_auto;  // no schedule chosen by the caller: fd_launch_variant picks by size
 };
 
 // Block schedules of the colour kernel (see launch_fd_colours) and the
 // thread-block sizes the pair passes accept.
 constexpr int kFdVariants = 5;
 __host__ __device__ constexpr int fd_default_variant(bool mixed) { return mixed ? 0 : 1; }
+// The block schedule of a handle's colour launches: the one set by the caller
+// or the autotuner, else by the blocks per colour.  Few blocks: a colour
+// lasts as long as its deepest block, which runs faster on a warp of its own
+// (variant 3; 32^3, 216 blocks per colour).  More blocks than resident warps:
+// two per warp use its lanes better (the defaults).
+constexpr int64_t kFdOwnWarpBlocks = 16 * 152;  // 16 warps on each of 152 SMs
+inline int fd_launch_variant(const Consts& c, bool mixed) {
+  if (!c.fd_auto && c.fd_variant >= 0 && c.fd_variant < kFdVariants) return c.fd_variant;
+  const int64_t nown = (int64_t)(c.nc[0] / 2) * (c.nc[1] / 2) * (c.nc[2] / 2);
+  return nown <= kFdOwnWarpBlocks ? 3 : fd_default_variant(mixed);
+}
 __host__ __device__ constexpr bool pair_threads_ok(int t) { return t == 32 || t == 64 || t == 128; }
 // whether a block schedule's shared memory fits a thread block (float64
 // blocks take twice the bytes of mixed ones)
@@ -318,10 +337,14 @@ struct Workspace {
   uint32_t* rcoord;     // Morton rank -> packed cell coordinates
   uint32_t* xmin[3];    // mixed: fixed-point lower edge of each cell, per axis
   // pair schedule of the fluctuation/dissipation sweep (per owner cell)
-  uint32_t* sched_hdr;    // npairs | nlevels << 16
-  uint16_t* sched_lvl;    // [ncell][kMaxLevels + 1] level offsets
-  uint16_t* sched_pair;   // [ncell][kMaxPairs] (local min-id | local max-id << 8)
-  uint8_t* level_of;      // [ncell][kMaxPairs] level of each pair in canonical order
+  uint32_t* sched_hdr;    // npairs | nrounds << 16
+  uint16_t* sched_canon;  // [ncell][kMaxPairs] owned pairs in canonical order (local min-id | local max-id << 8)
+  uint8_t* sched_rsize;   // [ncell][kRoundStride] pairs of each round
+  unsigned long long* sched_off;    // [ncell] where the block's pairs start in the arrays below
+  unsigned long long* sched_total;  // entries of those arrays in use
+  uint16_t* sched_pair;   // pairs round by round, block after block
+  void* st_geom;          // per scheduled pair: unit vector, F / (rho_i rho_j)
+  void* st_rnd;           // per scheduled pair: three normals and the uniform (EMS: its logarithm)
   // host <-> device staging in id order (float64)
   double* io_q;
   double* io_p;
@@ -386,10 +409,14 @@ void launch_density(const Consts& c, const Workspace& w, int cur, int update_eos
 template <class P>
 void launch_force(const Consts& c, const Workspace& w, int cur, double half_dt, double dt_drift,
                   double* force_by_id, cudaStream_t s);
+// the sweep schedule: P the state's storage policy, width the most pairs of a
+// round; the staged geometry (arithmetic policy A) completes it
 template <class P>
-void launch_fd_schedule(const Consts& c, const Workspace& w, int cur, cudaStream_t s);
-// the sweep's colour launches: P the state's storage policy, A the pair
-// arithmetic (A = Mixed on float64 state: float32 pair updates)
+void launch_fd_schedule(const Consts& c, const Workspace& w, int cur, int width, cudaStream_t s);
+template <class P, class A>
+void launch_stage_geometry(const Consts& c, const Workspace& w, int cur, cudaStream_t s);
+// one sweep (random numbers, then the colours): P the state's storage policy,
+// A the pair arithmetic (A = Mixed on float64 state: float32 pair updates)
 template <class P, class A = P>
 void fd_prepare();
 template <class P, class A = P>
@@ -397,6 +424,7 @@ void launch_fd_colours(const Consts& c, const Workspace& w, int cur, double dt, 
                        cudaStream_t s);
 template <class P>
 void launch_observables(const Consts& c, const Workspace& w, int cur, cudaStream_t s);
+int fd_round_width(int variant);  // lanes per block of a block schedule
 // sweep counter on the device: set to a value, or advanced by one
 void launch_set_sweep(const Workspace& w, unsigned long long value, cudaStream_t s);
 void launch_advance_sweep(const Workspace& w, cudaStream_t s);
