@@ -314,7 +314,7 @@ template <class P>
 void vv_step(sdpd_handle* s, double dt) {
   const Consts& c = s->c;
   {  // p^{n+1/2} = p^n + F^n dt/2, q^{n+1} = q^n + p^{n+1/2} dt/m
-    StageTimer t(s, 0, 2);
+    StageTimer t(s, 0, P::mixed ? 2 : 1);
     launch_force<P>(c, s->w, s->cur, 0.5 * dt, dt, nullptr, s->stream);
   }
   {
@@ -327,10 +327,10 @@ void vv_step(sdpd_handle* s, double dt) {
     launch_density<P>(c, s->w, s->cur, 1, nullptr, s->stream);
   }
   {  // p^{n+1} = p^{n+1/2} + F^{n+1} dt/2
-    StageTimer t(s, 3, 2);
+    StageTimer t(s, 3, P::mixed ? 2 : 1);
     launch_force<P>(c, s->w, s->cur, 0.5 * dt, 0.0, nullptr, s->stream);
   }
-  s->launches += 10;  // force + overflow, 5 sort, density, force + overflow
+  s->launches += P::mixed ? 10 : 8;  // force (mixed: + overflow), 5 sort, density, force (+ overflow)
   s->vv_step++;
   s->sched_valid = false;
 }
@@ -462,6 +462,7 @@ int sdpd_create(int64_t N, const double box[3], double m, double h, const sdpd_p
     c.L[d] = box[d];
     c.halfL[d] = 0.5 * box[d];
     c.cs[d] = box[d] / (double)n;
+    c.inv_cs[d] = 1.0 / c.cs[d];
     c.scale[d] = box[d] / 4294967296.0;
     c.inv_scale[d] = 4294967296.0 / box[d];
     ncell *= n;
@@ -498,6 +499,9 @@ int sdpd_create(int64_t N, const double box[3], double m, double h, const sdpd_p
     const double D = 8.0 * u * Lmax;
     const double rf = h + 3.0 * sqrt(3.0) * D;
     c.h2_filter = nextafterf((float)((1.0 + 8.0 * u) * rf * rf), INFINITY);
+    // by the same bounds r >= h implies r_f^2 >= (1 - 8u) (h - 3 sqrt(3) D)^2
+    const double ri = h - 3.0 * sqrt(3.0) * D;
+    c.h2_inner = ri > 0.0 ? nextafterf((float)((1.0 - 8.0 * u) * ri * ri), -INFINITY) : -1.0f;
     for (int d = 0; d < 3; ++d) {
       c.Lf[d] = (float)c.L[d];
       c.halfLf[d] = 0.5f * c.Lf[d];
@@ -506,7 +510,7 @@ int sdpd_create(int64_t N, const double box[3], double m, double h, const sdpd_p
   c.kernel = prm->kernel;
   c.fd_variant = fd_default_variant(prm->precision == SDPD_MIXED || prm->sweep_f32 != 0);
   c.pair_threads = 128;
-  c.fd_auto = true;
+  c.fd_auto = c.pair_auto = true;
   c.scheme = prm->scheme;
   s->prm = *prm;
   s->K = K;
@@ -824,6 +828,7 @@ int sdpd_set_tuning(sdpd_t* s, const sdpd_tuning* t) {
     return SDPD_ERR_INVALID_ARG;
   s->c.fd_variant = v;
   s->c.fd_auto = t->fd_variant < 0;
+  s->c.pair_auto = t->pair_threads == 0;
   s->c.pair_threads = pt;
   return SDPD_OK;
 }
@@ -848,7 +853,7 @@ int sdpd_autotune(sdpd_t* s, double dt, int64_t steps, uint64_t seed, sdpd_tunin
   // time per step of one candidate; infinity when it failed
   auto trial = [&](int v, int pt) -> double {
     s->c.fd_variant = v;
-    s->c.fd_auto = false;
+    s->c.fd_auto = s->c.pair_auto = false;
     s->c.pair_threads = pt;
     reload_handle(s, sv);
     if (mixed) do_steps<Mixed>(s, dt, 1, seed);
@@ -866,7 +871,7 @@ int sdpd_autotune(sdpd_t* s, double dt, int64_t steps, uint64_t seed, sdpd_tunin
     return (double)ms / (double)steps;
   };
   const int v0 = s->c.fd_variant, t0 = s->c.pair_threads;
-  const bool auto0 = s->c.fd_auto;
+  const bool fd_auto0 = s->c.fd_auto, pair_auto0 = s->c.pair_auto;
   int bv = v0, bt = 128;
   double bms = INFINITY;
   for (int v = 0; v < kFdVariants; ++v) {
@@ -882,7 +887,8 @@ int sdpd_autotune(sdpd_t* s, double dt, int64_t steps, uint64_t seed, sdpd_tunin
   cudaEventDestroy(ev[1]);
   if (!isfinite(bms)) { bv = v0; bt = t0; }
   s->c.fd_variant = bv;
-  s->c.fd_auto = !isfinite(bms) && auto0;
+  s->c.fd_auto = !isfinite(bms) && fd_auto0;
+  s->c.pair_auto = !isfinite(bms) && pair_auto0;
   s->c.pair_threads = bt;
   reload_handle(s, sv);  // back to the state and counters the call started from
   e = finish_restore(s, sv);
@@ -1287,7 +1293,7 @@ int debug_get(sdpd_handle* s, int what, void* dst, int64_t cap, int64_t* count) 
       if (cap < 3 * N) return SDPD_ERR_INVALID_ARG;
       if (mixed) launch_force<Mixed>(s->c, s->w, cur, 0.0, 0.0, s->w.io_p, st);
       else launch_force<Fp64>(s->c, s->w, cur, 0.0, 0.0, s->w.io_p, st);
-      s->launches += 2;
+      s->launches += mixed ? 2 : 1;
       if (N > 0 && cudaMemcpyAsync(dst, s->w.io_p, (size_t)N * 24, cudaMemcpyDeviceToHost, st) != cudaSuccess)
         return SDPD_ERR_CUDA;
       if (count) *count = 3 * N;
@@ -1476,7 +1482,7 @@ int sdpd_ensemble_step(sdpd_ens_t* e, double dt, int64_t nsteps, const uint64_t*
     // the graph holds the buffer pointers and launch shapes of its capture
     shape.push_back(h->cur);
     shape.push_back(h->c.fd_auto ? -1 : h->c.fd_variant);
-    shape.push_back(h->c.pair_threads);
+    shape.push_back(h->c.pair_auto ? -1 : h->c.pair_threads);
   }
   if (units > 0) {
     if (!e->exec || e->dt != dt || e->seeds != sv || e->phase != phase || e->shape != shape) {
@@ -1576,7 +1582,7 @@ int sdpd_ensemble_autotune(sdpd_ens_t* e, double dt, int64_t steps, const uint64
   for (size_t c = 0; c < cand.size() && !err; ++c) {
     for (size_t i = 0; i < n; ++i) {
       e->m[i]->c.fd_variant = cand[c][i].fd_variant;
-      e->m[i]->c.fd_auto = false;
+      e->m[i]->c.fd_auto = e->m[i]->c.pair_auto = false;
       e->m[i]->c.pair_threads = cand[c][i].pair_threads;
       reload_handle(e->m[i], sv[i]);
     }
@@ -1603,7 +1609,7 @@ int sdpd_ensemble_autotune(sdpd_ens_t* e, double dt, int64_t steps, const uint64
   // the chosen shapes, and every member back where the call found it
   for (size_t i = 0; i < n; ++i) {
     e->m[i]->c.fd_variant = cand[best][i].fd_variant;
-    e->m[i]->c.fd_auto = false;
+    e->m[i]->c.fd_auto = e->m[i]->c.pair_auto = false;
     e->m[i]->c.pair_threads = cand[best][i].pair_threads;
     reload_handle(e->m[i], sv[i]);
   }

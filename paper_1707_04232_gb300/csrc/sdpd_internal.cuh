@@ -41,7 +41,7 @@ struct Consts {
   int64_t N;
   int nc[3];
   int ncell;
-  double L[3], halfL[3], cs[3];
+  double L[3], halfL[3], cs[3], inv_cs[3];
   double scale[3];      // mixed precision: box side / 2^32 (fixed-point unit)
   double inv_scale[3];  // 2^32 / box side
   double h, h2, m, kB;
@@ -54,10 +54,13 @@ struct Consts {
   // whose float32 r^2 (from float32 copies of the positions) is >= h2_filter
   // has r^2 >= h^2 in float64 (bound on the conversion and rounding errors
   // set on the host), so it is skipped without float64 arithmetic.
-  float Lf[3], halfLf[3], h2_filter;
+  // Below h2_inner it has r^2 < h^2 for certain; only in between does the
+  // float64 predicate decide.
+  float Lf[3], halfLf[3], h2_filter, h2_inner;
   // launch shapes (results do not depend on them): the block schedule of the
   // sweep's colour launches and the threads per block of the pair passes
   int fd_variant, pair_threads;
+  bool pair_auto;  // no pair-pass block size chosen by the caller: by size (float64 path)
   bool fd_auto;  // no schedule chosen by the caller: fd_launch_variant picks by size
 };
 
@@ -127,6 +130,18 @@ __device__ __forceinline__ double pair_rinv(double r2) {
   return y * (1.5 - 0.5 * r2 * y * y);
 }
 __device__ __forceinline__ double pair_r(double r2) { return r2 > 1e-30 ? r2 * pair_rinv(r2) : sqrt(r2); }
+// The same with two float64 operations instead of four: the float32 root H,
+// then H + (r^2 - H^2) / (2 H) with the residual from one float64 FMA and the
+// small correction formed in float32 (Heron's step; relative error ~1e-14:
+// half the square of H's error and the rounding of the correction).
+__device__ __forceinline__ double pair_r64(double r2) {
+  const float f = (float)r2;
+  if (!(f > 1e-30f)) return sqrt(r2);
+  const float y = rsqrtf(f);
+  const double H = (double)(f * y);
+  const float d = (float)__fma_rn(-H, H, r2);
+  return H + (double)(0.5f * y * d);
+}
 __device__ __forceinline__ float pair_r(float r2) { return r2 > 0.0f ? r2 * rsqrtf(r2) : 0.0f; }
 
 // ---------------------------------------------------------------------------

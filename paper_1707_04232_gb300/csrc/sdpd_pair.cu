@@ -3,65 +3,21 @@
 // conservative force of Eq. (cons-forces) with the half kick (and, for the
 // first kick of a step, the drift and the cell binning of the new position).
 //
-// One thread per particle in storage order; the neighbour search walks the
-// 27 cells around the particle's cell (cell side >= h) with the predicate
-// r^2 < h^2 after the periodic minimum image.
+// The neighbour search walks the 27 cells around the particle's cell (cell
+// side >= h) with the predicate r^2 < h^2 after the periodic minimum image.
+// Mixed path: one thread per particle in storage order (k_density, k_force).
+// Float64 path: a group of kLanes64 lanes per particle (k_density64,
+// k_force64).
 #include "sdpd_internal.cuh"
 
 namespace sdpd {
 
 // Geometry of one home particle: displacement to a neighbour j.
-// Float64: absolute coordinates and the minimum image.
-// Mixed: coordinates relative to the own cell's lower corner; per axis and
+// Float64: Home64 below.  Mixed: coordinates relative to the own cell's lower corner; per axis and
 // neighbour offset o in {-1, 0, +1} the home coordinate shifted by the
 // (exact, fixed-point) distance between the two cells' corners.
 template <class P>
 struct Home;
-
-template <>
-struct Home<Fp64> {
-  double x, y, z;
-  int cx, cy, cz;
-  double mx, my, mz, px_, py_, pz_;  // image shifts of the neighbour offsets -1 and +1 per axis
-  double fx, fy, fz;                 // shifts of the current neighbour cell
-  __device__ void init(const Consts& c, const D4& q, int cx_, int cy_, int cz_, const uint32_t*, const uint32_t*,
-                       const uint32_t*) {
-    x = q.x; y = q.y; z = q.z;
-    cx = cx_; cy = cy_; cz = cz_;
-    mx = image_shift(cx, -1, c.nc[0], c.L[0]); px_ = image_shift(cx, 1, c.nc[0], c.L[0]);
-    my = image_shift(cy, -1, c.nc[1], c.L[1]); py_ = image_shift(cy, 1, c.nc[1], c.L[1]);
-    mz = image_shift(cz, -1, c.nc[2], c.L[2]); pz_ = image_shift(cz, 1, c.nc[2], c.L[2]);
-    fx = fy = fz = 0.0;
-  }
-  // neighbour cell (nx, ny, nz) = (cx + ox, ...) wrapped: its image shifts
-  __device__ __forceinline__ void frame(int nx, int ny, int nz) {
-    fx = nx - cx > 1 ? mx : (nx - cx < -1 ? px_ : 0.0);
-    fy = ny - cy > 1 ? my : (ny - cy < -1 ? py_ : 0.0);
-    fz = nz - cz > 1 ? mz : (nz - cz < -1 ? pz_ : 0.0);
-  }
-  __device__ __forceinline__ void frames_all(const Consts&) {}
-  __device__ __forceinline__ static double pick(uint32_t k, double m, double p) {
-    return k == 0 ? m : (k == 2 ? p : 0.0);
-  }
-  __device__ __forceinline__ void disp_code(uint32_t code, const D4& qj, double& dx, double& dy, double& dz) const {
-    const double sx = pick(code & 3u, mx, px_), sy = pick((code >> 2) & 3u, my, py_),
-                 sz = pick((code >> 4) & 3u, mz, pz_);
-    dx = __dsub_rn(x, qj.x);
-    dy = __dsub_rn(y, qj.y);
-    dz = __dsub_rn(z, qj.z);
-    if (sx != 0.0) dx = __dadd_rn(dx, sx);
-    if (sy != 0.0) dy = __dadd_rn(dy, sy);
-    if (sz != 0.0) dz = __dadd_rn(dz, sz);
-  }
-  __device__ __forceinline__ void disp(const D4& qj, double& dx, double& dy, double& dz) const {
-    dx = __dsub_rn(x, qj.x);
-    dy = __dsub_rn(y, qj.y);
-    dz = __dsub_rn(z, qj.z);
-    if (fx != 0.0) dx = __dadd_rn(dx, fx);
-    if (fy != 0.0) dy = __dadd_rn(dy, fy);
-    if (fz != 0.0) dz = __dadd_rn(dz, fz);
-  }
-};
 
 template <>
 struct Home<Mixed> {
@@ -120,7 +76,7 @@ __device__ __forceinline__ int wrapc(int v, int n) { return v < 0 ? v + n : (v >
 // P = c_rho rho eps / (C_K m).
 // ---------------------------------------------------------------------------
 template <class P, int KIND>
-__global__ void __launch_bounds__(128, P::mixed ? 12 : 1) k_density(Consts c, Arrays<P> a, typename P::V4* __restrict__ qp4,
+__global__ void __launch_bounds__(128, 12) k_density(Consts c, Arrays<P> a, typename P::V4* __restrict__ qp4,
                                                  const int32_t* __restrict__ cell_start,
                                                  const int32_t* __restrict__ mrank,
                                                  const uint32_t* __restrict__ xmx,
@@ -129,16 +85,15 @@ __global__ void __launch_bounds__(128, P::mixed ? 12 : 1) k_density(Consts c, Ar
                                                  int32_t* __restrict__ ncount_by_id,
                                                  uint32_t* __restrict__ nlist, int32_t* __restrict__ nn,
                                                  int32_t* __restrict__ ovf_list, int32_t* __restrict__ ovf_count,
-                                                 int32_t* __restrict__ ovf_other, const float4* __restrict__ qf4,
+                                                 int32_t* __restrict__ ovf_other,
                                                  typename P::V4* __restrict__ qr4, uint32_t* __restrict__ cend) {
+  static_assert(P::mixed, "the float64 path runs k_density64");
   using R = typename P::R;
   using V4 = typename P::V4;
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i == 0) *ovf_other = 0;  // the other slot: its readers have run
   if (i >= c.N) return;
   const V4 qi = ld4(&a.q4[i]);
-  float4 fi = make_float4(0.f, 0.f, 0.f, 0.f);
-  if constexpr (!P::mixed) fi = qf4[i];
   int cx, cy, cz;
   unpack_cell(w_to_cellbits(qi.w), cx, cy, cz);
   Home<P> home;
@@ -169,15 +124,6 @@ __global__ void __launch_bounds__(128, P::mixed ? 12 : 1) k_density(Consts c, Ar
         const uint32_t code = nbr_entry(0, ox, oy, oz);
 #pragma unroll 4
         for (int j = beg; j < end; ++j) {
-          if constexpr (!P::mixed) {  // float32 pre-test: skips only pairs with r >= h
-            if (j == i) continue;
-            const float4 fj = __ldg(&qf4[j]);
-            float ex = fi.x - fj.x, ey = fi.y - fj.y, ez = fi.z - fj.z;
-            ex = ex > c.halfLf[0] ? ex - c.Lf[0] : (ex < -c.halfLf[0] ? ex + c.Lf[0] : ex);
-            ey = ey > c.halfLf[1] ? ey - c.Lf[1] : (ey < -c.halfLf[1] ? ey + c.Lf[1] : ey);
-            ez = ez > c.halfLf[2] ? ez - c.Lf[2] : (ez < -c.halfLf[2] ? ez + c.Lf[2] : ez);
-            if (ex * ex + ey * ey + ez * ez >= c.h2_filter) continue;
-          }
           const V4 qj = ld4(&a.q4[j]);
           R dx, dy, dz;
           home.disp(qj, dx, dy, dz);
@@ -202,27 +148,232 @@ __global__ void __launch_bounds__(128, P::mixed ? 12 : 1) k_density(Consts c, Ar
   const R rho_new = (R)c.m * ((R)c.W0 + acc);
   double e = a.eps[i];
   if (update_eos) {
-    if constexpr (P::mixed) {
-      // eps * (rho_new / rho_old)^(c_rho / C_K), the factor minus one formed
-      // from log1p / expm1 of small arguments so float32 keeps it accurate
-      const float ro = a.rho[i];
-      const float g = expm1f((float)(c.c_rho / c.C_K) * log1pf((rho_new - ro) / ro));
-      e = fma(e, (double)g, e);
-    } else {
-      const double S = c.C_K * log(e) - c.c_rho * log((double)a.rho[i]);
-      e = exp((S + c.c_rho * log((double)rho_new)) / c.C_K);
-    }
+    // eps * (rho_new / rho_old)^(c_rho / C_K), the factor minus one formed
+    // from log1p / expm1 of small arguments so float32 keeps it accurate
+    const float ro = a.rho[i];
+    const float g = expm1f((float)(c.c_rho / c.C_K) * log1pf((rho_new - ro) / ro));
+    e = fma(e, (double)g, e);
     a.eps[i] = e;
   }
   a.rho[i] = rho_new;
-  R pi;
-  if constexpr (P::mixed) pi = (float)e * (float)(c.c_rho / (c.C_K * c.m)) / rho_new;
-  else pi = e * (c.c_rho / (c.C_K * c.m)) / rho_new;
+  const R pi = (float)e * (float)(c.c_rho / (c.C_K * c.m)) / rho_new;
   V4 o = qi;
   o.w = pi;
   st4(&qp4[i], o);
   o.w = rho_new;  // positions and density together for the sweep's pair geometry
   st4(&qr4[i], o);
+}
+
+// ---------------------------------------------------------------------------
+// Float64 pair passes.  GB300 issues one float64 instruction per 64 cycles on
+// each quarter of an SM whether 1 or 32 lanes are active, so a pass costs its
+// float64 instructions per warp.  With one thread per particle the kept
+// neighbour's branch ran on nearly every candidate of the 27 cells (one lane
+// in six keeps one): ~500 evaluations instead of ~80.  Here kLanes64 lanes
+// share a particle (a whole warp where particles are few).  The search is float32: r^2 from the float32 positions
+// decides a candidate unless it lies within its rounding bound of h^2 (then
+// the float64 predicate does), and the kept ones are appended in walk order
+// (ballot and prefix count) to a list in shared memory.  Only list entries
+// see float64 arithmetic, with all lanes at work.
+// ---------------------------------------------------------------------------
+constexpr int kLanes64 = 8;
+
+// Distance pieces of a float64 list entry: displacement with the periodic
+// image of its stencil code (edge: the home cell touches the box side on some
+// axis, else every image shift is zero; adding a zero shift changes nothing).
+struct Home64 {
+  double x, y, z;
+  double mx, my, mz, px_, py_, pz_;
+  bool edge;
+  __device__ __forceinline__ void init(const Consts& c, const D4& q, int cx, int cy, int cz) {
+    x = q.x; y = q.y; z = q.z;
+    mx = image_shift(cx, -1, c.nc[0], c.L[0]); px_ = image_shift(cx, 1, c.nc[0], c.L[0]);
+    my = image_shift(cy, -1, c.nc[1], c.L[1]); py_ = image_shift(cy, 1, c.nc[1], c.L[1]);
+    mz = image_shift(cz, -1, c.nc[2], c.L[2]); pz_ = image_shift(cz, 1, c.nc[2], c.L[2]);
+    edge = cx == 0 || cy == 0 || cz == 0 || cx == c.nc[0] - 1 || cy == c.nc[1] - 1 || cz == c.nc[2] - 1;
+  }
+  __device__ __forceinline__ static double pick(uint32_t k, double m, double p) {
+    return k == 0 ? m : (k == 2 ? p : 0.0);
+  }
+  __device__ __forceinline__ double r2(uint32_t code, const D4& qj, double& dx, double& dy, double& dz) const {
+    dx = __dsub_rn(x, qj.x);
+    dy = __dsub_rn(y, qj.y);
+    dz = __dsub_rn(z, qj.z);
+    if (edge) {
+      dx = __dadd_rn(dx, pick(code & 3u, mx, px_));
+      dy = __dadd_rn(dy, pick((code >> 2) & 3u, my, py_));
+      dz = __dadd_rn(dz, pick((code >> 4) & 3u, mz, pz_));
+    }
+    return r2_of(dx, dy, dz);
+  }
+};
+
+// The walk of a warp's particles (one per group of T lanes) over their 27
+// cells: calls keep(slot, j, code) on the lanes of kept candidates, slot
+// counting them in walk order, and row(row, word) with the list positions of
+// each row of three cells; returns the number kept.  The candidates of a
+// row's three cells are taken as one run, kBatch x T at a time, so that their
+// loads are in flight together.  The whole warp takes part (the groups'
+// particles mostly share their cell, so their loops have the same length);
+// a group with live = false meets no candidates.
+template <int T, class Row, class Keep>
+__device__ __forceinline__ int walk64(const Consts& c, bool live, const Home64& home, const float4& fi, int64_t i,
+                                      int cx, int cy, int cz, const D4* __restrict__ q4,
+                                      const float4* __restrict__ qf4, const int32_t* __restrict__ cell_start,
+                                      const int32_t* __restrict__ mrank, Row row, Keep keep) {
+  constexpr int kBatch = T == 32 ? 2 : 3;
+  constexpr unsigned kFull = T == 32 ? 0xffffffffu : (1u << (T & 31)) - 1u;
+  const int gl = threadIdx.x % T, shift = (threadIdx.x & 31) - gl;
+  const unsigned below = (1u << gl) - 1u;
+  auto first = [](int n) { return n <= 0 ? 0u : (n >= 32 ? 0xffffffffu : (1u << n) - 1u); };  // the lowest n bits
+  int cnt = 0;
+#pragma unroll 1
+  for (int oz = -1; oz <= 1; ++oz) {
+    const int nz = wrapc(cz + oz, c.nc[2]);
+#pragma unroll 1
+    for (int oy = -1; oy <= 1; ++oy) {
+      const int ny = wrapc(cy + oy, c.nc[1]);
+      int beg[3], off[4] = {0, 0, 0, 0};
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const int r = __ldg(&mrank[wrapc(cx + k - 1, c.nc[0]) + c.nc[0] * (ny + c.nc[1] * nz)]);
+        beg[k] = __ldg(&cell_start[r]);
+        off[k + 1] = __ldg(&cell_start[r + 1]) - beg[k];
+      }
+#pragma unroll
+      for (int k = 0; k < 3; ++k) off[k + 1] = live ? off[k + 1] + off[k] : 0;
+      const int start = cnt;
+      int c0 = 0, c1 = 0;  // kept in the first cell, in the first two
+      for (int b = 0; __any_sync(0xffffffffu, b < off[3]); b += kBatch * T) {
+        float4 fj[kBatch];
+        int js[kBatch];
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+          const int t = b + u * T + gl;
+          js[u] = t < off[1] ? beg[0] + t : (t < off[2] ? beg[1] + t - off[1] : beg[2] + t - off[2]);
+          if (t < off[3]) fj[u] = __ldg(&qf4[js[u]]);
+        }
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+          const int t0 = b + u * T, t = t0 + gl;
+          const uint32_t code = nbr_entry(0, (t >= off[1]) + (t >= off[2]) - 1, oy, oz);
+          bool in = false;
+          if (t < off[3] && js[u] != i) {
+            float ex = fi.x - fj[u].x, ey = fi.y - fj[u].y, ez = fi.z - fj[u].z;
+            ex = ex > c.halfLf[0] ? ex - c.Lf[0] : (ex < -c.halfLf[0] ? ex + c.Lf[0] : ex);
+            ey = ey > c.halfLf[1] ? ey - c.Lf[1] : (ey < -c.halfLf[1] ? ey + c.Lf[1] : ey);
+            ez = ez > c.halfLf[2] ? ez - c.Lf[2] : (ez < -c.halfLf[2] ? ez + c.Lf[2] : ez);
+            const float rf = ex * ex + ey * ey + ez * ez;
+            in = rf < c.h2_inner;
+            if (!in && rf < c.h2_filter) {  // within the rounding bound of h^2: float64 decides
+              double dx, dy, dz;
+              in = home.r2(code, ld4(&q4[js[u]]), dx, dy, dz) < c.h2;
+            }
+          }
+          const unsigned m = (__ballot_sync(0xffffffffu, in) >> shift) & kFull;
+          if (in) keep(cnt + __popc(m & below), js[u], code);
+          cnt += __popc(m);
+          c0 += __popc(m & first(off[1] - t0));
+          c1 += __popc(m & first(off[2] - t0));
+        }
+      }
+      row((oz + 1) * 3 + (oy + 1),
+          (uint32_t)min(start, 255) | (uint32_t)min(start + c0, 255) << 8 | (uint32_t)min(start + c1, 255) << 16 |
+              (uint32_t)min(cnt, 255) << 24);
+    }
+  }
+  return cnt;
+}
+
+// Sum of v over the lanes of a group, the same order for every group.
+template <int T>
+__device__ __forceinline__ double group_sum(double v) {
+#pragma unroll
+  for (int s = T / 2; s > 0; s >>= 1) v += __shfl_xor_sync(0xffffffffu, v, s);
+  return v;
+}
+
+// Density, equation of state and neighbour lists of PPB particles per thread
+// block (see k_density).  The list in shared memory has the layout of the
+// global one, so it is copied out in 16-byte pieces.  A particle with more
+// neighbours than a row holds sums the kernel over the cells again.  The
+// equation of state runs one particle per lane on the first warp.
+template <int KIND, int T, int PPB>
+__global__ void __launch_bounds__(PPB * T)
+    k_density64(Consts c, Arrays<Fp64> a, D4* __restrict__ qp4, const int32_t* __restrict__ cell_start,
+                const int32_t* __restrict__ mrank, int update_eos, int32_t* __restrict__ ncount_by_id,
+                uint32_t* __restrict__ nlist, int32_t* __restrict__ nn, int32_t* __restrict__ ovf_list,
+                int32_t* __restrict__ ovf_count, int32_t* __restrict__ ovf_other, const float4* __restrict__ qf4,
+                D4* __restrict__ qr4, uint32_t* __restrict__ cend) {
+  extern __shared__ uint32_t list_s[];  // [cap / 4][PPB][4]
+  __shared__ double acc_s[PPB];
+  __shared__ int cnt_s[PPB];
+  const int p = threadIdx.x / T, gl = threadIdx.x % T;
+  const int64_t i0 = blockIdx.x * (int64_t)PPB, i = i0 + p;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *ovf_other = 0;  // the other slot: its readers have run
+  const bool live = i < c.N;
+  const D4 qi = ld4(&a.q4[live ? i : 0]);
+  const float4 fi = qf4[live ? i : 0];
+  int cx, cy, cz;
+  unpack_cell(w_to_cellbits(qi.w), cx, cy, cz);
+  Home64 home;
+  home.init(c, qi, cx, cy, cz);
+  const int cnt = walk64<T>(
+      c, live, home, fi, i, cx, cy, cz, a.q4, qf4, cell_start, mrank,
+      [&](int r, uint32_t rw) { if (live && gl == 0) cend[(int64_t)r * c.N + i] = rw; },
+      [&](int k, int j, uint32_t code) {
+        if (k < c.nbr_cap) list_s[((k >> 2) * PPB + p) * 4 + (k & 3)] = ((uint32_t)j << 6) | code;
+      });
+  __syncwarp();
+  const double inv_h = 1.0 / c.h;
+  double acc = 0.0;
+  const bool over = cnt > c.nbr_cap;
+  for (int k = gl; k < (over ? 0 : cnt); k += T) {
+    const uint32_t e = list_s[((k >> 2) * PPB + p) * 4 + (k & 3)];
+    double dx, dy, dz;
+    const double r2 = home.r2(e & 63u, ld4(&a.q4[e >> 6]), dx, dy, dz);
+    acc += kernel_W<KIND>(pair_r64(r2) * inv_h, c.cW);
+  }
+  if (__any_sync(0xffffffffu, over))
+    walk64<T>(c, over, home, fi, i, cx, cy, cz, a.q4, qf4, cell_start, mrank, [](int, uint32_t) {},
+              [&](int, int j, uint32_t code) {
+                double dx, dy, dz;
+                acc += kernel_W<KIND>(pair_r64(home.r2(code, ld4(&a.q4[j]), dx, dy, dz)) * inv_h, c.cW);
+              });
+  acc = group_sum<T>(acc);
+  if (gl == 0) {
+    acc_s[p] = acc;
+    cnt_s[p] = cnt;
+  }
+  __syncthreads();
+  // the lists, row by row of four entries
+  const int kmax = c.nbr_cap >> 2;
+  for (int t = threadIdx.x; t < kmax * PPB; t += PPB * T) {
+    const int k4 = t / PPB, q = t % PPB;
+    if (4 * k4 < cnt_s[q])
+      *reinterpret_cast<uint4*>(nlist + nbr_slot(i0 + q, 4 * k4, c.nbr_cap)) = reinterpret_cast<const uint4*>(list_s)[t];
+  }
+  if (threadIdx.x < PPB && i0 + threadIdx.x < c.N) {
+    const int64_t g = i0 + threadIdx.x;
+    const int cnt = cnt_s[threadIdx.x];
+    if (ncount_by_id) ncount_by_id[a.id[g]] = cnt;
+    nn[g] = cnt;
+    if (cnt > c.nbr_cap) ovf_list[atomicAdd(ovf_count, 1)] = (int32_t)g;  // forces from the cells
+    const double rho_new = c.m * (c.W0 + acc_s[threadIdx.x]);
+    double e = a.eps[g];
+    if (update_eos) {
+      // eps' = E(S(eps, rho), rho') = eps (rho' / rho)^(c_rho / C_K)
+      const double ro = a.rho[g];
+      e *= exp(c.c_rho / c.C_K * log1p((rho_new - ro) / ro));
+      a.eps[g] = e;
+    }
+    a.rho[g] = rho_new;
+    D4 o = ld4(&a.q4[g]);
+    o.w = e * (c.c_rho / (c.C_K * c.m)) / rho_new;
+    st4(&qp4[g], o);
+    o.w = rho_new;  // positions and density together for the sweep's pair geometry
+    st4(&qr4[g], o);
+  }
 }
 
 // Kick (and, with dt_drift != 0, drift and binning) of particle i with the
@@ -250,28 +401,14 @@ __device__ __forceinline__ void kick_particle(const Consts& c, const Arrays<P>& 
   a.px[i] = px; a.py[i] = py; a.pz[i] = pz;
   if (dt_drift != 0.0) {
     int nc3[3];
-    if constexpr (P::mixed) {
-      // fixed point: the displacement in units of L / 2^32, wrap-around = periodic
-      uint32_t ux = a.qx[i] + (uint32_t)__float2int_rn(px * drift_f[0]);
-      uint32_t uy = a.qy[i] + (uint32_t)__float2int_rn(py * drift_f[1]);
-      uint32_t uz = a.qz[i] + (uint32_t)__float2int_rn(pz * drift_f[2]);
-      qdx[i] = ux; qdy[i] = uy; qdz[i] = uz;
-      nc3[0] = (int)__umulhi(ux, (uint32_t)c.nc[0]);
-      nc3[1] = (int)__umulhi(uy, (uint32_t)c.nc[1]);
-      nc3[2] = (int)__umulhi(uz, (uint32_t)c.nc[2]);
-    } else {
-      double pp[3] = {px, py, pz}, qq[3] = {a.qx[i], a.qy[i], a.qz[i]};
-      for (int d = 0; d < 3; ++d) {
-        double x = __dadd_rn(qq[d], __ddiv_rn(__dmul_rn(pp[d], dt_drift), c.m));
-        if (x >= c.L[d]) x = __dsub_rn(x, c.L[d]);
-        else if (x < 0.0) x = __dadd_rn(x, c.L[d]);
-        if (x >= c.L[d]) x = 0.0;
-        qq[d] = x;
-        int cc = (int)floor(__ddiv_rn(x, c.cs[d]));
-        nc3[d] = cc >= c.nc[d] ? c.nc[d] - 1 : (cc < 0 ? 0 : cc);
-      }
-      qdx[i] = qq[0]; qdy[i] = qq[1]; qdz[i] = qq[2];
-    }
+    // fixed point: the displacement in units of L / 2^32, wrap-around = periodic
+    uint32_t ux = a.qx[i] + (uint32_t)__float2int_rn(px * drift_f[0]);
+    uint32_t uy = a.qy[i] + (uint32_t)__float2int_rn(py * drift_f[1]);
+    uint32_t uz = a.qz[i] + (uint32_t)__float2int_rn(pz * drift_f[2]);
+    qdx[i] = ux; qdy[i] = uy; qdz[i] = uz;
+    nc3[0] = (int)__umulhi(ux, (uint32_t)c.nc[0]);
+    nc3[1] = (int)__umulhi(uy, (uint32_t)c.nc[1]);
+    nc3[2] = (int)__umulhi(uz, (uint32_t)c.nc[2]);
     const int r = mrank[nc3[0] + c.nc[0] * (nc3[1] + c.nc[1] * nc3[2])];
     key[i] = r;
     slot[i] = atomicAdd(&cell_count[r], 1);
@@ -338,7 +475,7 @@ __device__ __forceinline__ void force_from_cells(const Consts& c, const Arrays<P
 // by the density pass) is left to k_force_overflow.
 // ---------------------------------------------------------------------------
 template <class P, int KIND>
-__global__ void __launch_bounds__(128, P::mixed ? (KIND == SDPD_KERNEL_LUCY ? 16 : 12) : 1) k_force(Consts c, Arrays<P> a, const typename P::V4* __restrict__ qp4,
+__global__ void __launch_bounds__(128, KIND == SDPD_KERNEL_LUCY ? 16 : 12) k_force(Consts c, Arrays<P> a, const typename P::V4* __restrict__ qp4,
                                                const int32_t* __restrict__ cell_start,
                                                const int32_t* __restrict__ mrank,
                                                const uint32_t* __restrict__ xmx,
@@ -392,6 +529,83 @@ __global__ void __launch_bounds__(128, P::mixed ? (KIND == SDPD_KERNEL_LUCY ? 16
   }
 }
 
+// Force and kick of the float64 path: T lanes per particle over its list (see
+// k_force and the note at kLanes64), or over the cells when the list
+// overflowed its row; the kick, drift and binning one axis per lane.
+template <int KIND, int T>
+__global__ void __launch_bounds__(128)
+    k_force64(Consts c, Arrays<Fp64> a, const D4* __restrict__ qp4, const float4* __restrict__ qf4,
+              const int32_t* __restrict__ cell_start, const int32_t* __restrict__ mrank, double half_dt,
+              double dt_drift, double* __restrict__ qdx, double* __restrict__ qdy, double* __restrict__ qdz,
+              int32_t* __restrict__ key, int32_t* __restrict__ slot, int32_t* __restrict__ cell_count,
+              double* __restrict__ force_by_id, const uint32_t* __restrict__ nlist, const int32_t* __restrict__ nn) {
+  const int gl = threadIdx.x % T;
+  int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / T;
+  const bool mine = i < c.N;
+  if (!mine) i = 0;  // (the whole warp stays for the sums)
+  const int n = mine ? nn[i] : 0;
+  const bool over = n > c.nbr_cap;
+  const D4 qi = ld4(&qp4[i]);
+  int cx, cy, cz;
+  unpack_cell(w_to_cellbits(a.q4[i].w), cx, cy, cz);
+  Home64 home;
+  home.init(c, qi, cx, cy, cz);
+  const double inv_h = 1.0 / c.h;
+  double f[3] = {0.0, 0.0, 0.0};
+  auto add = [&](uint32_t code, const D4& qj) {
+    double dx, dy, dz;
+    const double r2 = home.r2(code, qj, dx, dy, dz);
+    const double s = (qi.w + qj.w) * kernel_F<KIND>(pair_r64(r2) * inv_h, 1.0);
+    f[0] += s * dx;
+    f[1] += s * dy;
+    f[2] += s * dz;
+  };
+#pragma unroll 2
+  for (int k = gl; k < (over ? 0 : n); k += T) {
+    const uint32_t e = __ldg(&nlist[nbr_slot(i, k, c.nbr_cap)]);
+    add(e & 63u, ld4(&qp4[e >> 6]));
+  }
+  if (__any_sync(0xffffffffu, over))
+    walk64<T>(c, over, home, qf4[i], i, cx, cy, cz, qp4, qf4, cell_start, mrank, [](int, uint32_t) {},
+              [&](int, int j, uint32_t code) { add(code, ld4(&qp4[j])); });
+#pragma unroll
+  for (int d = 0; d < 3; ++d) f[d] = group_sum<T>(f[d]);
+  // axis gl of the kick and drift (see kick_particle)
+  int cc = 0;
+  if (mine && gl < 3) {
+    const double fd = (gl == 0 ? f[0] : (gl == 1 ? f[1] : f[2])) * (c.m * c.m * c.cF);
+    if (force_by_id) force_by_id[3 * (int64_t)a.id[i] + gl] = fd;
+    double* pp = gl == 0 ? a.px : (gl == 1 ? a.py : a.pz);
+    const double pn = pp[i] + fd * half_dt;
+    pp[i] = pn;
+    if (dt_drift != 0.0) {
+      const double* qq = gl == 0 ? a.qx : (gl == 1 ? a.qy : a.qz);
+      const double L = c.L[gl];
+      const double step = __dmul_rn(pn, dt_drift);
+      double x = __dadd_rn(qq[i], c.m == 1.0 ? step : __ddiv_rn(step, c.m));
+      if (x >= L) x = __dsub_rn(x, L);
+      else if (x < 0.0) x = __dadd_rn(x, L);
+      if (x >= L) x = 0.0;
+      (gl == 0 ? qdx : (gl == 1 ? qdy : qdz))[i] = x;
+      // floor(x / cs): from a product unless it comes near a whole number
+      // (x / cs < 2^10, so the product is within 2^-40 of the quotient)
+      const double qt = x * c.inv_cs[gl];
+      cc = (int)qt;
+      const float fr = (float)(qt - (double)cc);
+      if (fr < 1e-6f || fr > 1.0f - 1e-6f) cc = (int)floor(__ddiv_rn(x, c.cs[gl]));
+      cc = cc >= c.nc[gl] ? c.nc[gl] - 1 : (cc < 0 ? 0 : cc);
+    }
+  }
+  if (dt_drift != 0.0) {
+    const int cy2 = __shfl_sync(0xffffffffu, cc, 1, T), cz2 = __shfl_sync(0xffffffffu, cc, 2, T);
+    if (mine && gl == 0) {
+      const int r = mrank[cc + c.nc[0] * (cy2 + c.nc[1] * cz2)];
+      key[i] = r;
+      slot[i] = atomicAdd(&cell_count[r], 1);
+    }
+  }
+}
+
 // The particles that k_force left: more neighbours than a list row holds.
 // A few thread blocks loop over the density pass's overflow list (usually
 // empty: the launch then ends at once).
@@ -422,57 +636,83 @@ static inline unsigned blocks_for(int64_t n, int t) { return (unsigned)((n + t -
 // memory, so any of the accepted sizes gives the same results)
 static inline int pair_block(const Consts& c) { return pair_threads_ok(c.pair_threads) ? c.pair_threads : 128; }
 
+// Lanes per particle of the float64 passes: with few particles a whole warp
+// each, which spreads them over the SM quarters and shortens every particle's
+// chain; else kLanes64, which costs fewer instructions in all.  The line lies
+// at four warps per SM quarter.
+static bool pair64_wide(const Consts& c) { return c.pair_auto && c.N <= 16 * 152; }
+
+template <int KIND>
+static void launch_density64(const Consts& c, const Workspace& w, const Arrays<Fp64>& a, int update_eos,
+                             int32_t* ncount_by_id, int32_t* ovf_list, int32_t* ovf_count, int32_t* ovf_other,
+                             cudaStream_t s) {
+  const bool wide = pair64_wide(c);
+  const int t = wide ? 128 : pair_block(c), ppb = wide ? 4 : t / kLanes64;
+  auto kern = wide ? k_density64<KIND, 32, 4>
+                   : (t == 32 ? k_density64<KIND, kLanes64, 32 / kLanes64>
+                              : (t == 64 ? k_density64<KIND, kLanes64, 64 / kLanes64>
+                                         : k_density64<KIND, kLanes64, 128 / kLanes64>));
+  kern<<<blocks_for(c.N, ppb), t, (size_t)c.nbr_cap * ppb * 4, s>>>(
+      c, a, (D4*)w.qp4, w.cell_start, w.mrank, update_eos, ncount_by_id, w.nlist, w.nn, ovf_list, ovf_count, ovf_other,
+      w.qf4, (D4*)w.qr4, w.cend);
+}
+
 template <class P>
 void launch_density(const Consts& c, const Workspace& w, int cur, int update_eos, int32_t* ncount_by_id,
                     cudaStream_t s) {
   if (c.N == 0) return;
   Arrays<P> a = view<P>(w, cur);
-  auto qp4 = (typename P::V4*)w.qp4;
-  const int t = pair_block(c);
   const int sl = (*w.ovf_slot ^= 1);  // this pass's slot of the overflow list
   int32_t* ovf_list = w.ovf_list + (size_t)sl * (size_t)c.N;
   int32_t* ovf_count = w.ovf_count + sl;
   int32_t* ovf_other = w.ovf_count + (sl ^ 1);
-  if (c.kernel == SDPD_KERNEL_LUCY)
-    k_density<P, SDPD_KERNEL_LUCY><<<blocks_for(c.N, t), t, 0, s>>>(
-        c, a, qp4, w.cell_start, w.mrank, w.xmin[0], w.xmin[1], w.xmin[2], update_eos, ncount_by_id, w.nlist,
-        w.nn, ovf_list, ovf_count, ovf_other, w.qf4, (typename P::V4*)w.qr4, w.cend);
-  else
-    k_density<P, SDPD_KERNEL_CUBIC><<<blocks_for(c.N, t), t, 0, s>>>(
-        c, a, qp4, w.cell_start, w.mrank, w.xmin[0], w.xmin[1], w.xmin[2], update_eos, ncount_by_id, w.nlist,
-        w.nn, ovf_list, ovf_count, ovf_other, w.qf4, (typename P::V4*)w.qr4, w.cend);
+  if constexpr (P::mixed) {
+    const int t = pair_block(c);
+    auto kern = c.kernel == SDPD_KERNEL_LUCY ? k_density<P, SDPD_KERNEL_LUCY> : k_density<P, SDPD_KERNEL_CUBIC>;
+    kern<<<blocks_for(c.N, t), t, 0, s>>>(c, a, (typename P::V4*)w.qp4, w.cell_start, w.mrank, w.xmin[0], w.xmin[1],
+                                          w.xmin[2], update_eos, ncount_by_id, w.nlist, w.nn, ovf_list, ovf_count,
+                                          ovf_other, (typename P::V4*)w.qr4, w.cend);
+  } else if (c.kernel == SDPD_KERNEL_LUCY) {
+    launch_density64<SDPD_KERNEL_LUCY>(c, w, a, update_eos, ncount_by_id, ovf_list, ovf_count, ovf_other, s);
+  } else {
+    launch_density64<SDPD_KERNEL_CUBIC>(c, w, a, update_eos, ncount_by_id, ovf_list, ovf_count, ovf_other, s);
+  }
+}
+
+template <class P, int KIND>
+static void launch_force_kind(const Consts& c, const Workspace& w, const Arrays<P>& a, double half_dt,
+                              double dt_drift, double* force_by_id, cudaStream_t s) {
+  auto qp4 = (const typename P::V4*)w.qp4;
+  auto qdx = (typename P::Q*)w.qdx;
+  auto qdy = (typename P::Q*)w.qdy;
+  auto qdz = (typename P::Q*)w.qdz;
+  if constexpr (P::mixed) {
+    const float3 drift3 =
+        make_float3((float)(dt_drift / c.m * c.inv_scale[0]), (float)(dt_drift / c.m * c.inv_scale[1]),
+                    (float)(dt_drift / c.m * c.inv_scale[2]));
+    const int sl = *w.ovf_slot;  // the overflow list of the latest density pass
+    const int t = pair_block(c);
+    k_force<P, KIND><<<blocks_for(c.N, t), t, 0, s>>>(
+        c, a, qp4, w.cell_start, w.mrank, w.xmin[0], w.xmin[1], w.xmin[2], half_dt, dt_drift, qdx, qdy, qdz, w.key,
+        w.slot, w.cell_count, force_by_id, w.nlist, w.nn, drift3);
+    k_force_overflow<P, KIND><<<kOverflowBlocks, 128, 0, s>>>(
+        c, a, qp4, w.cell_start, w.mrank, w.xmin[0], w.xmin[1], w.xmin[2], half_dt, dt_drift, qdx, qdy, qdz, w.key,
+        w.slot, w.cell_count, force_by_id, drift3, w.ovf_list + (size_t)sl * (size_t)c.N, w.ovf_count + sl);
+  } else {
+    const int t = pair_block(c), lanes = pair64_wide(c) ? 32 : kLanes64;
+    auto kern = lanes == 32 ? k_force64<KIND, 32> : k_force64<KIND, kLanes64>;
+    kern<<<blocks_for(c.N * lanes, t), t, 0, s>>>(c, a, qp4, w.qf4, w.cell_start, w.mrank, half_dt, dt_drift, qdx, qdy,
+                                                  qdz, w.key, w.slot, w.cell_count, force_by_id, w.nlist, w.nn);
+  }
 }
 
 template <class P>
 void launch_force(const Consts& c, const Workspace& w, int cur, double half_dt, double dt_drift,
                   double* force_by_id, cudaStream_t s) {
   if (c.N == 0) return;
-  Arrays<P> a = view<P>(w, cur);
-  auto qp4 = (const typename P::V4*)w.qp4;
-  auto qdx = (typename P::Q*)w.qdx;
-  auto qdy = (typename P::Q*)w.qdy;
-  auto qdz = (typename P::Q*)w.qdz;
-  const float3 drift3 = make_float3((float)(dt_drift / c.m * c.inv_scale[0]), (float)(dt_drift / c.m * c.inv_scale[1]),
-                                    (float)(dt_drift / c.m * c.inv_scale[2]));
-  const int sl = *w.ovf_slot;  // the overflow list of the latest density pass
-  const int32_t* ovf_list = w.ovf_list + (size_t)sl * (size_t)c.N;
-  const int32_t* ovf_count = w.ovf_count + sl;
-  const int t = pair_block(c);
-  if (c.kernel == SDPD_KERNEL_LUCY) {
-    k_force<P, SDPD_KERNEL_LUCY><<<blocks_for(c.N, t), t, 0, s>>>(
-        c, a, qp4, w.cell_start, w.mrank, w.xmin[0], w.xmin[1], w.xmin[2], half_dt, dt_drift, qdx, qdy,
-        qdz, w.key, w.slot, w.cell_count, force_by_id, w.nlist, w.nn, drift3);
-    k_force_overflow<P, SDPD_KERNEL_LUCY><<<kOverflowBlocks, 128, 0, s>>>(
-        c, a, qp4, w.cell_start, w.mrank, w.xmin[0], w.xmin[1], w.xmin[2], half_dt, dt_drift, qdx, qdy,
-        qdz, w.key, w.slot, w.cell_count, force_by_id, drift3, ovf_list, ovf_count);
-  } else {
-    k_force<P, SDPD_KERNEL_CUBIC><<<blocks_for(c.N, t), t, 0, s>>>(
-        c, a, qp4, w.cell_start, w.mrank, w.xmin[0], w.xmin[1], w.xmin[2], half_dt, dt_drift, qdx, qdy,
-        qdz, w.key, w.slot, w.cell_count, force_by_id, w.nlist, w.nn, drift3);
-    k_force_overflow<P, SDPD_KERNEL_CUBIC><<<kOverflowBlocks, 128, 0, s>>>(
-        c, a, qp4, w.cell_start, w.mrank, w.xmin[0], w.xmin[1], w.xmin[2], half_dt, dt_drift, qdx, qdy,
-        qdz, w.key, w.slot, w.cell_count, force_by_id, drift3, ovf_list, ovf_count);
-  }
+  const Arrays<P> a = view<P>(w, cur);
+  if (c.kernel == SDPD_KERNEL_LUCY) launch_force_kind<P, SDPD_KERNEL_LUCY>(c, w, a, half_dt, dt_drift, force_by_id, s);
+  else launch_force_kind<P, SDPD_KERNEL_CUBIC>(c, w, a, half_dt, dt_drift, force_by_id, s);
 }
 
 template void launch_density<Fp64>(const Consts&, const Workspace&, int, int, int32_t*, cudaStream_t);
