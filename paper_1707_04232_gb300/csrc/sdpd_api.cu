@@ -194,6 +194,7 @@ size_t layout(sdpd_handle* s, Workspace* w, char* base) {
   w->sched_pair = (uint16_t*)at(cap * 2);
   w->st_geom = at(cap * rec);
   w->st_rnd = at(cap * rec);
+  w->st_aux = rec == sizeof(D4) ? (double*)at(cap * 8) : nullptr;
   w->io_q = (double*)at(3 * N * 8);
   w->io_p = (double*)at(3 * N * 8);
   w->io_e = (double*)at(N * 8);
@@ -354,7 +355,7 @@ void fd_sweep_step(sdpd_handle* s, double dt_fd, uint64_t seed) {
   if (rec) cudaMemsetAsync(s->w.pair_rec_count, 0, 8, s->stream);
   if (!s->sched_valid) {  // positions unchanged since the last sweep: reuse it
     StageTimer t(s, 4, 5);
-    launch_fd_schedule<P>(c, s->w, s->cur, fd_round_width(fd_launch_variant(c, sweep_float(s))), s->stream);
+    launch_fd_schedule<P>(c, s->w, s->cur, fd_round_width(c, sweep_float(s)), s->stream);
     if constexpr (std::is_same<P, Fp64>::value) {
       if (s->prm.sweep_f32) launch_stage_geometry<Fp64, Mixed>(c, s->w, s->cur, s->stream);
       else launch_stage_geometry<Fp64, Fp64>(c, s->w, s->cur, s->stream);

@@ -584,19 +584,24 @@ __global__ void __launch_bounds__(kStageWarps * 32)
     v.y = (R)(ry * inv_r);
     v.z = (R)(rz * inv_r);
     v.w = (R)fm::div(stage_F<KIND>(r2 * inv_r, inv_h, cF), qa.w * qb.w);
+    if constexpr (!A::mixed)  // at r = h the pair does nothing: marked by base = 0
+      if (!(c.kperp_m2 * v.w > 0.0) || !(c.kpar_m2 * v.w > 0.0)) v.w = 0.0;
     st4(&geom[base + t], v);
   }
 }
 
 // Three normals and the uniform (its logarithm for EMS, whose Metropolis
 // test needs only that) of every scheduled pair at the current sweep.
+// float64: G split along and across e, (G - (e.G) e, e.G), and in aux
+// |G|^2 / 2 - ln U (see sdpd_fd_team64.cuh).
 template <class A>
 __global__ void __launch_bounds__(kStageWarps * 32)
     k_stage_random(Consts c, const int32_t* __restrict__ id, const int32_t* __restrict__ cell_start,
                    const int32_t* __restrict__ mrank, const uint32_t* __restrict__ hdr,
                    const unsigned long long* __restrict__ sched_off, const uint16_t* __restrict__ pairs,
                    uint64_t seed, const unsigned long long* __restrict__ sweep_ptr,
-                   typename A::V4* __restrict__ rnd) {
+                   const typename A::V4* __restrict__ geom, typename A::V4* __restrict__ rnd,
+                   double* __restrict__ aux) {
   using R = typename A::R;
   __shared__ FdCells cells_s[kStageWarps];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -615,10 +620,15 @@ __global__ void __launch_bounds__(kStageWarps * 32)
     R G[3], U;
     pair_randoms_fast(seed, sweep, (uint64_t)id[ga], (uint64_t)id[gb], G, &U);
     typename A::V4 v;
-    v.x = G[0];
-    v.y = G[1];
-    v.z = G[2];
-    v.w = c.scheme == SDPD_SCHEME_EMS ? fm::log(U) : U;
+    if constexpr (A::mixed) {
+      v = F4{G[0], G[1], G[2], c.scheme == SDPD_SCHEME_EMS ? fm::log(U) : U};
+    } else {
+      const D4 e = ld4(&geom[base + t]);
+      const double gp = e.x * G[0] + e.y * G[1] + e.z * G[2];
+      v = D4{G[0] - gp * e.x, G[1] - gp * e.y, G[2] - gp * e.z, gp};
+      aux[base + t] = c.scheme == SDPD_SCHEME_EMS
+                          ? 0.5 * (G[0] * G[0] + G[1] * G[1] + G[2] * G[2]) - fm::log(U) : 0.0;
+    }
     st4(&rnd[base + t], v);
   }
 }
@@ -810,19 +820,15 @@ static __device__ __noinline__ float fd_uniform_again(uint64_t seed, uint64_t sw
 // rounds (k_sched_rounds: at most 32 / OPW pairs of disjoint particles each).
 // A block's particles (momenta and energies) live in shared memory; the
 // pairs' staged data stream from global memory one round ahead of their use.
-// P is the storage policy of the state arrays, A the arithmetic policy of
-// the pair updates: A = P except for a float64 state swept with float32
-// pair arithmetic (P = Fp64, A = Mixed), where momenta and energies go back
-// as their float64 values plus the float32 increments of the visit.
-// REC: keep a record per pair (every Metropolis margin in float64).
-// Thread blocks of 1 to 4 warps; 128 registers per thread for float32
-// arithmetic (16 warps per SM), up to 168 for float64 (12 warps).
+// P is the storage policy of the state arrays, A = Mixed the arithmetic policy
+// of the pair updates (float64 pair arithmetic: k_fd_colour64).  A float64
+// state swept with float32 pair arithmetic (P = Fp64) gets its momenta and
+// energies back as their float64 values plus the float32 increments of the
+// visit.  REC: keep a record per pair (every Metropolis margin in float64).
+// Thread blocks of 1 to 4 warps, 128 registers per thread (16 warps per SM).
 // ---------------------------------------------------------------------------
-template <class A>
-constexpr int fd_min_blocks() { return A::mixed ? 4 : 3; }
-
 template <class P, class A, int OPW, bool REC>
-__global__ void __launch_bounds__(128, fd_min_blocks<A>())
+__global__ void __launch_bounds__(128, 4)
     k_fd_colour(Consts c, FDConst<typename A::R> k, Arrays<P> a, typename P::V4* __restrict__ qp4,
                 const int32_t* __restrict__ cell_start, const int32_t* __restrict__ mrank,
                 const uint32_t* __restrict__ xmx, const uint32_t* __restrict__ xmy,
@@ -837,6 +843,7 @@ __global__ void __launch_bounds__(128, fd_min_blocks<A>())
   using R = typename A::R;  // pair arithmetic
   using S = typename P::R;  // stored momenta, densities, geometry
   using AV4 = typename A::V4;
+  static_assert(A::mixed, "float64 pair arithmetic runs k_fd_colour64");
   constexpr bool kSame = std::is_same<R, S>::value;
   constexpr int kGroupLanes = 32 / OPW;
   extern __shared__ __align__(32) unsigned char fd_smem_raw[];
@@ -915,7 +922,7 @@ __global__ void __launch_bounds__(128, fd_min_blocks<A>())
       v.z = (R)a.pz[g];
       v.w = (R)a.eps[g];
       sm.s[q] = v;
-      if constexpr (A::mixed) sm.ec[q] = 0.0f;
+      sm.ec[q] = 0.0f;
     }
     __syncwarp();
     while (__any_sync(0xffffffffu, n > 0)) {
@@ -943,7 +950,7 @@ __global__ void __launch_bounds__(128, fd_min_blocks<A>())
         double margin;
         float m32 = 0.0f, tol = 0.0f;
         int dcs;
-        if constexpr (A::mixed) {
+        {
           const float eaf = sa.w, ebf = sb.w;
           auto exact_e = [&](double& ea, double& eb) { fd_exact_energies(a.eps, sm, ia, ib, eaf, ebf, ea, eb); };
           auto uniform = [&]() {
@@ -961,13 +968,6 @@ __global__ void __launch_bounds__(128, fd_min_blocks<A>())
             sm.ec[ib] = __fadd_rn(sm.ec[ib], __fadd_rn(e, dl));
             sm.s[ib] = F4{pb[0], pb[1], pb[2], s};
           }
-        } else {
-          double deps;
-          dcs = fd_pair(k, cg.x, cg.y, cg.z, cg.w, G, cr.w, pa, pb, sa.w, sb.w, deps, margin, negative);
-          if (dcs == 0) {
-            sm.s[ia] = D4{pa[0], pa[1], pa[2], sa.w + deps};
-            sm.s[ib] = D4{pb[0], pb[1], pb[2], sb.w + deps};
-          }
         }
         n_rb += dcs == 1;
         n_rm += dcs == 2;
@@ -982,7 +982,7 @@ __global__ void __launch_bounds__(128, fd_min_blocks<A>())
             rc.decision = dcs;
             rc.level = level;
             rc.margin = margin;
-            rc.margin_lo = A::mixed ? (double)m32 : margin;
+            rc.margin_lo = (double)m32;
             rc.margin_tol = (double)tol;
             recs[s] = rc;
           }
@@ -1000,12 +1000,9 @@ __global__ void __launch_bounds__(128, fd_min_blocks<A>())
         a.py[g] += (S)(v.y - (R)a.py[g]);
         a.pz[g] += (S)(v.z - (R)a.pz[g]);
       }
-      double e;
-      if constexpr (A::mixed) {  // once per visit: the load value plus the visit's exact change
-        const double e0 = a.eps[g];
-        e = e0 + (((double)v.w - (double)(float)e0) + (double)sm.ec[q]);
-      }
-      else e = v.w;
+      // once per visit: the load value plus the visit's exact change
+      const double e0 = a.eps[g];
+      const double e = e0 + (((double)v.w - (double)(float)e0) + (double)sm.ec[q]);
       bad |= !isfinite(v.w);  // (a sum that was not finite once never is again)
       a.eps[g] = e;
       // pressure over rho^2 of the new energy, Eq. (pg-eos): pi = c_rho eps / (C_K m rho)
@@ -1156,8 +1153,18 @@ void launch_colours_rec(const Consts& c, const Workspace& w, int cur, double dt,
 
 // Fills the resident-block counts of every block schedule ahead of time (a
 // host query, kept out of stream captures).
+template <bool REC>
+int team64_resident();
+template <bool REC>
+void launch_colours64(const Consts& c, const Workspace& w, int cur, double dt, uint64_t seed, cudaStream_t s);
+
 template <class P, class A>
 void fd_prepare() {
+  if constexpr (!A::mixed) {
+    team64_resident<false>();
+    team64_resident<true>();
+    return;
+  } else
   for (int v = 0; v < kFdVariants; ++v)
     if (fd_fits<A>(v)) {
       fd_resident<P, A, false>(v);
@@ -1188,12 +1195,17 @@ void launch_fd_colours(const Consts& c, const Workspace& w, int cur, double dt, 
     launch_advance_sweep(w, s);
     return;
   }
-  const int variant = fd_launch_variant(c, A::mixed);
   k_stage_random<A><<<stage_blocks(c), kStageWarps * 32, 0, s>>>(c, w.id[cur], w.cell_start, w.mrank, w.sched_hdr,
                                                                 w.sched_off, w.sched_pair, seed, w.sweep,
-                                                                (typename A::V4*)w.st_rnd);
-  if (record) launch_colours_rec<P, A, true>(c, w, cur, dt, seed, variant, s);
-  else launch_colours_rec<P, A, false>(c, w, cur, dt, seed, variant, s);
+                                                                (const typename A::V4*)w.st_geom,
+                                                                (typename A::V4*)w.st_rnd, w.st_aux);
+  if constexpr (!A::mixed) {
+    if (record) launch_colours64<true>(c, w, cur, dt, seed, s);
+    else launch_colours64<false>(c, w, cur, dt, seed, s);
+    return;
+  } else
+  if (record) launch_colours_rec<P, A, true>(c, w, cur, dt, seed, fd_launch_variant(c), s);
+  else launch_colours_rec<P, A, false>(c, w, cur, dt, seed, fd_launch_variant(c), s);
 }
 
 }  // namespace sdpd

@@ -1,7 +1,7 @@
 // sdpd_fd_colour_fp64.cu -- the colour kernels of the float64 state, every
 // block-schedule variant, with float64 or float32 pair arithmetic (kept apart
 // from the mixed state so that the variants compile in parallel).
-#include "sdpd_fd_colour.cuh"
+#include "sdpd_fd_team64.cuh"
 
 namespace sdpd {
 
@@ -15,7 +15,9 @@ template void launch_fd_colours<Fp64, Fp64>(const Consts&, const Workspace&, int
 template void launch_fd_colours<Fp64, Mixed>(const Consts&, const Workspace&, int, double, uint64_t, int,
                                            cudaStream_t);
 
-int fd_round_width(int variant) { return 32 / kFdOpw[variant]; }
+int fd_round_width(const Consts& c, bool float_arith) {
+  return float_arith ? 32 / kFdOpw[fd_launch_variant(c)] : kTeamPairs;
+}
 
 bool fd_variant_fits(bool mixed, int v) {
   return v >= 0 && v < kFdVariants && (mixed ? fd_fits<Mixed>(v) : fd_fits<Fp64>(v));

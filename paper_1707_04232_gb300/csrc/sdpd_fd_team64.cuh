@@ -1,0 +1,423 @@
+// sdpd_fd_team64.cuh -- the colour kernel of the float64 sweep: a team of two
+// warps per block, four lanes per pair.
+//
+// GB300 issues one float64 warp instruction per 64 cycles on each quarter of
+// an SM, whatever the number of active lanes and however independent the
+// instructions are, so a round of a block's schedule costs its float64
+// instructions times 64 cycles per warp: with one lane per pair about 340
+// (13 of 32 lanes in use).  Here the four lanes of a pair share its
+// arithmetic so that every lane of an instruction does a different part of
+// it: lanes 0 to 2 hold the components of the vectors and the direction
+// across e, lane 3 the energies and the direction along e.  The coefficients
+// (exponential, square root), the components of the proposal and of the
+// reverse noise, and the logarithms of the Metropolis ratio are each
+// evaluated once per instruction for the whole pair: about 95 float64
+// instructions per round.  Rounds hold at most 16 pairs (8 per warp).
+#pragma once
+#include "sdpd_fd_colour.cuh"
+
+namespace sdpd {
+
+// Elementary functions with few float64 instructions.  Each starts from a
+// hardware approximation or a float32 evaluation of its small terms.
+namespace f64 {
+__device__ __forceinline__ double rcp_seed(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  return y;
+}
+__device__ __forceinline__ double rsqrt_seed(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  return y;
+}
+// 1/x: one third-order (Householder) step y (1 + e + e^2), e = 1 - x y.
+__device__ __forceinline__ double rcp(double x) {
+  const double y = rcp_seed(x), e = __fma_rn(-x, y, 1.0);
+  return __fma_rn(y, __fma_rn(e, e, e), y);
+}
+// sqrt(x) and 1/sqrt(x): one third-order step, (1 - e)^(-1/2) =
+// 1 + e/2 + 3 e^2/8 + O(e^3) with e = 1 - x y^2.  Arguments whose seed could
+// be flushed take the library functions.
+__device__ __forceinline__ bool rsqrt_tiny(double x) { return __double2hiint(x) < 0x03f00000; }  // below 2^-960, <= 0
+__device__ __forceinline__ double sqrt_(double x) {
+  if (rsqrt_tiny(x)) return ::sqrt(x);
+  const double y = rsqrt_seed(x), h = __dmul_rn(x, y), e = __fma_rn(-h, y, 1.0);
+  return __fma_rn(__dmul_rn(h, e), __fma_rn(e, 0.375, 0.5), h);
+}
+__device__ __forceinline__ double rsqrt_(double x) {
+  if (rsqrt_tiny(x)) return 1.0 / ::sqrt(x);
+  const double y = rsqrt_seed(x), h = __dmul_rn(x, y), e = __fma_rn(-h, y, 1.0);
+  return __fma_rn(__dmul_rn(y, e), __fma_rn(e, 0.375, 0.5), y);
+}
+__device__ __forceinline__ bool below(double x, int hi) { return (__double2hiint(x) & 0x7fffffff) < hi; }
+constexpr int kHi2m6 = 0x3f900000, kHi2m3 = 0x3fc00000, kHi2m2 = 0x3fd00000;  // high words of 2^-6, 1/8, 1/4
+// expm1: Taylor series; below 2^-6 the terms from x^5/120 on, 2^-31 of the
+// result, in float32; below 1/4 twelve terms in float64.
+__device__ __forceinline__ double expm1(double x) {
+  if (below(x, kHi2m6)) {
+    const float f = (float)x;
+    const float t = f * (1.0f / 120.0f + f * (1.0f / 720.0f + f * (1.0f / 5040.0f)));
+    double p = 1.0 / 24.0 + (double)t;
+    p = __fma_rn(p, x, 1.0 / 6.0);
+    p = __fma_rn(p, x, 0.5);
+    return __fma_rn(__dmul_rn(p, x), x, x);
+  }
+  if (below(x, kHi2m2)) {
+    double p = 1.0 / 6227020800.0;
+    p = __fma_rn(p, x, 1.0 / 479001600.0);
+    p = __fma_rn(p, x, 1.0 / 39916800.0);
+    p = __fma_rn(p, x, 1.0 / 3628800.0);
+    p = __fma_rn(p, x, 1.0 / 362880.0);
+    p = __fma_rn(p, x, 1.0 / 40320.0);
+    p = __fma_rn(p, x, 1.0 / 5040.0);
+    p = __fma_rn(p, x, 1.0 / 720.0);
+    p = __fma_rn(p, x, 1.0 / 120.0);
+    p = __fma_rn(p, x, 1.0 / 24.0);
+    p = __fma_rn(p, x, 1.0 / 6.0);
+    p = __fma_rn(p, x, 0.5);
+    return __fma_rn(__dmul_rn(p, x), x, x);
+  }
+  return ::expm1(x);
+}
+// log1p: below 2^-6 the alternating series, its terms from x^6/6 on (2^-33 of
+// the result) in float32; below 1/8 2 atanh(u) with u = x / (2 + x), its
+// terms from u^7/7 on in float32.
+__device__ __forceinline__ double log1p(double x) {
+  if (below(x, kHi2m6)) {
+    const float f = (float)x;
+    const float t = f * (-1.0f / 6.0f + f * (1.0f / 7.0f + f * (-1.0f / 8.0f + f * (1.0f / 9.0f))));
+    double p = 0.2 + (double)t;
+    p = __fma_rn(p, x, -0.25);
+    p = __fma_rn(p, x, 1.0 / 3.0);
+    p = __fma_rn(p, x, -0.5);
+    return __fma_rn(__dmul_rn(p, x), x, x);
+  }
+  if (below(x, kHi2m3)) {
+    const double d = 2.0 + x, r = rcp(d);
+    double u = __dmul_rn(x, r);
+    u = __fma_rn(__fma_rn(-u, d, x), r, u);
+    const double w = __dmul_rn(u, u);
+    const float f = (float)w;
+    const float t = f * (1.0f / 7.0f + f * (1.0f / 9.0f + f * (1.0f / 11.0f + f * (1.0f / 13.0f))));
+    double p = 0.2 + (double)t;
+    p = __fma_rn(p, w, 1.0 / 3.0);
+    const double v = u + u;
+    return __fma_rn(__dmul_rn(p, w), v, v);
+  }
+  return ::log1p(x);
+}
+// comparisons with zero on the bits (a float64 comparison costs an issue)
+__device__ __forceinline__ bool positive(double x) {
+  const long long b = __double_as_longlong(x);
+  return b > 0 && b <= 0x7ff0000000000000ll;
+}
+__device__ __forceinline__ bool negative(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  return b > 0x8000000000000000ull && b <= 0xfff0000000000000ull;
+}
+}  // namespace f64
+
+// Constants of the team's arithmetic, in momentum units: with u = p_i - p_j,
+// dp = (m/2)(v' - v) = (alpha - 1) u / 2 + hz G per direction, hz = m zt / 2,
+// hz^2 = kB m / C_K * (eps_i eps_j / (eps_i + eps_j)) / (1 - d) * (1 - alpha^2).
+struct Team64Const {
+  double x_par, x_perp;  // log alpha per unit of base (1 - d): -2 kappa m^2 dt / m
+  double d2;             // 2 kB / C_K
+  double s;              // kB m / C_K
+  double de;             // -1 / (2 m)
+  double CKm1;
+  int scheme;
+};
+
+// alpha - 1 and (hz or, INV, 1 / hz) of this lane's direction at energies
+// with sum E, product P and 1/E = iE.
+template <bool INV>
+__device__ __forceinline__ void team_coeffs(const Team64Const& k, double x_dir, double base, double P, double iE,
+                                            double& m, double& z) {
+  const double a = P * iE;
+  const double omd = __fma_rn(-k.d2, a * iE, 1.0);
+  m = f64::expm1(x_dir * (base * omd));
+  const double s = k.s * a * f64::rcp(omd);
+  const double q = s * (-m * (2.0 + m));
+  z = INV ? f64::rsqrt_(q) : f64::sqrt_(q);
+}
+
+__device__ __forceinline__ double quad_sum(double v) {
+  v += __shfl_xor_sync(0xffffffffu, v, 1);
+  v += __shfl_xor_sync(0xffffffffu, v, 2);
+  return v;
+}
+
+// One pair update on the four lanes of a quad (whole warps call it).  l: the
+// lane's place in the quad; A, B: component l of the two particles' records
+// (px, py, pz, eps); ge: component l of (e, base); Gl: component l of
+// (G - (e.G) e, e.G); c0 = |G|^2 / 2 - ln U.  live: the pair exists and
+// base > 0.  Returns the decision (0 accept, 1 energy bound, 2 Metropolis);
+// dA, dB are the lane's changes of A and B.
+__device__ __forceinline__ int team_pair(const Team64Const& k, int l, bool live, double A, double B, double ge,
+                                         double Gl, double base, double c0, double& dA, double& dB, double& margin,
+                                         bool& neg) {
+  const double ei = __shfl_sync(0xffffffffu, A, 3, 4), ej = __shfl_sync(0xffffffffu, B, 3, 4);
+  const double x_dir = l == 3 ? k.x_par : k.x_perp;
+  const double el = l == 3 ? 0.0 : ge;
+  const double u = A - B;
+  const double E = ei + ej, P = ei * ej;
+  // lane 2 takes 1/P (for the entropy term) while the others take 1/E
+  const double r0 = f64::rcp(l == 2 ? P : E);
+  const double iE = __shfl_sync(0xffffffffu, r0, 0, 4);
+  double m, z;
+  team_coeffs<false>(k, x_dir, base, P, iE, m, z);
+  // u/2 split along and across e: lane 3 holds the component along it
+  const double upar = quad_sum(el * u);
+  const double U = 0.5 * (l == 3 ? upar : __fma_rn(-upar, el, u));
+  const double v = __fma_rn(m, U, z * Gl);
+  const double dpar = __shfl_sync(0xffffffffu, v, 3, 4);
+  const double dp = l == 3 ? 0.0 : __fma_rn(dpar, el, v);
+  // kinetic energy change of the pair: dp . (u + dp) / m
+  const double deps = k.de * quad_sum(dp * (u + dp));
+  const double fi = ei + deps, fj = ej + deps;
+  const bool bound = f64::positive(fi) && f64::positive(fj);
+  margin = fi < fj ? fi : fj;
+  int decision = 0;
+  if (k.scheme == SDPD_SCHEME_SSA) {
+    neg |= live && !bound;
+  } else {
+    decision = bound ? 0 : 1;
+    if (k.scheme == SDPD_SCHEME_EMS) {
+      // reverse move from v' with the coefficients at the proposed energies;
+      // reverse noise per direction [(1 - alpha' alpha) u/2 - alpha' hz G] / hz'
+      const double P2 = fi * fj;
+      double mr, iz;
+      team_coeffs<true>(k, x_dir, base, P2, f64::rcp(fi + fj), mr, iz);
+      const double cr = -__fma_rn(m, mr, m + mr);
+      const double g = __fma_rn(cr, U, -(__fma_rn(mr, z, z) * Gl)) * iz;
+      // ln|B(v)| - ln|B(v')| = ln(z z') along + 2 ln(z z') across e (lanes 3,
+      // 0, 1); entropy (C_K/kB - 1) ln(eps' products / eps products) (lane 2)
+      const double t = deps * (E + deps);
+      const double lg = f64::log1p(l == 2 ? t * r0 : __fma_rn(z, iz, -1.0));
+      const double mg = c0 + quad_sum(__fma_rn(-0.5 * g, g, l == 2 ? k.CKm1 * lg : lg));
+      if (bound) {
+        margin = mg;
+        if (f64::negative(mg)) decision = 2;  // U > exp(a)
+      }
+    }
+  }
+  dA = l == 3 ? deps : dp;
+  dB = l == 3 ? deps : -dp;
+  return decision;
+}
+
+constexpr int kTeamWarps = 2, kTeamPairs = 8 * kTeamWarps;
+
+template <bool REC>
+__global__ void __launch_bounds__(kTeamWarps * 32)
+    k_fd_colour64(Consts c, FDConst<double> kbig, Team64Const k, Arrays<Fp64> a, D4* __restrict__ qp4,
+                  const int32_t* __restrict__ cell_start, const int32_t* __restrict__ mrank,
+                  const uint32_t* __restrict__ hdr, const uint8_t* __restrict__ rsize,
+                  const unsigned long long* __restrict__ sched_off, const uint16_t* __restrict__ pairs,
+                  const double* __restrict__ geom, const double* __restrict__ rnd, const double* __restrict__ aux,
+                  int colour, uint64_t seed, unsigned long long* __restrict__ sweep_ptr, unsigned long long* counters,
+                  int* status, sdpd_pair_rec* recs, unsigned long long* rec_count, int64_t rec_cap,
+                  unsigned* __restrict__ queue, const int32_t* __restrict__ order, int32_t* __restrict__ big_perm,
+                  const int2* __restrict__ big_list, const uint32_t* __restrict__ big_count) {
+  __shared__ FdSmem<double> sm;
+  __shared__ uint8_t size_s[kRoundStride];
+  __shared__ unsigned next_s;
+  const uint64_t sweep = *sweep_ptr;
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  const int l = lane & 3, slot = warp * 8 + (lane >> 2);  // place in the quad, pair of the round
+  const int hx = c.nc[0] >> 1, hy = c.nc[1] >> 1, hz = c.nc[2] >> 1;
+  const int64_t nown = (int64_t)hx * hy * hz;
+  const double pi_coef = c.c_rho / (c.C_K * c.m);
+  unsigned n_tot = 0, n_rb = 0, n_rm = 0;
+  bool negative = false, bad = false;
+  double* rec = reinterpret_cast<double*>(sm.s);
+  // blocks from the colour's queue, deepest first (see k_fd_colour)
+  for (;;) {
+    if (t == 0) next_s = atomicAdd(queue, 1u);
+    __syncthreads();
+    const unsigned wi = next_s;
+    if ((int64_t)wi >= nown) break;
+    const int64_t w = order[colour * nown + wi];
+    const int ox = 2 * (int)(w % hx) + (colour & 1), oy = 2 * (int)((w / hx) % hy) + ((colour >> 1) & 1),
+              oz = 2 * (int)(w / ((int64_t)hx * hy)) + ((colour >> 2) & 1);
+    const int64_t o = ox + (int64_t)c.nc[0] * (oy + (int64_t)c.nc[1] * oz);
+    const uint32_t hd = hdr[o];
+    const int np = hd == kHdrBig ? 0 : (int)(hd & 0xffffu), nr = hd == kHdrBig ? 0 : (int)(hd >> 16);
+    if (np == 0) {  // (a block beyond capacity is swept below)
+      __syncthreads();
+      continue;
+    }
+    if (t == 0) n_tot += (unsigned)np;
+    const unsigned long long first = sched_off[o];
+    for (int r = t; r < nr; r += kTeamWarps * 32) size_s[r] = rsize[o * kRoundStride + r];
+    BlockCells b;
+    block_cells(c, ox, oy, oz, mrank, cell_start, b);
+    const int nb = b.base[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+      if (t == q) {
+        sm.cells.cst[q] = b.start[q];
+        sm.cells.cbs[q] = b.base[q];
+      }
+    __syncthreads();
+    for (int q = t; q < nb; q += kTeamWarps * 32) {
+      const int g = block_gidx(sm.cells, q);
+      sm.s[q] = D4{a.px[g], a.py[g], a.pz[g], a.eps[g]};
+    }
+    // this quad's pair of a round, loaded one round ahead
+    uint16_t pr = 0;
+    double ge = 0.0, Gl = 0.0, base = 0.0, c0 = 0.0;
+    int r = 0, pos = 0, left = size_s[0], n = min(left, kTeamPairs);
+    auto fetch = [&]() {
+      if (slot < n) {
+        const unsigned long long at = first + pos + slot;
+        pr = __ldg(&pairs[at]);
+        ge = __ldg(&geom[4 * at + l]);
+        base = __ldg(&geom[4 * at + 3]);
+        Gl = __ldg(&rnd[4 * at + l]);
+        c0 = __ldg(&aux[at]);
+      }
+    };
+    fetch();
+    __syncthreads();
+    while (n > 0) {
+      const bool act = slot < n;
+      const int busy = n - warp * 8, level = r;  // pairs of this warp
+      const uint16_t cpr = act ? pr : (uint16_t)0;
+      // (lanes without a pair run on values that keep to the short paths)
+      const double cge = ge, cG = act ? Gl : 0.0, cb = act ? base : 0.01, cc = c0;
+      pos += n;
+      left -= n;
+      if (left == 0) left = ++r < nr ? (int)size_s[r] : 0;
+      n = min(left, kTeamPairs);
+      fetch();
+      if (busy > 0) {
+        const int ia = cpr & 255, ib = cpr >> 8;
+        const double A = rec[4 * ia + l], B = rec[4 * ib + l];
+        const bool live = act && f64::positive(cb);  // at r = h the pair does nothing
+        double dA, dB, margin;
+        int dcs = team_pair(k, l, live, A, B, cge, cG, cb, cc, dA, dB, margin, negative);
+        if (!live) {
+          dcs = 0;
+          margin = 0.0;
+        } else if (dcs == 0) {
+          rec[4 * ia + l] = A + dA;
+          rec[4 * ib + l] = B + dB;
+        }
+        if (act && l == 0) {
+          n_rb += dcs == 1;
+          n_rm += dcs == 2;
+          if constexpr (REC) {
+            const unsigned long long s = atomicAdd(rec_count, 1ull);
+            if ((int64_t)s < rec_cap) {
+              sdpd_pair_rec rc;
+              rc.id_i = a.id[block_gidx(sm.cells, ia)];
+              rc.id_j = a.id[block_gidx(sm.cells, ib)];
+              rc.colour = colour;
+              rc.owner = (int32_t)o;
+              rc.decision = dcs;
+              rc.level = level;
+              rc.margin = margin;
+              rc.margin_lo = margin;
+              rc.margin_tol = 0.0;
+              recs[s] = rc;
+            }
+          }
+        }
+      }
+      __syncthreads();
+    }
+    for (int q = t; q < nb; q += kTeamWarps * 32) {
+      const int g = block_gidx(sm.cells, q);
+      const D4 v = lds4(&sm.s[q]);
+      a.px[g] = v.x; a.py[g] = v.y; a.pz[g] = v.z;
+      bad |= !isfinite(v.w);  // (an energy that was not finite once never is again)
+      a.eps[g] = v.w;
+      qp4[g].w = v.w * pi_coef / a.rho[g];  // pressure over rho^2 of the new energy, Eq. (pg-eos)
+    }
+    __syncthreads();  // the team's shared memory is refilled by the next block
+  }
+  // blocks beyond capacity, pair by pair, one per warp
+  for (;;) {
+    unsigned bi = 0;
+    if (lane == 0) bi = atomicAdd(&queue[2], 1u);
+    bi = __shfl_sync(0xffffffffu, bi, 0);
+    if (bi >= big_count[colour]) break;
+    const int2 ent = big_list[colour * nown + bi];
+    int bx, by, bz;
+    owner_coords(c, ent.x, bx, by, bz);
+    const BigCounts bc = fd_big_block<Fp64, Fp64>(c, kbig, a, qp4, cell_start, mrank, nullptr, nullptr, nullptr, ent.x,
+                                                  bx, by, bz, colour, seed, sweep, REC ? recs : nullptr, rec_count,
+                                                  rec_cap, big_perm + ent.y);
+    if (lane == 0) {  // (lane 0 made the updates)
+      atomicAdd(&counters[0], bc.tot);
+      atomicAdd(&counters[1], bc.acc);
+      atomicAdd(&counters[2], bc.rb);
+      atomicAdd(&counters[3], bc.rm);
+    }
+    negative |= bc.negative != 0;
+    bad |= bc.bad != 0;
+  }
+  if (lane == 0) {
+    const unsigned total = gridDim.x * (unsigned)kTeamWarps;
+    __threadfence();  // this warp's last take from the queue is performed before it counts as done
+    if (atomicAdd(&queue[1], 1u) == total - 1u) {
+      queue[0] = 0u;
+      queue[1] = 0u;
+      queue[2] = 0u;
+      if (colour == 7) *sweep_ptr = sweep + 1ull;  // (every warp has read it) the sweep is done
+    }
+  }
+  const unsigned c_tot = __reduce_add_sync(0xffffffffu, n_tot), c_rb = __reduce_add_sync(0xffffffffu, n_rb),
+                 c_rm = __reduce_add_sync(0xffffffffu, n_rm);
+  const unsigned any_neg = __any_sync(0xffffffffu, negative), any_bad = __any_sync(0xffffffffu, bad);
+  if (lane == 0) {
+    // (the team's pairs are counted on its first warp, rejections on both:
+    // accepted = pairs - rejected, added with wrap-around)
+    if (c_tot || c_rb || c_rm) {
+      atomicAdd(&counters[0], (unsigned long long)c_tot);
+      atomicAdd(&counters[1], (unsigned long long)c_tot - c_rb - c_rm);
+      atomicAdd(&counters[2], (unsigned long long)c_rb);
+      atomicAdd(&counters[3], (unsigned long long)c_rm);
+    }
+    if (any_neg) atomicOr(status, kStNegative);
+    if (any_bad) atomicOr(status, kStNaN);
+  }
+}
+
+// Thread blocks of the team kernel resident at once (see fd_resident_blocks).
+template <bool REC>
+int team64_resident() {
+  static const int n = [] {
+    int dev = 0, sms = 0, per_sm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fd_colour64<REC>, kTeamWarps * 32, 0);
+    return std::max(1, sms) * std::max(1, per_sm);
+  }();
+  return n;
+}
+
+template <bool REC>
+void launch_colours64(const Consts& c, const Workspace& w, int cur, double dt, uint64_t seed, cudaStream_t s) {
+  Team64Const k;
+  k.x_par = -2.0 * c.kpar_m2 * (dt / c.m);
+  k.x_perp = -2.0 * c.kperp_m2 * (dt / c.m);
+  k.d2 = 2.0 * c.kB / c.C_K;
+  k.s = c.kB * c.m / c.C_K;
+  k.de = -0.5 / c.m;
+  k.CKm1 = c.C_K / c.kB - 1.0;
+  k.scheme = c.scheme;
+  const int64_t nown = (int64_t)(c.nc[0] / 2) * (c.nc[1] / 2) * (c.nc[2] / 2);
+  const unsigned gf = (unsigned)std::max<int64_t>(1, std::min<int64_t>(nown, team64_resident<REC>()));
+  for (int col = 0; col < 8; ++col)
+    k_fd_colour64<REC><<<gf, kTeamWarps * 32, 0, s>>>(
+        c, fd_const<double>(c, dt), k, view<Fp64>(w, cur), (D4*)w.qp4, w.cell_start, w.mrank, w.sched_hdr,
+        w.sched_rsize, w.sched_off, w.sched_pair, (const double*)w.st_geom, (const double*)w.st_rnd, w.st_aux, col,
+        seed, w.sweep, w.counters, w.status, REC ? w.pair_recs : nullptr, w.pair_rec_count, w.pair_rec_cap,
+        w.fd_queue + 3 * col, w.blk_order, w.big_perm, w.big_list, w.big_count);
+}
+
+}  // namespace sdpd

@@ -68,16 +68,17 @@ struct Consts {
 // thread-block sizes the pair passes accept.
 constexpr int kFdVariants = 5;
 __host__ __device__ constexpr int fd_default_variant(bool mixed) { return mixed ? 0 : 1; }
-// The block schedule of a handle's colour launches: the one set by the caller
+// The block schedule of a handle's colour launches with float32 pair
+// arithmetic (float64 has one, k_fd_colour64): the one set by the caller
 // or the autotuner, else by the blocks per colour.  Few blocks: a colour
 // lasts as long as its deepest block, which runs faster on a warp of its own
 // (variant 3; 32^3, 216 blocks per colour).  More blocks than resident warps:
 // two per warp use its lanes better (the defaults).
 constexpr int64_t kFdOwnWarpBlocks = 16 * 152;  // 16 warps on each of 152 SMs
-inline int fd_launch_variant(const Consts& c, bool mixed) {
+inline int fd_launch_variant(const Consts& c) {
   if (!c.fd_auto && c.fd_variant >= 0 && c.fd_variant < kFdVariants) return c.fd_variant;
   const int64_t nown = (int64_t)(c.nc[0] / 2) * (c.nc[1] / 2) * (c.nc[2] / 2);
-  return nown <= kFdOwnWarpBlocks ? 3 : fd_default_variant(mixed);
+  return nown <= kFdOwnWarpBlocks ? 3 : fd_default_variant(true);
 }
 __host__ __device__ constexpr bool pair_threads_ok(int t) { return t == 32 || t == 64 || t == 128; }
 // whether a block schedule's shared memory fits a thread block (float64
@@ -359,7 +360,8 @@ struct Workspace {
   unsigned long long* sched_total;  // entries of those arrays in use
   uint16_t* sched_pair;   // pairs round by round, block after block
   void* st_geom;          // per scheduled pair: unit vector, F / (rho_i rho_j)
-  void* st_rnd;           // per scheduled pair: three normals and the uniform (EMS: its logarithm)
+  void* st_rnd;           // per scheduled pair: its random numbers (see k_stage_random)
+  double* st_aux;         // float64 pair arithmetic: |G|^2 / 2 - ln U per scheduled pair
   // host <-> device staging in id order (float64)
   double* io_q;
   double* io_p;
@@ -439,7 +441,7 @@ void launch_fd_colours(const Consts& c, const Workspace& w, int cur, double dt, 
                        cudaStream_t s);
 template <class P>
 void launch_observables(const Consts& c, const Workspace& w, int cur, cudaStream_t s);
-int fd_round_width(int variant);  // lanes per block of a block schedule
+int fd_round_width(const Consts& c, bool float_arith);  // pairs of a block that a colour launch updates at once
 // sweep counter on the device: set to a value, or advanced by one
 void launch_set_sweep(const Workspace& w, unsigned long long value, cudaStream_t s);
 void launch_advance_sweep(const Workspace& w, cudaStream_t s);
