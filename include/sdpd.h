@@ -157,8 +157,8 @@ int sdpd_get_state(sdpd_t* s, double* q, double* p, double* eps, int on_device);
  * and draws the pair's random numbers from Philox4x64-10 keyed by seed with
  * counter (sweep number, min id, max id, 0).  Any local density completes:
  * a particle with more than 160 neighbours has its forces summed from the
- * cells instead of its list, and a block with more than 256 particles, 2048
- * owned pairs or 255 dependency levels, or with a member of more than 160
+ * cells instead of its list, and a block with more than 512 particles, 4096
+ * owned pairs or 255 rounds of its schedule, or with a member of more than 160
  * neighbours, is swept pair by pair in the same order (slower, same
  * result; SDPD_DEBUG_BIG counts such blocks).  Asynchronous on the handle's
  * stream.
@@ -225,8 +225,8 @@ int sdpd_energy_histogram(sdpd_t* s, double lo, double hi, int nbins, double sca
  *                     one per pair in an order of the library's choosing
  *  SDPD_DEBUG_BIG     uint32[8]  per colour, the 2x2x2 cell blocks that the
  *                     latest sweep schedule left to the pair-by-pair sweep
- *                     (beyond its capacities: more than 256 particles, 2048
- *                     owned pairs or 255 dependency levels, or a member whose
+ *                     (beyond its capacities: more than 512 particles, 4096
+ *                     owned pairs or 255 rounds, or a member whose
  *                     neighbour list overflowed its row; Sections 3.2-3.3)
  * dst: host memory, cap = capacity in elements; *count receives the number
  * of elements written.  The capacity is checked before anything is copied.

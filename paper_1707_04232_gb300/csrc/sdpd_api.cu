@@ -191,7 +191,7 @@ size_t layout(sdpd_handle* s, Workspace* w, char* base) {
   w->sched_rsize = (uint8_t*)at(sweep * nc * kRoundStride);
   w->sched_off = (unsigned long long*)at(nc * 8);
   w->sched_total = (unsigned long long*)at(8);
-  w->sched_pair = (uint16_t*)at(cap * 2);
+  w->sched_pair = (uint32_t*)at(cap * 4);
   w->st_geom = at(cap * rec);
   w->st_rnd = at(cap * rec);
   w->st_aux = rec == sizeof(D4) ? (double*)at(cap * 8) : nullptr;
@@ -207,6 +207,9 @@ size_t layout(sdpd_handle* s, Workspace* w, char* base) {
   w->big_perm = (int32_t*)at(N * 4);
   w->big_list = (int2*)at(nc * 8);
   w->big_count = (uint32_t*)at(16 * 4);
+  w->large_cand = (int32_t*)at(nc * 4);
+  w->large_list = (int32_t*)at(nc * 4);
+  w->large_count = (uint32_t*)at(16 * 4);
   w->ovf_list = (int32_t*)at(2 * N * 4);
   w->ovf_count = (int32_t*)at(2 * 4);
   w->ovf_slot = &s->ovf_slot;
@@ -355,7 +358,8 @@ void fd_sweep_step(sdpd_handle* s, double dt_fd, uint64_t seed) {
   if (rec) cudaMemsetAsync(s->w.pair_rec_count, 0, 8, s->stream);
   if (!s->sched_valid) {  // positions unchanged since the last sweep: reuse it
     StageTimer t(s, 4, 5);
-    launch_fd_schedule<P>(c, s->w, s->cur, fd_round_width(c, sweep_float(s)), s->stream);
+    launch_fd_schedule<P>(c, s->w, s->cur, fd_round_width(c, sweep_float(s), false),
+                          fd_round_width(c, sweep_float(s), true), s->stream);
     if constexpr (std::is_same<P, Fp64>::value) {
       if (s->prm.sweep_f32) launch_stage_geometry<Fp64, Mixed>(c, s->w, s->cur, s->stream);
       else launch_stage_geometry<Fp64, Fp64>(c, s->w, s->cur, s->stream);
@@ -589,9 +593,11 @@ int sdpd_bind_workspace(sdpd_t* s, void* ptr, size_t bytes) {
   e |= cuda_ok(cudaMemsetAsync(s->w.sched_hdr, 0, (size_t)c.ncell * 4, st));
   e |= cuda_ok(cudaMemsetAsync(s->w.fd_queue, 0, 32 * 4, st));
   e |= cuda_ok(cudaMemsetAsync(s->w.ovf_count, 0, 2 * 4, st));
+  e |= cuda_ok(cudaMemsetAsync(s->w.large_count, 0, 16 * 4, st));
   e |= cuda_ok(cudaStreamSynchronize(st));
-  // launch sizes of the sweep's colour kernels, queried here rather than
-  // inside a later stream capture
+  // launch attributes and sizes of the sweep's kernels, set and queried here
+  // rather than inside a later stream capture
+  e |= sched_prepare();
   if (s->prm.precision == SDPD_MIXED) fd_prepare<Mixed, Mixed>();
   else if (s->prm.sweep_f32) fd_prepare<Fp64, Mixed>();
   else fd_prepare<Fp64, Fp64>();

@@ -27,13 +27,16 @@
 // positions only, which are fixed during the sweep): k_sched_enum (one
 // thread block per block: owned pairs in canonical order, from the
 // neighbour lists of the density pass), k_sched_rounds (one warp per block:
-// the round of every pair, and the pairs written round by round), two that
-// order each colour's blocks by their number of rounds (k_sched_order_scan,
-// k_sched_order_scatter) and k_stage_geometry (the pairs' unit vectors and
-// friction factors).  A sweep is then k_stage_random (the pairs' random
-// numbers) and k_fd_colour once per colour (sdpd_fd_colour.cuh): the pair
-// updates round by round in shared memory, one or two blocks per warp as the
-// launch's block schedule says.
+// the round of every pair, and the pairs written round by round),
+// k_sched_large (both for the blocks that are too large for those two, and
+// the depth histogram scanned), k_sched_order_scatter (each colour's blocks
+// ordered by their number of rounds) and k_stage_geometry (the pairs' unit
+// vectors and friction factors).  A sweep is then k_stage_random (the pairs'
+// random numbers) and one colour launch per colour (sdpd_fd_colour.cuh,
+// sdpd_fd_team64.cuh): the pair updates round by round in shared memory.
+#include <algorithm>
+#include <type_traits>
+
 #include "sdpd_fd_common.cuh"
 
 namespace sdpd {
@@ -70,52 +73,55 @@ namespace sdpd {
 // F(nb - 1) - F(nb - d) with F(n) = sum_{k <= n} ceil(k / 32)), which is then
 // read out row by row.
 // ---------------------------------------------------------------------------
-constexpr int kEnumThreads = 160;
-constexpr int kEnumWarps = kEnumThreads / 32;
-constexpr int kTriWords = 1152;   // >= F(255) = 1144: a triangle of 256 rows
+constexpr int kEnumThreads = 160;   // blocks of up to kMaxBlock particles
+constexpr int kLargeThreads = 256;  // blocks of up to kLargeBlock particles (two per thread)
 constexpr int kFlatEntries = 2048;  // group entries of one block per chunk
 
 // words of the first rows of the triangular bitmap: F(n) = sum_{k=1..n} ceil(k/32)
-__device__ __forceinline__ int tri_f(int n) {
-  const int q = n >> 5, s = n & 31;
-  return 16 * q * (q + 1) + s * (q + 1);
+__host__ __device__ constexpr int tri_f(int n) {
+  return 16 * (n >> 5) * ((n >> 5) + 1) + (n & 31) * ((n >> 5) + 1);
 }
 
+template <int CAP>
 struct EnumSmem {
-  uint32_t bits[kTriWords];
-  int32_t ids[2][kMaxBlock];  // merge rounds: the ids in run order
-  uint8_t ks[2][kMaxBlock];   // and the block-local index of each
-  uint8_t rank[kMaxBlock];    // rank of each block-local index
-  uint8_t perm[kMaxBlock];    // block-local index of each rank
-  uint8_t who[kFlatEntries];  // member of each flat entry
-  uint32_t rng[kMaxBlock];    // up to four slot ranges (first slot, length) of each member's group, packed
-  uint32_t rcum[kMaxBlock];   // cumulative lengths after ranges 0, 1, 2 (bytes)
-  uint8_t ncnt[kMaxBlock];    // entries of each member's group
-  uint8_t dk[kMaxBlock];      // block cell of each member
-  int64_t lbase[kMaxBlock];   // nbr_slot(member, 0) with the slot's in-row part removed
-  uint8_t dtab[8][64];        // partner cell of (member cell, stencil code); 8: not in the block
-  int32_t off[kMaxBlock + 1];  // first flat entry of each member
-  uint16_t rowbase[kMaxBlock];  // first word of each row of the bitmap
-  int32_t wtot[kEnumWarps];     // per-warp totals of the offset scan
-  int32_t ctot[8];              // row-scan chunk totals
+  using Idx = typename std::conditional<CAP <= 256, uint8_t, uint16_t>::type;  // block-local index
+  uint32_t bits[tri_f(CAP - 1) + 8];
+  int32_t ids[2][CAP];    // merge rounds: the ids in run order
+  Idx ks[2][CAP];         // and the block-local index of each
+  Idx rank[CAP];          // rank of each block-local index
+  Idx perm[CAP];          // block-local index of each rank
+  Idx who[kFlatEntries];  // member of each flat entry
+  uint32_t rng[CAP];      // up to four slot ranges (first slot, length) of each member's group, packed
+  uint32_t rcum[CAP];     // cumulative lengths after ranges 0, 1, 2 (bytes)
+  uint8_t ncnt[CAP];      // entries of each member's group
+  uint8_t dk[CAP];        // block cell of each member
+  int64_t lbase[CAP];     // nbr_slot(member, 0) with the slot's in-row part removed
+  uint8_t dtab[8][64];    // partner cell of (member cell, stencil code); 8: not in the block
+  int32_t off[CAP + 1];   // first flat entry of each member
+  uint16_t rowbase[CAP];  // first word of each row of the bitmap
+  int32_t wtot[8];        // per-warp totals of the offset scan
+  int32_t ctot[CAP / 32]; // row-scan chunk totals
   int32_t cstart[8], cbase[9], koff[9];
   int32_t nb, big;
 };
 
-__global__ void __launch_bounds__(kEnumThreads)
-    k_sched_enum(Consts c, const int32_t* __restrict__ pid, const int32_t* __restrict__ cell_start,
-                 const int32_t* __restrict__ mrank, const uint32_t* __restrict__ nlist,
-                 const int32_t* __restrict__ nn, const uint32_t* __restrict__ cend, uint32_t* __restrict__ hdr,
-                 uint16_t* __restrict__ canon, uint32_t* __restrict__ blk_hist, uint32_t* __restrict__ big_count,
-                 unsigned long long* __restrict__ sched_total) {
-  __shared__ EnumSmem sm;
+// Outcome of an enumeration that gives no list.
+enum : int { kEnumParticles = -1, kEnumPairs = -2, kEnumList = -3 };
+
+// Owned pairs of block o in canonical order by a thread block of THREADS
+// threads: emit(position, lower-ranked member, other member) per pair.
+// Returns their number, or kEnumParticles (more than CAP particles),
+// kEnumPairs (more than max_pairs pairs), kEnumList (a member's list
+// overflowed).  The same value on every thread.
+template <int CAP, int THREADS, class Emit>
+__device__ __forceinline__ int enum_block(EnumSmem<CAP>& sm, const Consts& c, int o, const int32_t* __restrict__ pid,
+                                          const int32_t* __restrict__ cell_start, const int32_t* __restrict__ mrank,
+                                          const uint32_t* __restrict__ nlist, const int32_t* __restrict__ nn,
+                                          const uint32_t* __restrict__ cend, int max_pairs, Emit emit) {
+  using Idx = typename EnumSmem<CAP>::Idx;
+  constexpr int kWarps = THREADS / 32;
+  static_assert(2 * THREADS >= CAP, "two rows and two members per thread");
   const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
-  if (blockIdx.x == 0) {  // what k_sched_rounds counts in: the depth histogram, the lists of blocks beyond capacity
-    if (t == 0) *sched_total = 0ull;
-    for (int k = t; k < 8 * 256; k += kEnumThreads) blk_hist[k] = 0u;
-    if (t < 16) big_count[t] = 0u;
-  }
-  const int o = blockIdx.x;  // owner cell (fewer than 2^31 cells)
   const int ox = o % c.nc[0], oy = (o / c.nc[0]) % c.nc[1], oz = o / (c.nc[0] * c.nc[1]);
   // the block's 8 cells: storage start, count and offset in the block
   if (t < 32) {
@@ -149,7 +155,7 @@ __global__ void __launch_bounds__(kEnumThreads)
       sm.koff[8] = -(1 << 30);  // a partner outside the block: out of range
     }
   }
-  for (int q = t; q < 8 * 64; q += kEnumThreads) {  // partner cell: member cell + (code - 1) per axis
+  for (int q = t; q < 8 * 64; q += THREADS) {  // partner cell: member cell + (code - 1) per axis
     const int dA = q >> 6, code = q & 63;
     int dB = 0;
     bool in = true;
@@ -163,25 +169,22 @@ __global__ void __launch_bounds__(kEnumThreads)
   }
   __syncthreads();
   const int nb = sm.nb;
-  if (nb > kMaxBlock) {  // beyond capacity: swept pair by pair (see kHdrBig)
-    if (t == 0) hdr[o] = kHdrBig;
-    return;
-  }
+  if (nb > CAP) return kEnumParticles;
   const int ntri = nb > 1 ? tri_f(nb - 1) : 0;  // words of the bitmap in use
-  for (int q = t; q < ntri; q += kEnumThreads) sm.bits[q] = 0u;
+  for (int q = t; q < ntri; q += THREADS) sm.bits[q] = 0u;
   int cb[9];
 #pragma unroll
   for (int u = 0; u < 9; ++u) cb[u] = sm.cbase[u];
   const int64_t N = c.N;
   // the members: id, and the slot ranges of the owner group in the list
-  for (int k = t; k < nb; k += kEnumThreads) {
+  for (int k = t; k < nb; k += THREADS) {
     int d = 0;
 #pragma unroll
     for (int u = 1; u < 8; ++u) d += (k >= cb[u]);
     const int g = sm.cstart[d] + (k - sm.cbase[d]);
     const int32_t id = __ldg(&pid[g]);
     sm.ids[0][k] = id;
-    sm.ks[0][k] = (uint8_t)k;
+    sm.ks[0][k] = (Idx)k;
     if (__ldg(&nn[g]) > c.nbr_cap) sm.big = 1;  // the list lost entries
     const unsigned ob = owner_bits(id);
     // per axis the cells of the group as indices [lo, hi) of the offsets
@@ -218,15 +221,12 @@ __global__ void __launch_bounds__(kEnumThreads)
     sm.lbase[k] = ((int64_t)(g >> 5) * (c.nbr_cap >> 2) << 7) + ((g & 31) << 2);
   }
   __syncthreads();
-  if (sm.big) {
-    if (t == 0) hdr[o] = kHdrBig;
-    return;
-  }
+  if (sm.big) return kEnumList;
   // the member of each flat entry of the chunk [E0, E0 + kFlatEntries), in
   // equal stretches per thread: one binary search for the stretch's first
   // entry, then a walk (members without entries are skipped)
   auto fill_who = [&](int E0) {
-    const int E = sm.off[nb], Ec = min(E - E0, kFlatEntries), per = (Ec + kEnumThreads - 1) / kEnumThreads;
+    const int E = sm.off[nb], Ec = min(E - E0, kFlatEntries), per = (Ec + THREADS - 1) / THREADS;
     const int e0 = E0 + t * per, e1 = min(E0 + Ec, e0 + per);
     if (e0 < e1) {
       int pos = 1, len = nb - 1;  // members 1 .. nb - 1 starting at or before e0
@@ -242,7 +242,7 @@ __global__ void __launch_bounds__(kEnumThreads)
           ++k;
           kend = sm.off[k] + sm.ncnt[k];
         }
-        sm.who[e - E0] = (uint8_t)k;
+        sm.who[e - E0] = (Idx)k;
       }
     }
   };
@@ -252,7 +252,7 @@ __global__ void __launch_bounds__(kEnumThreads)
 #pragma unroll 1
   for (int L = 0; L < 3; ++L) {
     const int src = L & 1, dst = src ^ 1;
-    for (int k = t; k < nb; k += kEnumThreads) {
+    for (int k = t; k < nb; k += THREADS) {
       const int d = sm.dk[k];
       const int run = d >> L, sib = run ^ 1;
       const int own0 = sm.cbase[run << L], m0 = sm.cbase[(run & ~1) << L];
@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(kEnumThreads)
     } else if (L == 1) {  // offsets in member order
       int before = 0, total = 0;
 #pragma unroll
-      for (int q = 0; q < kEnumWarps; ++q) {
+      for (int q = 0; q < kWarps; ++q) {
         before += q < wid ? sm.wtot[q] : 0;
         total += sm.wtot[q];
       }
@@ -295,12 +295,12 @@ __global__ void __launch_bounds__(kEnumThreads)
     }
     __syncthreads();
   }
-  for (int r = t; r < nb; r += kEnumThreads) {  // the merged run is ids[1]
+  for (int r = t; r < nb; r += THREADS) {  // the merged run is ids[1]
     const int k = sm.ks[1][r];
-    sm.perm[r] = (uint8_t)k;
-    sm.rank[k] = (uint8_t)r;
+    sm.perm[r] = (Idx)k;
+    sm.rank[k] = (Idx)r;
   }
-  for (int d = 1 + t; d < nb; d += kEnumThreads)  // row d of the bitmap starts at F(nb - 1) - F(nb - d)
+  for (int d = 1 + t; d < nb; d += THREADS)  // row d of the bitmap starts at F(nb - 1) - F(nb - d)
     sm.rowbase[d] = (uint16_t)(tri_f(nb - 1) - tri_f(nb - d));
   __syncthreads();
   // the flat entries: partner, rank test, bit; chunk by chunk (a block with
@@ -313,7 +313,7 @@ __global__ void __launch_bounds__(kEnumThreads)
     }
     const int E1 = min(E, E0 + kFlatEntries);
 #pragma unroll 4
-    for (int e = E0 + t; e < E1; e += kEnumThreads) {
+    for (int e = E0 + t; e < E1; e += THREADS) {
       const int A = sm.who[e - E0];
       const int m = e - sm.off[A];
       const uint32_t rng = sm.rng[A], cum = sm.rcum[A];
@@ -337,7 +337,7 @@ __global__ void __launch_bounds__(kEnumThreads)
   int rowex[2] = {0, 0};
 #pragma unroll
   for (int it = 0; it < 2; ++it) {
-    const int r0 = 1 + 32 * wid + it * kEnumThreads;
+    const int r0 = 1 + 32 * wid + it * THREADS;
     if (r0 >= nb) break;
     const int rr = r0 + lane;
     int n = 0;
@@ -358,15 +358,11 @@ __global__ void __launch_bounds__(kEnumThreads)
   const int nchunk = (nb - 1 + 31) >> 5;
   int npairs = 0;
   for (int ch = 0; ch < nchunk; ++ch) npairs += sm.ctot[ch];
-  if (npairs > kMaxPairs) {
-    if (t == 0) hdr[o] = kHdrBig;
-    return;
-  }
+  if (npairs > max_pairs) return kEnumPairs;
   // write the pairs row by row (difference ascending), lower rank ascending
-  uint16_t* out = canon + (int64_t)o * kMaxPairs;
 #pragma unroll
   for (int it = 0; it < 2; ++it) {
-    const int rr = 1 + t + it * kEnumThreads;
+    const int rr = 1 + t + it * THREADS;
     if (rr >= nb) break;
     const int chunk = (rr - 1) >> 5;
     int pos = rowex[it];
@@ -378,11 +374,36 @@ __global__ void __launch_bounds__(kEnumThreads)
         const int bit = __ffs(bits) - 1;
         bits &= bits - 1;
         const int lo = w * 32 + bit;
-        out[pos++] = (uint16_t)(sm.perm[lo] | (sm.perm[lo + rr] << 8));
+        emit(pos++, (int)sm.perm[lo], (int)sm.perm[lo + rr]);
       }
     }
   }
-  if (t == 0) hdr[o] = (uint32_t)npairs;
+  return npairs;
+}
+
+// The schedule's first launch: one thread block per block of cells.
+__global__ void __launch_bounds__(kEnumThreads)
+    k_sched_enum(const __grid_constant__ Consts c, const int32_t* __restrict__ pid,
+                 const int32_t* __restrict__ cell_start, const int32_t* __restrict__ mrank,
+                 const uint32_t* __restrict__ nlist, const int32_t* __restrict__ nn,
+                 const uint32_t* __restrict__ cend, uint32_t* __restrict__ hdr, uint16_t* __restrict__ canon,
+                 uint32_t* __restrict__ blk_hist, uint32_t* __restrict__ big_count, uint32_t* __restrict__ large_count,
+                 int32_t* __restrict__ large_cand, unsigned long long* __restrict__ sched_total) {
+  __shared__ EnumSmem<kMaxBlock> sm;
+  const int t = threadIdx.x, o = blockIdx.x;  // owner cell (fewer than 2^31 cells)
+  if (o == 0) {  // what the next launches count in: depth histogram, lists, dense pair arrays
+    if (t == 0) *sched_total = 0ull;
+    for (int k = t; k < 8 * 256; k += kEnumThreads) blk_hist[k] = 0u;
+    if (t < 16) big_count[t] = 0u;
+    if (t < 8) large_count[t] = 0u;
+  }
+  uint16_t* out = canon + (int64_t)o * kMaxPairs;
+  const int np = enum_block<kMaxBlock, kEnumThreads>(
+      sm, c, o, pid, cell_start, mrank, nlist, nn, cend, kMaxPairs,
+      [&](int pos, int lo, int hi) { out[pos] = (uint16_t)(lo | (hi << 8)); });
+  if (t != 0) return;
+  hdr[o] = np >= 0 ? (uint32_t)np : (np == kEnumList ? kHdrBig : kHdrLarge);
+  if (np == kEnumParticles || np == kEnumPairs) large_cand[atomicAdd(&large_count[8], 1u)] = o;
 }
 
 // Rounds: one warp per block takes the block's canonical list 32 pairs at a
@@ -402,40 +423,80 @@ __global__ void __launch_bounds__(kEnumThreads)
 // of ~190 cycles each).
 constexpr int kRoundWarps = 4;
 
+template <int CAP, int MAXP>
 struct RoundSmem {
-  uint32_t claim[kMaxBlock];
-  uint32_t cnt[kMaxLevels + 1];
-  uint16_t place[kMaxPairs];  // round << 5 | place in the round
-  uint8_t last[kMaxBlock];    // first round in which a particle is free
+  uint32_t claim[CAP];
+  uint32_t cnt[kRoundStride];
+  uint16_t place[MAXP];  // round << 5 | place in the round
+  uint8_t last[CAP];     // first round in which a particle is free
 };
 
-__global__ void __launch_bounds__(kRoundWarps * 32)
-    k_sched_rounds(int64_t ncell, int nc0, int nc1, int nc2, int width, uint32_t* __restrict__ hdr,
-                   const uint16_t* __restrict__ canon, uint8_t* __restrict__ rsize,
-                   unsigned long long* __restrict__ off, unsigned long long* __restrict__ total,
-                   unsigned long long cap, uint16_t* __restrict__ pairs, uint32_t* __restrict__ blk_hist,
-                   const int32_t* __restrict__ cell_start, const int32_t* __restrict__ mrank,
-                   uint32_t* __restrict__ big_count, int2* __restrict__ big_list) {
-  __shared__ RoundSmem sm_all[kRoundWarps];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t o = (int64_t)blockIdx.x * kRoundWarps + warp;
-  if (o >= ncell) return;
-  RoundSmem& sm = sm_all[warp];
-  const uint32_t hd = hdr[o];
-  bool big = hd == kHdrBig;
-  const int np = big ? 0 : (int)(hd & 0xffffu);
-  for (int k = lane; k < kMaxBlock; k += 32) sm.claim[k] = 0xffffffffu;
-  for (int k = lane; k <= kMaxLevels; k += 32) sm.cnt[k] = 0u;
-  for (int k = lane; k < kMaxBlock / 4; k += 32) reinterpret_cast<uint32_t*>(sm.last)[k] = 0u;
+// The dense arrays and lists a schedule is written to.
+struct SchedOut {
+  int64_t ncell;
+  int nc[3];
+  unsigned long long cap;  // entries of the dense pair arrays
+  uint32_t* hdr;
+  uint8_t* rsize;
+  unsigned long long* off;
+  unsigned long long* total;
+  uint32_t* pairs;
+  uint32_t* blk_hist;
+  const int32_t* cell_start;
+  const int32_t* mrank;
+  uint32_t* big_count;
+  int2* big_list;
+};
+
+// the block's colour is the parity pattern of its owner cell
+__device__ __forceinline__ int block_colour(const int nc[3], int64_t o, int& ox, int& oy, int& oz) {
+  ox = (int)(o % nc[0]);
+  oy = (int)((o / nc[0]) % nc[1]);
+  oz = (int)(o / ((int64_t)nc[0] * nc[1]));
+  return (ox & 1) | ((oy & 1) << 1) | ((oz & 1) << 2);
+}
+
+// One thread: block o goes pair by pair after its colour's other blocks,
+// listed with the place of its particles in big_perm (blocks of a colour are
+// disjoint).
+__device__ __noinline__ void list_big(const SchedOut& out, int64_t o) {
+  int ox, oy, oz;
+  const int colour = block_colour(out.nc, o, ox, oy, oz);
+  out.hdr[o] = kHdrBig;
+  int nb = 0;
+  for (int d = 0; d < 8; ++d) {
+    int cx = ox + (d & 1), cy = oy + ((d >> 1) & 1), cz = oz + ((d >> 2) & 1);
+    if (cx >= out.nc[0]) cx -= out.nc[0];
+    if (cy >= out.nc[1]) cy -= out.nc[1];
+    if (cz >= out.nc[2]) cz -= out.nc[2];
+    const int r = out.mrank[cx + out.nc[0] * (cy + out.nc[1] * cz)];
+    nb += out.cell_start[r + 1] - out.cell_start[r];
+  }
+  const uint32_t first = atomicAdd(&out.big_count[8 + colour], (uint32_t)nb);
+  const uint32_t slot = atomicAdd(&out.big_count[colour], 1u);
+  out.big_list[colour * (out.ncell >> 3) + slot] = make_int2((int)o, (int)first);
+  atomicAdd(&out.blk_hist[colour * 256 + kMaxLevels], 1u);
+}
+
+// The rounds of block o's canonical list (np pairs, in(k) = lower | other <<
+// 16 for pair k) by one warp, written to the dense arrays; flag is or-ed into
+// the header.  False: more rounds than kMaxLevels, or the dense arrays are
+// full (their capacity covers every schedule of symmetric lists).
+template <int CAP, int MAXP, class In>
+__device__ __forceinline__ bool assign_rounds(RoundSmem<CAP, MAXP>& sm, const SchedOut& out, int64_t o, int np,
+                                              int width, uint32_t flag, In in) {
+  const int lane = threadIdx.x & 31;
+  for (int k = lane; k < CAP; k += 32) sm.claim[k] = 0xffffffffu;
+  for (int k = lane; k < kRoundStride; k += 32) sm.cnt[k] = 0u;
+  for (int k = lane; k < CAP / 4; k += 32) reinterpret_cast<uint32_t*>(sm.last)[k] = 0u;
   __syncwarp();
-  const uint16_t* in = canon + o * kMaxPairs;
   int full = 0;  // rounds below are full
   bool overflow = false;
-  uint16_t nxt = lane < np ? in[lane] : (uint16_t)0;
+  uint32_t nxt = lane < np ? in(lane) : 0u;
   for (int k0 = 0; k0 < np; k0 += 32) {
-    const uint16_t pr = nxt;
-    if (k0 + 32 + lane < np) nxt = in[k0 + 32 + lane];
-    const int u = pr & 255, v = pr >> 8;
+    const uint32_t pr = nxt;
+    if (k0 + 32 + lane < np) nxt = in(k0 + 32 + lane);
+    const int u = pr & 0xffffu, v = pr >> 16;
     bool pending = k0 + lane < np;
     while (__any_sync(0xffffffffu, pending)) {
       if (pending) {
@@ -460,41 +521,13 @@ __global__ void __launch_bounds__(kRoundWarps * 32)
       }
       __syncwarp();
     }
-    if (__any_sync(0xffffffffu, overflow)) break;
+    if (__any_sync(0xffffffffu, overflow)) return false;
     while (full < kMaxLevels && sm.cnt[full] >= (uint32_t)width) ++full;
   }
-  big = big || __any_sync(0xffffffffu, overflow);
-  __syncwarp();
-  // the block's place in the dense pair arrays (their capacity covers every
-  // schedule; a block past it would be swept pair by pair)
   unsigned long long at = 0ull;
-  if (!big && lane == 0) at = atomicAdd(total, (unsigned long long)((np + 7) & ~7));
+  if (lane == 0) at = atomicAdd(out.total, (unsigned long long)((np + 7) & ~7));
   at = __shfl_sync(0xffffffffu, at, 0);
-  big = big || at + (unsigned long long)np > cap;
-  // the block's colour is the parity pattern of its owner cell
-  const int ox = (int)(o % nc0), oy = (int)((o / nc0) % nc1), oz = (int)(o / ((int64_t)nc0 * nc1));
-  const int colour = (ox & 1) | ((oy & 1) << 1) | ((oz & 1) << 2);
-  if (big) {
-    // swept pair by pair after the colour's other blocks: listed with the
-    // place of its particles in big_perm (blocks of a colour are disjoint)
-    if (lane == 0) {
-      hdr[o] = kHdrBig;
-      int nb = 0;
-      for (int d = 0; d < 8; ++d) {
-        int cx = ox + (d & 1), cy = oy + ((d >> 1) & 1), cz = oz + ((d >> 2) & 1);
-        if (cx >= nc0) cx -= nc0;
-        if (cy >= nc1) cy -= nc1;
-        if (cz >= nc2) cz -= nc2;
-        const int r = mrank[cx + nc0 * (cy + nc1 * cz)];
-        nb += cell_start[r + 1] - cell_start[r];
-      }
-      const uint32_t first = atomicAdd(&big_count[8 + colour], (uint32_t)nb);
-      const uint32_t slot = atomicAdd(&big_count[colour], 1u);
-      big_list[colour * (ncell >> 3) + slot] = make_int2((int)o, (int)first);
-      atomicAdd(&blk_hist[colour * 256 + kMaxLevels], 1u);
-    }
-    return;
-  }
+  if (at + (unsigned long long)np > out.cap) return false;
   // round sizes and their first positions: 8 consecutive rounds per lane
   // (rounds are contiguous: a pair enters round L > 0 only after a pair in
   // round L - 1 or because that round is full)
@@ -514,24 +547,116 @@ __global__ void __launch_bounds__(kRoundWarps * 32)
   }
   nr = __reduce_add_sync(0xffffffffu, nr);
   if (lane == 0) {
-    off[o] = at;
-    hdr[o] = (uint32_t)np | ((uint32_t)nr << 16);
-    atomicAdd(&blk_hist[colour * 256 + nr], 1u);
+    int ox, oy, oz;
+    out.off[o] = at;
+    out.hdr[o] = (uint32_t)np | ((uint32_t)nr << 16) | flag;
+    atomicAdd(&out.blk_hist[block_colour(out.nc, o, ox, oy, oz) * 256 + nr], 1u);
   }
   int run = incl - sum;
   uint32_t packed[2] = {0u, 0u};
+  __syncwarp();
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
     packed[q >> 2] |= (uint32_t)v[q] << (8 * (q & 3));
     sm.cnt[lane * 8 + q] = (uint32_t)run;
     run += v[q];
   }
-  if (lane * 8 < nr) reinterpret_cast<uint2*>(rsize + o * kRoundStride)[lane] = make_uint2(packed[0], packed[1]);
+  if (lane * 8 < nr) reinterpret_cast<uint2*>(out.rsize + o * kRoundStride)[lane] = make_uint2(packed[0], packed[1]);
   __syncwarp();
 #pragma unroll 4
   for (int k = lane; k < np; k += 32) {
     const int pl = sm.place[k];
-    pairs[at + sm.cnt[pl >> 5] + (pl & 31)] = in[k];
+    out.pairs[at + sm.cnt[pl >> 5] + (pl & 31)] = in(k);
+  }
+  return true;
+}
+
+__global__ void __launch_bounds__(kRoundWarps * 32)
+    k_sched_rounds(const __grid_constant__ SchedOut out, int width, const uint16_t* __restrict__ canon) {
+  __shared__ RoundSmem<kMaxBlock, kMaxPairs> sm_all[kRoundWarps];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t o = (int64_t)blockIdx.x * kRoundWarps + warp;
+  if (o >= out.ncell) return;
+  const uint32_t hd = out.hdr[o];
+  if (hd == kHdrLarge) return;  // k_sched_large
+  const uint16_t* in = canon + o * kMaxPairs;
+  const bool ok = hd != kHdrBig &&
+                  assign_rounds(sm_all[warp], out, o, (int)hd, width, 0u, [&](int k) {
+                    const uint32_t pr = __ldg(&in[k]);
+                    return (pr & 255u) | (pr >> 8) << 16;
+                  });
+  if (!ok && lane == 0) list_big(out, o);
+}
+
+// ---------------------------------------------------------------------------
+// Large blocks: more particles or owned pairs than k_sched_enum holds, as in
+// boxes whose side lies between two cell counts (14 / 2.5: cells of 3.5,
+// blocks of 343).  One thread block takes them in turn, pairs and rounds with
+// the list in shared memory.  (Swept pair by pair on one lane they took 40 ms
+// per sweep of 14^3 particles.)  width: as k_sched_rounds.  The last thread
+// block then turns the depth histogram into each depth's first position,
+// deepest first (one warp per colour; see below).
+// ---------------------------------------------------------------------------
+struct LargeSmem {
+  EnumSmem<kLargeBlock> e;
+  RoundSmem<kLargeBlock, kLargePairs> r;
+  uint32_t canon[kLargePairs];
+  int np;
+  uint32_t last;
+};
+
+__global__ void __launch_bounds__(kLargeThreads)
+    k_sched_large(const __grid_constant__ Consts c, const __grid_constant__ SchedOut out, int width,
+                  const int32_t* __restrict__ pid, const uint32_t* __restrict__ nlist, const int32_t* __restrict__ nn,
+                  const uint32_t* __restrict__ cend, const int32_t* __restrict__ cand,
+                  uint32_t* __restrict__ large_count, int32_t* __restrict__ large_list) {
+  extern __shared__ __align__(16) unsigned char large_smem_raw[];
+  LargeSmem& sm = *reinterpret_cast<LargeSmem*>(large_smem_raw);
+  const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+  const int n = (int)large_count[8];
+  for (int q = blockIdx.x; q < n; q += gridDim.x) {
+    const int o = cand[q];
+    const int np = enum_block<kLargeBlock, kLargeThreads>(
+        sm.e, c, o, pid, out.cell_start, out.mrank, nlist, nn, cend, kLargePairs,
+        [&](int pos, int lo, int hi) { sm.canon[pos] = (uint32_t)lo | (uint32_t)hi << 16; });
+    __syncthreads();
+    if (wid == 0) {
+      const bool ok = np >= 0 && assign_rounds(sm.r, out, o, np, width, kHdrLargeFlag, [&](int k) { return sm.canon[k]; });
+      if (lane == 0) {
+        int ox, oy, oz;
+        const int colour = block_colour(out.nc, o, ox, oy, oz);
+        if (ok) large_list[colour * (out.ncell >> 3) + atomicAdd(&large_count[colour], 1u)] = o;
+        else list_big(out, o);
+      }
+    }
+    __syncthreads();
+  }
+  if (t == 0) {
+    __threadfence();
+    sm.last = atomicAdd(&large_count[9], 1u) == gridDim.x - 1u;
+  }
+  __syncthreads();
+  if (!sm.last) return;
+  __threadfence();
+  // place k of warp `wid`'s colour is depth 255 - k, eight places per lane
+  uint32_t* h = out.blk_hist + wid * 256;
+  uint32_t v[8], sum = 0;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    v[q] = __ldcg(&h[255 - (lane * 8 + q)]);
+    sum += v[q];
+  }
+  uint32_t incl = sum;
+#pragma unroll
+  for (int sh = 1; sh < 32; sh <<= 1) {
+    const uint32_t x = __shfl_up_sync(0xffffffffu, incl, sh);
+    if (lane >= sh) incl += x;
+  }
+  uint32_t run = incl - sum;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    h[255 - (lane * 8 + q)] = run;
+    run += v[q];
   }
 }
 
@@ -541,32 +666,13 @@ __global__ void __launch_bounds__(kRoundWarps * 32)
 // deepest, so neighbours in this order have similar depth, and the deep
 // blocks start first, which keeps the launch's tail short.  Blocks of a colour
 // are independent, so the order changes no result.
-// Step 1 (8 thread blocks of 256, one per colour): the depth histogram turned
-// into each depth's first position, deepest first.
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_sched_order_scan(uint32_t* __restrict__ blk_hist) {
-  __shared__ uint32_t warp_sum[8];
-  const int t = threadIdx.x, lane = t & 31, wp = t >> 5;
-  uint32_t* h = blk_hist + blockIdx.x * 256;
-  const uint32_t v = h[255 - t];  // thread t takes depth 255 - t
-  uint32_t incl = v;
-#pragma unroll
-  for (int sh = 1; sh < 32; sh <<= 1) {
-    const uint32_t x = __shfl_up_sync(0xffffffffu, incl, sh);
-    if (lane >= sh) incl += x;
-  }
-  if (lane == 31) warp_sum[wp] = incl;
-  __syncthreads();
-  uint32_t before = 0;
-  for (int k = 0; k < wp; ++k) before += warp_sum[k];
-  __syncthreads();
-  h[255 - t] = before + incl - v;
-}
-
-// Step 2 (one thread per owner cell): each block's place in its colour's
-// order, by depth; the order among blocks of equal depth is free.
+// One thread per owner cell: each block's place in its colour's order, by
+// depth (from the positions that k_sched_large left in the histogram); the
+// order among blocks of equal depth is free.
 __global__ void k_sched_order_scatter(int64_t ncell, int nc0, int nc1, const uint32_t* __restrict__ hdr,
-                                      uint32_t* __restrict__ blk_hist, int32_t* __restrict__ blk_order) {
+                                      uint32_t* __restrict__ blk_hist, int32_t* __restrict__ blk_order,
+                                      uint32_t* __restrict__ large_count) {
+  if (blockIdx.x == 0 && threadIdx.x < 2) large_count[8 + threadIdx.x] = 0u;  // for the next schedule
   const int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (o >= ncell) return;
   const int ox = (int)(o % nc0), oy = (int)((o / nc0) % nc1), oz = (int)(o / ((int64_t)nc0 * nc1));
@@ -574,24 +680,48 @@ __global__ void k_sched_order_scatter(int64_t ncell, int nc0, int nc1, const uin
   const int hx = nc0 >> 1, hy = nc1 >> 1;
   const int32_t w = (ox >> 1) + hx * ((oy >> 1) + hy * (oz >> 1));  // index among the colour's blocks
   const uint32_t hd = hdr[o];
-  const int nlev = hd == kHdrBig ? kMaxLevels : (int)(hd >> 16);
+  const int nlev = hd == kHdrBig ? kMaxLevels : (int)(hd >> 16 & 255u);
   const uint32_t pos = atomicAdd(&blk_hist[colour * 256 + nlev], 1u);
   blk_order[colour * (ncell >> 3) + pos] = w;
 }
 
 template <class P>
-void launch_fd_schedule(const Consts& c, const Workspace& w, int cur, int width, cudaStream_t s) {
+void launch_fd_schedule(const Consts& c, const Workspace& w, int cur, int width, int large_width, cudaStream_t s) {
   if (c.N == 0) return;
   Arrays<P> a = view<P>(w, cur);
+  SchedOut out;
+  out.ncell = c.ncell;
+  for (int d = 0; d < 3; ++d) out.nc[d] = c.nc[d];
+  out.cap = (unsigned long long)sched_pair_capacity(c.N, c.nbr_cap, c.ncell);
+  out.hdr = w.sched_hdr;
+  out.rsize = w.sched_rsize;
+  out.off = w.sched_off;
+  out.total = w.sched_total;
+  out.pairs = w.sched_pair;
+  out.blk_hist = w.blk_hist;
+  out.cell_start = w.cell_start;
+  out.mrank = w.mrank;
+  out.big_count = w.big_count;
+  out.big_list = w.big_list;
   k_sched_enum<<<(unsigned)c.ncell, kEnumThreads, 0, s>>>(c, a.id, w.cell_start, w.mrank, w.nlist, w.nn, w.cend,
-                                                          w.sched_hdr, w.sched_canon, w.blk_hist, w.big_count,
-                                                          w.sched_total);
-  k_sched_rounds<<<(unsigned)((c.ncell + kRoundWarps - 1) / kRoundWarps), kRoundWarps * 32, 0, s>>>(
-      c.ncell, c.nc[0], c.nc[1], c.nc[2], width, w.sched_hdr, w.sched_canon, w.sched_rsize, w.sched_off,
-      w.sched_total, (unsigned long long)sched_pair_capacity(c.N, c.nbr_cap, c.ncell), w.sched_pair, w.blk_hist, w.cell_start, w.mrank, w.big_count, w.big_list);
-  k_sched_order_scan<<<8, 256, 0, s>>>(w.blk_hist);
+                                                          w.sched_hdr, w.sched_canon, w.blk_hist, w.big_count, w.large_count,
+                                                          w.large_cand, w.sched_total);
+  k_sched_rounds<<<(unsigned)((c.ncell + kRoundWarps - 1) / kRoundWarps), kRoundWarps * 32, 0, s>>>(out, width,
+                                                                                                   w.sched_canon);
+  // (a large block has a whole warp of the colour launch, or its team)
+  k_sched_large<<<(unsigned)std::min(c.ncell, 152), kLargeThreads, sizeof(LargeSmem), s>>>(
+      c, out, std::max(width, large_width), a.id, w.nlist, w.nn, w.cend, w.large_cand, w.large_count, w.large_list);
   k_sched_order_scatter<<<(unsigned)((c.ncell + 255) / 256), 256, 0, s>>>(c.ncell, c.nc[0], c.nc[1], w.sched_hdr,
-                                                                         w.blk_hist, w.blk_order);
+                                                                         w.blk_hist, w.blk_order, w.large_count);
+}
+
+// Launch attributes of the schedule's kernels (once per device and process;
+// kept out of stream captures).
+int sched_prepare() {
+  return cudaFuncSetAttribute(k_sched_large, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(LargeSmem)) ==
+                 cudaSuccess
+             ? SDPD_OK
+             : SDPD_ERR_CUDA;
 }
 
 __global__ void k_sweep_set(unsigned long long* sweep, unsigned long long v) { *sweep = v; }
@@ -602,7 +732,7 @@ void launch_set_sweep(const Workspace& w, unsigned long long value, cudaStream_t
 }
 void launch_advance_sweep(const Workspace& w, cudaStream_t s) { k_sweep_advance<<<1, 1, 0, s>>>(w.sweep); }
 
-template void launch_fd_schedule<Fp64>(const Consts&, const Workspace&, int, int, cudaStream_t);
-template void launch_fd_schedule<Mixed>(const Consts&, const Workspace&, int, int, cudaStream_t);
+template void launch_fd_schedule<Fp64>(const Consts&, const Workspace&, int, int, int, cudaStream_t);
+template void launch_fd_schedule<Mixed>(const Consts&, const Workspace&, int, int, int, cudaStream_t);
 
 }  // namespace sdpd

@@ -445,24 +445,15 @@ __device__ __forceinline__ int block_code(T w, int ox, int oy, int oz) {
   return (cx != ox) | ((cy != oy) << 1) | ((cz != oz) << 2);
 }
 
-// Shared memory of one block in a colour launch: momenta and energy of each
-// particle in one record (so a pair reads two records with wide loads).
-// float64 pair arithmetic: (p, eps).  float32: (p, es) with es the energy at
-// load rounded to float32 plus the visit's changes, and its compensation ec
-// (the rounding errors of that sum and the low parts of the changes), so
-// that the energy is eps(load) + (es - (float)eps(load)) + ec.
 struct FdCells {
   int32_t cst[8], cbs[8];  // the block's cells: first storage index, offset in the block
 };
-template <class R>
-struct FdSmem;
-template <>
-struct FdSmem<double> {
-  D4 s[kMaxBlock];
-  FdCells cells;
-};
-template <>
-struct FdSmem<float> {
+// Shared memory of one block in a colour launch with float32 pair arithmetic:
+// each particle's record (px, py, pz, es), es the energy at load rounded to
+// float32 plus the visit's changes (one wide load per particle and pair), and
+// its compensation ec (the rounding errors of that sum and the low parts of
+// the changes), so that the energy is eps(load) + (es - (float)eps(load)) + ec.
+struct FdSmem {
   F4 s[kMaxBlock];
   float ec[kMaxBlock];
   FdCells cells;
@@ -549,7 +540,7 @@ __global__ void __launch_bounds__(kStageWarps * 32)
                      const int32_t* __restrict__ mrank, const uint32_t* __restrict__ xmx,
                      const uint32_t* __restrict__ xmy, const uint32_t* __restrict__ xmz,
                      const uint32_t* __restrict__ hdr, const unsigned long long* __restrict__ sched_off,
-                     const uint16_t* __restrict__ pairs, typename A::V4* __restrict__ geom) {
+                     const uint32_t* __restrict__ pairs, typename A::V4* __restrict__ geom) {
   using R = typename A::R;
   using S = typename P::R;
   __shared__ FdCells cells_s[kStageWarps];
@@ -568,9 +559,9 @@ __global__ void __launch_bounds__(kStageWarps * 32)
   const S inv_h = (S)(1.0 / c.h), cF = (S)c.cF;
   const unsigned long long base = sched_off[o];
   for (int t = lane; t < np; t += 32) {
-    const uint16_t pr = pairs[base + t];
+    const uint32_t pr = pairs[base + t];
     int da, db;
-    const int ga = block_gidx(cells, pr & 255, da), gb = block_gidx(cells, pr >> 8, db);
+    const int ga = block_gidx(cells, pr & 0xffffu, da), gb = block_gidx(cells, pr >> 16, db);
     S xa, ya, za, xb, yb, zb, rx, ry, rz;
     // positions and densities of the latest density pass (one load each)
     const typename P::V4 qa = ld4(&qr4[ga]), qb = ld4(&qr4[gb]);
@@ -598,7 +589,7 @@ template <class A>
 __global__ void __launch_bounds__(kStageWarps * 32)
     k_stage_random(Consts c, const int32_t* __restrict__ id, const int32_t* __restrict__ cell_start,
                    const int32_t* __restrict__ mrank, const uint32_t* __restrict__ hdr,
-                   const unsigned long long* __restrict__ sched_off, const uint16_t* __restrict__ pairs,
+                   const unsigned long long* __restrict__ sched_off, const uint32_t* __restrict__ pairs,
                    uint64_t seed, const unsigned long long* __restrict__ sweep_ptr,
                    const typename A::V4* __restrict__ geom, typename A::V4* __restrict__ rnd,
                    double* __restrict__ aux) {
@@ -615,8 +606,8 @@ __global__ void __launch_bounds__(kStageWarps * 32)
   const uint64_t sweep = *sweep_ptr;
   const unsigned long long base = sched_off[o];
   for (int t = lane; t < np; t += 32) {
-    const uint16_t pr = pairs[base + t];
-    const int ga = block_gidx(cells, pr & 255), gb = block_gidx(cells, pr >> 8);  // pr & 255 holds the lower id
+    const uint32_t pr = pairs[base + t];
+    const int ga = block_gidx(cells, pr & 0xffffu), gb = block_gidx(cells, pr >> 16);  // ga holds the lower id
     R G[3], U;
     pair_randoms_fast(seed, sweep, (uint64_t)id[ga], (uint64_t)id[gb], G, &U);
     typename A::V4 v;
@@ -634,7 +625,8 @@ __global__ void __launch_bounds__(kStageWarps * 32)
 }
 
 // A block beyond the capacities of the shared-memory schedule (kHdrBig: more
-// than kMaxBlock particles, kMaxPairs owned pairs or kMaxLevels levels).
+// than kLargeBlock particles, kLargePairs owned pairs or kMaxLevels rounds, or
+// a member whose neighbour list overflowed its row).
 // The whole warp sweeps its owned pairs in canonical order, one pair after
 // the other, on the state in global memory; slow, but any block completes
 // with the result of the sequential sweep.  The block's particles in rank
@@ -802,11 +794,11 @@ __device__ __noinline__ BigCounts fd_big_block(const Consts& c, const FDConst<ty
 // stored energies plus the visit's changes.  The pair's uniform drawn again.
 // Both serve the rare float64 decisions (near ties of the bound or the
 // ratio) and are kept out of the hot loop.
-static __device__ __noinline__ void fd_exact_energies(const double* eps, const FdSmem<float>& sm, int ia, int ib,
-                                                      float eaf, float ebf, double& ea, double& eb) {
-  const double ga = eps[block_gidx(sm.cells, ia)], gb = eps[block_gidx(sm.cells, ib)];
-  ea = ga + (((double)eaf - (double)(float)ga) + (double)sm.ec[ia]);
-  eb = gb + (((double)ebf - (double)(float)gb) + (double)sm.ec[ib]);
+static __device__ __noinline__ void fd_exact_energies(const double* eps, const FdCells& cells, const float* ec, int ia,
+                                                      int ib, float eaf, float ebf, double& ea, double& eb) {
+  const double ga = eps[block_gidx(cells, ia)], gb = eps[block_gidx(cells, ib)];
+  ea = ga + (((double)eaf - (double)(float)ga) + (double)ec[ia]);
+  eb = gb + (((double)ebf - (double)(float)gb) + (double)ec[ib]);
 }
 static __device__ __noinline__ float fd_uniform_again(uint64_t seed, uint64_t sweep, int32_t ida, int32_t idb) {
   float G[3], U;
@@ -827,189 +819,336 @@ static __device__ __noinline__ float fd_uniform_again(uint64_t seed, uint64_t sw
 // visit.  REC: keep a record per pair (every Metropolis margin in float64).
 // Thread blocks of 1 to 4 warps, 128 registers per thread (16 warps per SM).
 // ---------------------------------------------------------------------------
-template <class P, class A, int OPW, bool REC>
-__global__ void __launch_bounds__(128, 4)
-    k_fd_colour(Consts c, FDConst<typename A::R> k, Arrays<P> a, typename P::V4* __restrict__ qp4,
-                const int32_t* __restrict__ cell_start, const int32_t* __restrict__ mrank,
-                const uint32_t* __restrict__ xmx, const uint32_t* __restrict__ xmy,
-                const uint32_t* __restrict__ xmz, const uint32_t* __restrict__ hdr,
-                const uint8_t* __restrict__ rsize, const unsigned long long* __restrict__ sched_off,
-                const uint16_t* __restrict__ pairs, const typename A::V4* __restrict__ geom,
-                const typename A::V4* __restrict__ rnd, int colour, uint64_t seed,
-                unsigned long long* __restrict__ sweep_ptr, unsigned long long* counters, int* status,
-                sdpd_pair_rec* recs, unsigned long long* rec_count, int64_t rec_cap, unsigned* __restrict__ queue,
-                const int32_t* __restrict__ order, int32_t* __restrict__ big_perm,
-                const int2* __restrict__ big_list, const uint32_t* __restrict__ big_count) {
-  using R = typename A::R;  // pair arithmetic
+// What the lanes of a colour launch count.
+struct FdTally {
+  unsigned n_tot = 0, n_rb = 0, n_rm = 0;  // pairs, rejections (accepted = pairs - rejected)
+  bool negative = false, bad = false;
+};
+
+// Launch-wide arguments of the block runs.
+template <class P>
+struct FdRun {
+  Consts c;
+  FDConst<float> k;
+  Arrays<P> a;
+  typename P::V4* qp4;
+  const int32_t *cell_start, *mrank;
+  const uint32_t *xmx, *xmy, *xmz;
+  const uint32_t* hdr;
+  const uint8_t* rsize;
+  const unsigned long long* sched_off;
+  const uint32_t* pairs;
+  const F4 *geom, *rnd;
+  int colour;
+  uint64_t seed;
+  unsigned long long* sweep_ptr;
+  unsigned long long* counters;
+  int* status;
+  sdpd_pair_rec* recs;
+  unsigned long long* rec_count;
+  int64_t rec_cap;
+  unsigned* queue;
+  const int32_t* order;
+  int32_t* big_perm;
+  const int2* big_list;
+  const uint32_t* big_count;
+  const int32_t* large_list;
+  const uint32_t* large_count;
+};
+
+// Runs one block per group of GL lanes (live: this group has one, of owner
+// cell o with header hd): state into shared memory (s, ec, cells), the rounds,
+// state back.  All lanes of the warp take part.
+template <class P, int GL, bool REC>
+__device__ __forceinline__ void fd_run_block(const FdRun<P>& f, bool live, int64_t o, int ox, int oy, int oz,
+                                             uint32_t hd, uint64_t sweep, F4* s, float* ec, FdCells& cells,
+                                             FdTally& tally) {
   using S = typename P::R;  // stored momenta, densities, geometry
-  using AV4 = typename A::V4;
-  static_assert(A::mixed, "float64 pair arithmetic runs k_fd_colour64");
-  constexpr bool kSame = std::is_same<R, S>::value;
-  constexpr int kGroupLanes = 32 / OPW;
+  constexpr bool kSame = std::is_same<S, float>::value;
+  const Consts& c = f.c;
+  const Arrays<P>& a = f.a;
+  const int gl = (threadIdx.x & 31) % GL;
+  const int np = live ? (int)(hd & 0xffffu) : 0, nr = live ? (int)(hd >> 16 & 255u) : 0;
+  if (gl == 0) tally.n_tot += (unsigned)np;
+  // the pairs' staged data: this lane's element of the next round, loaded
+  // one round ahead (`left` pairs of the current round not yet loaded)
+  const unsigned long long first = np > 0 ? f.sched_off[o] : 0ull;
+  const uint8_t* rs = f.rsize + o * kRoundStride;
+  int r = 0, sizes = gl < nr ? (int)rs[gl] : 0;  // sizes of rounds [r - r % GL, ...)
+  int left = __shfl_sync(0xffffffffu, sizes, 0, GL);
+  int pos = 0, n = min(left, GL);
+  uint32_t pr = 0;
+  F4 ge{}, rn{};
+  auto fetch = [&]() {
+    if (gl < n) {
+      pr = __ldg(&f.pairs[first + pos + gl]);
+      ge = ld4(&f.geom[first + pos + gl]);
+      rn = ld4(&f.rnd[first + pos + gl]);
+    }
+  };
+  fetch();
+  BlockCells b;
+  b.base[8] = 0;
+  if (np > 0) block_cells(c, ox, oy, oz, f.mrank, f.cell_start, b);
+  const int nb = np > 0 ? b.base[8] : 0;
+#pragma unroll
+  for (int t = 0; t < 8; ++t)
+    if (gl == t) {
+      cells.cst[t] = b.start[t];
+      cells.cbs[t] = b.base[t];
+    }
+  __syncwarp();
+  for (int q = gl; q < nb; q += GL) {
+    const int g = block_gidx(cells, q);
+    s[q] = F4{(float)a.px[g], (float)a.py[g], (float)a.pz[g], (float)a.eps[g]};
+    ec[q] = 0.0f;
+  }
+  __syncwarp();
+  while (__any_sync(0xffffffffu, n > 0)) {
+    const bool act = gl < n;
+    const int level = r;
+    const uint32_t cpr = pr;
+    const F4 cg = ge, cr = rn;
+    // advance to the next round (or the rest of a wide one) and load it
+    pos += n;
+    left -= n;
+    if (left == 0 && r < nr) {
+      ++r;
+      if (r % GL == 0) sizes = r + gl < nr ? (int)rs[r + gl] : 0;
+    }
+    const int nx = __shfl_sync(0xffffffffu, sizes, r % GL, GL);
+    if (left == 0) left = r < nr ? nx : 0;
+    n = min(left, GL);
+    fetch();
+    if (act) {
+      const int ia = cpr & 0xffffu, ib = cpr >> 16;
+      const F4 sa = lds4(&s[ia]), sb = lds4(&s[ib]);
+      float pa[3] = {sa.x, sa.y, sa.z};
+      float pb[3] = {sb.x, sb.y, sb.z};
+      const float G[3] = {cr.x, cr.y, cr.z};
+      double margin;
+      float m32 = 0.0f, tol = 0.0f;
+      const float eaf = sa.w, ebf = sb.w;
+      auto exact_e = [&](double& ea, double& eb) { fd_exact_energies(a.eps, cells, ec, ia, ib, eaf, ebf, ea, eb); };
+      auto uniform = [&]() {
+        return fd_uniform_again(f.seed, sweep, a.id[block_gidx(cells, ia)], a.id[block_gidx(cells, ib)]);
+      };
+      float dh, dl;
+      const int dcs = fd_pair_mixed<false>(f.k, cg.x, cg.y, cg.z, cg.w, G, uniform, cr.w, pa, pb, eaf, ebf, exact_e, dh,
+                                         dl, margin, m32, tol, REC, tally.negative);
+      if (dcs == 0) {
+        float t, e;
+        eft::two_sum(eaf, dh, t, e);
+        ec[ia] = __fadd_rn(ec[ia], __fadd_rn(e, dl));
+        s[ia] = F4{pa[0], pa[1], pa[2], t};
+        eft::two_sum(ebf, dh, t, e);
+        ec[ib] = __fadd_rn(ec[ib], __fadd_rn(e, dl));
+        s[ib] = F4{pb[0], pb[1], pb[2], t};
+      }
+      tally.n_rb += dcs == 1;
+      tally.n_rm += dcs == 2;
+      if constexpr (REC) {
+        const unsigned long long at = atomicAdd(f.rec_count, 1ull);
+        if ((int64_t)at < f.rec_cap) {
+          sdpd_pair_rec rc;
+          rc.id_i = a.id[block_gidx(cells, ia)];
+          rc.id_j = a.id[block_gidx(cells, ib)];
+          rc.colour = f.colour;
+          rc.owner = (int32_t)o;
+          rc.decision = dcs;
+          rc.level = level;
+          rc.margin = margin;
+          rc.margin_lo = (double)m32;
+          rc.margin_tol = (double)tol;
+          f.recs[at] = rc;
+        }
+      }
+    }
+    __syncwarp();
+  }
+  const S pi_coef = (S)(c.c_rho / (c.C_K * c.m));
+  for (int q = gl; q < nb; q += GL) {
+    const int g = block_gidx(cells, q);
+    const F4 v = lds4(&s[q]);
+    if constexpr (kSame) {
+      a.px[g] = v.x; a.py[g] = v.y; a.pz[g] = v.z;
+    } else {  // the stored value plus this visit's increment
+      a.px[g] += (S)(v.x - (float)a.px[g]);
+      a.py[g] += (S)(v.y - (float)a.py[g]);
+      a.pz[g] += (S)(v.z - (float)a.pz[g]);
+    }
+    // once per visit: the load value plus the visit's exact change
+    const double e0 = a.eps[g];
+    const double e = e0 + (((double)v.w - (double)(float)e0) + (double)ec[q]);
+    tally.bad |= !isfinite(v.w);  // (a sum that was not finite once never is again)
+    a.eps[g] = e;
+    // pressure over rho^2 of the new energy, Eq. (pg-eos): pi = c_rho eps / (C_K m rho)
+    // (from the stored float64 energy, as a restart recomputes it)
+    f.qp4[g].w = (S)e * pi_coef / a.rho[g];
+  }
+  __syncwarp();  // the group's shared memory is refilled by the next block
+}
+
+// Shared memory of a large block: momenta as stored and float64 energies.
+template <class P>
+struct FdLargeSmem {
+  typename P::R p[3][kLargeBlock];
+  double e[kLargeBlock];
+  FdCells cells;
+};
+
+// One of the colour's large blocks on a whole warp, its rounds at most 32
+// pairs wide.  The pair updates are those of the pair-by-pair sweep
+// (fd_big_block): float32 arithmetic on the stored momenta and float64
+// energies, which take each pair's change.
+template <class P, bool REC>
+__device__ __noinline__ void fd_large_block(const FdRun<P>& f, int64_t o, uint64_t sweep, unsigned char* smem,
+                                            FdTally& tally) {
+  using S = typename P::R;
+  FdLargeSmem<P>& sm = *reinterpret_cast<FdLargeSmem<P>*>(smem);
+  const Consts& c = f.c;
+  const Arrays<P>& a = f.a;
+  const int lane = threadIdx.x & 31;
+  const uint32_t hd = f.hdr[o];
+  const int np = (int)(hd & 0xffffu), nr = (int)(hd >> 16 & 255u);
+  if (lane == 0) tally.n_tot += (unsigned)np;
+  stage_cells(c, o, f.mrank, f.cell_start, lane, sm.cells);
+  int nb = 0;  // particles: the last cell's offset and count
+  {
+    int ox, oy, oz;
+    owner_coords(c, o, ox, oy, oz);
+    BlockCells b;
+    block_cells(c, ox, oy, oz, f.mrank, f.cell_start, b);
+    nb = b.base[8];
+  }
+  for (int q = lane; q < nb; q += 32) {
+    const int g = block_gidx(sm.cells, q);
+    sm.p[0][q] = a.px[g];
+    sm.p[1][q] = a.py[g];
+    sm.p[2][q] = a.pz[g];
+    sm.e[q] = a.eps[g];
+  }
+  __syncwarp();
+  const uint8_t* rs = f.rsize + o * kRoundStride;
+  unsigned long long at = f.sched_off[o];
+  for (int r = 0; r < nr; ++r) {
+    const int n = rs[r];
+    for (int t = lane; t < n; t += 32) {
+      const uint32_t pr = __ldg(&f.pairs[at + t]);
+      const F4 ge = ld4(&f.geom[at + t]), rn = ld4(&f.rnd[at + t]);
+      const int ia = pr & 0xffffu, ib = pr >> 16;
+      float pa[3], pb[3], pa0[3], pb0[3];
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        pa0[d] = pa[d] = (float)sm.p[d][ia];
+        pb0[d] = pb[d] = (float)sm.p[d][ib];
+      }
+      const double ea = sm.e[ia], eb = sm.e[ib];
+      const float G[3] = {rn.x, rn.y, rn.z};
+      auto exact_e = [&](double& x, double& y) { x = ea; y = eb; };
+      auto uniform = [&]() {
+        return fd_uniform_again(f.seed, sweep, a.id[block_gidx(sm.cells, ia)], a.id[block_gidx(sm.cells, ib)]);
+      };
+      double margin;
+      float dh, dl, m32 = 0.0f, tol = 0.0f;
+      const int dcs = fd_pair_mixed<true>(f.k, ge.x, ge.y, ge.z, ge.w, G, uniform, rn.w, pa, pb, (float)ea, (float)eb,
+                                          exact_e, dh, dl, margin, m32, tol, REC, tally.negative);
+      if (dcs == 0) {
+        const double de = (double)dh + (double)dl;
+        sm.e[ia] = ea + de;
+        sm.e[ib] = eb + de;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          if constexpr (std::is_same<S, float>::value) {
+            sm.p[d][ia] = pa[d];
+            sm.p[d][ib] = pb[d];
+          } else {  // the stored value plus the increment
+            sm.p[d][ia] += (S)(pa[d] - pa0[d]);
+            sm.p[d][ib] += (S)(pb[d] - pb0[d]);
+          }
+        }
+      }
+      tally.n_rb += dcs == 1;
+      tally.n_rm += dcs == 2;
+      if constexpr (REC) {
+        const unsigned long long k = atomicAdd(f.rec_count, 1ull);
+        if ((int64_t)k < f.rec_cap) {
+          sdpd_pair_rec rc;
+          rc.id_i = a.id[block_gidx(sm.cells, ia)];
+          rc.id_j = a.id[block_gidx(sm.cells, ib)];
+          rc.colour = f.colour;
+          rc.owner = (int32_t)o;
+          rc.decision = dcs;
+          rc.level = r;
+          rc.margin = margin;
+          rc.margin_lo = (double)m32;
+          rc.margin_tol = (double)tol;
+          f.recs[k] = rc;
+        }
+      }
+    }
+    at += n;
+    __syncwarp();
+  }
+  const S pi_coef = (S)(c.c_rho / (c.C_K * c.m));
+  for (int q = lane; q < nb; q += 32) {
+    const int g = block_gidx(sm.cells, q);
+    a.px[g] = sm.p[0][q];
+    a.py[g] = sm.p[1][q];
+    a.pz[g] = sm.p[2][q];
+    tally.bad |= !isfinite(sm.e[q]);
+    a.eps[g] = sm.e[q];
+    f.qp4[g].w = (S)sm.e[q] * pi_coef / a.rho[g];
+  }
+  __syncwarp();
+}
+
+template <class P, int OPW, bool REC>
+__global__ void __launch_bounds__(128, 4) k_fd_colour(const __grid_constant__ FdRun<P> f) {
+  constexpr int GL = 32 / OPW;
   extern __shared__ __align__(32) unsigned char fd_smem_raw[];
-  const uint64_t sweep = *sweep_ptr;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int grp = lane / kGroupLanes, gl = lane % kGroupLanes;
+  const uint64_t sweep = *f.sweep_ptr;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, grp = lane / GL;
+  const Consts& c = f.c;
+  const int colour = f.colour;
   const int hx = c.nc[0] >> 1, hy = c.nc[1] >> 1, hz = c.nc[2] >> 1;
   const int64_t nown = (int64_t)hx * hy * hz;
-  FdSmem<R>& sm = reinterpret_cast<FdSmem<R>*>(fd_smem_raw)[warp * OPW + grp];
-  const S pi_coef = (S)(c.c_rho / (c.C_K * c.m));
-  unsigned n_tot = 0, n_rb = 0, n_rm = 0;  // per lane (accepted = total - rejected)
-  bool negative = false, bad = false;
+  FdSmem& sm = reinterpret_cast<FdSmem*>(fd_smem_raw)[warp * OPW + grp];
+  unsigned* queue = f.queue;
+  FdTally tally;
   // The grid holds as many thread blocks as fit on the GPU at once; each
   // warp takes the colour's blocks OPW at a time from queue[0] until they
   // run out, so no partial last wave of thread blocks idles the GPU and
   // blocks of uneven depth balance out.  The blocks come in the order of
   // `order` (deepest first), so the blocks a warp runs in lockstep have
   // similar depth.  queue[1] counts the warps that are done; the last one
-  // sets them back to zero for the next launch (queue[2]: the next entry of
-  // the colour's list of blocks beyond capacity).
+  // sets them back to zero for the next launch (queue[2], queue[3]: the next
+  // entries of the colour's lists of blocks beyond capacity and of large blocks).
   for (;;) {
     unsigned w0 = 0;
     if (lane == 0) w0 = atomicAdd(queue, (unsigned)OPW);
     w0 = __shfl_sync(0xffffffffu, w0, 0);
     if ((int64_t)w0 >= nown) break;
     const int64_t wi = (int64_t)w0 + grp;
-    const int64_t w = wi < nown ? (int64_t)order[colour * nown + wi] : nown;
-    int np = 0, nlev = 0;
-    int64_t o = 0;
-    int ox = 0, oy = 0, oz = 0;
-    if (w < nown) {
-      ox = 2 * (int)(w % hx) + (colour & 1);
-      oy = 2 * (int)((w / hx) % hy) + ((colour >> 1) & 1);
-      oz = 2 * (int)(w / ((int64_t)hx * hy)) + ((colour >> 2) & 1);
-      o = ox + (int64_t)c.nc[0] * (oy + (int64_t)c.nc[1] * oz);
-      const uint32_t hd = hdr[o];
-      if (hd != kHdrBig) {  // (a block beyond capacity is swept below)
-        np = (int)(hd & 0xffffu);
-        nlev = (int)(hd >> 16);
-      }
+    const int64_t w = wi < nown ? (int64_t)f.order[colour * nown + wi] : 0;
+    const int ox = 2 * (int)(w % hx) + (colour & 1), oy = 2 * (int)((w / hx) % hy) + ((colour >> 1) & 1),
+              oz = 2 * (int)(w / ((int64_t)hx * hy)) + ((colour >> 2) & 1);
+    const int64_t o = ox + (int64_t)c.nc[0] * (oy + (int64_t)c.nc[1] * oz);
+    const uint32_t hd = f.hdr[o];
+    // (large blocks and those beyond capacity, which have the flag's bit set too, come below)
+    const bool live = wi < nown && !(hd & kHdrLargeFlag);
+    fd_run_block<P, GL, REC>(f, live, o, ox, oy, oz, hd, sweep, sm.s, sm.ec, sm.cells, tally);
+  }
+  // large blocks: one warp of the thread block, on all of its shared memory
+  if (f.large_count[colour] > 0) {
+    __syncthreads();
+    for (; warp == 0;) {
+      unsigned li = 0;
+      if (lane == 0) li = atomicAdd(&queue[3], 1u);
+      li = __shfl_sync(0xffffffffu, li, 0);
+      if (li >= f.large_count[colour]) break;
+      fd_large_block<P, REC>(f, f.large_list[colour * nown + li], sweep, fd_smem_raw, tally);
     }
-    if (gl == 0) n_tot += (unsigned)np;
-    // the pairs' staged data: this lane's element of the next round, loaded
-    // one round ahead (`left` pairs of the current round not yet loaded)
-    const unsigned long long first = np > 0 ? sched_off[o] : 0ull;
-    const uint8_t* rs = rsize + o * kRoundStride;
-    int r = 0, sizes = gl < nlev ? (int)rs[gl] : 0;  // sizes of rounds [r - r % kGroupLanes, ...)
-    int left = __shfl_sync(0xffffffffu, sizes, 0, kGroupLanes);
-    int pos = 0, n = min(left, kGroupLanes);
-    uint16_t pr = 0;
-    AV4 ge{}, rn{};
-    auto fetch = [&]() {
-      if (gl < n) {
-        pr = __ldg(&pairs[first + pos + gl]);
-        ge = ld4(&geom[first + pos + gl]);
-        rn = ld4(&rnd[first + pos + gl]);
-      }
-    };
-    fetch();
-    BlockCells b;
-    b.base[8] = 0;
-    if (np > 0) block_cells(c, ox, oy, oz, mrank, cell_start, b);
-    const int nb = np > 0 ? b.base[8] : 0;
-#pragma unroll
-    for (int t = 0; t < 8; ++t)
-      if (gl == t % kGroupLanes) {
-        sm.cells.cst[t] = b.start[t];
-        sm.cells.cbs[t] = b.base[t];
-      }
-    __syncwarp();
-    for (int q = gl; q < nb; q += kGroupLanes) {
-      const int g = block_gidx(sm.cells, q);
-      AV4 v;
-      v.x = (R)a.px[g];
-      v.y = (R)a.py[g];
-      v.z = (R)a.pz[g];
-      v.w = (R)a.eps[g];
-      sm.s[q] = v;
-      sm.ec[q] = 0.0f;
-    }
-    __syncwarp();
-    while (__any_sync(0xffffffffu, n > 0)) {
-      const bool act = gl < n;
-      const int level = r;
-      const uint16_t cpr = pr;
-      const AV4 cg = ge, cr = rn;
-      // advance to the next round (or the rest of a wide one) and load it
-      pos += n;
-      left -= n;
-      if (left == 0 && r < nlev) {
-        ++r;
-        if (r % kGroupLanes == 0) sizes = r + gl < nlev ? (int)rs[r + gl] : 0;
-      }
-      const int nx = __shfl_sync(0xffffffffu, sizes, r % kGroupLanes, kGroupLanes);
-      if (left == 0) left = r < nlev ? nx : 0;
-      n = min(left, kGroupLanes);
-      fetch();
-      if (act) {
-        const int ia = cpr & 255, ib = cpr >> 8;
-        const AV4 sa = lds4(&sm.s[ia]), sb = lds4(&sm.s[ib]);
-        R pa[3] = {sa.x, sa.y, sa.z};
-        R pb[3] = {sb.x, sb.y, sb.z};
-        const R G[3] = {cr.x, cr.y, cr.z};
-        double margin;
-        float m32 = 0.0f, tol = 0.0f;
-        int dcs;
-        {
-          const float eaf = sa.w, ebf = sb.w;
-          auto exact_e = [&](double& ea, double& eb) { fd_exact_energies(a.eps, sm, ia, ib, eaf, ebf, ea, eb); };
-          auto uniform = [&]() {
-            return fd_uniform_again(seed, sweep, a.id[block_gidx(sm.cells, ia)], a.id[block_gidx(sm.cells, ib)]);
-          };
-          float dh, dl;
-          dcs = fd_pair_mixed<false>(k, cg.x, cg.y, cg.z, cg.w, G, uniform, cr.w, pa, pb, eaf, ebf, exact_e, dh, dl, margin,
-                              m32, tol, REC, negative);
-          if (dcs == 0) {
-            float s, e;
-            eft::two_sum(eaf, dh, s, e);
-            sm.ec[ia] = __fadd_rn(sm.ec[ia], __fadd_rn(e, dl));
-            sm.s[ia] = F4{pa[0], pa[1], pa[2], s};
-            eft::two_sum(ebf, dh, s, e);
-            sm.ec[ib] = __fadd_rn(sm.ec[ib], __fadd_rn(e, dl));
-            sm.s[ib] = F4{pb[0], pb[1], pb[2], s};
-          }
-        }
-        n_rb += dcs == 1;
-        n_rm += dcs == 2;
-        if constexpr (REC) {
-          const unsigned long long s = atomicAdd(rec_count, 1ull);
-          if ((int64_t)s < rec_cap) {
-            sdpd_pair_rec rc;
-            rc.id_i = a.id[block_gidx(sm.cells, ia)];
-            rc.id_j = a.id[block_gidx(sm.cells, ib)];
-            rc.colour = colour;
-            rc.owner = (int32_t)o;
-            rc.decision = dcs;
-            rc.level = level;
-            rc.margin = margin;
-            rc.margin_lo = (double)m32;
-            rc.margin_tol = (double)tol;
-            recs[s] = rc;
-          }
-        }
-      }
-      __syncwarp();
-    }
-    for (int q = gl; q < nb; q += kGroupLanes) {
-      const int g = block_gidx(sm.cells, q);
-      const AV4 v = lds4(&sm.s[q]);
-      if constexpr (kSame) {
-        a.px[g] = v.x; a.py[g] = v.y; a.pz[g] = v.z;
-      } else {  // the stored value plus this visit's increment
-        a.px[g] += (S)(v.x - (R)a.px[g]);
-        a.py[g] += (S)(v.y - (R)a.py[g]);
-        a.pz[g] += (S)(v.z - (R)a.pz[g]);
-      }
-      // once per visit: the load value plus the visit's exact change
-      const double e0 = a.eps[g];
-      const double e = e0 + (((double)v.w - (double)(float)e0) + (double)sm.ec[q]);
-      bad |= !isfinite(v.w);  // (a sum that was not finite once never is again)
-      a.eps[g] = e;
-      // pressure over rho^2 of the new energy, Eq. (pg-eos): pi = c_rho eps / (C_K m rho)
-      // (from the stored float64 energy, as a restart recomputes it)
-      qp4[g].w = (S)e * pi_coef / a.rho[g];
-    }
-    __syncwarp();  // the group's shared memory is refilled by the next block
   }
   // the colour's blocks beyond capacity (listed by the schedule), swept pair
   // by pair by whole warps once the queue is empty
@@ -1017,28 +1156,21 @@ __global__ void __launch_bounds__(128, 4)
     unsigned bi = 0;
     if (lane == 0) bi = atomicAdd(&queue[2], 1u);
     bi = __shfl_sync(0xffffffffu, bi, 0);
-    if (bi >= big_count[colour]) break;
-    const int2 ent = big_list[colour * nown + bi];
-    const int64_t ob = ent.x;
+    if (bi >= f.big_count[colour]) break;
+    const int2 ent = f.big_list[colour * nown + bi];
     int bx, by, bz;
-    owner_coords(c, ob, bx, by, bz);
-    const BigCounts bc = fd_big_block<P, A>(c, k, a, qp4, cell_start, mrank, xmx, xmy, xmz, ob, bx, by, bz, colour,
-                                            seed, sweep, REC ? recs : nullptr, rec_count, rec_cap, big_perm + ent.y);
-    unsigned long long bt = bc.tot, ba = bc.acc, bb = bc.rb, bm = bc.rm;  // (rare: counted at once)
-    for (int s = 16; s > 0; s >>= 1) {
-      bt += __shfl_xor_sync(0xffffffffu, bt, s);
-      ba += __shfl_xor_sync(0xffffffffu, ba, s);
-      bb += __shfl_xor_sync(0xffffffffu, bb, s);
-      bm += __shfl_xor_sync(0xffffffffu, bm, s);
+    owner_coords(c, ent.x, bx, by, bz);
+    const BigCounts bc = fd_big_block<P, Mixed>(c, f.k, f.a, f.qp4, f.cell_start, f.mrank, f.xmx, f.xmy, f.xmz, ent.x,
+                                                bx, by, bz, colour, f.seed, sweep, REC ? f.recs : nullptr, f.rec_count,
+                                                f.rec_cap, f.big_perm + ent.y);
+    if (lane == 0) {  // (rare: counted at once; lane 0 made the updates)
+      atomicAdd(&f.counters[0], bc.tot);
+      atomicAdd(&f.counters[1], bc.acc);
+      atomicAdd(&f.counters[2], bc.rb);
+      atomicAdd(&f.counters[3], bc.rm);
     }
-    if (lane == 0 && bt) {
-      atomicAdd(&counters[0], bt);
-      atomicAdd(&counters[1], ba);
-      atomicAdd(&counters[2], bb);
-      atomicAdd(&counters[3], bm);
-    }
-    negative |= bc.negative != 0;
-    bad |= bc.bad != 0;
+    tally.negative |= bc.negative != 0;
+    tally.bad |= bc.bad != 0;
   }
   if (lane == 0) {
     const unsigned total = gridDim.x * (blockDim.x >> 5);
@@ -1047,26 +1179,27 @@ __global__ void __launch_bounds__(128, 4)
       queue[0] = 0u;
       queue[1] = 0u;
       queue[2] = 0u;
-      if (colour == 7) *sweep_ptr = sweep + 1ull;  // (every warp has read it) the sweep is done
+      queue[3] = 0u;
+      if (colour == 7) *f.sweep_ptr = sweep + 1ull;  // (every warp has read it) the sweep is done
     }
   }
   // counters
-  unsigned long long c_tot = n_tot, c_rb = n_rb, c_rm = n_rm;
+  unsigned long long c_tot = tally.n_tot, c_rb = tally.n_rb, c_rm = tally.n_rm;
   for (int s = 16; s > 0; s >>= 1) {
     c_tot += __shfl_xor_sync(0xffffffffu, c_tot, s);
     c_rb += __shfl_xor_sync(0xffffffffu, c_rb, s);
     c_rm += __shfl_xor_sync(0xffffffffu, c_rm, s);
   }
-  const unsigned any_neg = __any_sync(0xffffffffu, negative), any_bad = __any_sync(0xffffffffu, bad);
+  const unsigned any_neg = __any_sync(0xffffffffu, tally.negative), any_bad = __any_sync(0xffffffffu, tally.bad);
   if (lane == 0) {
     if (c_tot) {
-      atomicAdd(&counters[0], c_tot);
-      atomicAdd(&counters[1], c_tot - c_rb - c_rm);
-      atomicAdd(&counters[2], c_rb);
-      atomicAdd(&counters[3], c_rm);
+      atomicAdd(&f.counters[0], c_tot);
+      atomicAdd(&f.counters[1], c_tot - c_rb - c_rm);
+      atomicAdd(&f.counters[2], c_rb);
+      atomicAdd(&f.counters[3], c_rm);
     }
-    if (any_neg) atomicOr(status, kStNegative);
-    if (any_bad) atomicOr(status, kStNaN);
+    if (any_neg) atomicOr(f.status, kStNegative);
+    if (any_bad) atomicOr(f.status, kStNaN);
   }
 }
 
@@ -1099,56 +1232,81 @@ static FDConst<R> fd_const(const Consts& c, double dt) {
 constexpr int kFdOpw[kFdVariants] = {2, 2, 1, 1, 1};
 constexpr int kFdWarps[kFdVariants] = {2, 1, 1, 2, 4};
 
-// A block schedule fits when its groups' shared memory stays within 48 KB.
-template <class A>
-constexpr bool fd_fits(int v) { return sizeof(FdSmem<typename A::R>) * kFdOpw[v] * kFdWarps[v] <= 48 * 1024; }
+// Shared memory of a thread block: its groups' blocks, at least one large block.
+template <class P>
+constexpr size_t fd_smem_bytes(int v) {
+  return std::max(sizeof(FdSmem) * kFdOpw[v] * kFdWarps[v], sizeof(FdLargeSmem<P>));
+}
 
 // Thread blocks of a colour kernel that the device holds at once (SMs x
 // blocks per SM, from the occupancy calculator; at least one), computed once
-// per kernel and warps per thread block on the device current at the first
-// launch.
-template <class P, class A, int OPW, bool REC, int W>
+// per kernel and schedule on the device current at the first launch.
+template <class P, bool REC, int V>
 int fd_resident_blocks() {
   static const int n = [] {
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fd_colour<P, A, OPW, REC>, W * 32,
-                                                  sizeof(FdSmem<typename A::R>) * OPW * W);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fd_colour<P, kFdOpw[V], REC>, kFdWarps[V] * 32,
+                                                  fd_smem_bytes<P>(V));
     return std::max(1, sms) * std::max(1, per_sm);
   }();
   return n;
 }
-template <class P, class A, bool REC>
+template <class P, bool REC>
 int fd_resident(int variant) {
   switch (variant) {
-    case 0: return fd_resident_blocks<P, A, 2, REC, 2>();
-    case 1: return fd_resident_blocks<P, A, 2, REC, 1>();
-    case 2: return fd_resident_blocks<P, A, 1, REC, 1>();
-    case 3: return fd_resident_blocks<P, A, 1, REC, 2>();
-    default: return fd_resident_blocks<P, A, 1, REC, 4>();
+    case 0: return fd_resident_blocks<P, REC, 0>();
+    case 1: return fd_resident_blocks<P, REC, 1>();
+    case 2: return fd_resident_blocks<P, REC, 2>();
+    case 3: return fd_resident_blocks<P, REC, 3>();
+    default: return fd_resident_blocks<P, REC, 4>();
   }
 }
 
-// The eight colour launches of one sweep.
-template <class P, class A, bool REC>
-void launch_colours_rec(const Consts& c, const Workspace& w, int cur, double dt, uint64_t seed, int variant,
-                        cudaStream_t s) {
-  const FDConst<typename A::R> k = fd_const<typename A::R>(c, dt);
-  const Arrays<P> a = view<P>(w, cur);
+// The eight colour launches of one sweep with float32 pair arithmetic.  Few
+// blocks spread over as many thread blocks (a warp that finds none left ends).
+template <class P, bool REC>
+void launch_colours32(const Consts& c, const Workspace& w, int cur, double dt, uint64_t seed, int variant,
+                      cudaStream_t s) {
   const int64_t nown = (int64_t)(c.nc[0] / 2) * (c.nc[1] / 2) * (c.nc[2] / 2);
   const int opw = kFdOpw[variant], W = kFdWarps[variant];
-  const int64_t need = (nown + W * opw - 1) / (W * opw);
-  const unsigned gf = (unsigned)std::max<int64_t>(1, std::min<int64_t>(need, fd_resident<P, A, REC>(variant)));
-  const size_t smem = sizeof(FdSmem<typename A::R>) * (size_t)(opw * W);
-  auto kern = opw == 2 ? k_fd_colour<P, A, 2, REC> : k_fd_colour<P, A, 1, REC>;
-  for (int col = 0; col < 8; ++col)
-    kern<<<gf, W * 32, smem, s>>>(c, k, a, (typename P::V4*)w.qp4, w.cell_start, w.mrank, w.xmin[0], w.xmin[1],
-                                  w.xmin[2], w.sched_hdr, w.sched_rsize, w.sched_off, w.sched_pair,
-                                  (const typename A::V4*)w.st_geom, (const typename A::V4*)w.st_rnd, col, seed,
-                                  w.sweep, w.counters, w.status, REC ? w.pair_recs : nullptr, w.pair_rec_count,
-                                  w.pair_rec_cap, w.fd_queue + 3 * col, w.blk_order, w.big_perm, w.big_list,
-                                  w.big_count);
+  const unsigned gf = (unsigned)std::max<int64_t>(1, std::min<int64_t>((nown + opw - 1) / opw, fd_resident<P, REC>(variant)));
+  FdRun<P> f;
+  f.c = c;
+  f.k = fd_const<float>(c, dt);
+  f.a = view<P>(w, cur);
+  f.qp4 = (typename P::V4*)w.qp4;
+  f.cell_start = w.cell_start;
+  f.mrank = w.mrank;
+  f.xmx = w.xmin[0];
+  f.xmy = w.xmin[1];
+  f.xmz = w.xmin[2];
+  f.hdr = w.sched_hdr;
+  f.rsize = w.sched_rsize;
+  f.sched_off = w.sched_off;
+  f.pairs = w.sched_pair;
+  f.geom = (const F4*)w.st_geom;
+  f.rnd = (const F4*)w.st_rnd;
+  f.seed = seed;
+  f.sweep_ptr = w.sweep;
+  f.counters = w.counters;
+  f.status = w.status;
+  f.recs = REC ? w.pair_recs : nullptr;
+  f.rec_count = w.pair_rec_count;
+  f.rec_cap = w.pair_rec_cap;
+  f.order = w.blk_order;
+  f.big_perm = w.big_perm;
+  f.big_list = w.big_list;
+  f.big_count = w.big_count;
+  f.large_list = w.large_list;
+  f.large_count = w.large_count;
+  auto kern = opw == 2 ? k_fd_colour<P, 2, REC> : k_fd_colour<P, 1, REC>;
+  for (int col = 0; col < 8; ++col) {
+    f.colour = col;
+    f.queue = w.fd_queue + 4 * col;
+    kern<<<gf, W * 32, fd_smem_bytes<P>(variant), s>>>(f);
+  }
 }
 
 // Fills the resident-block counts of every block schedule ahead of time (a
@@ -1163,13 +1321,12 @@ void fd_prepare() {
   if constexpr (!A::mixed) {
     team64_resident<false>();
     team64_resident<true>();
-    return;
-  } else
-  for (int v = 0; v < kFdVariants; ++v)
-    if (fd_fits<A>(v)) {
-      fd_resident<P, A, false>(v);
-      fd_resident<P, A, true>(v);
+  } else {
+    for (int v = 0; v < kFdVariants; ++v) {
+      fd_resident<P, false>(v);
+      fd_resident<P, true>(v);
     }
+  }
 }
 
 static inline unsigned stage_blocks(const Consts& c) { return (unsigned)((c.ncell + kStageWarps - 1) / kStageWarps); }
@@ -1202,10 +1359,10 @@ void launch_fd_colours(const Consts& c, const Workspace& w, int cur, double dt, 
   if constexpr (!A::mixed) {
     if (record) launch_colours64<true>(c, w, cur, dt, seed, s);
     else launch_colours64<false>(c, w, cur, dt, seed, s);
-    return;
-  } else
-  if (record) launch_colours_rec<P, A, true>(c, w, cur, dt, seed, fd_launch_variant(c), s);
-  else launch_colours_rec<P, A, false>(c, w, cur, dt, seed, fd_launch_variant(c), s);
+  } else {
+    if (record) launch_colours32<P, true>(c, w, cur, dt, seed, fd_launch_variant(c), s);
+    else launch_colours32<P, false>(c, w, cur, dt, seed, fd_launch_variant(c), s);
+  }
 }
 
 }  // namespace sdpd

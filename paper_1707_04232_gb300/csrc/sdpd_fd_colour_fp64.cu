@@ -15,12 +15,10 @@ template void launch_fd_colours<Fp64, Fp64>(const Consts&, const Workspace&, int
 template void launch_fd_colours<Fp64, Mixed>(const Consts&, const Workspace&, int, double, uint64_t, int,
                                            cudaStream_t);
 
-int fd_round_width(const Consts& c, bool float_arith) {
-  return float_arith ? 32 / kFdOpw[fd_launch_variant(c)] : kTeamPairs;
+int fd_round_width(const Consts& c, bool float_arith, bool large) {
+  return float_arith ? (large ? 32 : 32 / kFdOpw[fd_launch_variant(c)]) : kTeamPairs;
 }
 
-bool fd_variant_fits(bool mixed, int v) {
-  return v >= 0 && v < kFdVariants && (mixed ? fd_fits<Mixed>(v) : fd_fits<Fp64>(v));
-}
+bool fd_variant_fits(bool, int v) { return v >= 0 && v < kFdVariants; }
 
 }  // namespace sdpd

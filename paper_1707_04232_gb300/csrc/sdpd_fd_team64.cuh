@@ -208,20 +208,27 @@ __device__ __forceinline__ int team_pair(const Team64Const& k, int l, bool live,
   return decision;
 }
 
+// Shared memory of a team's block: records (px, py, pz, eps).
+struct Team64Smem {
+  D4 s[kLargeBlock];
+  FdCells cells;
+};
+
 constexpr int kTeamWarps = 2, kTeamPairs = 8 * kTeamWarps;
 
 template <bool REC>
 __global__ void __launch_bounds__(kTeamWarps * 32)
-    k_fd_colour64(Consts c, FDConst<double> kbig, Team64Const k, Arrays<Fp64> a, D4* __restrict__ qp4,
+    k_fd_colour64(const __grid_constant__ Consts c, const __grid_constant__ FDConst<double> kbig, Team64Const k,
+                  const __grid_constant__ Arrays<Fp64> a, D4* __restrict__ qp4,
                   const int32_t* __restrict__ cell_start, const int32_t* __restrict__ mrank,
                   const uint32_t* __restrict__ hdr, const uint8_t* __restrict__ rsize,
-                  const unsigned long long* __restrict__ sched_off, const uint16_t* __restrict__ pairs,
+                  const unsigned long long* __restrict__ sched_off, const uint32_t* __restrict__ pairs,
                   const double* __restrict__ geom, const double* __restrict__ rnd, const double* __restrict__ aux,
                   int colour, uint64_t seed, unsigned long long* __restrict__ sweep_ptr, unsigned long long* counters,
                   int* status, sdpd_pair_rec* recs, unsigned long long* rec_count, int64_t rec_cap,
                   unsigned* __restrict__ queue, const int32_t* __restrict__ order, int32_t* __restrict__ big_perm,
                   const int2* __restrict__ big_list, const uint32_t* __restrict__ big_count) {
-  __shared__ FdSmem<double> sm;
+  __shared__ Team64Smem sm;
   __shared__ uint8_t size_s[kRoundStride];
   __shared__ unsigned next_s;
   const uint64_t sweep = *sweep_ptr;
@@ -244,7 +251,7 @@ __global__ void __launch_bounds__(kTeamWarps * 32)
               oz = 2 * (int)(w / ((int64_t)hx * hy)) + ((colour >> 2) & 1);
     const int64_t o = ox + (int64_t)c.nc[0] * (oy + (int64_t)c.nc[1] * oz);
     const uint32_t hd = hdr[o];
-    const int np = hd == kHdrBig ? 0 : (int)(hd & 0xffffu), nr = hd == kHdrBig ? 0 : (int)(hd >> 16);
+    const int np = hd == kHdrBig ? 0 : (int)(hd & 0xffffu), nr = hd == kHdrBig ? 0 : (int)(hd >> 16 & 255u);
     if (np == 0) {  // (a block beyond capacity is swept below)
       __syncthreads();
       continue;
@@ -267,7 +274,7 @@ __global__ void __launch_bounds__(kTeamWarps * 32)
       sm.s[q] = D4{a.px[g], a.py[g], a.pz[g], a.eps[g]};
     }
     // this quad's pair of a round, loaded one round ahead
-    uint16_t pr = 0;
+    uint32_t pr = 0;
     double ge = 0.0, Gl = 0.0, base = 0.0, c0 = 0.0;
     int r = 0, pos = 0, left = size_s[0], n = min(left, kTeamPairs);
     auto fetch = [&]() {
@@ -285,7 +292,7 @@ __global__ void __launch_bounds__(kTeamWarps * 32)
     while (n > 0) {
       const bool act = slot < n;
       const int busy = n - warp * 8, level = r;  // pairs of this warp
-      const uint16_t cpr = act ? pr : (uint16_t)0;
+      const uint32_t cpr = act ? pr : 0u;
       // (lanes without a pair run on values that keep to the short paths)
       const double cge = ge, cG = act ? Gl : 0.0, cb = act ? base : 0.01, cc = c0;
       pos += n;
@@ -294,7 +301,7 @@ __global__ void __launch_bounds__(kTeamWarps * 32)
       n = min(left, kTeamPairs);
       fetch();
       if (busy > 0) {
-        const int ia = cpr & 255, ib = cpr >> 8;
+        const int ia = cpr & 0xffffu, ib = cpr >> 16;
         const double A = rec[4 * ia + l], B = rec[4 * ib + l];
         const bool live = act && f64::positive(cb);  // at r = h the pair does nothing
         double dA, dB, margin;
@@ -417,7 +424,7 @@ void launch_colours64(const Consts& c, const Workspace& w, int cur, double dt, u
         c, fd_const<double>(c, dt), k, view<Fp64>(w, cur), (D4*)w.qp4, w.cell_start, w.mrank, w.sched_hdr,
         w.sched_rsize, w.sched_off, w.sched_pair, (const double*)w.st_geom, (const double*)w.st_rnd, w.st_aux, col,
         seed, w.sweep, w.counters, w.status, REC ? w.pair_recs : nullptr, w.pair_rec_count, w.pair_rec_cap,
-        w.fd_queue + 3 * col, w.blk_order, w.big_perm, w.big_list, w.big_count);
+        w.fd_queue + 4 * col, w.blk_order, w.big_perm, w.big_list, w.big_count);
 }
 
 }  // namespace sdpd

@@ -14,11 +14,15 @@ namespace sdpd {
 // ---------------------------------------------------------------------------
 constexpr int kMaxBlock = 256;   // particles in a block (8-bit local index)
 constexpr int kMaxPairs = 2048;  // owned pairs of a block
-constexpr int kMaxLevels = 255;  // dependency levels of a block's pair schedule
+constexpr int kLargeBlock = 512;   // the same of a large block (k_sched_large; in a
+constexpr int kLargePairs = 4096;  // colour launch it has a whole warp or team)
+constexpr int kMaxLevels = 255;  // rounds of a block's pair schedule
 // Schedule header of a block beyond one of these capacities: its sweep runs
 // in canonical order, one pair after the other, on the whole warp that takes
 // it (no shared-memory schedule), so any block size completes.
 constexpr uint32_t kHdrBig = 0xFFFFFFFFu;
+constexpr uint32_t kHdrLarge = 0xFFFFFFFEu;    // between k_sched_enum and k_sched_large: not scheduled yet
+constexpr uint32_t kHdrLargeFlag = 1u << 24;  // header of a large block: npairs | nrounds << 16 | this
 constexpr int kRoundStride = 256;  // bytes per block of the round sizes (>= kMaxLevels)
 // Entries of the dense pair arrays: the scheduled blocks own at most half the
 // neighbour-list entries (a member whose list overflowed leaves its block to
@@ -358,7 +362,7 @@ struct Workspace {
   uint8_t* sched_rsize;   // [ncell][kRoundStride] pairs of each round
   unsigned long long* sched_off;    // [ncell] where the block's pairs start in the arrays below
   unsigned long long* sched_total;  // entries of those arrays in use
-  uint16_t* sched_pair;   // pairs round by round, block after block
+  uint32_t* sched_pair;   // pairs round by round, block after block (local min-id | local max-id << 16)
   void* st_geom;          // per scheduled pair: unit vector, F / (rho_i rho_j)
   void* st_rnd;           // per scheduled pair: its random numbers (see k_stage_random)
   double* st_aux;         // float64 pair arithmetic: |G|^2 / 2 - ln U per scheduled pair
@@ -374,12 +378,15 @@ struct Workspace {
   int* status;
   uint32_t* blk_hist;            // [8][256]: blocks of each colour by dependency depth, then cursors
   int32_t* blk_order;            // [8][ncell / 8]: each colour's blocks, deepest first
-  unsigned* fd_queue;            // [8][3]: next block, finished warps and next entry of
-                                 // big_list of each colour launch; zero between launches
+  unsigned* fd_queue;            // [8][4]: next block, finished warps and next entries of
+                                 // big_list and large_list of each colour launch; zero between launches
   int32_t* big_perm;             // [N]: rank order of the particles of blocks beyond capacity
   int2* big_list;                // [8][ncell / 8]: each colour's blocks beyond capacity (owner
                                  // cell, offset in big_perm)
   uint32_t* big_count;           // [8] entries of big_list, then [8] entries of big_perm in use
+  int32_t* large_cand;           // [ncell] blocks left to k_sched_large
+  int32_t* large_list;           // [8][ncell / 8]: each colour's large blocks
+  uint32_t* large_count;         // [8] entries of large_list, then of large_cand, then finished thread blocks
   // particles whose neighbour list overflows its row, listed by the density
   // pass into one of two slots: [2][N] entries and [2] counts.  A density
   // pass fills slot *ovf_slot (toggled on the host before each launch) and
@@ -427,9 +434,10 @@ template <class P>
 void launch_force(const Consts& c, const Workspace& w, int cur, double half_dt, double dt_drift,
                   double* force_by_id, cudaStream_t s);
 // the sweep schedule: P the state's storage policy, width the most pairs of a
-// round; the staged geometry (arithmetic policy A) completes it
+// round (large_width: of a large block's); the staged geometry (arithmetic policy A) completes it
 template <class P>
-void launch_fd_schedule(const Consts& c, const Workspace& w, int cur, int width, cudaStream_t s);
+void launch_fd_schedule(const Consts& c, const Workspace& w, int cur, int width, int large_width, cudaStream_t s);
+int sched_prepare();  // launch attributes of the schedule's kernels (SDPD_OK or SDPD_ERR_CUDA)
 template <class P, class A>
 void launch_stage_geometry(const Consts& c, const Workspace& w, int cur, cudaStream_t s);
 // one sweep (random numbers, then the colours): P the state's storage policy,
@@ -441,7 +449,7 @@ void launch_fd_colours(const Consts& c, const Workspace& w, int cur, double dt, 
                        cudaStream_t s);
 template <class P>
 void launch_observables(const Consts& c, const Workspace& w, int cur, cudaStream_t s);
-int fd_round_width(const Consts& c, bool float_arith);  // pairs of a block that a colour launch updates at once
+int fd_round_width(const Consts& c, bool float_arith, bool large);  // pairs of a block that a colour launch updates at once
 // sweep counter on the device: set to a value, or advanced by one
 void launch_set_sweep(const Workspace& w, unsigned long long value, cudaStream_t s);
 void launch_advance_sweep(const Workspace& w, cudaStream_t s);
