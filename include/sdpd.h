@@ -313,11 +313,11 @@ typedef struct {
   int fd_variant;   /* blocks per warp x warps per thread block of the colour
                        launches: 0 (2 x 2), 1 (2 x 1), 2 (1 x 1), 3 (1 x 2),
                        4 (1 x 4); -1 = chosen at launch by the blocks per
-                       colour (3 up to 2432 of them, else 0;
+                       colour (2 up to 912 of them, 1 up to 4864, else 0;
                        sdpd_get_tuning then reports 0 for float32 and 1 for
                        float64 pair arithmetic); a new handle starts with -1.
-                       Float64 pair arithmetic has one schedule, two warps
-                       per block, whatever the value */
+                       Float64 pair arithmetic has one schedule, a team of
+                       warps per block, whatever the value */
   int pair_threads; /* threads per block of the density and force passes:
                        32, 64 or 128; 0 = 128 (and, float64 with at most 2432
                        particles, a warp per particle instead of 8 lanes) */

@@ -73,16 +73,16 @@ struct Consts {
 constexpr int kFdVariants = 5;
 __host__ __device__ constexpr int fd_default_variant(bool mixed) { return mixed ? 0 : 1; }
 // The block schedule of a handle's colour launches with float32 pair
-// arithmetic (float64 has one, k_fd_colour64): the one set by the caller
-// or the autotuner, else by the blocks per colour.  Few blocks: a colour
-// lasts as long as its deepest block, which runs faster on a warp of its own
-// (variant 3; 32^3, 216 blocks per colour).  More blocks than resident warps:
-// two per warp use its lanes better (the defaults).
-constexpr int64_t kFdOwnWarpBlocks = 16 * 152;  // 16 warps on each of 152 SMs
+// arithmetic (float64 has one, k_fd_colour64): the one set by the caller or
+// the autotuner, else by the blocks per colour.  Few blocks: a colour lasts as
+// long as its deepest block, which runs fastest on a warp of its own; from
+// about six blocks per SM on two per warp use its lanes better.  Microseconds
+// per sweep with schedules 0 / 1 / 2: 512 blocks 613 / 636 / 594, 1331 blocks
+// 791 / 756 / 785, 4096 blocks 1091 / 1069 / 1457, 6859 blocks 1711 / 1734 / 2340.
 inline int fd_launch_variant(const Consts& c) {
   if (!c.fd_auto && c.fd_variant >= 0 && c.fd_variant < kFdVariants) return c.fd_variant;
   const int64_t nown = (int64_t)(c.nc[0] / 2) * (c.nc[1] / 2) * (c.nc[2] / 2);
-  return nown <= kFdOwnWarpBlocks ? 3 : fd_default_variant(true);
+  return nown <= 6 * 152 ? 2 : (nown <= 32 * 152 ? 1 : 0);
 }
 __host__ __device__ constexpr bool pair_threads_ok(int t) { return t == 32 || t == 64 || t == 128; }
 // whether a block schedule's shared memory fits a thread block (float64
