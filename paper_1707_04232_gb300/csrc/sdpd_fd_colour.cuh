@@ -1311,16 +1311,13 @@ void launch_colours32(const Consts& c, const Workspace& w, int cur, double dt, u
 
 // Fills the resident-block counts of every block schedule ahead of time (a
 // host query, kept out of stream captures).
-template <bool REC>
-int team64_resident();
-template <bool REC>
-void launch_colours64(const Consts& c, const Workspace& w, int cur, double dt, uint64_t seed, cudaStream_t s);
+void team64_prepare();
+void launch_team64(const Consts& c, const Workspace& w, int cur, double dt, uint64_t seed, int record, cudaStream_t s);
 
 template <class P, class A>
 void fd_prepare() {
   if constexpr (!A::mixed) {
-    team64_resident<false>();
-    team64_resident<true>();
+    team64_prepare();
   } else {
     for (int v = 0; v < kFdVariants; ++v) {
       fd_resident<P, false>(v);
@@ -1357,8 +1354,7 @@ void launch_fd_colours(const Consts& c, const Workspace& w, int cur, double dt, 
                                                                 (const typename A::V4*)w.st_geom,
                                                                 (typename A::V4*)w.st_rnd, w.st_aux);
   if constexpr (!A::mixed) {
-    if (record) launch_colours64<true>(c, w, cur, dt, seed, s);
-    else launch_colours64<false>(c, w, cur, dt, seed, s);
+    launch_team64(c, w, cur, dt, seed, record, s);
   } else {
     if (record) launch_colours32<P, true>(c, w, cur, dt, seed, fd_launch_variant(c), s);
     else launch_colours32<P, false>(c, w, cur, dt, seed, fd_launch_variant(c), s);

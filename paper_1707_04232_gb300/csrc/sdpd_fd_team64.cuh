@@ -1,4 +1,4 @@
-// sdpd_fd_team64.cuh -- the colour kernel of the float64 sweep: a team of two
+// sdpd_fd_team64.cuh -- the colour kernel of the float64 sweep: a team of
 // warps per block, four lanes per pair.
 //
 // GB300 issues one float64 warp instruction per 64 cycles on each quarter of
@@ -13,6 +13,13 @@
 // reverse noise, and the logarithms of the Metropolis ratio are each
 // evaluated once per instruction for the whole pair: about 95 float64
 // instructions per round.  Rounds hold at most 16 pairs (8 per warp).
+//
+// EMS: the proposal (about 45 of them) and the Metropolis test (50) run on
+// different warps, one round apart.  Two warps propose round r and write its
+// moves into the shared state at once; while they go on to round r + 1, two
+// others test round r.  When they reject a move (1e-4 to 3e-2 of the pairs)
+// the proposers take round r + 1 back, then the rejected moves, and propose
+// round r + 1 again, so the result is the sequential one.
 #pragma once
 #include "sdpd_fd_colour.cuh"
 
@@ -149,75 +156,81 @@ __device__ __forceinline__ double quad_sum(double v) {
   return v;
 }
 
-// One pair update on the four lanes of a quad (whole warps call it).  l: the
-// lane's place in the quad; A, B: component l of the two particles' records
-// (px, py, pz, eps); ge: component l of (e, base); Gl: component l of
-// (G - (e.G) e, e.G); c0 = |G|^2 / 2 - ln U.  live: the pair exists and
-// base > 0.  Returns the decision (0 accept, 1 energy bound, 2 Metropolis);
-// dA, dB are the lane's changes of A and B.
-__device__ __forceinline__ int team_pair(const Team64Const& k, int l, bool live, double A, double B, double ge,
-                                         double Gl, double base, double c0, double& dA, double& dB, double& margin,
-                                         bool& neg) {
-  const double ei = __shfl_sync(0xffffffffu, A, 3, 4), ej = __shfl_sync(0xffffffffu, B, 3, 4);
-  const double x_dir = l == 3 ? k.x_par : k.x_perp;
+// What the test of a move needs from its proposal, per lane and per pair.
+struct Team64Move {
+  double m, z, U;            // this lane's alpha - 1, hz, half velocity component (momentum units)
+  double deps, ei, ej, r0;   // r0: 1/P on lane 2
+  bool bound;                // both new energies positive
+};
+
+// The proposal of one pair on the four lanes of a quad (whole warps call it).
+// l: the lane's place in the quad; A, B: component l of the two particles'
+// records (px, py, pz, eps); ge: component l of (e, base); Gl: component l of
+// (G - (e.G) e, e.G).  dA, dB: the lane's changes of A and B.
+__device__ __forceinline__ Team64Move team_propose(const Team64Const& k, int l, double A, double B, double ge,
+                                                   double Gl, double base, double& dA, double& dB) {
+  Team64Move v;
+  v.ei = __shfl_sync(0xffffffffu, A, 3, 4);
+  v.ej = __shfl_sync(0xffffffffu, B, 3, 4);
   const double el = l == 3 ? 0.0 : ge;
   const double u = A - B;
-  const double E = ei + ej, P = ei * ej;
+  const double E = v.ei + v.ej, P = v.ei * v.ej;
   // lane 2 takes 1/P (for the entropy term) while the others take 1/E
-  const double r0 = f64::rcp(l == 2 ? P : E);
-  const double iE = __shfl_sync(0xffffffffu, r0, 0, 4);
-  double m, z;
-  team_coeffs<false>(k, x_dir, base, P, iE, m, z);
+  v.r0 = f64::rcp(l == 2 ? P : E);
+  const double iE = __shfl_sync(0xffffffffu, v.r0, 0, 4);
+  team_coeffs<false>(k, l == 3 ? k.x_par : k.x_perp, base, P, iE, v.m, v.z);
   // u/2 split along and across e: lane 3 holds the component along it
   const double upar = quad_sum(el * u);
-  const double U = 0.5 * (l == 3 ? upar : __fma_rn(-upar, el, u));
-  const double v = __fma_rn(m, U, z * Gl);
-  const double dpar = __shfl_sync(0xffffffffu, v, 3, 4);
-  const double dp = l == 3 ? 0.0 : __fma_rn(dpar, el, v);
+  v.U = 0.5 * (l == 3 ? upar : __fma_rn(-upar, el, u));
+  const double w = __fma_rn(v.m, v.U, v.z * Gl);
+  const double wpar = __shfl_sync(0xffffffffu, w, 3, 4);
+  const double dp = l == 3 ? 0.0 : __fma_rn(wpar, el, w);
   // kinetic energy change of the pair: dp . (u + dp) / m
-  const double deps = k.de * quad_sum(dp * (u + dp));
-  const double fi = ei + deps, fj = ej + deps;
-  const bool bound = f64::positive(fi) && f64::positive(fj);
-  margin = fi < fj ? fi : fj;
-  int decision = 0;
-  if (k.scheme == SDPD_SCHEME_SSA) {
-    neg |= live && !bound;
-  } else {
-    decision = bound ? 0 : 1;
-    if (k.scheme == SDPD_SCHEME_EMS) {
-      // reverse move from v' with the coefficients at the proposed energies;
-      // reverse noise per direction [(1 - alpha' alpha) u/2 - alpha' hz G] / hz'
-      const double P2 = fi * fj;
-      double mr, iz;
-      team_coeffs<true>(k, x_dir, base, P2, f64::rcp(fi + fj), mr, iz);
-      const double cr = -__fma_rn(m, mr, m + mr);
-      const double g = __fma_rn(cr, U, -(__fma_rn(mr, z, z) * Gl)) * iz;
-      // ln|B(v)| - ln|B(v')| = ln(z z') along + 2 ln(z z') across e (lanes 3,
-      // 0, 1); entropy (C_K/kB - 1) ln(eps' products / eps products) (lane 2)
-      const double t = deps * (E + deps);
-      const double lg = f64::log1p(l == 2 ? t * r0 : __fma_rn(z, iz, -1.0));
-      const double mg = c0 + quad_sum(__fma_rn(-0.5 * g, g, l == 2 ? k.CKm1 * lg : lg));
-      if (bound) {
-        margin = mg;
-        if (f64::negative(mg)) decision = 2;  // U > exp(a)
-      }
-    }
-  }
-  dA = l == 3 ? deps : dp;
-  dB = l == 3 ? deps : -dp;
-  return decision;
+  v.deps = k.de * quad_sum(dp * (u + dp));
+  v.bound = f64::positive(v.ei + v.deps) && f64::positive(v.ej + v.deps);
+  dA = l == 3 ? v.deps : dp;
+  dB = l == 3 ? v.deps : -dp;
+  return v;
 }
 
-// Shared memory of a team's block: records (px, py, pz, eps).
+// The Metropolis margin a - ln U of Eq. (metropolis-ratio) of a move: the
+// reverse move from v' with the coefficients at the proposed energies, its
+// noise per direction [(1 - alpha' alpha) u/2 - alpha' hz G] / hz'.
+// c0 = |G|^2 / 2 - ln U.
+__device__ __forceinline__ double team_margin(const Team64Const& k, int l, const Team64Move& v, double Gl, double base,
+                                              double c0) {
+  const double fi = v.ei + v.deps, fj = v.ej + v.deps;
+  double mr, iz;
+  team_coeffs<true>(k, l == 3 ? k.x_par : k.x_perp, base, fi * fj, f64::rcp(fi + fj), mr, iz);
+  const double cr = -__fma_rn(v.m, mr, v.m + mr);
+  const double g = __fma_rn(cr, v.U, -(__fma_rn(mr, v.z, v.z) * Gl)) * iz;
+  // ln|B(v)| - ln|B(v')| = ln(z z') along + 2 ln(z z') across e (lanes 3, 0,
+  // 1); entropy (C_K/kB - 1) ln(eps' products / eps products) (lane 2)
+  const double t = v.deps * ((v.ei + v.ej) + v.deps);
+  const double lg = f64::log1p(l == 2 ? t * v.r0 : __fma_rn(v.z, iz, -1.0));
+  return c0 + quad_sum(__fma_rn(-0.5 * g, g, l == 2 ? k.CKm1 * lg : lg));
+}
+
+constexpr int kTeamPairs = 16;    // pairs of a round
+constexpr int kTeamThreads = 64;  // a quad per pair
+template <bool EMS>
+constexpr int team_threads() { return EMS ? 2 * kTeamThreads : kTeamThreads; }
+
+// Shared memory of a team: the block's records (px, py, pz, eps), and the
+// moves of two rounds.
 struct Team64Smem {
   D4 s[kLargeBlock];
   FdCells cells;
+  uint8_t rsize[kRoundStride];
+  double m[2][kTeamThreads], z[2][kTeamThreads], U[2][kTeamThreads], r0[2][kTeamPairs];
+  double deps[2][kTeamPairs], ei[2][kTeamPairs], ej[2][kTeamPairs];
+  uint8_t bound[2][kTeamPairs];
+  unsigned rejected[2];  // quads (their lanes' bits) of the last tested round, per warp
+  unsigned next;
 };
 
-constexpr int kTeamWarps = 2, kTeamPairs = 8 * kTeamWarps;
-
-template <bool REC>
-__global__ void __launch_bounds__(kTeamWarps * 32)
+template <bool EMS, bool REC>
+__global__ void __launch_bounds__(team_threads<EMS>())
     k_fd_colour64(const __grid_constant__ Consts c, const __grid_constant__ FDConst<double> kbig, Team64Const k,
                   const __grid_constant__ Arrays<Fp64> a, D4* __restrict__ qp4,
                   const int32_t* __restrict__ cell_start, const int32_t* __restrict__ mrank,
@@ -228,12 +241,12 @@ __global__ void __launch_bounds__(kTeamWarps * 32)
                   int* status, sdpd_pair_rec* recs, unsigned long long* rec_count, int64_t rec_cap,
                   unsigned* __restrict__ queue, const int32_t* __restrict__ order, int32_t* __restrict__ big_perm,
                   const int2* __restrict__ big_list, const uint32_t* __restrict__ big_count) {
+  constexpr int kThreads = team_threads<EMS>();
   __shared__ Team64Smem sm;
-  __shared__ uint8_t size_s[kRoundStride];
-  __shared__ unsigned next_s;
   const uint64_t sweep = *sweep_ptr;
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-  const int l = lane & 3, slot = warp * 8 + (lane >> 2);  // place in the quad, pair of the round
+  const bool tester = EMS && t >= kTeamThreads;
+  const int tt = t % kTeamThreads, l = tt & 3, slot = tt >> 2;  // quad lane, pair of the round
   const int hx = c.nc[0] >> 1, hy = c.nc[1] >> 1, hz = c.nc[2] >> 1;
   const int64_t nown = (int64_t)hx * hy * hz;
   const double pi_coef = c.c_rho / (c.C_K * c.m);
@@ -242,9 +255,9 @@ __global__ void __launch_bounds__(kTeamWarps * 32)
   double* rec = reinterpret_cast<double*>(sm.s);
   // blocks from the colour's queue, deepest first (see k_fd_colour)
   for (;;) {
-    if (t == 0) next_s = atomicAdd(queue, 1u);
+    if (t == 0) sm.next = atomicAdd(queue, 1u);
     __syncthreads();
-    const unsigned wi = next_s;
+    const unsigned wi = sm.next;
     if ((int64_t)wi >= nown) break;
     const int64_t w = order[colour * nown + wi];
     const int ox = 2 * (int)(w % hx) + (colour & 1), oy = 2 * (int)((w / hx) % hy) + ((colour >> 1) & 1),
@@ -258,7 +271,7 @@ __global__ void __launch_bounds__(kTeamWarps * 32)
     }
     if (t == 0) n_tot += (unsigned)np;
     const unsigned long long first = sched_off[o];
-    for (int r = t; r < nr; r += kTeamWarps * 32) size_s[r] = rsize[o * kRoundStride + r];
+    for (int r = t; r < nr; r += kThreads) sm.rsize[r] = rsize[o * kRoundStride + r];
     BlockCells b;
     block_cells(c, ox, oy, oz, mrank, cell_start, b);
     const int nb = b.base[8];
@@ -269,74 +282,147 @@ __global__ void __launch_bounds__(kTeamWarps * 32)
         sm.cells.cbs[q] = b.base[q];
       }
     __syncthreads();
-    for (int q = t; q < nb; q += kTeamWarps * 32) {
+    for (int q = t; q < nb; q += kThreads) {
       const int g = block_gidx(sm.cells, q);
       sm.s[q] = D4{a.px[g], a.py[g], a.pz[g], a.eps[g]};
     }
-    // this quad's pair of a round, loaded one round ahead
+    // this quad's pair of a round, loaded one round ahead; a tester meets
+    // round r one step after its proposer.  The round sizes never exceed the
+    // team's pairs (the schedule's width).
     uint32_t pr = 0;
     double ge = 0.0, Gl = 0.0, base = 0.0, c0 = 0.0;
-    int r = 0, pos = 0, left = size_s[0], n = min(left, kTeamPairs);
+    int pos = 0, n = sm.rsize[0];
     auto fetch = [&]() {
       if (slot < n) {
         const unsigned long long at = first + pos + slot;
-        pr = __ldg(&pairs[at]);
-        ge = __ldg(&geom[4 * at + l]);
+        if (!tester || REC) pr = __ldg(&pairs[at]);
+        if (!tester) ge = __ldg(&geom[4 * at + l]);
         base = __ldg(&geom[4 * at + 3]);
         Gl = __ldg(&rnd[4 * at + l]);
-        c0 = __ldg(&aux[at]);
+        if (tester) c0 = __ldg(&aux[at]);
       }
     };
     fetch();
     __syncthreads();
-    while (n > 0) {
-      const bool act = slot < n;
-      const int busy = n - warp * 8, level = r;  // pairs of this warp
+    uint32_t last_pr = 0;  // the proposer's pair of the round before, and its values before the move
+    double lastA = 0.0, lastB = 0.0;
+    const int steps = EMS ? nr + 1 : nr;
+    for (int st = 0; st < steps; ++st) {
+      const int r = tester ? st - 1 : st;  // this warp's round
+      const bool on = r >= 0 && r < nr;
+      const int cn = on ? n : 0, buf = r & 1;
+      const bool act = slot < cn, busy = (tt & 32) / 4 < cn;  // this quad, this warp has a pair
       const uint32_t cpr = act ? pr : 0u;
       // (lanes without a pair run on values that keep to the short paths)
       const double cge = ge, cG = act ? Gl : 0.0, cb = act ? base : 0.01, cc = c0;
-      pos += n;
-      left -= n;
-      if (left == 0) left = ++r < nr ? (int)size_s[r] : 0;
-      n = min(left, kTeamPairs);
-      fetch();
-      if (busy > 0) {
-        const int ia = cpr & 0xffffu, ib = cpr >> 16;
-        const double A = rec[4 * ia + l], B = rec[4 * ib + l];
-        const bool live = act && f64::positive(cb);  // at r = h the pair does nothing
-        double dA, dB, margin;
-        int dcs = team_pair(k, l, live, A, B, cge, cG, cb, cc, dA, dB, margin, negative);
-        if (!live) {
-          dcs = 0;
-          margin = 0.0;
-        } else if (dcs == 0) {
+      if (on) {
+        pos += n;
+        n = r + 1 < nr ? (int)sm.rsize[r + 1] : 0;
+        fetch();
+      }
+      const bool live = act && f64::positive(cb);  // at r = h the pair does nothing
+      const int ia = cpr & 0xffffu, ib = cpr >> 16;
+      double A = 0.0, B = 0.0;
+      bool moved = false;
+      Team64Move v;
+      // proposes round r on the current state and moves it
+      auto propose = [&]() {
+        A = rec[4 * ia + l];
+        B = rec[4 * ib + l];
+        double dA, dB;
+        v = team_propose(k, l, A, B, cge, cG, cb, dA, dB);
+        moved = live && (v.bound || k.scheme == SDPD_SCHEME_SSA);
+        if (moved) {
           rec[4 * ia + l] = A + dA;
           rec[4 * ib + l] = B + dB;
         }
-        if (act && l == 0) {
-          n_rb += dcs == 1;
-          n_rm += dcs == 2;
-          if constexpr (REC) {
-            const unsigned long long s = atomicAdd(rec_count, 1ull);
-            if ((int64_t)s < rec_cap) {
-              sdpd_pair_rec rc;
-              rc.id_i = a.id[block_gidx(sm.cells, ia)];
-              rc.id_j = a.id[block_gidx(sm.cells, ib)];
-              rc.colour = colour;
-              rc.owner = (int32_t)o;
-              rc.decision = dcs;
-              rc.level = level;
-              rc.margin = margin;
-              rc.margin_lo = margin;
-              rc.margin_tol = 0.0;
-              recs[s] = rc;
-            }
+        if (EMS && act) {
+          sm.m[buf][tt] = v.m;
+          sm.z[buf][tt] = v.z;
+          sm.U[buf][tt] = v.U;
+          if (l == 2) sm.r0[buf][slot] = v.r0;
+          if (l == 0) {
+            sm.deps[buf][slot] = v.deps;
+            sm.ei[buf][slot] = v.ei;
+            sm.ej[buf][slot] = v.ej;
+            sm.bound[buf][slot] = v.bound;
+          }
+        }
+      };
+      int dcs = 0;
+      double margin = 0.0;
+      if (!tester) {
+        if (busy) propose();
+        if (!EMS && live) {
+          margin = fmin(v.ei + v.deps, v.ej + v.deps);
+          if (k.scheme == SDPD_SCHEME_SSA) negative |= !v.bound;
+          else dcs = v.bound ? 0 : 1;
+        }
+      } else {
+        if (busy) {
+          v.m = sm.m[buf][tt];
+          v.z = sm.z[buf][tt];
+          v.U = sm.U[buf][tt];
+          v.r0 = sm.r0[buf][slot];
+          v.deps = sm.deps[buf][slot];
+          v.ei = sm.ei[buf][slot];
+          v.ej = sm.ej[buf][slot];
+          v.bound = sm.bound[buf][slot];
+          const double mg = team_margin(k, l, v, cG, cb, cc);
+          if (live) {
+            dcs = !v.bound ? 1 : (f64::negative(mg) ? 2 : 0);  // 2: U > exp(a)
+            margin = v.bound ? mg : fmin(v.ei + v.deps, v.ej + v.deps);
+          }
+        }
+        const unsigned rej = __ballot_sync(0xffffffffu, dcs == 2);
+        if (lane == 0) sm.rejected[warp & 1] = rej;
+      }
+      if ((tester || !EMS) && act && l == 0) {
+        n_rb += dcs == 1;
+        n_rm += dcs == 2;
+        if constexpr (REC) {
+          const unsigned long long at = atomicAdd(rec_count, 1ull);
+          if ((int64_t)at < rec_cap) {
+            sdpd_pair_rec rc;
+            rc.id_i = a.id[block_gidx(sm.cells, ia)];
+            rc.id_j = a.id[block_gidx(sm.cells, ib)];
+            rc.colour = colour;
+            rc.owner = (int32_t)o;
+            rc.decision = dcs;
+            rc.level = r;
+            rc.margin = margin;
+            rc.margin_lo = margin;
+            rc.margin_tol = 0.0;
+            recs[at] = rc;
           }
         }
       }
       __syncthreads();
+      if constexpr (EMS) {
+        if (sm.rejected[0] | sm.rejected[1]) {
+          // a move of the round before was rejected: this round's moves back,
+          // then the rejected ones, then this round once more
+          if (!tester && moved) {
+            rec[4 * ia + l] = A;
+            rec[4 * ib + l] = B;
+          }
+          __syncthreads();
+          if (!tester && (sm.rejected[warp] >> lane & 1u)) {
+            rec[4 * (last_pr & 0xffffu) + l] = lastA;
+            rec[4 * (last_pr >> 16) + l] = lastB;
+          }
+          __syncthreads();
+          if (t < 2) sm.rejected[t] = 0u;
+          if (!tester && busy) propose();
+          __syncthreads();
+        }
+        last_pr = cpr;
+        lastA = A;
+        lastB = B;
+      }
     }
-    for (int q = t; q < nb; q += kTeamWarps * 32) {
+    __syncthreads();
+    for (int q = t; q < nb; q += kThreads) {
       const int g = block_gidx(sm.cells, q);
       const D4 v = lds4(&sm.s[q]);
       a.px[g] = v.x; a.py[g] = v.y; a.pz[g] = v.z;
@@ -368,7 +454,7 @@ __global__ void __launch_bounds__(kTeamWarps * 32)
     bad |= bc.bad != 0;
   }
   if (lane == 0) {
-    const unsigned total = gridDim.x * (unsigned)kTeamWarps;
+    const unsigned total = gridDim.x * (unsigned)(kThreads / 32);
     __threadfence();  // this warp's last take from the queue is performed before it counts as done
     if (atomicAdd(&queue[1], 1u) == total - 1u) {
       queue[0] = 0u;
@@ -381,7 +467,7 @@ __global__ void __launch_bounds__(kTeamWarps * 32)
                  c_rm = __reduce_add_sync(0xffffffffu, n_rm);
   const unsigned any_neg = __any_sync(0xffffffffu, negative), any_bad = __any_sync(0xffffffffu, bad);
   if (lane == 0) {
-    // (the team's pairs are counted on its first warp, rejections on both:
+    // (the team's pairs are counted on its first warp, rejections on others:
     // accepted = pairs - rejected, added with wrap-around)
     if (c_tot || c_rb || c_rm) {
       atomicAdd(&counters[0], (unsigned long long)c_tot);
@@ -395,19 +481,25 @@ __global__ void __launch_bounds__(kTeamWarps * 32)
 }
 
 // Thread blocks of the team kernel resident at once (see fd_resident_blocks).
-template <bool REC>
+template <bool EMS, bool REC>
 int team64_resident() {
   static const int n = [] {
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fd_colour64<REC>, kTeamWarps * 32, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fd_colour64<EMS, REC>, team_threads<EMS>(), 0);
     return std::max(1, sms) * std::max(1, per_sm);
   }();
   return n;
 }
+void team64_prepare() {
+  team64_resident<true, true>();
+  team64_resident<true, false>();
+  team64_resident<false, true>();
+  team64_resident<false, false>();
+}
 
-template <bool REC>
+template <bool EMS, bool REC>
 void launch_colours64(const Consts& c, const Workspace& w, int cur, double dt, uint64_t seed, cudaStream_t s) {
   Team64Const k;
   k.x_par = -2.0 * c.kpar_m2 * (dt / c.m);
@@ -418,13 +510,21 @@ void launch_colours64(const Consts& c, const Workspace& w, int cur, double dt, u
   k.CKm1 = c.C_K / c.kB - 1.0;
   k.scheme = c.scheme;
   const int64_t nown = (int64_t)(c.nc[0] / 2) * (c.nc[1] / 2) * (c.nc[2] / 2);
-  const unsigned gf = (unsigned)std::max<int64_t>(1, std::min<int64_t>(nown, team64_resident<REC>()));
+  const unsigned gf = (unsigned)std::max<int64_t>(1, std::min<int64_t>(nown, team64_resident<EMS, REC>()));
   for (int col = 0; col < 8; ++col)
-    k_fd_colour64<REC><<<gf, kTeamWarps * 32, 0, s>>>(
+    k_fd_colour64<EMS, REC><<<gf, team_threads<EMS>(), 0, s>>>(
         c, fd_const<double>(c, dt), k, view<Fp64>(w, cur), (D4*)w.qp4, w.cell_start, w.mrank, w.sched_hdr,
         w.sched_rsize, w.sched_off, w.sched_pair, (const double*)w.st_geom, (const double*)w.st_rnd, w.st_aux, col,
         seed, w.sweep, w.counters, w.status, REC ? w.pair_recs : nullptr, w.pair_rec_count, w.pair_rec_cap,
         w.fd_queue + 4 * col, w.blk_order, w.big_perm, w.big_list, w.big_count);
+}
+void launch_team64(const Consts& c, const Workspace& w, int cur, double dt, uint64_t seed, int record,
+                   cudaStream_t s) {
+  const bool ems = c.scheme == SDPD_SCHEME_EMS;
+  if (ems && record) launch_colours64<true, true>(c, w, cur, dt, seed, s);
+  else if (ems) launch_colours64<true, false>(c, w, cur, dt, seed, s);
+  else if (record) launch_colours64<false, true>(c, w, cur, dt, seed, s);
+  else launch_colours64<false, false>(c, w, cur, dt, seed, s);
 }
 
 }  // namespace sdpd
