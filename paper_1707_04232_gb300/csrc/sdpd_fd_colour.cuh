@@ -506,6 +506,14 @@ __device__ __forceinline__ S stage_F(S r, S inv_h, S cF) {
   return kernel_F<KIND>(r * inv_h, cF);
 }
 
+// Warps per block of the staging kernels: one, or as many (up to 16) as fill
+// the GPU's 608 SM quarters eight times where blocks are few (10^3 particles,
+// 64 blocks: the float64 random numbers take 189 us with one).
+inline int stage_split(int64_t ncell) {
+  const int64_t n = 8 * 608 / (ncell > 0 ? ncell : 1);
+  return (int)(n < 1 ? 1 : (n > 16 ? 16 : n));
+}
+
 // The block's cells into shared memory, by the whole warp.
 __device__ __forceinline__ void stage_cells(const Consts& c, int64_t o, const int32_t* __restrict__ mrank,
                                             const int32_t* __restrict__ cell_start, int lane, FdCells& cells) {
@@ -540,16 +548,17 @@ __global__ void __launch_bounds__(kStageWarps * 32)
                      const int32_t* __restrict__ mrank, const uint32_t* __restrict__ xmx,
                      const uint32_t* __restrict__ xmy, const uint32_t* __restrict__ xmz,
                      const uint32_t* __restrict__ hdr, const unsigned long long* __restrict__ sched_off,
-                     const uint32_t* __restrict__ pairs, typename A::V4* __restrict__ geom) {
+                     const uint32_t* __restrict__ pairs, int split, typename A::V4* __restrict__ geom) {
   using R = typename A::R;
   using S = typename P::R;
   __shared__ FdCells cells_s[kStageWarps];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t o = (int64_t)blockIdx.x * kStageWarps + warp;
+  const int64_t wg = (int64_t)blockIdx.x * kStageWarps + warp, o = wg / split;
   if (o >= c.ncell) return;
+  const int part = (int)(wg - o * split);
   const uint32_t hd = hdr[o];
   const int np = hd == kHdrBig ? 0 : (int)(hd & 0xffffu);
-  if (np == 0) return;
+  if (32 * part >= np) return;
   FdCells& cells = cells_s[warp];
   stage_cells(c, o, mrank, cell_start, lane, cells);
   int ox, oy, oz;
@@ -558,7 +567,7 @@ __global__ void __launch_bounds__(kStageWarps * 32)
   geo.init(c, ox, oy, oz, xmx, xmy, xmz);
   const S inv_h = (S)(1.0 / c.h), cF = (S)c.cF;
   const unsigned long long base = sched_off[o];
-  for (int t = lane; t < np; t += 32) {
+  for (int t = 32 * part + lane; t < np; t += 32 * split) {
     const uint32_t pr = pairs[base + t];
     int da, db;
     const int ga = block_gidx(cells, pr & 0xffffu, da), gb = block_gidx(cells, pr >> 16, db);
@@ -590,26 +599,28 @@ __global__ void __launch_bounds__(kStageWarps * 32)
     k_stage_random(Consts c, const int32_t* __restrict__ id, const int32_t* __restrict__ cell_start,
                    const int32_t* __restrict__ mrank, const uint32_t* __restrict__ hdr,
                    const unsigned long long* __restrict__ sched_off, const uint32_t* __restrict__ pairs,
-                   uint64_t seed, const unsigned long long* __restrict__ sweep_ptr,
+                   int split, uint64_t seed, const unsigned long long* __restrict__ sweep_ptr,
                    const typename A::V4* __restrict__ geom, typename A::V4* __restrict__ rnd,
                    double* __restrict__ aux) {
   using R = typename A::R;
   __shared__ FdCells cells_s[kStageWarps];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t o = (int64_t)blockIdx.x * kStageWarps + warp;
+  const int64_t wg = (int64_t)blockIdx.x * kStageWarps + warp, o = wg / split;
   if (o >= c.ncell) return;
+  const int part = (int)(wg - o * split);
   const uint32_t hd = hdr[o];
   const int np = hd == kHdrBig ? 0 : (int)(hd & 0xffffu);
-  if (np == 0) return;
+  if (32 * part >= np) return;
   FdCells& cells = cells_s[warp];
   stage_cells(c, o, mrank, cell_start, lane, cells);
   const uint64_t sweep = *sweep_ptr;
   const unsigned long long base = sched_off[o];
-  for (int t = lane; t < np; t += 32) {
+  for (int t = 32 * part + lane; t < np; t += 32 * split) {
     const uint32_t pr = pairs[base + t];
     const int ga = block_gidx(cells, pr & 0xffffu), gb = block_gidx(cells, pr >> 16);  // ga holds the lower id
     R G[3], U;
-    pair_randoms_fast(seed, sweep, (uint64_t)id[ga], (uint64_t)id[gb], G, &U);
+    // (ids as unsigned 32-bit numbers: the high words of the counter are known to be zero)
+    pair_randoms_fast(seed, sweep, (uint32_t)id[ga], (uint32_t)id[gb], G, &U);
     typename A::V4 v;
     if constexpr (A::mixed) {
       v = F4{G[0], G[1], G[2], c.scheme == SDPD_SCHEME_EMS ? fm::log(U) : U};
@@ -1326,7 +1337,9 @@ void fd_prepare() {
   }
 }
 
-static inline unsigned stage_blocks(const Consts& c) { return (unsigned)((c.ncell + kStageWarps - 1) / kStageWarps); }
+static inline unsigned stage_blocks(const Consts& c) {
+  return (unsigned)(((int64_t)c.ncell * stage_split(c.ncell) + kStageWarps - 1) / kStageWarps);
+}
 
 // The staged geometry of every scheduled pair (the last launch of a schedule).
 template <class P, class A>
@@ -1336,7 +1349,7 @@ void launch_stage_geometry(const Consts& c, const Workspace& w, int cur, cudaStr
   auto kern = c.kernel == SDPD_KERNEL_LUCY ? k_stage_geometry<P, A, SDPD_KERNEL_LUCY>
                                            : k_stage_geometry<P, A, SDPD_KERNEL_CUBIC>;
   kern<<<stage_blocks(c), kStageWarps * 32, 0, s>>>(c, (const typename P::V4*)w.qr4, w.cell_start, w.mrank, w.xmin[0],
-                                                   w.xmin[1], w.xmin[2], w.sched_hdr, w.sched_off, w.sched_pair,
+                                                   w.xmin[1], w.xmin[2], w.sched_hdr, w.sched_off, w.sched_pair, stage_split(c.ncell),
                                                    (typename A::V4*)w.st_geom);
 }
 
@@ -1350,7 +1363,8 @@ void launch_fd_colours(const Consts& c, const Workspace& w, int cur, double dt, 
     return;
   }
   k_stage_random<A><<<stage_blocks(c), kStageWarps * 32, 0, s>>>(c, w.id[cur], w.cell_start, w.mrank, w.sched_hdr,
-                                                                w.sched_off, w.sched_pair, seed, w.sweep,
+                                                                w.sched_off, w.sched_pair, stage_split(c.ncell), seed,
+                                                                w.sweep,
                                                                 (const typename A::V4*)w.st_geom,
                                                                 (typename A::V4*)w.st_rnd, w.st_aux);
   if constexpr (!A::mixed) {
