@@ -407,14 +407,13 @@ __global__ void __launch_bounds__(kEnumThreads)
 }
 
 // Rounds: one warp per block takes the block's canonical list 32 pairs at a
-// time.  A pair may go after all earlier pairs of its two particles, so the
-// lanes of a chunk first claim their particles (smallest lane wins, in
-// shared memory); a lane that holds both of its claims has no earlier pair
-// of the chunk left in its way and takes the first round >= the ones its
-// particles are free from that still has room, by an atomic count.  The
-// others try again; a chunk takes as many passes as its longest chain of
-// pairs sharing particles (mostly one or two: a row of the canonical order
-// shares particles only between pairs one row distance apart).
+// time.  A pair may go after all earlier pairs of its two particles.  The
+// lanes of a chunk set their bit in a mask per particle (shared memory), which
+// gives each lane the earlier lanes that share a particle with it; a lane
+// whose earlier lanes are done takes the first round >= the ones its
+// particles are free from that still has room, by an atomic count.  A chunk
+// takes as many passes as its longest chain of pairs sharing particles (four
+// to five on the lattice).
 // Round width: the lanes that a colour launch gives a block.  Limiting the
 // rounds here instead of splitting wide dependency levels there fills the
 // lanes better (16 lanes, 32^3 lattice: 53 rounds per block instead of 68).
@@ -425,9 +424,9 @@ constexpr int kRoundWarps = 4;
 
 template <int CAP, int MAXP>
 struct RoundSmem {
-  uint32_t claim[CAP];
+  uint32_t claim[CAP];   // lanes of the current chunk that hold a particle
   uint32_t cnt[kRoundStride];
-  uint16_t place[MAXP];  // round << 5 | place in the round
+  uint8_t place[MAXP];   // round of each pair (the order inside a round is free)
   uint8_t last[CAP];     // first round in which a particle is free
 };
 
@@ -486,7 +485,7 @@ template <int CAP, int MAXP, class In>
 __device__ __forceinline__ bool assign_rounds(RoundSmem<CAP, MAXP>& sm, const SchedOut& out, int64_t o, int np,
                                               int width, uint32_t flag, In in) {
   const int lane = threadIdx.x & 31;
-  for (int k = lane; k < CAP; k += 32) sm.claim[k] = 0xffffffffu;
+  for (int k = lane; k < CAP; k += 32) sm.claim[k] = 0u;
   for (int k = lane; k < kRoundStride; k += 32) sm.cnt[k] = 0u;
   for (int k = lane; k < CAP / 4; k += 32) reinterpret_cast<uint32_t*>(sm.last)[k] = 0u;
   __syncwarp();
@@ -497,28 +496,29 @@ __device__ __forceinline__ bool assign_rounds(RoundSmem<CAP, MAXP>& sm, const Sc
     const uint32_t pr = nxt;
     if (k0 + 32 + lane < np) nxt = in(k0 + 32 + lane);
     const int u = pr & 0xffffu, v = pr >> 16;
-    bool pending = k0 + lane < np;
-    while (__any_sync(0xffffffffu, pending)) {
-      if (pending) {
-        atomicMin(&sm.claim[u], (uint32_t)lane);
-        atomicMin(&sm.claim[v], (uint32_t)lane);
-      }
-      __syncwarp();
-      const bool ready = pending && sm.claim[u] == (uint32_t)lane && sm.claim[v] == (uint32_t)lane;
-      __syncwarp();
-      if (pending) sm.claim[u] = sm.claim[v] = 0xffffffffu;
+    const bool valid = k0 + lane < np;
+    if (valid) {
+      atomicOr(&sm.claim[u], 1u << lane);
+      atomicOr(&sm.claim[v], 1u << lane);
+    }
+    __syncwarp();
+    const unsigned before = valid ? (sm.claim[u] | sm.claim[v]) & ((1u << lane) - 1u) : 0u;
+    unsigned pending = __ballot_sync(0xffffffffu, valid);
+    __syncwarp();
+    if (valid) sm.claim[u] = sm.claim[v] = 0u;
+    while (pending) {
+      const bool ready = (pending >> lane & 1u) && !(before & pending);
       if (ready) {
         int L = max(full, max((int)sm.last[u], (int)sm.last[v]));
-        uint32_t s = 0;
-        while (L < kMaxLevels && (s = atomicAdd(&sm.cnt[L], 1u)) >= (uint32_t)width) ++L;
+        while (L < kMaxLevels && atomicAdd(&sm.cnt[L], 1u) >= (uint32_t)width) ++L;
         if (L >= kMaxLevels) {
           overflow = true;
         } else {
           sm.last[u] = sm.last[v] = (uint8_t)(L + 1);
-          sm.place[k0 + lane] = (uint16_t)(L << 5 | (int)s);
+          sm.place[k0 + lane] = (uint8_t)L;
         }
-        pending = false;
       }
+      pending &= ~__ballot_sync(0xffffffffu, ready);
       __syncwarp();
     }
     if (__any_sync(0xffffffffu, overflow)) return false;
@@ -564,10 +564,7 @@ __device__ __forceinline__ bool assign_rounds(RoundSmem<CAP, MAXP>& sm, const Sc
   if (lane * 8 < nr) reinterpret_cast<uint2*>(out.rsize + o * kRoundStride)[lane] = make_uint2(packed[0], packed[1]);
   __syncwarp();
 #pragma unroll 4
-  for (int k = lane; k < np; k += 32) {
-    const int pl = sm.place[k];
-    out.pairs[at + sm.cnt[pl >> 5] + (pl & 31)] = in(k);
-  }
+  for (int k = lane; k < np; k += 32) out.pairs[at + atomicAdd(&sm.cnt[sm.place[k]], 1u)] = in(k);
   return true;
 }
 
