@@ -15,51 +15,16 @@
 //                             - m F (rbar_i + rbar_j) r_ij ],  c_ij = wt m^2 (pi_i + pi_j)
 //           and dL/dh = sum_{i<j} [ c_ij t_ij dF/dh + m dW/dh (rbar_i + rbar_j) ]
 //                       + sum_i rbar_i m dW/dh(0).
-// Each pass is a gather over the neighbour list of particle i (one thread per
-// particle, no atomics); every pair is met from both sides, so the symmetric
+// Each pass is a gather over the neighbour list of particle i (a group of
+// lanes per particle, no atomics); every pair is met from both sides, so the symmetric
 // h terms are halved.  Cotangents of particles are kept in id order.
 #include <math.h>
 
-#include "sdpd_internal.cuh"
+#include "sdpd_f64.cuh"
 
 namespace sdpd {
 
 namespace {
-
-// dF/dr: Lucy -2 cF (1 - x)/h; cubic -3 cF/h (x <= 1/2), -(cF/h)(1 - x)(1 + x)/x^2
-template <int KIND>
-__device__ __forceinline__ double kernel_dF(double x, double cF, double inv_h) {
-  if (KIND == SDPD_KERNEL_LUCY) return -2.0 * cF * (1.0 - x) * inv_h;
-  if (x <= 0.5) return -3.0 * cF * inv_h;
-  return -cF * inv_h * (1.0 - x) * (1.0 + x) / (x * x);
-}
-
-// Displacement r_ij with the periodic image taken from the neighbour-list
-// entry's stencil code (offset + 1 per axis, 2 bits each) and the home cell.
-struct Images {
-  double m[3], p[3];  // shifts of the offsets -1 and +1 per axis
-  __device__ void init(const Consts& c, double cellbits_w) {
-    int ci[3];
-    unpack_cell(w_to_cellbits(cellbits_w), ci[0], ci[1], ci[2]);
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      m[d] = image_shift(ci[d], -1, c.nc[d], c.L[d]);
-      p[d] = image_shift(ci[d], 1, c.nc[d], c.L[d]);
-    }
-  }
-};
-
-__device__ __forceinline__ void pair_disp(const Images& im, uint32_t code, const D4& qi, const D4& qj, double& dx,
-                                          double& dy, double& dz) {
-  double d[3] = {__dsub_rn(qi.x, qj.x), __dsub_rn(qi.y, qj.y), __dsub_rn(qi.z, qj.z)};
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    const uint32_t k = (code >> (2 * a)) & 3u;
-    const double s = k == 0 ? im.m[a] : (k == 2 ? im.p[a] : 0.0);
-    if (s != 0.0) d[a] = __dadd_rn(d[a], s);
-  }
-  dx = d[0]; dy = d[1]; dz = d[2];
-}
 
 // v_i = scale * pbar[id_i], rbar slot cleared
 __global__ void k_adj_gather(int64_t N, const int32_t* __restrict__ id, const double* __restrict__ pbar,
@@ -70,33 +35,36 @@ __global__ void k_adj_gather(int64_t N, const int32_t* __restrict__ id, const do
   st4(&vs4[i], D4{scale * pbar[3 * k], scale * pbar[3 * k + 1], scale * pbar[3 * k + 2], 0.0});
 }
 
-// pass A: A_i = m^2 sum_j F(r_ij) t_ij
-template <int KIND, int MODE>
-__global__ void __launch_bounds__(128) k_adj_pairsum(Consts c, const D4* __restrict__ qp4, const D4* __restrict__ q4,
-                                                     const D4* __restrict__ vs4, const uint32_t* __restrict__ nlist,
+// pass A: A_i = m^2 sum_j F(r_ij) t_ij, T lanes per particle over its list
+// (see kLanes64; with one thread per particle the pass took 198 us at 32^3).
+template <int KIND, int MODE, int T>
+__global__ void __launch_bounds__(128) k_adj_pairsum(Consts c, const D4* __restrict__ qp4,
+                                                     const float4* __restrict__ qf4, const D4* __restrict__ vs4,
+                                                     const uint32_t* __restrict__ nlist,
                                                      const int32_t* __restrict__ nn, double* __restrict__ A,
                                                      int* __restrict__ status) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= c.N) return;
+  const int gl = threadIdx.x % T;
+  int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / T;
+  const bool mine = i < c.N;
+  if (!mine) i = 0;  // (the whole warp stays for the sums)
   const D4 qi = ld4(&qp4[i]);
-  Images im;
-  im.init(c, q4[i].w);
+  int cx, cy, cz;
+  unpack_cell(__float_as_uint(qf4[i].w), cx, cy, cz);
+  Home64 home;
+  home.init(c, qi, cx, cy, cz);
   D4 vi{0.0, 0.0, 0.0, 0.0};
   if (MODE == 0) vi = ld4(&vs4[i]);
-  const double inv_h = 1.0 / c.h;
   double acc = 0.0;
-  int n = nn[i];
+  int n = mine ? nn[i] : 0;
   if (n > c.nbr_cap) {  // the gradient passes walk the list only
     atomicOr(status, kStNbrCap);
     n = c.nbr_cap;
   }
 #pragma unroll 2
-  for (int k = 0; k < n; ++k) {
+  for (int k = gl; k < n; k += T) {
     const uint32_t e = __ldg(&nlist[nbr_slot(i, k, c.nbr_cap)]);
-    const D4 qj = ld4(&qp4[e >> 6]);
     double dx, dy, dz;
-    pair_disp(im, e & 63u, qi, qj, dx, dy, dz);
-    const double r2 = r2_of(dx, dy, dz);
+    const double r2 = home.r2(e & 63u, ld4(&qp4[e >> 6]), dx, dy, dz);
     double t;
     if (MODE == 0) {
       const D4 vj = ld4(&vs4[e >> 6]);
@@ -104,9 +72,10 @@ __global__ void __launch_bounds__(128) k_adj_pairsum(Consts c, const D4* __restr
     } else {
       t = r2;
     }
-    acc += kernel_F<KIND>(pair_r(r2) * inv_h, c.cF) * t;
+    acc += F64<KIND>(pair_r64(r2), c.inv_h) * t;
   }
-  A[i] = c.m * c.m * acc;
+  acc = group_sum<T>(acc);
+  if (mine && gl == 0) A[i] = c.m * c.m * c.cF * acc;
 }
 
 // Elementwise step of the trajectory's reverse pass at position k (state
@@ -239,43 +208,57 @@ __global__ void k_adj_mid_virial(Consts c, const D4* __restrict__ qp4, const dou
   vs4[i].w = -g / rho[i];
 }
 
-// pass B (MODE 0: kick pulled back along v; 1: virial; 2: density term only)
-template <int KIND, int MODE>
-__global__ void __launch_bounds__(128) k_adj_back(Consts c, const D4* __restrict__ qp4, const D4* __restrict__ q4,
-                                                  const D4* __restrict__ vs4, const int32_t* __restrict__ id,
-                                                  const uint32_t* __restrict__ nlist,
+// pass B (MODE 0: kick pulled back along v; 1: virial; 2: density term only),
+// T lanes per particle over its list
+template <int KIND, int MODE, int T>
+__global__ void __launch_bounds__(128) k_adj_back(Consts c, const D4* __restrict__ qp4,
+                                                  const float4* __restrict__ qf4, const D4* __restrict__ vs4,
+                                                  const int32_t* __restrict__ id, const uint32_t* __restrict__ nlist,
                                                   const int32_t* __restrict__ nn, double wt, int accumulate,
                                                   double* __restrict__ qbar, double* __restrict__ thbar,
                                                   int* __restrict__ status) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= c.N) return;
+  const int gl = threadIdx.x % T;
+  int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / T;
+  const bool mine = i < c.N;
+  if (!mine) i = 0;  // (the whole warp stays for the sums)
   const D4 qi = ld4(&qp4[i]);
   const D4 vi = ld4(&vs4[i]);
-  Images im;
-  im.init(c, q4[i].w);
-  const double inv_h = 1.0 / c.h, m = c.m, cm2 = wt * c.m * c.m;
-  double gx = 0.0, gy = 0.0, gz = 0.0, gh = 0.0;
-  int n = nn[i];
+  int cx, cy, cz;
+  unpack_cell(__float_as_uint(qf4[i].w), cx, cy, cz);
+  Home64 home;
+  home.init(c, qi, cx, cy, cz);
+  const double inv_h = c.inv_h, mF = c.m * c.cF, w3 = 3.0 * c.cW / c.cF, cm2 = wt * c.m * c.m * c.cF;
+  double gx = 0.0, gy = 0.0, gz = 0.0, gd = 0.0, gf = 0.0;
+  int n = mine ? nn[i] : 0;
   if (n > c.nbr_cap) {  // the gradient passes walk the list only
     atomicOr(status, kStNbrCap);
     n = c.nbr_cap;
   }
 #pragma unroll 2
-  for (int k = 0; k < n; ++k) {
+  for (int k = gl; k < n; k += T) {
     const uint32_t e = __ldg(&nlist[nbr_slot(i, k, c.nbr_cap)]);
     const D4 qj = ld4(&qp4[e >> 6]);
     const D4 vj = ld4(&vs4[e >> 6]);
-    double dx, dy, dz;
-    pair_disp(im, e & 63u, qi, qj, dx, dy, dz);
-    const double r2 = r2_of(dx, dy, dz);
-    const double r = pair_r(r2), x = r * inv_h;
-    const double f = kernel_F<KIND>(x, c.cF);
-    const double rb = vi.w + vj.w;
+    double dx, dy, dz, rinv;
+    const double r2 = home.r2(e & 63u, qj, dx, dy, dz);
+    const double r = MODE == 2 ? pair_r64(r2) : pair_r64(r2, rinv);
+    const double f = F64<KIND>(r, inv_h);
+    const double rb = mF * (vi.w + vj.w);
     // density: d rho / d q along r_ij, and dW/dh = (r^2 F - 3 W)/h
-    double s = -m * f * rb;
-    gh += m * (r2 * f - 3.0 * kernel_W<KIND>(x, c.cW)) * inv_h * rb;
+    double s = -f * rb;
+    gd += __fma_rn(-w3, W64<KIND>(r, inv_h), r2 * f) * rb;
     if (MODE != 2) {
-      const double fp = kernel_dF<KIND>(x, c.cF, inv_h);
+      // F'/cF: Lucy -2 (1 - x)/h; cubic -3/h (x <= 1/2), -(1 - x)(1 + x)/(h x^2)
+      const double x = r * inv_h;
+      double fp;
+      if (KIND == SDPD_KERNEL_LUCY) {
+        fp = -2.0 * inv_h * (1.0 - x);
+      } else if (inner_half(x)) {
+        fp = -3.0 * inv_h;
+      } else {
+        const double u = c.h * rinv;  // 1/x
+        fp = inv_h * (1.0 - u * u);
+      }
       const double cc = cm2 * (qi.w + qj.w);
       double t, ux, uy, uz;
       if (MODE == 0) {
@@ -285,14 +268,19 @@ __global__ void __launch_bounds__(128) k_adj_back(Consts c, const D4* __restrict
         ux = 2.0 * dx; uy = 2.0 * dy; uz = 2.0 * dz;
         t = r2;
       }
-      // F'/r t vanishes with r at coincident particles
-      s += r2 > 0.0 ? cc * fp / r * t : 0.0;
-      const double cf = cc * f;
+      const double ct = cc * t, cf = cc * f;
+      // F'/r t vanishes with r at coincident particles (rinv = 0 there)
+      s = __fma_rn(ct * fp, rinv, s);
       gx += cf * ux; gy += cf * uy; gz += cf * uz;
-      gh -= cc * t * (5.0 * f + r * fp) * inv_h;  // dF/dh = -(5 F + r F')/h
+      gf += ct * __fma_rn(5.0, f, r * fp);  // dF/dh = -(5 F + r F')/h
     }
     gx += s * dx; gy += s * dy; gz += s * dz;
   }
+  gx = group_sum<T>(gx);
+  gy = group_sum<T>(gy);
+  gz = group_sum<T>(gz);
+  const double gh = group_sum<T>((gd - gf) * inv_h);
+  if (!mine || gl != 0) return;
   const int64_t k = id[i];
   if (accumulate) {
     qbar[3 * k] += gx; qbar[3 * k + 1] += gy; qbar[3 * k + 2] += gz;
@@ -300,7 +288,7 @@ __global__ void __launch_bounds__(128) k_adj_back(Consts c, const D4* __restrict
     qbar[3 * k] = gx; qbar[3 * k + 1] = gy; qbar[3 * k + 2] = gz;
   }
   // self term of rho_i: m dW/dh(0) = -3 m W(0)/h
-  thbar[3 * k] += 0.5 * gh - 3.0 * m * c.W0 * inv_h * vi.w;
+  thbar[3 * k] += 0.5 * gh - 3.0 * c.m * c.W0 * inv_h * vi.w;
 }
 
 __global__ void k_adj_axpy(int64_t n, double a, const double* __restrict__ x, double* __restrict__ y) {
@@ -353,18 +341,24 @@ void launch_adj_gather(const Consts& c, const Workspace& w, int cur, const doubl
   k_adj_gather<<<nblocks(c.N, 256), 256, 0, s>>>(c.N, w.id[cur], pbar_id, scale, vs4);
 }
 
+template <int KIND, int MODE>
+static void launch_pairsum(const Consts& c, const Workspace& w, const D4* vs4, double* A, cudaStream_t s) {
+  const bool wide = pair64_wide(c);
+  auto kern = wide ? k_adj_pairsum<KIND, MODE, 32> : k_adj_pairsum<KIND, MODE, kLanes64>;
+  kern<<<nblocks(c.N * (wide ? 32 : kLanes64), 128), 128, 0, s>>>(c, (const D4*)w.qp4, w.qf4, vs4, w.nlist, w.nn, A,
+                                                                 w.status);
+}
+
 void launch_adj_pairsum(const Consts& c, const Workspace& w, int cur, int mode, const D4* vs4, double* A,
                         cudaStream_t s) {
   if (c.N == 0) return;
-  const D4* qp4 = (const D4*)w.qp4;
-  const D4* q4 = (const D4*)w.q4[cur];
-  const unsigned nb = nblocks(c.N, 128);
+  (void)cur;
   if (c.kernel == SDPD_KERNEL_LUCY) {
-    if (mode == 0) k_adj_pairsum<SDPD_KERNEL_LUCY, 0><<<nb, 128, 0, s>>>(c, qp4, q4, vs4, w.nlist, w.nn, A, w.status);
-    else k_adj_pairsum<SDPD_KERNEL_LUCY, 1><<<nb, 128, 0, s>>>(c, qp4, q4, vs4, w.nlist, w.nn, A, w.status);
+    if (mode == 0) launch_pairsum<SDPD_KERNEL_LUCY, 0>(c, w, vs4, A, s);
+    else launch_pairsum<SDPD_KERNEL_LUCY, 1>(c, w, vs4, A, s);
   } else {
-    if (mode == 0) k_adj_pairsum<SDPD_KERNEL_CUBIC, 0><<<nb, 128, 0, s>>>(c, qp4, q4, vs4, w.nlist, w.nn, A, w.status);
-    else k_adj_pairsum<SDPD_KERNEL_CUBIC, 1><<<nb, 128, 0, s>>>(c, qp4, q4, vs4, w.nlist, w.nn, A, w.status);
+    if (mode == 0) launch_pairsum<SDPD_KERNEL_CUBIC, 0>(c, w, vs4, A, s);
+    else launch_pairsum<SDPD_KERNEL_CUBIC, 1>(c, w, vs4, A, s);
   }
 }
 
@@ -402,25 +396,30 @@ void launch_adj_mid_virial(const Consts& c, const Workspace& w, int cur, const d
       (const double*)w.py[cur], (const double*)w.pz[cur], w.id[cur], A, wt, vs4, val_id, gp, geps, thbar);
 }
 
+template <int KIND, int MODE>
+static void launch_back(const Consts& c, const Workspace& w, int cur, double wt, const D4* vs4, int accumulate,
+                        double* qbar, double* thbar, cudaStream_t s) {
+  const bool wide = pair64_wide(c);
+  auto kern = wide ? k_adj_back<KIND, MODE, 32> : k_adj_back<KIND, MODE, kLanes64>;
+  kern<<<nblocks(c.N * (wide ? 32 : kLanes64), 128), 128, 0, s>>>(c, (const D4*)w.qp4, w.qf4, vs4, w.id[cur], w.nlist,
+                                                                 w.nn, wt, accumulate, qbar, thbar, w.status);
+}
+
+template <int KIND>
+static void launch_back_mode(const Consts& c, const Workspace& w, int cur, int mode, double wt, const D4* vs4,
+                             int accumulate, double* qbar, double* thbar, cudaStream_t s) {
+  if (mode == 0) launch_back<KIND, 0>(c, w, cur, wt, vs4, accumulate, qbar, thbar, s);
+  else if (mode == 1) launch_back<KIND, 1>(c, w, cur, wt, vs4, accumulate, qbar, thbar, s);
+  else launch_back<KIND, 2>(c, w, cur, wt, vs4, accumulate, qbar, thbar, s);
+}
+
 void launch_adj_back(const Consts& c, const Workspace& w, int cur, int mode, double wt, const D4* vs4,
                      int accumulate, double* qbar, double* thbar, cudaStream_t s) {
   if (c.N == 0) return;
-  const D4* qp4 = (const D4*)w.qp4;
-  const D4* q4 = (const D4*)w.q4[cur];
-  const unsigned nb = nblocks(c.N, 128);
-  const int32_t* id = w.id[cur];
-#define SDPD_ADJ_BACK(KIND, MODE) \
-  k_adj_back<KIND, MODE><<<nb, 128, 0, s>>>(c, qp4, q4, vs4, id, w.nlist, w.nn, wt, accumulate, qbar, thbar, w.status)
-  if (c.kernel == SDPD_KERNEL_LUCY) {
-    if (mode == 0) SDPD_ADJ_BACK(SDPD_KERNEL_LUCY, 0);
-    else if (mode == 1) SDPD_ADJ_BACK(SDPD_KERNEL_LUCY, 1);
-    else SDPD_ADJ_BACK(SDPD_KERNEL_LUCY, 2);
-  } else {
-    if (mode == 0) SDPD_ADJ_BACK(SDPD_KERNEL_CUBIC, 0);
-    else if (mode == 1) SDPD_ADJ_BACK(SDPD_KERNEL_CUBIC, 1);
-    else SDPD_ADJ_BACK(SDPD_KERNEL_CUBIC, 2);
-  }
-#undef SDPD_ADJ_BACK
+  if (c.kernel == SDPD_KERNEL_LUCY)
+    launch_back_mode<SDPD_KERNEL_LUCY>(c, w, cur, mode, wt, vs4, accumulate, qbar, thbar, s);
+  else
+    launch_back_mode<SDPD_KERNEL_CUBIC>(c, w, cur, mode, wt, vs4, accumulate, qbar, thbar, s);
 }
 
 void launch_adj_axpy(int64_t n, double a, const double* x, double* y, cudaStream_t s) {

@@ -475,6 +475,7 @@ int sdpd_create(int64_t N, const double box[3], double m, double h, const sdpd_p
   c.ncell = (int)ncell;
   c.h = h;
   c.h2 = h * h;
+  c.inv_h = 1.0 / h;
   c.m = m;
   c.kB = prm->kB;
   c.C_K = 1.5 * (K - 1.0) * prm->kB;

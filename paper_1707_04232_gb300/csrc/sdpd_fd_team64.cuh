@@ -21,109 +21,10 @@
 // the proposers take round r + 1 back, then the rejected moves, and propose
 // round r + 1 again, so the result is the sequential one.
 #pragma once
+#include "sdpd_f64.cuh"
 #include "sdpd_fd_colour.cuh"
 
 namespace sdpd {
-
-// Elementary functions with few float64 instructions.  Each starts from a
-// hardware approximation or a float32 evaluation of its small terms.
-namespace f64 {
-__device__ __forceinline__ double rcp_seed(double x) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  return y;
-}
-__device__ __forceinline__ double rsqrt_seed(double x) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  return y;
-}
-// 1/x: one third-order (Householder) step y (1 + e + e^2), e = 1 - x y.
-__device__ __forceinline__ double rcp(double x) {
-  const double y = rcp_seed(x), e = __fma_rn(-x, y, 1.0);
-  return __fma_rn(y, __fma_rn(e, e, e), y);
-}
-// sqrt(x) and 1/sqrt(x): one third-order step, (1 - e)^(-1/2) =
-// 1 + e/2 + 3 e^2/8 + O(e^3) with e = 1 - x y^2.  Arguments whose seed could
-// be flushed take the library functions.
-__device__ __forceinline__ bool rsqrt_tiny(double x) { return __double2hiint(x) < 0x03f00000; }  // below 2^-960, <= 0
-__device__ __forceinline__ double sqrt_(double x) {
-  if (rsqrt_tiny(x)) return ::sqrt(x);
-  const double y = rsqrt_seed(x), h = __dmul_rn(x, y), e = __fma_rn(-h, y, 1.0);
-  return __fma_rn(__dmul_rn(h, e), __fma_rn(e, 0.375, 0.5), h);
-}
-__device__ __forceinline__ double rsqrt_(double x) {
-  if (rsqrt_tiny(x)) return 1.0 / ::sqrt(x);
-  const double y = rsqrt_seed(x), h = __dmul_rn(x, y), e = __fma_rn(-h, y, 1.0);
-  return __fma_rn(__dmul_rn(y, e), __fma_rn(e, 0.375, 0.5), y);
-}
-__device__ __forceinline__ bool below(double x, int hi) { return (__double2hiint(x) & 0x7fffffff) < hi; }
-constexpr int kHi2m6 = 0x3f900000, kHi2m3 = 0x3fc00000, kHi2m2 = 0x3fd00000;  // high words of 2^-6, 1/8, 1/4
-// expm1: Taylor series; below 2^-6 the terms from x^5/120 on, 2^-31 of the
-// result, in float32; below 1/4 twelve terms in float64.
-__device__ __forceinline__ double expm1(double x) {
-  if (below(x, kHi2m6)) {
-    const float f = (float)x;
-    const float t = f * (1.0f / 120.0f + f * (1.0f / 720.0f + f * (1.0f / 5040.0f)));
-    double p = 1.0 / 24.0 + (double)t;
-    p = __fma_rn(p, x, 1.0 / 6.0);
-    p = __fma_rn(p, x, 0.5);
-    return __fma_rn(__dmul_rn(p, x), x, x);
-  }
-  if (below(x, kHi2m2)) {
-    double p = 1.0 / 6227020800.0;
-    p = __fma_rn(p, x, 1.0 / 479001600.0);
-    p = __fma_rn(p, x, 1.0 / 39916800.0);
-    p = __fma_rn(p, x, 1.0 / 3628800.0);
-    p = __fma_rn(p, x, 1.0 / 362880.0);
-    p = __fma_rn(p, x, 1.0 / 40320.0);
-    p = __fma_rn(p, x, 1.0 / 5040.0);
-    p = __fma_rn(p, x, 1.0 / 720.0);
-    p = __fma_rn(p, x, 1.0 / 120.0);
-    p = __fma_rn(p, x, 1.0 / 24.0);
-    p = __fma_rn(p, x, 1.0 / 6.0);
-    p = __fma_rn(p, x, 0.5);
-    return __fma_rn(__dmul_rn(p, x), x, x);
-  }
-  return ::expm1(x);
-}
-// log1p: below 2^-6 the alternating series, its terms from x^6/6 on (2^-33 of
-// the result) in float32; below 1/8 2 atanh(u) with u = x / (2 + x), its
-// terms from u^7/7 on in float32.
-__device__ __forceinline__ double log1p(double x) {
-  if (below(x, kHi2m6)) {
-    const float f = (float)x;
-    const float t = f * (-1.0f / 6.0f + f * (1.0f / 7.0f + f * (-1.0f / 8.0f + f * (1.0f / 9.0f))));
-    double p = 0.2 + (double)t;
-    p = __fma_rn(p, x, -0.25);
-    p = __fma_rn(p, x, 1.0 / 3.0);
-    p = __fma_rn(p, x, -0.5);
-    return __fma_rn(__dmul_rn(p, x), x, x);
-  }
-  if (below(x, kHi2m3)) {
-    const double d = 2.0 + x, r = rcp(d);
-    double u = __dmul_rn(x, r);
-    u = __fma_rn(__fma_rn(-u, d, x), r, u);
-    const double w = __dmul_rn(u, u);
-    const float f = (float)w;
-    const float t = f * (1.0f / 7.0f + f * (1.0f / 9.0f + f * (1.0f / 11.0f + f * (1.0f / 13.0f))));
-    double p = 0.2 + (double)t;
-    p = __fma_rn(p, w, 1.0 / 3.0);
-    const double v = u + u;
-    return __fma_rn(__dmul_rn(p, w), v, v);
-  }
-  return ::log1p(x);
-}
-// comparisons with zero on the bits (a float64 comparison costs an issue)
-__device__ __forceinline__ bool positive(double x) {
-  const long long b = __double_as_longlong(x);
-  return b > 0 && b <= 0x7ff0000000000000ll;
-}
-__device__ __forceinline__ bool negative(double x) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  return b > 0x8000000000000000ull && b <= 0xfff0000000000000ull;
-}
-}  // namespace f64
 
 // Constants of the team's arithmetic, in momentum units: with u = p_i - p_j,
 // dp = (m/2)(v' - v) = (alpha - 1) u / 2 + hz G per direction, hz = m zt / 2,

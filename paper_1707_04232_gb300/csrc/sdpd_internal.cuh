@@ -48,7 +48,7 @@ struct Consts {
   double L[3], halfL[3], cs[3], inv_cs[3];
   double scale[3];      // mixed precision: box side / 2^32 (fixed-point unit)
   double inv_scale[3];  // 2^32 / box side
-  double h, h2, m, kB;
+  double h, h2, inv_h, m, kB;
   double C_K, c_rho;
   double kpar_m2, kperp_m2;  // (10/3 eta + 4 zeta) m^2 and (5/3 eta - zeta) m^2
   double cW, cF, W0;         // kernel constants and W(0)
@@ -135,18 +135,6 @@ __device__ __forceinline__ double pair_rinv(double r2) {
   return y * (1.5 - 0.5 * r2 * y * y);
 }
 __device__ __forceinline__ double pair_r(double r2) { return r2 > 1e-30 ? r2 * pair_rinv(r2) : sqrt(r2); }
-// The same with two float64 operations instead of four: the float32 root H,
-// then H + (r^2 - H^2) / (2 H) with the residual from one float64 FMA and the
-// small correction formed in float32 (Heron's step; relative error ~1e-14:
-// half the square of H's error and the rounding of the correction).
-__device__ __forceinline__ double pair_r64(double r2) {
-  const float f = (float)r2;
-  if (!(f > 1e-30f)) return sqrt(r2);
-  const float y = rsqrtf(f);
-  const double H = (double)(f * y);
-  const float d = (float)__fma_rn(-H, H, r2);
-  return H + (double)(0.5f * y * d);
-}
 __device__ __forceinline__ float pair_r(float r2) { return r2 > 0.0f ? r2 * rsqrtf(r2) : 0.0f; }
 
 // ---------------------------------------------------------------------------
@@ -339,7 +327,7 @@ struct Workspace {
   int32_t* id[2];
   void* qp4;            // sorted (x, y, z, pi): positions and p/rho^2 for force passes
   void* qr4;            // sorted (x, y, z, rho) of the latest density pass: the sweep's geometry
-  float4* qf4;          // float64 path: float32 copies (x, y, z, 0) of the sorted positions
+  float4* qf4;          // float64 path: float32 copies of the sorted positions and the cell bits
   uint32_t* nlist;      // neighbour lists, entry k of particle i at nlist[nbr_slot(i, k, nbr_cap)]
   int32_t* nn;          // neighbour count per particle
   uint32_t* cend;       // [9][N]: per particle and row of 3 cells, where its list stands (see k_density)

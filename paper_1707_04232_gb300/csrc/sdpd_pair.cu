@@ -8,7 +8,7 @@
 // Mixed path: one thread per particle in storage order (k_density, k_force).
 // Float64 path: a group of kLanes64 lanes per particle (k_density64,
 // k_force64).
-#include "sdpd_internal.cuh"
+#include "sdpd_f64.cuh"
 
 namespace sdpd {
 
@@ -164,135 +164,6 @@ __global__ void __launch_bounds__(128, 12) k_density(Consts c, Arrays<P> a, type
   st4(&qr4[i], o);
 }
 
-// ---------------------------------------------------------------------------
-// Float64 pair passes.  GB300 issues one float64 instruction per 64 cycles on
-// each quarter of an SM whether 1 or 32 lanes are active, so a pass costs its
-// float64 instructions per warp.  With one thread per particle the kept
-// neighbour's branch ran on nearly every candidate of the 27 cells (one lane
-// in six keeps one): ~500 evaluations instead of ~80.  Here kLanes64 lanes
-// share a particle (a whole warp where particles are few).  The search is float32: r^2 from the float32 positions
-// decides a candidate unless it lies within its rounding bound of h^2 (then
-// the float64 predicate does), and the kept ones are appended in walk order
-// (ballot and prefix count) to a list in shared memory.  Only list entries
-// see float64 arithmetic, with all lanes at work.
-// ---------------------------------------------------------------------------
-constexpr int kLanes64 = 8;
-
-// Distance pieces of a float64 list entry: displacement with the periodic
-// image of its stencil code (edge: the home cell touches the box side on some
-// axis, else every image shift is zero; adding a zero shift changes nothing).
-struct Home64 {
-  double x, y, z;
-  double mx, my, mz, px_, py_, pz_;
-  bool edge;
-  __device__ __forceinline__ void init(const Consts& c, const D4& q, int cx, int cy, int cz) {
-    x = q.x; y = q.y; z = q.z;
-    mx = image_shift(cx, -1, c.nc[0], c.L[0]); px_ = image_shift(cx, 1, c.nc[0], c.L[0]);
-    my = image_shift(cy, -1, c.nc[1], c.L[1]); py_ = image_shift(cy, 1, c.nc[1], c.L[1]);
-    mz = image_shift(cz, -1, c.nc[2], c.L[2]); pz_ = image_shift(cz, 1, c.nc[2], c.L[2]);
-    edge = cx == 0 || cy == 0 || cz == 0 || cx == c.nc[0] - 1 || cy == c.nc[1] - 1 || cz == c.nc[2] - 1;
-  }
-  __device__ __forceinline__ static double pick(uint32_t k, double m, double p) {
-    return k == 0 ? m : (k == 2 ? p : 0.0);
-  }
-  __device__ __forceinline__ double r2(uint32_t code, const D4& qj, double& dx, double& dy, double& dz) const {
-    dx = __dsub_rn(x, qj.x);
-    dy = __dsub_rn(y, qj.y);
-    dz = __dsub_rn(z, qj.z);
-    if (edge) {
-      dx = __dadd_rn(dx, pick(code & 3u, mx, px_));
-      dy = __dadd_rn(dy, pick((code >> 2) & 3u, my, py_));
-      dz = __dadd_rn(dz, pick((code >> 4) & 3u, mz, pz_));
-    }
-    return r2_of(dx, dy, dz);
-  }
-};
-
-// The walk of a warp's particles (one per group of T lanes) over their 27
-// cells: calls keep(slot, j, code) on the lanes of kept candidates, slot
-// counting them in walk order, and row(row, word) with the list positions of
-// each row of three cells; returns the number kept.  The candidates of a
-// row's three cells are taken as one run, kBatch x T at a time, so that their
-// loads are in flight together.  The whole warp takes part (the groups'
-// particles mostly share their cell, so their loops have the same length);
-// a group with live = false meets no candidates.
-template <int T, class Row, class Keep>
-__device__ __forceinline__ int walk64(const Consts& c, bool live, const Home64& home, const float4& fi, int64_t i,
-                                      int cx, int cy, int cz, const D4* __restrict__ q4,
-                                      const float4* __restrict__ qf4, const int32_t* __restrict__ cell_start,
-                                      const int32_t* __restrict__ mrank, Row row, Keep keep) {
-  constexpr int kBatch = T == 32 ? 2 : 3;
-  constexpr unsigned kFull = T == 32 ? 0xffffffffu : (1u << (T & 31)) - 1u;
-  const int gl = threadIdx.x % T, shift = (threadIdx.x & 31) - gl;
-  const unsigned below = (1u << gl) - 1u;
-  auto first = [](int n) { return n <= 0 ? 0u : (n >= 32 ? 0xffffffffu : (1u << n) - 1u); };  // the lowest n bits
-  int cnt = 0;
-#pragma unroll 1
-  for (int oz = -1; oz <= 1; ++oz) {
-    const int nz = wrapc(cz + oz, c.nc[2]);
-#pragma unroll 1
-    for (int oy = -1; oy <= 1; ++oy) {
-      const int ny = wrapc(cy + oy, c.nc[1]);
-      int beg[3], off[4] = {0, 0, 0, 0};
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        const int r = __ldg(&mrank[wrapc(cx + k - 1, c.nc[0]) + c.nc[0] * (ny + c.nc[1] * nz)]);
-        beg[k] = __ldg(&cell_start[r]);
-        off[k + 1] = __ldg(&cell_start[r + 1]) - beg[k];
-      }
-#pragma unroll
-      for (int k = 0; k < 3; ++k) off[k + 1] = live ? off[k + 1] + off[k] : 0;
-      const int start = cnt;
-      int c0 = 0, c1 = 0;  // kept in the first cell, in the first two
-      for (int b = 0; __any_sync(0xffffffffu, b < off[3]); b += kBatch * T) {
-        float4 fj[kBatch];
-        int js[kBatch];
-#pragma unroll
-        for (int u = 0; u < kBatch; ++u) {
-          const int t = b + u * T + gl;
-          js[u] = t < off[1] ? beg[0] + t : (t < off[2] ? beg[1] + t - off[1] : beg[2] + t - off[2]);
-          if (t < off[3]) fj[u] = __ldg(&qf4[js[u]]);
-        }
-#pragma unroll
-        for (int u = 0; u < kBatch; ++u) {
-          const int t0 = b + u * T, t = t0 + gl;
-          const uint32_t code = nbr_entry(0, (t >= off[1]) + (t >= off[2]) - 1, oy, oz);
-          bool in = false;
-          if (t < off[3] && js[u] != i) {
-            float ex = fi.x - fj[u].x, ey = fi.y - fj[u].y, ez = fi.z - fj[u].z;
-            ex = ex > c.halfLf[0] ? ex - c.Lf[0] : (ex < -c.halfLf[0] ? ex + c.Lf[0] : ex);
-            ey = ey > c.halfLf[1] ? ey - c.Lf[1] : (ey < -c.halfLf[1] ? ey + c.Lf[1] : ey);
-            ez = ez > c.halfLf[2] ? ez - c.Lf[2] : (ez < -c.halfLf[2] ? ez + c.Lf[2] : ez);
-            const float rf = ex * ex + ey * ey + ez * ez;
-            in = rf < c.h2_inner;
-            if (!in && rf < c.h2_filter) {  // within the rounding bound of h^2: float64 decides
-              double dx, dy, dz;
-              in = home.r2(code, ld4(&q4[js[u]]), dx, dy, dz) < c.h2;
-            }
-          }
-          const unsigned m = (__ballot_sync(0xffffffffu, in) >> shift) & kFull;
-          if (in) keep(cnt + __popc(m & below), js[u], code);
-          cnt += __popc(m);
-          c0 += __popc(m & first(off[1] - t0));
-          c1 += __popc(m & first(off[2] - t0));
-        }
-      }
-      row((oz + 1) * 3 + (oy + 1),
-          (uint32_t)min(start, 255) | (uint32_t)min(start + c0, 255) << 8 | (uint32_t)min(start + c1, 255) << 16 |
-              (uint32_t)min(cnt, 255) << 24);
-    }
-  }
-  return cnt;
-}
-
-// Sum of v over the lanes of a group, the same order for every group.
-template <int T>
-__device__ __forceinline__ double group_sum(double v) {
-#pragma unroll
-  for (int s = T / 2; s > 0; s >>= 1) v += __shfl_xor_sync(0xffffffffu, v, s);
-  return v;
-}
-
 // Density, equation of state and neighbour lists of PPB particles per thread
 // block (see k_density).  The list in shared memory has the layout of the
 // global one, so it is copied out in 16-byte pieces.  A particle with more
@@ -315,7 +186,7 @@ __global__ void __launch_bounds__(PPB * T)
   const D4 qi = ld4(&a.q4[live ? i : 0]);
   const float4 fi = qf4[live ? i : 0];
   int cx, cy, cz;
-  unpack_cell(w_to_cellbits(qi.w), cx, cy, cz);
+  unpack_cell(__float_as_uint(fi.w), cx, cy, cz);
   Home64 home;
   home.init(c, qi, cx, cy, cz);
   const int cnt = walk64<T>(
@@ -325,20 +196,19 @@ __global__ void __launch_bounds__(PPB * T)
         if (k < c.nbr_cap) list_s[((k >> 2) * PPB + p) * 4 + (k & 3)] = ((uint32_t)j << 6) | code;
       });
   __syncwarp();
-  const double inv_h = 1.0 / c.h;
   double acc = 0.0;
   const bool over = cnt > c.nbr_cap;
   for (int k = gl; k < (over ? 0 : cnt); k += T) {
     const uint32_t e = list_s[((k >> 2) * PPB + p) * 4 + (k & 3)];
     double dx, dy, dz;
     const double r2 = home.r2(e & 63u, ld4(&a.q4[e >> 6]), dx, dy, dz);
-    acc += kernel_W<KIND>(pair_r64(r2) * inv_h, c.cW);
+    acc += W64<KIND>(pair_r64(r2), c.inv_h);
   }
   if (__any_sync(0xffffffffu, over))
     walk64<T>(c, over, home, fi, i, cx, cy, cz, a.q4, qf4, cell_start, mrank, [](int, uint32_t) {},
               [&](int, int j, uint32_t code) {
                 double dx, dy, dz;
-                acc += kernel_W<KIND>(pair_r64(home.r2(code, ld4(&a.q4[j]), dx, dy, dz)) * inv_h, c.cW);
+                acc += W64<KIND>(pair_r64(home.r2(code, ld4(&a.q4[j]), dx, dy, dz)), c.inv_h);
               });
   acc = group_sum<T>(acc);
   if (gl == 0) {
@@ -359,7 +229,7 @@ __global__ void __launch_bounds__(PPB * T)
     if (ncount_by_id) ncount_by_id[a.id[g]] = cnt;
     nn[g] = cnt;
     if (cnt > c.nbr_cap) ovf_list[atomicAdd(ovf_count, 1)] = (int32_t)g;  // forces from the cells
-    const double rho_new = c.m * (c.W0 + acc_s[threadIdx.x]);
+    const double rho_new = c.m * __fma_rn(c.cW, acc_s[threadIdx.x], c.W0);
     double e = a.eps[g];
     if (update_eos) {
       // eps' = E(S(eps, rho), rho') = eps (rho' / rho)^(c_rho / C_K)
@@ -546,16 +416,16 @@ __global__ void __launch_bounds__(128)
   const int n = mine ? nn[i] : 0;
   const bool over = n > c.nbr_cap;
   const D4 qi = ld4(&qp4[i]);
+  const float4 fi = qf4[i];
   int cx, cy, cz;
-  unpack_cell(w_to_cellbits(a.q4[i].w), cx, cy, cz);
+  unpack_cell(__float_as_uint(fi.w), cx, cy, cz);
   Home64 home;
   home.init(c, qi, cx, cy, cz);
-  const double inv_h = 1.0 / c.h;
   double f[3] = {0.0, 0.0, 0.0};
   auto add = [&](uint32_t code, const D4& qj) {
     double dx, dy, dz;
     const double r2 = home.r2(code, qj, dx, dy, dz);
-    const double s = (qi.w + qj.w) * kernel_F<KIND>(pair_r64(r2) * inv_h, 1.0);
+    const double s = (qi.w + qj.w) * F64<KIND>(pair_r64(r2), c.inv_h);
     f[0] += s * dx;
     f[1] += s * dy;
     f[2] += s * dz;
@@ -566,7 +436,7 @@ __global__ void __launch_bounds__(128)
     add(e & 63u, ld4(&qp4[e >> 6]));
   }
   if (__any_sync(0xffffffffu, over))
-    walk64<T>(c, over, home, qf4[i], i, cx, cy, cz, qp4, qf4, cell_start, mrank, [](int, uint32_t) {},
+    walk64<T>(c, over, home, fi, i, cx, cy, cz, qp4, qf4, cell_start, mrank, [](int, uint32_t) {},
               [&](int, int j, uint32_t code) { add(code, ld4(&qp4[j])); });
 #pragma unroll
   for (int d = 0; d < 3; ++d) f[d] = group_sum<T>(f[d]);
@@ -635,12 +505,6 @@ static inline unsigned blocks_for(int64_t n, int t) { return (unsigned)((n + t -
 // threads per block of the pair passes (one thread per particle, no shared
 // memory, so any of the accepted sizes gives the same results)
 static inline int pair_block(const Consts& c) { return pair_threads_ok(c.pair_threads) ? c.pair_threads : 128; }
-
-// Lanes per particle of the float64 passes: with few particles a whole warp
-// each, which spreads them over the SM quarters and shortens every particle's
-// chain; else kLanes64, which costs fewer instructions in all.  The line lies
-// at four warps per SM quarter.
-static bool pair64_wide(const Consts& c) { return c.pair_auto && c.N <= 16 * 152; }
 
 template <int KIND>
 static void launch_density64(const Consts& c, const Workspace& w, const Arrays<Fp64>& a, int update_eos,

@@ -185,7 +185,7 @@ __global__ void k_gather(Consts c, const int32_t* __restrict__ tmp, const int32_
     v.z = __uint2float_rn(z - xmz[cz]) * (float)c.scale[2];
   } else {
     v.x = x; v.y = y; v.z = z;
-    qf4[d] = make_float4((float)x, (float)y, (float)z, 0.0f);
+    qf4[d] = make_float4((float)x, (float)y, (float)z, __uint_as_float(cb));
   }
   v.w = cellbits_to_w(cb, (V4*)nullptr);
   st4(&dst.q4[d], v);
