@@ -146,7 +146,8 @@ __device__ __forceinline__ double pair_r64(double r2) {
   const double H = f64::widen(f * y);
   return __fma_rn(__fma_rn(-H, H, r2), f64::widen(0.5f * y), H);
 }
-// The same and 1/r: y - y (r y - 1) (1 - (r y - 1)) with y in float32.
+// The same with a second Heron step, and 1/r = y (1 + e + e^2), e = 1 - r y,
+// y in float32.
 __device__ __forceinline__ double pair_r64(double r2, double& rinv) {
   const float f = f64::trunc_abs(r2);
   if (!(f > 1e-30f)) {
@@ -156,7 +157,9 @@ __device__ __forceinline__ double pair_r64(double r2, double& rinv) {
   }
   const float y = rsqrtf(f);
   const double H = f64::widen(f * y), yd = f64::widen(y);
-  const double r = __fma_rn(__fma_rn(-H, H, r2), 0.5 * yd, H);
+  const double yh = f64::widen(0.5f * y);
+  double r = __fma_rn(__fma_rn(-H, H, r2), yh, H);
+  r = __fma_rn(__fma_rn(-r, r, r2), yh, r);
   const double e = __fma_rn(-r, yd, 1.0);
   rinv = __fma_rn(yd, __fma_rn(e, e, e), yd);
   return r;

@@ -82,46 +82,48 @@ __host__ __device__ constexpr int tri_f(int n) {
   return 16 * (n >> 5) * ((n >> 5) + 1) + (n & 31) * ((n >> 5) + 1);
 }
 
+// What an enumeration keeps in shared memory: ranks, bitmap and the block's
+// cells; with the lists' group entries (EnumSmem) or the members' positions
+// (LargeEnumSmem).
 template <int CAP>
-struct EnumSmem {
+struct EnumBase {
   using Idx = typename std::conditional<CAP <= 256, uint8_t, uint16_t>::type;  // block-local index
   uint32_t bits[tri_f(CAP - 1) + 8];
   int32_t ids[2][CAP];    // merge rounds: the ids in run order
   Idx ks[2][CAP];         // and the block-local index of each
   Idx rank[CAP];          // rank of each block-local index
   Idx perm[CAP];          // block-local index of each rank
-  Idx who[kFlatEntries];  // member of each flat entry
-  uint32_t rng[CAP];      // up to four slot ranges (first slot, length) of each member's group, packed
-  uint32_t rcum[CAP];     // cumulative lengths after ranges 0, 1, 2 (bytes)
-  uint8_t ncnt[CAP];      // entries of each member's group
   uint8_t dk[CAP];        // block cell of each member
-  int64_t lbase[CAP];     // nbr_slot(member, 0) with the slot's in-row part removed
-  uint8_t dtab[8][64];    // partner cell of (member cell, stencil code); 8: not in the block
-  int32_t off[CAP + 1];   // first flat entry of each member
   uint16_t rowbase[CAP];  // first word of each row of the bitmap
-  int32_t wtot[8];        // per-warp totals of the offset scan
   int32_t ctot[CAP / 32]; // row-scan chunk totals
   int32_t cstart[8], cbase[9], koff[9];
   int32_t nb, big;
+};
+struct EnumSmem : EnumBase<kMaxBlock> {
+  Idx who[kFlatEntries];       // member of each flat entry
+  uint32_t rng[kMaxBlock];     // up to four slot ranges (first slot, length) of each member's group, packed
+  uint32_t rcum[kMaxBlock];    // cumulative lengths after ranges 0, 1, 2 (bytes)
+  uint8_t ncnt[kMaxBlock];     // entries of each member's group
+  int64_t lbase[kMaxBlock];    // nbr_slot(member, 0) with the slot's in-row part removed
+  uint8_t dtab[8][64];         // partner cell of (member cell, stencil code); 8: not in the block
+  int32_t off[kMaxBlock + 1];  // first flat entry of each member
+  int32_t wtot[8];             // per-warp totals of the offset scan
+};
+template <class P>
+struct LargeEnumSmem : EnumBase<kLargeBlock> {
+  typename P::R x[kLargeBlock], y[kLargeBlock], z[kLargeBlock];  // block-local position of each rank
+  uint8_t own[kLargeBlock];  // block cell | owner bits << 3 of each rank
 };
 
 // Outcome of an enumeration that gives no list.
 enum : int { kEnumParticles = -1, kEnumPairs = -2, kEnumList = -3 };
 
-// Owned pairs of block o in canonical order by a thread block of THREADS
-// threads: emit(position, lower-ranked member, other member) per pair.
-// Returns their number, or kEnumParticles (more than CAP particles),
-// kEnumPairs (more than max_pairs pairs), kEnumList (a member's list
-// overflowed).  The same value on every thread.
-template <int CAP, int THREADS, class Emit>
-__device__ __forceinline__ int enum_block(EnumSmem<CAP>& sm, const Consts& c, int o, const int32_t* __restrict__ pid,
-                                          const int32_t* __restrict__ cell_start, const int32_t* __restrict__ mrank,
-                                          const uint32_t* __restrict__ nlist, const int32_t* __restrict__ nn,
-                                          const uint32_t* __restrict__ cend, int max_pairs, Emit emit) {
-  using Idx = typename EnumSmem<CAP>::Idx;
-  constexpr int kWarps = THREADS / 32;
-  static_assert(2 * THREADS >= CAP, "two rows and two members per thread");
-  const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+// The block's 8 cells (first warp; the thread block synchronises after it).
+template <int CAP>
+__device__ __forceinline__ void enum_cells(EnumBase<CAP>& sm, const Consts& c, int o,
+                                           const int32_t* __restrict__ cell_start,
+                                           const int32_t* __restrict__ mrank) {
+  const int t = threadIdx.x, lane = t & 31;
   const int ox = o % c.nc[0], oy = (o / c.nc[0]) % c.nc[1], oz = o / (c.nc[0] * c.nc[1]);
   // the block's 8 cells: storage start, count and offset in the block
   if (t < 32) {
@@ -155,6 +157,103 @@ __device__ __forceinline__ int enum_block(EnumSmem<CAP>& sm, const Consts& c, in
       sm.koff[8] = -(1 << 30);  // a partner outside the block: out of range
     }
   }
+}
+
+// One round of the pairwise merges of the sorted cells (level L = 0, 1, 2).
+template <int CAP, int THREADS>
+__device__ __forceinline__ void enum_merge(EnumBase<CAP>& sm, int nb, int L) {
+  const int t = threadIdx.x;
+  const int src = L & 1, dst = src ^ 1;
+  for (int k = t; k < nb; k += THREADS) {
+    const int d = sm.dk[k];
+    const int run = d >> L, sib = run ^ 1;
+    const int own0 = sm.cbase[run << L], m0 = sm.cbase[(run & ~1) << L];
+    int pos = sm.cbase[sib << L], len = sm.cbase[(sib + 1) << L] - pos;
+    const int sib0 = pos;
+    const int32_t myid = sm.ids[src][k];
+    while (len > 0) {
+      const int half = len >> 1;
+      const bool below = sm.ids[src][pos + half] < myid;
+      pos = below ? pos + half + 1 : pos;
+      len = below ? len - half - 1 : half;
+    }
+    const int np = m0 + (k - own0) + (pos - sib0);
+    sm.ids[dst][np] = myid;
+    sm.ks[dst][np] = sm.ks[src][k];
+  }
+}
+
+// The bitmap read out row by row (difference ascending), lower rank
+// ascending: emit(position, lower-ranked member, other member) per pair.
+// Returns the number of pairs, or kEnumPairs above max_pairs.
+template <int CAP, int THREADS, class Emit>
+__device__ __forceinline__ int enum_rows(EnumBase<CAP>& sm, int nb, int max_pairs, Emit emit) {
+  const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+  static_assert(2 * THREADS >= CAP, "two rows per thread");
+  // row populations (rows 1 .. nb - 1): each warp scans 32 rows at a time
+  // (row 1 + t is thread t's in every phase below), then the chunk totals
+  // are added in
+  int rowex[2] = {0, 0};
+#pragma unroll
+  for (int it = 0; it < 2; ++it) {
+    const int r0 = 1 + 32 * wid + it * THREADS;
+    if (r0 >= nb) break;
+    const int rr = r0 + lane;
+    int n = 0;
+    if (rr < nb) {
+      const int w0 = sm.rowbase[rr], nwr = (nb - rr + 31) >> 5;
+      for (int w = 0; w < nwr; ++w) n += __popc(sm.bits[w0 + w]);
+    }
+    int inc = n;
+#pragma unroll
+    for (int sh = 1; sh < 32; sh <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, inc, sh);
+      if (lane >= sh) inc += v;
+    }
+    rowex[it] = inc - n;
+    if (lane == 31) sm.ctot[(r0 - 1) >> 5] = inc;
+  }
+  __syncthreads();
+  const int nchunk = (nb - 1 + 31) >> 5;
+  int npairs = 0;
+  for (int ch = 0; ch < nchunk; ++ch) npairs += sm.ctot[ch];
+  if (npairs > max_pairs) return kEnumPairs;
+  // write the pairs row by row (difference ascending), lower rank ascending
+#pragma unroll
+  for (int it = 0; it < 2; ++it) {
+    const int rr = 1 + t + it * THREADS;
+    if (rr >= nb) break;
+    const int chunk = (rr - 1) >> 5;
+    int pos = rowex[it];
+    for (int ch = 0; ch < chunk; ++ch) pos += sm.ctot[ch];
+    const int w0 = sm.rowbase[rr], nwr = (nb - rr + 31) >> 5;
+    for (int w = 0; w < nwr; ++w) {
+      uint32_t bits = sm.bits[w0 + w];
+      while (bits) {
+        const int bit = __ffs(bits) - 1;
+        bits &= bits - 1;
+        const int lo = w * 32 + bit;
+        emit(pos++, (int)sm.perm[lo], (int)sm.perm[lo + rr]);
+      }
+    }
+  }
+  return npairs;
+}
+
+// Owned pairs of block o in canonical order from the neighbour lists, by a
+// thread block of kEnumThreads threads.  Returns their number, or
+// kEnumParticles (more than kMaxBlock particles), kEnumPairs (more than
+// max_pairs pairs), kEnumList (a member's list overflowed).  The same value
+// on every thread.
+template <class Emit>
+__device__ __forceinline__ int enum_block(EnumSmem& sm, const Consts& c, int o, const int32_t* __restrict__ pid,
+                                          const int32_t* __restrict__ cell_start, const int32_t* __restrict__ mrank,
+                                          const uint32_t* __restrict__ nlist, const int32_t* __restrict__ nn,
+                                          const uint32_t* __restrict__ cend, int max_pairs, Emit emit) {
+  constexpr int CAP = kMaxBlock, THREADS = kEnumThreads, kWarps = THREADS / 32;
+  using Idx = EnumSmem::Idx;
+  const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+  enum_cells<CAP>(sm, c, o, cell_start, mrank);
   for (int q = t; q < 8 * 64; q += THREADS) {  // partner cell: member cell + (code - 1) per axis
     const int dA = q >> 6, code = q & 63;
     int dB = 0;
@@ -251,24 +350,7 @@ __device__ __forceinline__ int enum_block(EnumSmem<CAP>& sm, const Consts& c, in
   int cnt0 = 0, incl = 0;
 #pragma unroll 1
   for (int L = 0; L < 3; ++L) {
-    const int src = L & 1, dst = src ^ 1;
-    for (int k = t; k < nb; k += THREADS) {
-      const int d = sm.dk[k];
-      const int run = d >> L, sib = run ^ 1;
-      const int own0 = sm.cbase[run << L], m0 = sm.cbase[(run & ~1) << L];
-      int pos = sm.cbase[sib << L], len = sm.cbase[(sib + 1) << L] - pos;
-      const int sib0 = pos;
-      const int32_t myid = sm.ids[src][k];
-      while (len > 0) {
-        const int half = len >> 1;
-        const bool below = sm.ids[src][pos + half] < myid;
-        pos = below ? pos + half + 1 : pos;
-        len = below ? len - half - 1 : half;
-      }
-      const int np = m0 + (k - own0) + (pos - sib0);
-      sm.ids[dst][np] = myid;
-      sm.ks[dst][np] = sm.ks[src][k];
-    }
+    enum_merge<CAP, THREADS>(sm, nb, L);
     if (L == 0) {  // counts of members 2t and 2t + 1: per-warp inclusive scan
       cnt0 = 2 * t < nb ? sm.ncnt[2 * t] : 0;
       const int cnt1 = 2 * t + 1 < nb ? sm.ncnt[2 * t + 1] : 0;
@@ -331,65 +413,94 @@ __device__ __forceinline__ int enum_block(EnumSmem<CAP>& sm, const Consts& c, in
     }
     __syncthreads();
   }
-  // row populations (rows 1 .. nb - 1): each warp scans 32 rows at a time
-  // (row 1 + t is thread t's in every phase below), then the chunk totals
-  // are added in
-  int rowex[2] = {0, 0};
-#pragma unroll
-  for (int it = 0; it < 2; ++it) {
-    const int r0 = 1 + 32 * wid + it * THREADS;
-    if (r0 >= nb) break;
-    const int rr = r0 + lane;
-    int n = 0;
-    if (rr < nb) {
-      const int w0 = sm.rowbase[rr], nwr = (nb - rr + 31) >> 5;
-      for (int w = 0; w < nwr; ++w) n += __popc(sm.bits[w0 + w]);
-    }
-    int inc = n;
-#pragma unroll
-    for (int sh = 1; sh < 32; sh <<= 1) {
-      const int v = __shfl_up_sync(0xffffffffu, inc, sh);
-      if (lane >= sh) inc += v;
-    }
-    rowex[it] = inc - n;
-    if (lane == 31) sm.ctot[(r0 - 1) >> 5] = inc;
-  }
-  __syncthreads();
-  const int nchunk = (nb - 1 + 31) >> 5;
-  int npairs = 0;
-  for (int ch = 0; ch < nchunk; ++ch) npairs += sm.ctot[ch];
-  if (npairs > max_pairs) return kEnumPairs;
-  // write the pairs row by row (difference ascending), lower rank ascending
-#pragma unroll
-  for (int it = 0; it < 2; ++it) {
-    const int rr = 1 + t + it * THREADS;
-    if (rr >= nb) break;
-    const int chunk = (rr - 1) >> 5;
-    int pos = rowex[it];
-    for (int ch = 0; ch < chunk; ++ch) pos += sm.ctot[ch];
-    const int w0 = sm.rowbase[rr], nwr = (nb - rr + 31) >> 5;
-    for (int w = 0; w < nwr; ++w) {
-      uint32_t bits = sm.bits[w0 + w];
-      while (bits) {
-        const int bit = __ffs(bits) - 1;
-        bits &= bits - 1;
-        const int lo = w * 32 + bit;
-        emit(pos++, (int)sm.perm[lo], (int)sm.perm[lo + rr]);
-      }
-    }
-  }
-  return npairs;
+  return enum_rows<CAP, THREADS>(sm, nb, max_pairs, emit);
 }
 
-// The schedule's first launch: one thread block per block of cells.
-__global__ void __launch_bounds__(kEnumThreads)
+// The same for a large block, from positions: the members in rank order with
+// their block-local coordinates, then every pair of ranks by the owner rule
+// and the distance (32 pairs of one row per warp, whose ballot is a word of
+// the bitmap).  The predicate is the one of the pair-by-pair sweep.
+template <class P, class Emit>
+__device__ __forceinline__ int enum_large(LargeEnumSmem<P>& sm, const Consts& c, int o,
+                                          const int32_t* __restrict__ pid, const int32_t* __restrict__ cell_start,
+                                          const int32_t* __restrict__ mrank, const typename P::V4* __restrict__ q4,
+                                          const uint32_t* xmx, const uint32_t* xmy, const uint32_t* xmz,
+                                          const int32_t* __restrict__ nn, int max_pairs, Emit emit) {
+  using R = typename P::R;
+  constexpr int CAP = kLargeBlock, THREADS = kLargeThreads;
+  using Idx = typename EnumBase<CAP>::Idx;
+  const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+  enum_cells<CAP>(sm, c, o, cell_start, mrank);
+  __syncthreads();
+  const int nb = sm.nb;
+  if (nb > CAP) return kEnumParticles;
+  auto member = [&](int k, int& d) {
+    d = 0;
+#pragma unroll
+    for (int u = 1; u < 8; ++u) d += (k >= sm.cbase[u]);
+    return sm.cstart[d] + (k - sm.cbase[d]);
+  };
+  for (int k = t; k < nb; k += THREADS) {
+    int d;
+    const int g = member(k, d);
+    sm.ids[0][k] = __ldg(&pid[g]);
+    sm.ks[0][k] = (Idx)k;
+    sm.dk[k] = (uint8_t)d;
+    if (__ldg(&nn[g]) > c.nbr_cap) sm.big = 1;  // (left to the pair-by-pair sweep)
+  }
+  __syncthreads();
+  if (sm.big) return kEnumList;
+#pragma unroll 1
+  for (int L = 0; L < 3; ++L) {
+    enum_merge<CAP, THREADS>(sm, nb, L);
+    __syncthreads();
+  }
+  BlockGeom<P> geo;
+  geo.init(c, o % c.nc[0], (o / c.nc[0]) % c.nc[1], o / (c.nc[0] * c.nc[1]), xmx, xmy, xmz);
+  for (int r = t; r < nb; r += THREADS) {  // the merged run is ids[1]
+    const int k = sm.ks[1][r];
+    int d;
+    const int g = member(k, d);
+    sm.perm[r] = (Idx)k;
+    R x, y, z;
+    geo.local(ld4(&q4[g]), d, x, y, z);
+    sm.x[r] = x;
+    sm.y[r] = y;
+    sm.z[r] = z;
+    sm.own[r] = (uint8_t)(d | (int)owner_bits(sm.ids[1][r]) << 3);
+  }
+  for (int d = 1 + t; d < nb; d += THREADS) sm.rowbase[d] = (uint16_t)(tri_f(nb - 1) - tri_f(nb - d));
+  __syncthreads();
+  const R h2 = (R)c.h2;
+  for (int d = 1 + wid; d < nb; d += THREADS / 32)
+    for (int r0 = 0; r0 < nb - d; r0 += 32) {
+      const int r = r0 + lane;
+      bool hit = false;
+      if (r < nb - d) {
+        const int a = sm.own[r], dA = a & 7, dB = sm.own[r + d] & 7;
+        if ((((dA ^ (a >> 3)) & ~(dA ^ dB)) & 7) == 0) {  // on shared axes the cell bit equals the owner bit
+          R dx, dy, dz;
+          geo.disp(sm.x[r], sm.y[r], sm.z[r], sm.x[r + d], sm.y[r + d], sm.z[r + d], dx, dy, dz);
+          hit = r2_of(dx, dy, dz) < h2;
+        }
+      }
+      const unsigned m = __ballot_sync(0xffffffffu, hit);
+      if (lane == 0) sm.bits[sm.rowbase[d] + (r0 >> 5)] = m;
+    }
+  __syncthreads();
+  return enum_rows<CAP, THREADS>(sm, nb, max_pairs, emit);
+}
+
+// The schedule's first launch: one thread block per block of cells (12 per SM:
+// 32 registers; 1520 us instead of 1313 at 2M particles with 38).
+__global__ void __launch_bounds__(kEnumThreads, 12)
     k_sched_enum(const __grid_constant__ Consts c, const int32_t* __restrict__ pid,
                  const int32_t* __restrict__ cell_start, const int32_t* __restrict__ mrank,
                  const uint32_t* __restrict__ nlist, const int32_t* __restrict__ nn,
                  const uint32_t* __restrict__ cend, uint32_t* __restrict__ hdr, uint16_t* __restrict__ canon,
                  uint32_t* __restrict__ blk_hist, uint32_t* __restrict__ big_count, uint32_t* __restrict__ large_count,
                  int32_t* __restrict__ large_cand, unsigned long long* __restrict__ sched_total) {
-  __shared__ EnumSmem<kMaxBlock> sm;
+  __shared__ EnumSmem sm;
   const int t = threadIdx.x, o = blockIdx.x;  // owner cell (fewer than 2^31 cells)
   if (o == 0) {  // what the next launches count in: depth histogram, lists, dense pair arrays
     if (t == 0) *sched_total = 0ull;
@@ -398,7 +509,7 @@ __global__ void __launch_bounds__(kEnumThreads)
     if (t < 8) large_count[t] = 0u;
   }
   uint16_t* out = canon + (int64_t)o * kMaxPairs;
-  const int np = enum_block<kMaxBlock, kEnumThreads>(
+  const int np = enum_block(
       sm, c, o, pid, cell_start, mrank, nlist, nn, cend, kMaxPairs,
       [&](int pos, int lo, int hi) { out[pos] = (uint16_t)(lo | (hi << 8)); });
   if (t != 0) return;
@@ -588,33 +699,36 @@ __global__ void __launch_bounds__(kRoundWarps * 32)
 // ---------------------------------------------------------------------------
 // Large blocks: more particles or owned pairs than k_sched_enum holds, as in
 // boxes whose side lies between two cell counts (14 / 2.5: cells of 3.5,
-// blocks of 343).  One thread block takes them in turn, pairs and rounds with
-// the list in shared memory.  (Swept pair by pair on one lane they took 40 ms
+// blocks of 343).  One thread block takes them in turn, pairs (enum_large) and
+// rounds with the list in shared memory.  (Swept pair by pair on one lane they took 40 ms
 // per sweep of 14^3 particles.)  width: as k_sched_rounds.  The last thread
 // block then turns the depth histogram into each depth's first position,
 // deepest first (one warp per colour; see below).
 // ---------------------------------------------------------------------------
+template <class P>
 struct LargeSmem {
-  EnumSmem<kLargeBlock> e;
+  LargeEnumSmem<P> e;
   RoundSmem<kLargeBlock, kLargePairs> r;
   uint32_t canon[kLargePairs];
   int np;
   uint32_t last;
 };
 
+template <class P>
 __global__ void __launch_bounds__(kLargeThreads)
     k_sched_large(const __grid_constant__ Consts c, const __grid_constant__ SchedOut out, int width,
-                  const int32_t* __restrict__ pid, const uint32_t* __restrict__ nlist, const int32_t* __restrict__ nn,
-                  const uint32_t* __restrict__ cend, const int32_t* __restrict__ cand,
+                  const int32_t* __restrict__ pid, const typename P::V4* __restrict__ q4, const uint32_t* xmx,
+                  const uint32_t* xmy, const uint32_t* xmz, const int32_t* __restrict__ nn,
+                  const int32_t* __restrict__ cand,
                   uint32_t* __restrict__ large_count, int32_t* __restrict__ large_list) {
   extern __shared__ __align__(16) unsigned char large_smem_raw[];
-  LargeSmem& sm = *reinterpret_cast<LargeSmem*>(large_smem_raw);
+  LargeSmem<P>& sm = *reinterpret_cast<LargeSmem<P>*>(large_smem_raw);
   const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
   const int n = (int)large_count[8];
   for (int q = blockIdx.x; q < n; q += gridDim.x) {
     const int o = cand[q];
-    const int np = enum_block<kLargeBlock, kLargeThreads>(
-        sm.e, c, o, pid, out.cell_start, out.mrank, nlist, nn, cend, kLargePairs,
+    const int np = enum_large<P>(
+        sm.e, c, o, pid, out.cell_start, out.mrank, q4, xmx, xmy, xmz, nn, kLargePairs,
         [&](int pos, int lo, int hi) { sm.canon[pos] = (uint32_t)lo | (uint32_t)hi << 16; });
     __syncthreads();
     if (wid == 0) {
@@ -706,8 +820,9 @@ void launch_fd_schedule(const Consts& c, const Workspace& w, int cur, int width,
   k_sched_rounds<<<(unsigned)((c.ncell + kRoundWarps - 1) / kRoundWarps), kRoundWarps * 32, 0, s>>>(out, width,
                                                                                                    w.sched_canon);
   // (a large block has a whole warp of the colour launch, or its team)
-  k_sched_large<<<(unsigned)std::min(c.ncell, 152), kLargeThreads, sizeof(LargeSmem), s>>>(
-      c, out, std::max(width, large_width), a.id, w.nlist, w.nn, w.cend, w.large_cand, w.large_count, w.large_list);
+  k_sched_large<P><<<(unsigned)std::min(c.ncell, 152), kLargeThreads, sizeof(LargeSmem<P>), s>>>(
+      c, out, std::max(width, large_width), a.id, a.q4, w.xmin[0], w.xmin[1], w.xmin[2], w.nn, w.large_cand,
+      w.large_count, w.large_list);
   k_sched_order_scatter<<<(unsigned)((c.ncell + 255) / 256), 256, 0, s>>>(c.ncell, c.nc[0], c.nc[1], w.sched_hdr,
                                                                          w.blk_hist, w.blk_order, w.large_count);
 }
@@ -715,10 +830,11 @@ void launch_fd_schedule(const Consts& c, const Workspace& w, int cur, int width,
 // Launch attributes of the schedule's kernels (once per device and process;
 // kept out of stream captures).
 int sched_prepare() {
-  return cudaFuncSetAttribute(k_sched_large, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(LargeSmem)) ==
-                 cudaSuccess
-             ? SDPD_OK
-             : SDPD_ERR_CUDA;
+  const cudaError_t a = cudaFuncSetAttribute(k_sched_large<Fp64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)sizeof(LargeSmem<Fp64>)),
+                    b = cudaFuncSetAttribute(k_sched_large<Mixed>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)sizeof(LargeSmem<Mixed>));
+  return a == cudaSuccess && b == cudaSuccess ? SDPD_OK : SDPD_ERR_CUDA;
 }
 
 __global__ void k_sweep_set(unsigned long long* sweep, unsigned long long v) { *sweep = v; }
