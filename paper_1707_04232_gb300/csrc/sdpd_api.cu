@@ -246,7 +246,7 @@ void do_load(sdpd_handle* s) {
   launch_sort<P>(s->c, s->w, 0, s->stream);
   s->cur = 1;
   launch_density<P>(s->c, s->w, s->cur, 0, nullptr, s->stream);
-  s->launches += 7;
+  s->launches += 2 + sort_launches(s->c);  // load, sort, density
   s->sched_valid = false;
 }
 
@@ -322,7 +322,7 @@ void vv_step(sdpd_handle* s, double dt) {
     launch_force<P>(c, s->w, s->cur, 0.5 * dt, dt, nullptr, s->stream);
   }
   {
-    StageTimer t(s, 1, 5);
+    StageTimer t(s, 1, sort_launches(c));
     launch_sort<P>(c, s->w, s->cur, s->stream);
   }
   s->cur = 1 - s->cur;
@@ -334,7 +334,7 @@ void vv_step(sdpd_handle* s, double dt) {
     StageTimer t(s, 3, P::mixed ? 2 : 1);
     launch_force<P>(c, s->w, s->cur, 0.5 * dt, 0.0, nullptr, s->stream);
   }
-  s->launches += P::mixed ? 10 : 8;  // force (mixed: + overflow), 5 sort, density, force (+ overflow)
+  s->launches += (P::mixed ? 5 : 3) + sort_launches(c);  // force (mixed: + overflow), sort, density, force (+ overflow)
   s->vv_step++;
   s->sched_valid = false;
 }
@@ -492,6 +492,17 @@ int sdpd_create(int64_t N, const double box[3], double m, double h, const sdpd_p
   }
   c.W0 = c.cW;
   c.nbr_cap = 160;
+  c.pi_coef = c.c_rho / (c.C_K * c.m);
+  c.f_h2 = (float)c.h2;
+  c.f_inv_h = 1.0f / (float)c.h;
+  c.f_cW = (float)c.cW;
+  c.f_cF = (float)c.cF;
+  c.f_m = (float)c.m;
+  c.f_m2 = (float)(c.m * c.m);
+  c.f_W0 = (float)c.W0;
+  for (int d = 0; d < 3; ++d) c.f_scale[d] = (float)c.scale[d];
+  c.f_eos = (float)(c.c_rho / c.C_K);
+  c.f_pi_coef = (float)c.pi_coef;
   {
     // Float32 pre-test of r^2 < h^2 (float64 path).  With u = 2^-24, each
     // float32 coordinate, the float32 difference and the float32 minimum
@@ -977,7 +988,7 @@ void load_state(sdpd_handle* s, const double* slot) {
   launch_sort<Fp64>(s->c, s->w, 0, s->stream);
   s->cur = 1;
   launch_density<Fp64>(s->c, s->w, s->cur, 0, nullptr, s->stream);
-  s->launches += 7;
+  s->launches += 2 + sort_launches(s->c);  // load, sort, density
   s->sched_valid = false;
 }
 
@@ -1104,16 +1115,16 @@ int sdpd_vv_adjoint(sdpd_t* s, void* tape, size_t tape_bytes, const double* gq, 
   double* Sbar_prev = t.Sbar2;
   for (int64_t k = ns; k >= 0; --k) {
     if (k == ns) {
-      StageTimer tm(s, 6, 7);
+      StageTimer tm(s, 6, 2 + sort_launches(c));
       load_state(s, t.final_state());
     } else if (k % every == 0) {
-      StageTimer tm(s, 6, 7);
+      StageTimer tm(s, 6, 2 + sort_launches(c));
       load_state(s, t.ckpt(k / every));
     } else {
       const int64_t sg = k / every, k0 = sg * every;
       if (sg != seg_loaded) {  // replay the segment from its checkpoint
         {
-          StageTimer tm(s, 6, 7);
+          StageTimer tm(s, 6, 2 + sort_launches(c));
           load_state(s, t.ckpt(sg));
         }
         const int64_t k1 = std::min(k0 + every, ns);
@@ -1126,7 +1137,7 @@ int sdpd_vv_adjoint(sdpd_t* s, void* tape, size_t tape_bytes, const double* gq, 
         }
         seg_loaded = sg;
       }
-      StageTimer tm(s, 6, 7);
+      StageTimer tm(s, 6, 2 + sort_launches(c));
       load_state(s, t.seg(k - k0 - 1));
     }
     // the first kick of step k (k < n) and the second of step k - 1 (k > 0)

@@ -565,7 +565,7 @@ __global__ void __launch_bounds__(kStageWarps * 32)
   owner_coords(c, o, ox, oy, oz);
   BlockGeom<P> geo;
   geo.init(c, ox, oy, oz, xmx, xmy, xmz);
-  const S inv_h = (S)(1.0 / c.h), cF = (S)c.cF;
+  const S inv_h = (S)c.inv_h, cF = (S)c.cF;
   const unsigned long long base = sched_off[o];
   for (int t = 32 * part + lane; t < np; t += 32 * split) {
     const uint32_t pr = pairs[base + t];
@@ -792,7 +792,7 @@ __device__ __noinline__ BigCounts fd_big_block(const Consts& c, const FDConst<ty
     }
   }
   // pressure over rho^2 of the new energies, Eq. (pg-eos)
-  const S pi_coef = (S)(c.c_rho / (c.C_K * c.m));
+  const S pi_coef = std::is_same<S, float>::value ? (S)c.f_pi_coef : (S)c.pi_coef;
   for (int q = lane; q < nb; q += 32) {
     const int g = perm[q];
     qp4[g].w = (S)a.eps[g] * pi_coef / a.rho[g];
@@ -977,7 +977,7 @@ __device__ __forceinline__ void fd_run_block(const FdRun<P>& f, bool live, int64
     }
     __syncwarp();
   }
-  const S pi_coef = (S)(c.c_rho / (c.C_K * c.m));
+  const S pi_coef = std::is_same<S, float>::value ? (S)c.f_pi_coef : (S)c.pi_coef;
   for (int q = gl; q < nb; q += GL) {
     const int g = block_gidx(cells, q);
     const F4 v = lds4(&s[q]);
@@ -1101,7 +1101,7 @@ __device__ __noinline__ void fd_large_block(const FdRun<P>& f, int64_t o, uint64
     at += n;
     __syncwarp();
   }
-  const S pi_coef = (S)(c.c_rho / (c.C_K * c.m));
+  const S pi_coef = std::is_same<S, float>::value ? (S)c.f_pi_coef : (S)c.pi_coef;
   for (int q = lane; q < nb; q += 32) {
     const int g = block_gidx(sm.cells, q);
     a.px[g] = sm.p[0][q];

@@ -71,7 +71,7 @@ struct BlockGeom<Mixed> {
     const uint32_t* xm[3] = {xmx, xmy, xmz};
     for (int d = 0; d < 3; ++d) {
       int up = o[d] + 1 >= c.nc[d] ? 0 : o[d] + 1;
-      off[d] = (float)(int32_t)(xm[d][up] - xm[d][o[d]]) * (float)c.scale[d];
+      off[d] = (float)(int32_t)(xm[d][up] - xm[d][o[d]]) * c.f_scale[d];
     }
   }
   __device__ __forceinline__ void local(const F4& q, int code, float& x, float& y, float& z) const {

@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(team_threads<EMS>())
   const int tt = t % kTeamThreads, l = tt & 3, slot = tt >> 2;  // quad lane, pair of the round
   const int hx = c.nc[0] >> 1, hy = c.nc[1] >> 1, hz = c.nc[2] >> 1;
   const int64_t nown = (int64_t)hx * hy * hz;
-  const double pi_coef = c.c_rho / (c.C_K * c.m);
+  const double pi_coef = c.pi_coef;
   unsigned n_tot = 0, n_rb = 0, n_rm = 0;
   bool negative = false, bad = false;
   double* rec = reinterpret_cast<double*>(sm.s);

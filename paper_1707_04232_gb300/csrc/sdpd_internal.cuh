@@ -50,6 +50,10 @@ struct Consts {
   double inv_scale[3];  // 2^32 / box side
   double h, h2, inv_h, m, kB;
   double C_K, c_rho;
+  double pi_coef;            // pressure over rho^2: pi = pi_coef eps / rho, c_rho / (C_K m)
+  // the same for float32 arithmetic (a conversion or a division of these by
+  // every thread would cost float64 issues)
+  float f_h2, f_inv_h, f_cW, f_cF, f_m, f_m2, f_W0, f_scale[3], f_eos, f_pi_coef;
   double kpar_m2, kperp_m2;  // (10/3 eta + 4 zeta) m^2 and (5/3 eta - zeta) m^2
   double cW, cF, W0;         // kernel constants and W(0)
   int kernel, scheme;
@@ -413,6 +417,7 @@ template <class P>
 void launch_load(const Consts& c, const Workspace& w, cudaStream_t s);
 template <class P>
 void launch_sort(const Consts& c, const Workspace& w, int from, cudaStream_t s);
+int sort_launches(const Consts& c);  // kernels of launch_sort
 template <class P>
 void launch_unload(const Consts& c, const Workspace& w, int cur, cudaStream_t s);
 template <class P>

@@ -28,7 +28,7 @@ struct Home<Mixed> {
   __device__ void init(const Consts& c, const F4& q, int cx_, int cy_, int cz_, const uint32_t* xmx_,
                        const uint32_t* xmy_, const uint32_t* xmz_) {
     x = q.x; y = q.y; z = q.z;
-    sx = (float)c.scale[0]; sy = (float)c.scale[1]; sz = (float)c.scale[2];
+    sx = c.f_scale[0]; sy = c.f_scale[1]; sz = c.f_scale[2];
     cx = cx_; cy = cy_; cz = cz_;
     xmx = xmx_; xmy = xmy_; xmz = xmz_;
   }
@@ -145,18 +145,18 @@ __global__ void __launch_bounds__(128, 12) k_density(Consts c, Arrays<P> a, type
   if (ncount_by_id) ncount_by_id[a.id[i]] = cnt;
   nn[i] = cnt;
   if (cnt > c.nbr_cap) ovf_list[atomicAdd(ovf_count, 1)] = (int32_t)i;  // forces from the cells
-  const R rho_new = (R)c.m * ((R)c.W0 + acc);
+  const R rho_new = c.f_m * (c.f_W0 + acc);
   double e = a.eps[i];
   if (update_eos) {
     // eps * (rho_new / rho_old)^(c_rho / C_K), the factor minus one formed
     // from log1p / expm1 of small arguments so float32 keeps it accurate
     const float ro = a.rho[i];
-    const float g = expm1f((float)(c.c_rho / c.C_K) * log1pf((rho_new - ro) / ro));
+    const float g = expm1f(c.f_eos * log1pf((rho_new - ro) / ro));
     e = fma(e, (double)g, e);
     a.eps[i] = e;
   }
   a.rho[i] = rho_new;
-  const R pi = (float)e * (float)(c.c_rho / (c.C_K * c.m)) / rho_new;
+  const R pi = (float)e * c.f_pi_coef / rho_new;
   V4 o = qi;
   o.w = pi;
   st4(&qp4[i], o);
@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(PPB * T)
     }
     a.rho[g] = rho_new;
     D4 o = ld4(&a.q4[g]);
-    o.w = e * (c.c_rho / (c.C_K * c.m)) / rho_new;
+    o.w = e * c.pi_coef / rho_new;
     st4(&qp4[g], o);
     o.w = rho_new;  // positions and density together for the sweep's pair geometry
     st4(&qr4[g], o);
@@ -258,7 +258,7 @@ __device__ __forceinline__ void kick_particle(const Consts& c, const Arrays<P>& 
                                               const int32_t* __restrict__ mrank, double* __restrict__ force_by_id,
                                               const float drift_f[3]) {
   using R = typename P::R;
-  const R m2 = (R)(c.m * c.m);
+  const R m2 = c.f_m2;
   fx *= m2; fy *= m2; fz *= m2;
   if (force_by_id) {
     const int64_t k = a.id[i];
@@ -305,7 +305,7 @@ __device__ __forceinline__ void force_from_cells(const Consts& c, const Arrays<P
   unpack_cell(w_to_cellbits(ld4(&a.q4[i]).w), cx, cy, cz);
   Home<P> home;
   home.init(c, qi, cx, cy, cz, xmx, xmy, xmz);
-  const R h2 = (R)c.h2, inv_h = R(1) / (R)c.h, cF = (R)c.cF;
+  const R h2 = c.f_h2, inv_h = c.f_inv_h, cF = c.f_cF;
   R fx = R(0), fy = R(0), fz = R(0);
   for (int oz = -1; oz <= 1; ++oz) {
     const int nz = wrapc(cz + oz, c.nc[2]);
@@ -371,7 +371,7 @@ __global__ void __launch_bounds__(128, KIND == SDPD_KERNEL_LUCY ? 16 : 12) k_for
     unpack_cell(w_to_cellbits(qi.w), cx, cy, cz);
     Home<P> home;
     home.init(c, qi, cx, cy, cz, xmx, xmy, xmz);
-    const R inv_h = R(1) / (R)c.h, cF = (R)c.cF;
+    const R inv_h = c.f_inv_h, cF = c.f_cF;
     R fx = R(0), fy = R(0), fz = R(0);
     home.frames_all(c);
     // four entries per 16-byte load (a warp's loads are contiguous, see
