@@ -312,7 +312,9 @@ void sdpd_ensemble_destroy(sdpd_ens_t* e);
 typedef struct {
   int fd_variant;   /* blocks per warp x warps per thread block of the colour
                        launches: 0 (2 x 2), 1 (2 x 1), 2 (1 x 1), 3 (1 x 2),
-                       4 (1 x 4); -1 = chosen at launch by the blocks per
+                       4 (1 x 4); with 2 to 4 the Metropolised scheme runs
+                       a team of two warps per block instead.  -1 = chosen at
+                       launch by the blocks per
                        colour (2 up to 912 of them, 1 up to 4864, else 0;
                        sdpd_get_tuning then reports 0 for float32 and 1 for
                        float64 pair arithmetic); a new handle starts with -1.

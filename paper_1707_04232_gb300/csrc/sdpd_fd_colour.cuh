@@ -293,29 +293,39 @@ static __device__ __noinline__ double mixed_margin_fp64(const MixedRatioIn& r, d
 // evaluated (always when `exact` is set).  exact_e(ei, ej) gives the two
 // current energies in float64 and uniform() the pair's uniform U (both for
 // the rare float64 evaluations).
-template <bool SEQ, class ExactE, class Uniform>
-__device__ __forceinline__ int fd_pair_mixed(const FDConst<float>& k, float ex, float ey, float ez, float base,
-                                             const float G[3], Uniform uniform, float lnU, float* pi, float* pj,
-                                             float eif, float ejf, ExactE exact_e, float& dh, float& dl,
-                                             double& margin, float& m32, float& tol, bool exact,
-                                             bool& negative) {
+// The proposal of one mixed-path pair: what its Metropolis test needs, and the
+// new momenta.
+struct MixedMove {
+  float vx, vy, vz, mpar, mperp, zpar, zperp;  // velocity, alpha - 1 and zt per direction
+  float dh, dl, dhf;                           // energy change (float-float), its float32 estimate
+  float nn[6];                                 // new momenta of i and j
+};
+
+// e . v and e . G (the rounding order is written out so that it does not
+// depend on the code around it; SEQ: the order of the pair-by-pair sweep).
+__device__ __forceinline__ float mixed_vpar(float ex, float ey, float ez, float vx, float vy, float vz) {
+  return __fmaf_rn(ez, vz, __fmaf_rn(ex, vx, __fmul_rn(ey, vy)));
+}
+template <bool SEQ>
+__device__ __forceinline__ float mixed_gpar(float ex, float ey, float ez, const float G[3]) {
+  return __fmaf_rn(ez, G[2], SEQ ? __fmaf_rn(ey, G[1], __fmul_rn(ex, G[0])) : __fmaf_rn(ex, G[0], __fmul_rn(ey, G[1])));
+}
+
+// Returns 2 when the pair does nothing (r = h), else 1 when both new energies
+// are positive and 0 when the energy bound rejects the move.
+template <bool SEQ, class ExactE>
+__device__ __forceinline__ int mixed_propose(const FDConst<float>& k, float ex, float ey, float ez, float base,
+                                             const float G[3], const float* pi, const float* pj, float eif, float ejf,
+                                             ExactE exact_e, MixedMove& mv, float& emn) {
+  emn = 0.0f;
   const float kpar = k.kpar_m2 * base, kperp = k.kperp_m2 * base;
-  margin = 0.0;
-  dh = 0.0f;
-  dl = 0.0f;
-  m32 = 0.0f;
-  tol = 0.0f;
-  if (!(kperp > 0.0f) || !(kpar > 0.0f)) return 0;  // at r = h the pair does nothing
+  if (!(kperp > 0.0f) || !(kpar > 0.0f)) return 2;  // at r = h the pair does nothing
   const float vx = (pi[0] - pj[0]) * k.inv_m, vy = (pi[1] - pj[1]) * k.inv_m, vz = (pi[2] - pj[2]) * k.inv_m;
   float mpar, mperp, zpar, zperp;  // alpha - 1 and zt per direction
   pair_coeffs(k, kpar, kperp, eif, ejf, mpar, mperp, zpar, zperp);
   // proposal, Eq. (proposal), as the velocity change
   // v' - v = m_perp v + zt_perp G + [(m_par - m_perp) v_par + (zt_par - zt_perp) G_par] e
-  // (the rounding order is written out so that it does not depend on the code
-  // around it; SEQ: the order of the pair-by-pair sweep)
-  const float vpar = __fmaf_rn(ez, vz, __fmaf_rn(ex, vx, __fmul_rn(ey, vy)));
-  const float gpar = __fmaf_rn(ez, G[2], SEQ ? __fmaf_rn(ey, G[1], __fmul_rn(ex, G[0]))
-                                             : __fmaf_rn(ex, G[0], __fmul_rn(ey, G[1])));
+  const float vpar = mixed_vpar(ex, ey, ez, vx, vy, vz), gpar = mixed_gpar<SEQ>(ex, ey, ez, G);
   const float cpar = (mpar - mperp) * vpar + (zpar - zperp) * gpar;
   const float dvx = mperp * vx + zperp * G[0] + cpar * ex;
   const float dvy = mperp * vy + zperp * G[1] + cpar * ey;
@@ -337,6 +347,7 @@ __device__ __forceinline__ int fd_pair_mixed(const FDConst<float>& k, float ex, 
     }
     dhf = k.nq_hi * dk;
   }
+  float dh, dl;
   {  // deps = -1/2 of the kinetic-energy change of the stored momenta, exactly
     const float oo[6] = {pi[0], pi[1], pi[2], pj[0], pj[1], pj[2]};
     float d[6], lo[6];  // new^2 - old^2 per component as d + lo, exactly
@@ -368,70 +379,108 @@ __device__ __forceinline__ int fd_pair_mixed(const FDConst<float>& k, float ex, 
   // energy bound, Eq. (energy-bound): both new internal energies > 0;
   // float32 decides unless the margin is within its rounding of zero
   const float eminf = eif < ejf ? eif : ejf;
-  float emn = eminf + dh;
+  emn = eminf + dh;
   if (fabsf(emn) <= 32.0f * 5.9604645e-8f * (eminf + fabsf(dh))) {
     double ei, ej;
     exact_e(ei, ej);
     emn = ((ei < ej ? ei : ej) + ((double)dh + (double)dl)) > 0.0 ? 1.0f : -1.0f;
   }
+  mv.vx = vx; mv.vy = vy; mv.vz = vz;
+  mv.mpar = mpar; mv.mperp = mperp; mv.zpar = zpar; mv.zperp = zperp;
+  mv.dh = dh; mv.dl = dl; mv.dhf = dhf;
+#pragma unroll
+  for (int t = 0; t < 6; ++t) mv.nn[t] = nn[t];
+  return emn > 0.0f ? 1 : 0;
+}
+
+// The Metropolis test of a move: true when it is rejected.  margin receives
+// the float64 margin whenever it was evaluated (always when `exact` is set).
+template <bool SEQ, class ExactE, class Uniform>
+__device__ __forceinline__ bool mixed_rejects(const FDConst<float>& k, float ex, float ey, float ez, float base,
+                                              const float G[3], Uniform uniform, float lnU, float eif, float ejf,
+                                              ExactE exact_e, const MixedMove& mv, double& margin, float& m32,
+                                              float& tol, bool exact) {
+  const float kpar = k.kpar_m2 * base, kperp = k.kperp_m2 * base;
+  const float vx = mv.vx, vy = mv.vy, vz = mv.vz, mpar = mv.mpar, mperp = mv.mperp, zpar = mv.zpar, zperp = mv.zperp;
+  const float dh = mv.dh, dhf = mv.dhf;
+  const float vpar = mixed_vpar(ex, ey, ez, vx, vy, vz), gpar = mixed_gpar<SEQ>(ex, ey, ez, G);
+  // reverse move from v' with the coefficients at the proposed energies
+  float mrpar, mrperp, ypar, yperp;
+  pair_coeffs(k, kpar, kperp, eif + dhf, ejf + dhf, mrpar, mrperp, ypar, yperp);
+  // 1 - alpha' alpha = -(m + m' + m m') (both m <= 0: no cancellation), alpha' zt
+  const float cpr = -(mpar + mrpar + mpar * mrpar), cqr = -(mperp + mrperp + mperp * mrperp);
+  const float bzpar = fmaf(mrpar, zpar, zpar), bzperp = fmaf(mrperp, zperp, zperp);
+  const float ryy = fm::div(1.0f, ypar * yperp);
+  const float ipar = yperp * ryy, ip = ypar * ryy;  // 1 / zt'_par, 1 / zt'_perp
+  // reverse noise B'^-1 (v - A' v') = B'^-1 [(I - A' A) v - A' B G] per
+  // direction: no cancellation when zt' -> 0 (pairs near the cut-off)
+  const float qpar = (cpr * vpar - bzpar * gpar) * ipar;
+  const float qx = (cqr * (vx - vpar * ex) - bzperp * (G[0] - gpar * ex)) * ip;
+  const float qy = (cqr * (vy - vpar * ey) - bzperp * (G[1] - gpar * ey)) * ip;
+  const float qz = (cqr * (vz - vpar * ez) - bzperp * (G[2] - gpar * ez)) * ip;
+  const float quad = qpar * qpar + qx * qx + qy * qy + qz * qz;
+  const float g2 = G[0] * G[0] + G[1] * G[1] + G[2] * G[2];
+  // log|B(v)| - log|B(v')| with |B| = zt_par zt_perp^2
+  const float ldet = fm::log(zpar * zperp * zperp * (ipar * ip * ip));
+  // (S(eps') - S(eps))/kB - (log T(eps') - log T(eps)) over both particles
+  const float x = fm::div(dh * (eif + ejf + dh), eif * ejf);
+  const float ent = k.CKm1 * fm::log1p(x);
+  const float mg = 0.5f * (g2 - quad) + ldet + ent - lnU;
+  // error bound of mg against its exact value for these inputs (u = 2^-24;
+  // 3.6e-7 bounds the absolute error of the hardware logarithm on
+  // [0.5, 2], 3 ulp elsewhere)
+  const float u = 5.9604645e-8f, elog = 3.6e-7f;
+  const float V = fabsf(vx) + fabsf(vy) + fabsf(vz), Gs = fabsf(G[0]) + fabsf(G[1]) + fabsf(G[2]);
+  const float qm = fabsf(qpar) * ipar * (fabsf(cpr) * V + bzpar * Gs) +
+                   (fabsf(qx) + fabsf(qy) + fabsf(qz)) * ip * (fabsf(cqr) * V + bzperp * Gs);
+  const float T = 8.0f * g2 + 23.0f * quad + 32.0f * qm + 11.0f * fabsf(ldet) + 25.0f * fabsf(ent) +
+                  11.0f * fabsf(lnU) + 23.0f;
+  tol = 2.0f * (u * T + 2.0f * elog);
+  if (fabsf(x) >= 0.0625f) tol += 2.0f * k.CKm1 * (elog + 16.0f * u);
+  m32 = mg;
+  if (exact || !(fabsf(mg) > tol)) {  // float32 not decisive (or NaN): float64
+    MixedRatioIn r;
+    r.ex = ex; r.ey = ey; r.ez = ez; r.vx = vx; r.vy = vy; r.vz = vz;
+    r.g0 = G[0]; r.g1 = G[1]; r.g2 = G[2]; r.u = uniform();
+    r.mpar = mpar; r.mperp = mperp; r.zpar = zpar; r.zperp = zperp;
+    r.mrpar = mrpar; r.mrperp = mrperp; r.ypar = ypar; r.yperp = yperp;
+    exact_e(r.ei, r.ej);
+    r.deps = (double)dh + (double)mv.dl;
+    margin = mixed_margin_fp64(r, k.CKm1_d);
+    return margin < 0.0;  // U > exp(a)
+  }
+  return mg < 0.0f;  // decided in float32: |mg| exceeds its error bound
+}
+
+template <bool SEQ, class ExactE, class Uniform>
+__device__ __forceinline__ int fd_pair_mixed(const FDConst<float>& k, float ex, float ey, float ez, float base,
+                                             const float G[3], Uniform uniform, float lnU, float* pi, float* pj,
+                                             float eif, float ejf, ExactE exact_e, float& dh, float& dl,
+                                             double& margin, float& m32, float& tol, bool exact,
+                                             bool& negative) {
+  margin = 0.0;
+  m32 = 0.0f;
+  tol = 0.0f;
+  MixedMove mv;
+  mv.dh = mv.dl = 0.0f;
+  float emn;
+  const int ok = mixed_propose<SEQ>(k, ex, ey, ez, base, G, pi, pj, eif, ejf, exact_e, mv, emn);
+  dh = mv.dh;
+  dl = mv.dl;
+  if (ok == 2) return 0;
   if (exact) margin = (double)emn;  // (float64 work only where it is asked for)
   int decision = 0;
   if (k.scheme == SDPD_SCHEME_SSA) {
-    if (!(emn > 0.0f)) negative = true;
-  } else if (!(emn > 0.0f)) {
+    if (!ok) negative = true;
+  } else if (!ok) {
     decision = 1;
   } else if (k.scheme == SDPD_SCHEME_EMS) {
-    // reverse move from v' with the coefficients at the proposed energies
-    float mrpar, mrperp, ypar, yperp;
-    pair_coeffs(k, kpar, kperp, eif + dhf, ejf + dhf, mrpar, mrperp, ypar, yperp);
-    // 1 - alpha' alpha = -(m + m' + m m') (both m <= 0: no cancellation), alpha' zt
-    const float cpr = -(mpar + mrpar + mpar * mrpar), cqr = -(mperp + mrperp + mperp * mrperp);
-    const float bzpar = fmaf(mrpar, zpar, zpar), bzperp = fmaf(mrperp, zperp, zperp);
-    const float ryy = fm::div(1.0f, ypar * yperp);
-    const float ipar = yperp * ryy, ip = ypar * ryy;  // 1 / zt'_par, 1 / zt'_perp
-    // reverse noise B'^-1 (v - A' v') = B'^-1 [(I - A' A) v - A' B G] per
-    // direction: no cancellation when zt' -> 0 (pairs near the cut-off)
-    const float qpar = (cpr * vpar - bzpar * gpar) * ipar;
-    const float qx = (cqr * (vx - vpar * ex) - bzperp * (G[0] - gpar * ex)) * ip;
-    const float qy = (cqr * (vy - vpar * ey) - bzperp * (G[1] - gpar * ey)) * ip;
-    const float qz = (cqr * (vz - vpar * ez) - bzperp * (G[2] - gpar * ez)) * ip;
-    const float quad = qpar * qpar + qx * qx + qy * qy + qz * qz;
-    const float g2 = G[0] * G[0] + G[1] * G[1] + G[2] * G[2];
-    // log|B(v)| - log|B(v')| with |B| = zt_par zt_perp^2
-    const float ldet = fm::log(zpar * zperp * zperp * (ipar * ip * ip));
-    // (S(eps') - S(eps))/kB - (log T(eps') - log T(eps)) over both particles
-    const float x = fm::div(dh * (eif + ejf + dh), eif * ejf);
-    const float ent = k.CKm1 * fm::log1p(x);
-    const float mg = 0.5f * (g2 - quad) + ldet + ent - lnU;
-    // error bound of mg against its exact value for these inputs (u = 2^-24;
-    // 3.6e-7 bounds the absolute error of the hardware logarithm on
-    // [0.5, 2], 3 ulp elsewhere)
-    const float u = 5.9604645e-8f, elog = 3.6e-7f;
-    const float V = fabsf(vx) + fabsf(vy) + fabsf(vz), Gs = fabsf(G[0]) + fabsf(G[1]) + fabsf(G[2]);
-    const float qm = fabsf(qpar) * ipar * (fabsf(cpr) * V + bzpar * Gs) +
-                     (fabsf(qx) + fabsf(qy) + fabsf(qz)) * ip * (fabsf(cqr) * V + bzperp * Gs);
-    const float T = 8.0f * g2 + 23.0f * quad + 32.0f * qm + 11.0f * fabsf(ldet) + 25.0f * fabsf(ent) +
-                    11.0f * fabsf(lnU) + 23.0f;
-    tol = 2.0f * (u * T + 2.0f * elog);
-    if (fabsf(x) >= 0.0625f) tol += 2.0f * k.CKm1 * (elog + 16.0f * u);
-    m32 = mg;
-    if (exact || !(fabsf(mg) > tol)) {  // float32 not decisive (or NaN): float64
-      MixedRatioIn r;
-      r.ex = ex; r.ey = ey; r.ez = ez; r.vx = vx; r.vy = vy; r.vz = vz;
-      r.g0 = G[0]; r.g1 = G[1]; r.g2 = G[2]; r.u = uniform();
-      r.mpar = mpar; r.mperp = mperp; r.zpar = zpar; r.zperp = zperp;
-      r.mrpar = mrpar; r.mrperp = mrperp; r.ypar = ypar; r.yperp = yperp;
-      exact_e(r.ei, r.ej);
-      r.deps = (double)dh + (double)dl;
-      margin = mixed_margin_fp64(r, k.CKm1_d);
-      if (margin < 0.0) decision = 2;  // U > exp(a)
-    } else if (mg < 0.0f) {  // decided in float32: |mg| exceeds its error bound
+    if (mixed_rejects<SEQ>(k, ex, ey, ez, base, G, uniform, lnU, eif, ejf, exact_e, mv, margin, m32, tol, exact))
       decision = 2;
-    }
   }
   if (decision == 0) {
-    pi[0] = nn[0]; pi[1] = nn[1]; pi[2] = nn[2];
-    pj[0] = nn[3]; pj[1] = nn[4]; pj[2] = nn[5];
+    pi[0] = mv.nn[0]; pi[1] = mv.nn[1]; pi[2] = mv.nn[2];
+    pj[0] = mv.nn[3]; pj[1] = mv.nn[4]; pj[2] = mv.nn[5];
   }
   return decision;
 }
@@ -1040,13 +1089,30 @@ __device__ __noinline__ void fd_large_block(const FdRun<P>& f, int64_t o, uint64
     sm.e[q] = a.eps[g];
   }
   __syncwarp();
+  // each lane's pair of a round (at most 32 pairs), loaded one round ahead
   const uint8_t* rs = f.rsize + o * kRoundStride;
   unsigned long long at = f.sched_off[o];
+  uint32_t nxt_pr = 0;
+  F4 nxt_ge{}, nxt_rn{};
+  int n = nr > 0 ? (int)rs[0] : 0;
+  auto fetch = [&]() {
+    if (lane < n) {
+      nxt_pr = __ldg(&f.pairs[at + lane]);
+      nxt_ge = ld4(&f.geom[at + lane]);
+      nxt_rn = ld4(&f.rnd[at + lane]);
+    }
+  };
+  fetch();
+  int n1 = nr > 1 ? (int)rs[1] : 0;  // size of the round after
   for (int r = 0; r < nr; ++r) {
-    const int n = rs[r];
-    for (int t = lane; t < n; t += 32) {
-      const uint32_t pr = __ldg(&f.pairs[at + t]);
-      const F4 ge = ld4(&f.geom[at + t]), rn = ld4(&f.rnd[at + t]);
+    const bool act = lane < n;
+    const uint32_t pr = nxt_pr;
+    const F4 ge = nxt_ge, rn = nxt_rn;
+    at += n;
+    n = n1;
+    n1 = r + 2 < nr ? (int)rs[r + 2] : 0;
+    fetch();
+    if (act) {
       const int ia = pr & 0xffffu, ib = pr >> 16;
       float pa[3], pb[3], pa0[3], pb0[3];
 #pragma unroll
@@ -1098,7 +1164,6 @@ __device__ __noinline__ void fd_large_block(const FdRun<P>& f, int64_t o, uint64
         }
       }
     }
-    at += n;
     __syncwarp();
   }
   const S pi_coef = std::is_same<S, float>::value ? (S)c.f_pi_coef : (S)c.pi_coef;
@@ -1114,42 +1179,15 @@ __device__ __noinline__ void fd_large_block(const FdRun<P>& f, int64_t o, uint64
   __syncwarp();
 }
 
-template <class P, int OPW, bool REC>
-__global__ void __launch_bounds__(128, 4) k_fd_colour(const __grid_constant__ FdRun<P> f) {
-  constexpr int GL = 32 / OPW;
-  extern __shared__ __align__(32) unsigned char fd_smem_raw[];
-  const uint64_t sweep = *f.sweep_ptr;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, grp = lane / GL;
+// The end of a colour launch, by all warps: large blocks, blocks beyond
+// capacity, the queue's reset and the counters.
+template <class P, bool REC>
+__device__ __forceinline__ void fd_finish(const FdRun<P>& f, uint64_t sweep, unsigned char* fd_smem_raw,
+                                          FdTally& tally) {
   const Consts& c = f.c;
-  const int colour = f.colour;
-  const int hx = c.nc[0] >> 1, hy = c.nc[1] >> 1, hz = c.nc[2] >> 1;
-  const int64_t nown = (int64_t)hx * hy * hz;
-  FdSmem& sm = reinterpret_cast<FdSmem*>(fd_smem_raw)[warp * OPW + grp];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, colour = f.colour;
+  const int64_t nown = (int64_t)(c.nc[0] >> 1) * (c.nc[1] >> 1) * (c.nc[2] >> 1);
   unsigned* queue = f.queue;
-  FdTally tally;
-  // The grid holds as many thread blocks as fit on the GPU at once; each
-  // warp takes the colour's blocks OPW at a time from queue[0] until they
-  // run out, so no partial last wave of thread blocks idles the GPU and
-  // blocks of uneven depth balance out.  The blocks come in the order of
-  // `order` (deepest first), so the blocks a warp runs in lockstep have
-  // similar depth.  queue[1] counts the warps that are done; the last one
-  // sets them back to zero for the next launch (queue[2], queue[3]: the next
-  // entries of the colour's lists of blocks beyond capacity and of large blocks).
-  for (;;) {
-    unsigned w0 = 0;
-    if (lane == 0) w0 = atomicAdd(queue, (unsigned)OPW);
-    w0 = __shfl_sync(0xffffffffu, w0, 0);
-    if ((int64_t)w0 >= nown) break;
-    const int64_t wi = (int64_t)w0 + grp;
-    const int64_t w = wi < nown ? (int64_t)f.order[colour * nown + wi] : 0;
-    const int ox = 2 * (int)(w % hx) + (colour & 1), oy = 2 * (int)((w / hx) % hy) + ((colour >> 1) & 1),
-              oz = 2 * (int)(w / ((int64_t)hx * hy)) + ((colour >> 2) & 1);
-    const int64_t o = ox + (int64_t)c.nc[0] * (oy + (int64_t)c.nc[1] * oz);
-    const uint32_t hd = f.hdr[o];
-    // (large blocks and those beyond capacity, which have the flag's bit set too, come below)
-    const bool live = wi < nown && !(hd & kHdrLargeFlag);
-    fd_run_block<P, GL, REC>(f, live, o, ox, oy, oz, hd, sweep, sm.s, sm.ec, sm.cells, tally);
-  }
   // large blocks: one warp of the thread block, on all of its shared memory
   if (f.large_count[colour] > 0) {
     __syncthreads();
@@ -1203,7 +1241,7 @@ __global__ void __launch_bounds__(128, 4) k_fd_colour(const __grid_constant__ Fd
   }
   const unsigned any_neg = __any_sync(0xffffffffu, tally.negative), any_bad = __any_sync(0xffffffffu, tally.bad);
   if (lane == 0) {
-    if (c_tot) {
+    if (c_tot | c_rb | c_rm) {  // (accepted = pairs - rejected, added with wrap-around)
       atomicAdd(&f.counters[0], c_tot);
       atomicAdd(&f.counters[1], c_tot - c_rb - c_rm);
       atomicAdd(&f.counters[2], c_rb);
@@ -1212,6 +1250,288 @@ __global__ void __launch_bounds__(128, 4) k_fd_colour(const __grid_constant__ Fd
     if (any_neg) atomicOr(f.status, kStNegative);
     if (any_bad) atomicOr(f.status, kStNaN);
   }
+}
+
+template <class P, int OPW, bool REC>
+__global__ void __launch_bounds__(128, 4) k_fd_colour(const __grid_constant__ FdRun<P> f) {
+  constexpr int GL = 32 / OPW;
+  extern __shared__ __align__(32) unsigned char fd_smem_raw[];
+  const uint64_t sweep = *f.sweep_ptr;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, grp = lane / GL;
+  const Consts& c = f.c;
+  const int colour = f.colour;
+  const int hx = c.nc[0] >> 1, hy = c.nc[1] >> 1, hz = c.nc[2] >> 1;
+  const int64_t nown = (int64_t)hx * hy * hz;
+  FdSmem& sm = reinterpret_cast<FdSmem*>(fd_smem_raw)[warp * OPW + grp];
+  unsigned* queue = f.queue;
+  FdTally tally;
+  // The grid holds as many thread blocks as fit on the GPU at once; each
+  // warp takes the colour's blocks OPW at a time from queue[0] until they
+  // run out, so no partial last wave of thread blocks idles the GPU and
+  // blocks of uneven depth balance out.  The blocks come in the order of
+  // `order` (deepest first), so the blocks a warp runs in lockstep have
+  // similar depth.  queue[1] counts the warps that are done; the last one
+  // sets them back to zero for the next launch (queue[2], queue[3]: the next
+  // entries of the colour's lists of blocks beyond capacity and of large blocks).
+  for (;;) {
+    unsigned w0 = 0;
+    if (lane == 0) w0 = atomicAdd(queue, (unsigned)OPW);
+    w0 = __shfl_sync(0xffffffffu, w0, 0);
+    if ((int64_t)w0 >= nown) break;
+    const int64_t wi = (int64_t)w0 + grp;
+    const int64_t w = wi < nown ? (int64_t)f.order[colour * nown + wi] : 0;
+    const int ox = 2 * (int)(w % hx) + (colour & 1), oy = 2 * (int)((w / hx) % hy) + ((colour >> 1) & 1),
+              oz = 2 * (int)(w / ((int64_t)hx * hy)) + ((colour >> 2) & 1);
+    const int64_t o = ox + (int64_t)c.nc[0] * (oy + (int64_t)c.nc[1] * oz);
+    const uint32_t hd = f.hdr[o];
+    // (large blocks and those beyond capacity, which have the flag's bit set too, come below)
+    const bool live = wi < nown && !(hd & kHdrLargeFlag);
+    fd_run_block<P, GL, REC>(f, live, o, ox, oy, oz, hd, sweep, sm.s, sm.ec, sm.cells, tally);
+  }
+  fd_finish<P, REC>(f, sweep, fd_smem_raw, tally);
+}
+
+// ---------------------------------------------------------------------------
+// EMS with one block per team of two warps, for launches with few blocks,
+// where a colour lasts as long as its deepest block.  A round on one warp is a
+// chain of about 560 instructions that issue at a third of the rate; here the
+// first warp proposes round r and moves it at once, and the second tests it
+// while the first is at round r + 1.  When it rejects a move (1e-4 to 3e-2 of
+// the pairs) the first takes round r + 1 back, then the rejected moves, and
+// proposes round r + 1 again, so the result is that of the sequential sweep,
+// bit for bit that of k_fd_colour.  64,000 particles (512 blocks per colour):
+// 63 us per launch, with one warp per block 70.
+// ---------------------------------------------------------------------------
+struct FdSpecSmem {
+  FdSmem b;
+  float mv[2][14][32];   // moves of two rounds: v, m, z, dh, dl, dhf, the energies and compensations before
+  uint8_t ok[2][32];     // mixed_propose's answer
+  uint8_t rsize[kRoundStride];
+  unsigned rejected[2];  // lanes of the round tested in a step, by the step's parity
+  unsigned next;
+};
+
+template <class P, bool REC>
+__global__ void __launch_bounds__(64) k_fd_colour_spec(const __grid_constant__ FdRun<P> f) {
+  using S = typename P::R;
+  constexpr bool kSame = std::is_same<S, float>::value;
+  extern __shared__ __align__(32) unsigned char fd_smem_raw[];
+  FdSpecSmem& sm = *reinterpret_cast<FdSpecSmem*>(fd_smem_raw);
+  const uint64_t sweep = *f.sweep_ptr;
+  const int t = threadIdx.x, lane = t & 31;
+  const bool tester = t >= 32;
+  const Consts& c = f.c;
+  const Arrays<P>& a = f.a;
+  const int colour = f.colour;
+  const int hx = c.nc[0] >> 1, hy = c.nc[1] >> 1, hz = c.nc[2] >> 1;
+  const int64_t nown = (int64_t)hx * hy * hz;
+  const S pi_coef = kSame ? (S)c.f_pi_coef : (S)c.pi_coef;
+  unsigned* queue = f.queue;
+  FdTally tally;
+  F4* s = sm.b.s;
+  float* ec = sm.b.ec;
+  FdCells& cells = sm.b.cells;
+  for (;;) {  // blocks from the colour's queue, deepest first (see k_fd_colour)
+    if (t == 0) sm.next = atomicAdd(queue, 1u);
+    __syncthreads();
+    const unsigned wi = sm.next;
+    if ((int64_t)wi >= nown) break;
+    const int64_t w = f.order[colour * nown + wi];
+    const int ox = 2 * (int)(w % hx) + (colour & 1), oy = 2 * (int)((w / hx) % hy) + ((colour >> 1) & 1),
+              oz = 2 * (int)(w / ((int64_t)hx * hy)) + ((colour >> 2) & 1);
+    const int64_t o = ox + (int64_t)c.nc[0] * (oy + (int64_t)c.nc[1] * oz);
+    const uint32_t hd = f.hdr[o];
+    const int np = hd & kHdrLargeFlag ? 0 : (int)(hd & 0xffffu), nr = (int)(hd >> 16 & 255u);
+    if (np == 0) {  // (large blocks and those beyond capacity come below)
+      __syncthreads();
+      continue;
+    }
+    if (t == 0) tally.n_tot += (unsigned)np;
+    const unsigned long long first = f.sched_off[o];
+    for (int r = t; r < nr; r += 64) sm.rsize[r] = f.rsize[o * kRoundStride + r];
+    BlockCells b;
+    block_cells(c, ox, oy, oz, f.mrank, f.cell_start, b);
+    const int nb = b.base[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+      if (t == q) {
+        cells.cst[q] = b.start[q];
+        cells.cbs[q] = b.base[q];
+      }
+    __syncthreads();
+    for (int q = t; q < nb; q += 64) {
+      const int g = block_gidx(cells, q);
+      s[q] = F4{(float)a.px[g], (float)a.py[g], (float)a.pz[g], (float)a.eps[g]};
+      ec[q] = 0.0f;
+    }
+    // this lane's pair of a round, loaded one round ahead; the tester meets
+    // round r one step after the proposer
+    uint32_t pr = 0;
+    F4 ge{}, rn{};
+    int pos = 0, n = sm.rsize[0];
+    auto fetch = [&]() {
+      if (lane < n) {
+        pr = __ldg(&f.pairs[first + pos + lane]);
+        ge = ld4(&f.geom[first + pos + lane]);
+        rn = ld4(&f.rnd[first + pos + lane]);
+      }
+    };
+    fetch();
+    __syncthreads();
+    // the proposer's pairs of this round and the one before, with the records
+    // before their moves
+    int ia = 0, ib = 0, last_a = 0, last_b = 0;
+    F4 sa{}, sb{}, last_sa{}, last_sb{};
+    float ca = 0.0f, cb = 0.0f, last_ca = 0.0f, last_cb = 0.0f;
+    for (int st = 0; st <= nr; ++st) {
+      const int r = tester ? st - 1 : st;
+      const bool on = r >= 0 && r < nr;
+      const int buf = r & 1;
+      const bool act = on && lane < n;
+      const uint32_t cpr = pr;
+      const F4 cg = ge, cr = rn;
+      if (on) {
+        pos += n;
+        n = r + 1 < nr ? (int)sm.rsize[r + 1] : 0;
+        fetch();
+      }
+      const float G[3] = {cr.x, cr.y, cr.z};
+      ia = cpr & 0xffffu;
+      ib = cpr >> 16;
+      bool moved = false;
+      auto propose = [&]() {
+        sa = lds4(&s[ia]);
+        sb = lds4(&s[ib]);
+        ca = ec[ia];
+        cb = ec[ib];
+        const float pa[3] = {sa.x, sa.y, sa.z}, pb[3] = {sb.x, sb.y, sb.z};
+        auto exact_e = [&](double& x, double& y) { fd_exact_energies(a.eps, cells, ec, ia, ib, sa.w, sb.w, x, y); };
+        MixedMove mv;
+        mv.dh = mv.dl = 0.0f;
+        float emn;
+        const int ok = mixed_propose<false>(f.k, cg.x, cg.y, cg.z, cg.w, G, pa, pb, sa.w, sb.w, exact_e, mv, emn);
+        moved = ok == 1;
+        if (moved) {
+          float v, e;
+          eft::two_sum(sa.w, mv.dh, v, e);
+          ec[ia] = __fadd_rn(ca, __fadd_rn(e, mv.dl));
+          s[ia] = F4{mv.nn[0], mv.nn[1], mv.nn[2], v};
+          eft::two_sum(sb.w, mv.dh, v, e);
+          ec[ib] = __fadd_rn(cb, __fadd_rn(e, mv.dl));
+          s[ib] = F4{mv.nn[3], mv.nn[4], mv.nn[5], v};
+          const float out[14] = {mv.vx, mv.vy, mv.vz, mv.mpar, mv.mperp, mv.zpar, mv.zperp, mv.dh, mv.dl, mv.dhf,
+                                 sa.w, sb.w, ca, cb};
+#pragma unroll
+          for (int q = 0; q < 14; ++q) sm.mv[buf][q][lane] = out[q];
+        }
+        sm.ok[buf][lane] = (uint8_t)ok;
+        if (REC) sm.mv[buf][7][lane] = moved ? mv.dh : emn;
+      };
+      if (!tester) {
+        if (act) propose();
+      } else {
+        int dcs = 0;
+        if (act) {
+          const int ok = sm.ok[buf][lane];
+          double margin = 0.0;
+          float m32 = 0.0f, tol = 0.0f;
+          if (ok == 1) {
+            MixedMove mv;
+            const float* in = &sm.mv[buf][0][lane];
+            mv.vx = in[0]; mv.vy = in[32]; mv.vz = in[64];
+            mv.mpar = in[96]; mv.mperp = in[128]; mv.zpar = in[160]; mv.zperp = in[192];
+            mv.dh = in[224]; mv.dl = in[256]; mv.dhf = in[288];
+            const float eaf = in[320], ebf = in[352], eca = in[384], ecb = in[416];
+            auto exact_e = [&](double& x, double& y) {  // the energies before the move
+              const double ga = a.eps[block_gidx(cells, ia)], gb = a.eps[block_gidx(cells, ib)];
+              x = ga + (((double)eaf - (double)(float)ga) + (double)eca);
+              y = gb + (((double)ebf - (double)(float)gb) + (double)ecb);
+            };
+            auto uniform = [&]() {
+              return fd_uniform_again(f.seed, sweep, a.id[block_gidx(cells, ia)], a.id[block_gidx(cells, ib)]);
+            };
+            if (mixed_rejects<false>(f.k, cg.x, cg.y, cg.z, cg.w, G, uniform, cr.w, eaf, ebf, exact_e, mv, margin, m32,
+                                     tol, REC))
+              dcs = 2;
+          } else if (ok == 0) {
+            dcs = 1;
+            if (REC) margin = (double)sm.mv[buf][7][lane];
+          }
+          tally.n_rb += dcs == 1;
+          tally.n_rm += dcs == 2;
+          if constexpr (REC) {
+            const unsigned long long at = atomicAdd(f.rec_count, 1ull);
+            if ((int64_t)at < f.rec_cap) {
+              sdpd_pair_rec rc;
+              rc.id_i = a.id[block_gidx(cells, ia)];
+              rc.id_j = a.id[block_gidx(cells, ib)];
+              rc.colour = colour;
+              rc.owner = (int32_t)o;
+              rc.decision = dcs;
+              rc.level = r;
+              rc.margin = margin;
+              rc.margin_lo = (double)m32;
+              rc.margin_tol = (double)tol;
+              f.recs[at] = rc;
+            }
+          }
+        }
+        const unsigned rej = __ballot_sync(0xffffffffu, dcs == 2);
+        if (lane == 0) sm.rejected[st & 1] = rej;
+      }
+      __syncthreads();
+      const unsigned rej = sm.rejected[st & 1];
+      if (rej) {  // (uniform: both warps)
+        if (!tester) {
+          if (moved) {  // this round back,
+            s[ia] = sa;
+            s[ib] = sb;
+            ec[ia] = ca;
+            ec[ib] = cb;
+          }
+          __syncwarp();
+          if (rej >> lane & 1u) {  // the rejected moves of the round before,
+            s[last_a] = last_sa;
+            s[last_b] = last_sb;
+            ec[last_a] = last_ca;
+            ec[last_b] = last_cb;
+          }
+          __syncwarp();
+          if (act) propose();  // this round once more
+        }
+        __syncthreads();
+      }
+      if (!tester) {
+        __syncwarp();
+        last_a = ia;
+        last_b = ib;
+        last_sa = sa;
+        last_sb = sb;
+        last_ca = ca;
+        last_cb = cb;
+      }
+    }
+    __syncthreads();
+    for (int q = t; q < nb; q += 64) {
+      const int g = block_gidx(cells, q);
+      const F4 v = lds4(&s[q]);
+      if constexpr (kSame) {
+        a.px[g] = v.x; a.py[g] = v.y; a.pz[g] = v.z;
+      } else {  // the stored value plus this visit's increment
+        a.px[g] += (S)(v.x - (float)a.px[g]);
+        a.py[g] += (S)(v.y - (float)a.py[g]);
+        a.pz[g] += (S)(v.z - (float)a.pz[g]);
+      }
+      // once per visit: the load value plus the visit's exact change
+      const double e0 = a.eps[g];
+      const double e = e0 + (((double)v.w - (double)(float)e0) + (double)ec[q]);
+      tally.bad |= !isfinite(v.w);
+      a.eps[g] = e;
+      f.qp4[g].w = (S)e * pi_coef / a.rho[g];  // as in fd_run_block
+    }
+    __syncthreads();  // the team's shared memory is refilled by the next block
+  }
+  fd_finish<P, REC>(f, sweep, fd_smem_raw, tally);
 }
 
 template <class R>
@@ -1238,7 +1558,8 @@ static FDConst<R> fd_const(const Consts& c, double dt) {
 }
 
 // Block schedules of the colour launches: blocks per warp and warps per
-// thread block of each variant (see sdpd_tuning).  The mapping onto the GPU
+// thread block of each variant (see sdpd_tuning); EMS with one block per warp
+// runs k_fd_colour_spec, a two-warp team per block.  The mapping onto the GPU
 // differs, the pair updates and their order per particle do not.
 constexpr int kFdOpw[kFdVariants] = {2, 2, 1, 1, 1};
 constexpr int kFdWarps[kFdVariants] = {2, 1, 1, 2, 4};
@@ -1273,6 +1594,20 @@ int fd_resident(int variant) {
     case 3: return fd_resident_blocks<P, REC, 3>();
     default: return fd_resident_blocks<P, REC, 4>();
   }
+}
+
+template <class P>
+constexpr size_t fd_spec_bytes() { return std::max(sizeof(FdSpecSmem), sizeof(FdLargeSmem<P>)); }
+template <class P, bool REC>
+int fd_spec_resident() {
+  static const int n = [] {
+    int dev = 0, sms = 0, per_sm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fd_colour_spec<P, REC>, 64, fd_spec_bytes<P>());
+    return std::max(1, sms) * std::max(1, per_sm);
+  }();
+  return n;
 }
 
 // The eight colour launches of one sweep with float32 pair arithmetic.  Few
@@ -1313,10 +1648,15 @@ void launch_colours32(const Consts& c, const Workspace& w, int cur, double dt, u
   f.large_list = w.large_list;
   f.large_count = w.large_count;
   auto kern = opw == 2 ? k_fd_colour<P, 2, REC> : k_fd_colour<P, 1, REC>;
+  // a team per block where a warp per block would run it (EMS: only there has
+  // the test its own work)
+  const bool spec = opw == 1 && c.scheme == SDPD_SCHEME_EMS;
+  const unsigned gs = (unsigned)std::max<int64_t>(1, std::min<int64_t>(nown, fd_spec_resident<P, REC>()));
   for (int col = 0; col < 8; ++col) {
     f.colour = col;
     f.queue = w.fd_queue + 4 * col;
-    kern<<<gf, W * 32, fd_smem_bytes<P>(variant), s>>>(f);
+    if (spec) k_fd_colour_spec<P, REC><<<gs, 64, fd_spec_bytes<P>(), s>>>(f);
+    else kern<<<gf, W * 32, fd_smem_bytes<P>(variant), s>>>(f);
   }
 }
 
@@ -1330,6 +1670,8 @@ void fd_prepare() {
   if constexpr (!A::mixed) {
     team64_prepare();
   } else {
+    fd_spec_resident<P, false>();
+    fd_spec_resident<P, true>();
     for (int v = 0; v < kFdVariants; ++v) {
       fd_resident<P, false>(v);
       fd_resident<P, true>(v);

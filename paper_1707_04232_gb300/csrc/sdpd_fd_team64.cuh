@@ -126,7 +126,7 @@ struct Team64Smem {
   double m[2][kTeamThreads], z[2][kTeamThreads], U[2][kTeamThreads], r0[2][kTeamPairs];
   double deps[2][kTeamPairs], ei[2][kTeamPairs], ej[2][kTeamPairs];
   uint8_t bound[2][kTeamPairs];
-  unsigned rejected[2];  // quads (their lanes' bits) of the last tested round, per warp
+  unsigned rejected[2][2];  // quads (their lanes' bits) of the round tested in a step, by its parity and per warp
   unsigned next;
 };
 
@@ -276,7 +276,7 @@ __global__ void __launch_bounds__(team_threads<EMS>())
           }
         }
         const unsigned rej = __ballot_sync(0xffffffffu, dcs == 2);
-        if (lane == 0) sm.rejected[warp & 1] = rej;
+        if (lane == 0) sm.rejected[st & 1][warp & 1] = rej;
       }
       if ((tester || !EMS) && act && l == 0) {
         n_rb += dcs == 1;
@@ -300,7 +300,7 @@ __global__ void __launch_bounds__(team_threads<EMS>())
       }
       __syncthreads();
       if constexpr (EMS) {
-        if (sm.rejected[0] | sm.rejected[1]) {
+        if (sm.rejected[st & 1][0] | sm.rejected[st & 1][1]) {
           // a move of the round before was rejected: this round's moves back,
           // then the rejected ones, then this round once more
           if (!tester && moved) {
@@ -308,12 +308,11 @@ __global__ void __launch_bounds__(team_threads<EMS>())
             rec[4 * ib + l] = B;
           }
           __syncthreads();
-          if (!tester && (sm.rejected[warp] >> lane & 1u)) {
+          if (!tester && (sm.rejected[st & 1][warp & 1] >> lane & 1u)) {
             rec[4 * (last_pr & 0xffffu) + l] = lastA;
             rec[4 * (last_pr >> 16) + l] = lastB;
           }
           __syncthreads();
-          if (t < 2) sm.rejected[t] = 0u;
           if (!tester && busy) propose();
           __syncthreads();
         }

@@ -79,10 +79,12 @@ __host__ __device__ constexpr int fd_default_variant(bool mixed) { return mixed 
 // The block schedule of a handle's colour launches with float32 pair
 // arithmetic (float64 has one, k_fd_colour64): the one set by the caller or
 // the autotuner, else by the blocks per colour.  Few blocks: a colour lasts as
-// long as its deepest block, which runs fastest on a warp of its own; from
-// about six blocks per SM on two per warp use its lanes better.  Microseconds
-// per sweep with schedules 0 / 1 / 2: 512 blocks 613 / 636 / 594, 1331 blocks
-// 791 / 756 / 785, 4096 blocks 1091 / 1069 / 1457, 6859 blocks 1711 / 1734 / 2340.
+// long as its deepest block, which runs fastest on warps of its own (EMS: two,
+// k_fd_colour_spec); from about six blocks per SM on two blocks per warp use
+// its lanes better.  Microseconds per sweep (EMS, with the random numbers) with
+// schedules 0 / 1 / 2: 216 blocks 621 / 646 / 484, 512 blocks 633 / 653 / 540,
+// 729 blocks 723 / 747 / 645, 1000 blocks 772 / 754 / 867, 1331 blocks 805 /
+// 777 / 962, 2744 blocks 1041 / 966 / 1645; 6859 blocks 1711 / 1734 / 2340.
 inline int fd_launch_variant(const Consts& c) {
   if (!c.fd_auto && c.fd_variant >= 0 && c.fd_variant < kFdVariants) return c.fd_variant;
   const int64_t nown = (int64_t)(c.nc[0] / 2) * (c.nc[1] / 2) * (c.nc[2] / 2);

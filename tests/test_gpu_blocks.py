@@ -60,3 +60,23 @@ def test_block_sizes_match_oracle(kind):
         assert m.observables()["n_pairs"] == 2 * stats.n_pairs
         ref = ref or x
         assert all(np.array_equal(u, w) for u, w in zip(x, ref))
+
+
+@pytest.mark.parametrize("precision,K,dt", [(sdpd.MIXED, 50.0, 0.05), (sdpd.MIXED, 5.0, 0.45), (sdpd.FP64, 5.0, 0.22)])
+def test_tested_one_round_late_is_the_sequential_sweep(precision, K, dt):
+    """One block per team (moves made before their test, taken back when it
+    rejects them) against two blocks per warp (each round tested before the
+    next), float32 pair arithmetic: the same counts and, bit for bit, the same
+    state, with moves rejected on the way."""
+    w = Workload(n=16, K=K, jitter=0.2, seed=4)
+    out = []
+    for v in (1, 2):
+        s = sdpd.SDPD(w.N, w.L, h=w.h, K=K, precision=precision, fd_only=True, **(
+            {"sweep_f32": True} if precision == sdpd.FP64 else {}))
+        s.set_tuning(v, 128)
+        s.set_state(*lattice_state(w))
+        s.step(dt, 3, seed=13)
+        o = s.observables()
+        out.append((s.get_state(), [o[k] for k in ("n_pairs", "n_accept", "n_reject_bound", "n_reject_metropolis")]))
+    assert out[0][1] == out[1][1] and out[0][1][3] > 0
+    assert all(np.array_equal(a, b) for a, b in zip(out[0][0], out[1][0]))
