@@ -314,15 +314,14 @@ typedef struct {
                        launches: 0 (2 x 2), 1 (2 x 1), 2 (1 x 1), 3 (1 x 2),
                        4 (1 x 4); with 2 to 4 the Metropolised scheme runs
                        a team of two warps per block instead.  -1 = chosen at
-                       launch by the blocks per
-                       colour (2 up to 912 of them, 1 up to 4864, else 0;
-                       sdpd_get_tuning then reports 0 for float32 and 1 for
-                       float64 pair arithmetic); a new handle starts with -1.
-                       Float64 pair arithmetic has one schedule, a team of
-                       warps per block, whatever the value */
+                       launch by the blocks per colour (2 up to 912 of them,
+                       1 up to 4864, else 0; sdpd_get_tuning then reports 0
+                       for float32 and 1 for float64 pair arithmetic); a new
+                       handle starts with -1.
+                       Float64 pair arithmetic takes 1, 2 and 3 and has one
+                       schedule, a team of warps per block */
   int pair_threads; /* threads per block of the density and force passes:
-                       32, 64 or 128; 0 = 128 (and, float64 with at most 2432
-                       particles, a warp per particle instead of 8 lanes) */
+                       32, 64 or 128; 0 = 128 */
 } sdpd_tuning;
 
 /* Current launch shapes.  Errors: SDPD_ERR_INVALID_ARG. */

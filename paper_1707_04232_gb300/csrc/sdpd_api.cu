@@ -527,7 +527,7 @@ int sdpd_create(int64_t N, const double box[3], double m, double h, const sdpd_p
   c.kernel = prm->kernel;
   c.fd_variant = fd_default_variant(prm->precision == SDPD_MIXED || prm->sweep_f32 != 0);
   c.pair_threads = 128;
-  c.fd_auto = c.pair_auto = true;
+  c.fd_auto = true;
   c.scheme = prm->scheme;
   s->prm = *prm;
   s->K = K;
@@ -847,7 +847,6 @@ int sdpd_set_tuning(sdpd_t* s, const sdpd_tuning* t) {
     return SDPD_ERR_INVALID_ARG;
   s->c.fd_variant = v;
   s->c.fd_auto = t->fd_variant < 0;
-  s->c.pair_auto = t->pair_threads == 0;
   s->c.pair_threads = pt;
   return SDPD_OK;
 }
@@ -872,7 +871,7 @@ int sdpd_autotune(sdpd_t* s, double dt, int64_t steps, uint64_t seed, sdpd_tunin
   // time per step of one candidate; infinity when it failed
   auto trial = [&](int v, int pt) -> double {
     s->c.fd_variant = v;
-    s->c.fd_auto = s->c.pair_auto = false;
+    s->c.fd_auto = false;
     s->c.pair_threads = pt;
     reload_handle(s, sv);
     if (mixed) do_steps<Mixed>(s, dt, 1, seed);
@@ -890,7 +889,7 @@ int sdpd_autotune(sdpd_t* s, double dt, int64_t steps, uint64_t seed, sdpd_tunin
     return (double)ms / (double)steps;
   };
   const int v0 = s->c.fd_variant, t0 = s->c.pair_threads;
-  const bool fd_auto0 = s->c.fd_auto, pair_auto0 = s->c.pair_auto;
+  const bool fd_auto0 = s->c.fd_auto;
   int bv = v0, bt = 128;
   double bms = INFINITY;
   for (int v = 0; v < kFdVariants; ++v) {
@@ -907,7 +906,6 @@ int sdpd_autotune(sdpd_t* s, double dt, int64_t steps, uint64_t seed, sdpd_tunin
   if (!isfinite(bms)) { bv = v0; bt = t0; }
   s->c.fd_variant = bv;
   s->c.fd_auto = !isfinite(bms) && fd_auto0;
-  s->c.pair_auto = !isfinite(bms) && pair_auto0;
   s->c.pair_threads = bt;
   reload_handle(s, sv);  // back to the state and counters the call started from
   e = finish_restore(s, sv);
@@ -1501,7 +1499,7 @@ int sdpd_ensemble_step(sdpd_ens_t* e, double dt, int64_t nsteps, const uint64_t*
     // the graph holds the buffer pointers and launch shapes of its capture
     shape.push_back(h->cur);
     shape.push_back(h->c.fd_auto ? -1 : h->c.fd_variant);
-    shape.push_back(h->c.pair_auto ? -1 : h->c.pair_threads);
+    shape.push_back(h->c.pair_threads);
   }
   if (units > 0) {
     if (!e->exec || e->dt != dt || e->seeds != sv || e->phase != phase || e->shape != shape) {
@@ -1601,7 +1599,7 @@ int sdpd_ensemble_autotune(sdpd_ens_t* e, double dt, int64_t steps, const uint64
   for (size_t c = 0; c < cand.size() && !err; ++c) {
     for (size_t i = 0; i < n; ++i) {
       e->m[i]->c.fd_variant = cand[c][i].fd_variant;
-      e->m[i]->c.fd_auto = e->m[i]->c.pair_auto = false;
+      e->m[i]->c.fd_auto = false;
       e->m[i]->c.pair_threads = cand[c][i].pair_threads;
       reload_handle(e->m[i], sv[i]);
     }
@@ -1628,7 +1626,7 @@ int sdpd_ensemble_autotune(sdpd_ens_t* e, double dt, int64_t steps, const uint64
   // the chosen shapes, and every member back where the call found it
   for (size_t i = 0; i < n; ++i) {
     e->m[i]->c.fd_variant = cand[best][i].fd_variant;
-    e->m[i]->c.fd_auto = e->m[i]->c.pair_auto = false;
+    e->m[i]->c.fd_auto = false;
     e->m[i]->c.pair_threads = cand[best][i].pair_threads;
     reload_handle(e->m[i], sv[i]);
   }

@@ -322,6 +322,6 @@ __device__ __forceinline__ double group_sum(double v) {
 // each, which spreads them over the SM quarters and shortens every particle's
 // chain; else kLanes64, which costs fewer instructions in all.  The line lies
 // at four warps per SM quarter.
-inline bool pair64_wide(const Consts& c) { return c.pair_auto && c.N <= 16 * 152; }
+inline bool pair64_wide(const Consts& c) { return c.N <= 16 * 152; }
 
 }  // namespace sdpd

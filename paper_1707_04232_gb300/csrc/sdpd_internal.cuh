@@ -68,7 +68,6 @@ struct Consts {
   // launch shapes (results do not depend on them): the block schedule of the
   // sweep's colour launches and the threads per block of the pair passes
   int fd_variant, pair_threads;
-  bool pair_auto;  // no pair-pass block size chosen by the caller: by size (float64 path)
   bool fd_auto;  // no schedule chosen by the caller: fd_launch_variant picks by size
 };
 
@@ -91,9 +90,9 @@ inline int fd_launch_variant(const Consts& c) {
   return nown <= 6 * 152 ? 2 : (nown <= 32 * 152 ? 1 : 0);
 }
 __host__ __device__ constexpr bool pair_threads_ok(int t) { return t == 32 || t == 64 || t == 128; }
-// whether a block schedule's shared memory fits a thread block (float64
-// blocks take twice the bytes of mixed ones)
-bool fd_variant_fits(bool mixed, int v);
+// whether a handle takes a block schedule (float64 pair arithmetic: 1 to 3, all
+// of them its one team kernel)
+bool fd_variant_fits(bool float_arith, int v);
 
 // Neighbour-list entry: neighbour index << 6 | stencil offset code, the code
 // holding (o + 1) per axis in 2 bits (x lowest) for o in {-1, 0, +1}.

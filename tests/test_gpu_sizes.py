@@ -41,3 +41,23 @@ def test_sort_density_and_forces(N, side):
             if prec == sdpd.FP64:
                 assert (s.order() == O.sorted_order(P, q)).all()
                 assert (s.cells() == O.cells(P, q)).all()
+
+
+@pytest.mark.parametrize("N", [700, 2433])
+def test_float64_launch_shapes_are_bitwise_alike(N):
+    """Block sizes of the passes, set or left alone, on both sides of the line
+    of a warp per particle; float64 handles take schedules 1 to 3 only."""
+    q, p, e = random_box_state(N, 1.0, 1.0, 1.0, 30.0, seed=N)
+    out = []
+    for pt in (None, 32, 64, 128):
+        s = sdpd.SDPD(N, 13.0, h=2.5, K=20.0, precision=sdpd.FP64)
+        if pt is not None:
+            s.set_tuning(1, pt)
+            for v in (0, 4):
+                with pytest.raises(sdpd.SDPDError):
+                    s.set_tuning(v, pt)
+        s.set_state(q * 13.0, p, e)
+        s.step(0.002, 3, seed=3)
+        out.append(s.get_state())
+    for x in out[1:]:
+        assert all(np.array_equal(a, b) for a, b in zip(x, out[0]))
