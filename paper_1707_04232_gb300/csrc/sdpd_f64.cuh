@@ -56,27 +56,22 @@ __device__ __forceinline__ double rsqrt_(double x) {
 __device__ __forceinline__ bool below(double x, int hi) { return (__double2hiint(x) & 0x7fffffff) < hi; }
 constexpr int kHi2m6 = 0x3f900000, kHi2m3 = 0x3fc00000, kHi2m2 = 0x3fd00000;  // high words of 2^-6, 1/8, 1/4
 // expm1: Taylor series; below 2^-6 the terms from x^5/120 on, 2^-31 of the
-// result, in float32; below 1/4 twelve terms in float64.
+// result, in float32; below 1/4 those from x^8/40320 on, 2^-29 of it.
 __device__ __forceinline__ double expm1(double x) {
-  if (below(x, kHi2m6)) {
-    const float f = copysignf(trunc_abs(x), __int_as_float(__double2hiint(x)));
-    const float t = f * (1.0f / 120.0f + f * (1.0f / 720.0f + f * (1.0f / 5040.0f)));
-    double p = 1.0 / 24.0 + widen_signed(t);
-    p = __fma_rn(p, x, 1.0 / 6.0);
-    p = __fma_rn(p, x, 0.5);
-    return __fma_rn(__dmul_rn(p, x), x, x);
-  }
   if (below(x, kHi2m2)) {
-    double p = 1.0 / 6227020800.0;
-    p = __fma_rn(p, x, 1.0 / 479001600.0);
-    p = __fma_rn(p, x, 1.0 / 39916800.0);
-    p = __fma_rn(p, x, 1.0 / 3628800.0);
-    p = __fma_rn(p, x, 1.0 / 362880.0);
-    p = __fma_rn(p, x, 1.0 / 40320.0);
-    p = __fma_rn(p, x, 1.0 / 5040.0);
-    p = __fma_rn(p, x, 1.0 / 720.0);
-    p = __fma_rn(p, x, 1.0 / 120.0);
-    p = __fma_rn(p, x, 1.0 / 24.0);
+    const float f = copysignf(trunc_abs(x), __int_as_float(__double2hiint(x)));
+    double p;
+    if (below(x, kHi2m6)) {
+      const float t = f * (1.0f / 120.0f + f * (1.0f / 720.0f + f * (1.0f / 5040.0f)));
+      p = 1.0 / 24.0 + widen_signed(t);
+    } else {
+      const float t = f * (1.0f / 40320.0f +
+                           f * (1.0f / 362880.0f + f * (1.0f / 3628800.0f + f * (1.0f / 39916800.0f))));
+      p = 1.0 / 5040.0 + widen_signed(t);
+      p = __fma_rn(p, x, 1.0 / 720.0);
+      p = __fma_rn(p, x, 1.0 / 120.0);
+      p = __fma_rn(p, x, 1.0 / 24.0);
+    }
     p = __fma_rn(p, x, 1.0 / 6.0);
     p = __fma_rn(p, x, 0.5);
     return __fma_rn(__dmul_rn(p, x), x, x);

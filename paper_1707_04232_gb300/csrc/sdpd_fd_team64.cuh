@@ -27,28 +27,29 @@
 namespace sdpd {
 
 // Constants of the team's arithmetic, in momentum units: with u = p_i - p_j,
-// dp = (m/2)(v' - v) = (alpha - 1) u / 2 + hz G per direction, hz = m zt / 2,
-// hz^2 = kB m / C_K * (eps_i eps_j / (eps_i + eps_j)) / (1 - d) * (1 - alpha^2).
+// 2 dp = m (v' - v) = (alpha - 1) u + z G per direction, z = m zt,
+// z^2 = 4 kB m / C_K * (eps_i eps_j / (eps_i + eps_j)) / (1 - d) * (1 - alpha^2).
 struct Team64Const {
   double x_par, x_perp;  // log alpha per unit of base (1 - d): -2 kappa m^2 dt / m
   double d2;             // 2 kB / C_K
-  double s;              // kB m / C_K
-  double de;             // -1 / (2 m)
+  double s;              // 4 kB m / C_K
+  double de;             // -1 / (4 m)
   double CKm1;
   int scheme;
 };
 
-// alpha - 1 and (hz or, INV, 1 / hz) of this lane's direction at energies
-// with sum E, product P and 1/E = iE.
+// alpha - 1 and (z or, INV, 1 / z) of this lane's direction at energies with
+// sum E, product P and 1/E = iE.  With q = 1 - d and n = q z^2, z is
+// n / sqrt(n q) and 1/z is q / sqrt(n q): one reciprocal square root.
 template <bool INV>
 __device__ __forceinline__ void team_coeffs(const Team64Const& k, double x_dir, double base, double P, double iE,
                                             double& m, double& z) {
   const double a = P * iE;
-  const double omd = __fma_rn(-k.d2, a * iE, 1.0);
-  m = f64::expm1(x_dir * (base * omd));
-  const double s = k.s * a * f64::rcp(omd);
-  const double q = s * (-m * (2.0 + m));
-  z = INV ? f64::rsqrt_(q) : f64::sqrt_(q);
+  const double q = __fma_rn(-k.d2, a * iE, 1.0);
+  m = f64::expm1(x_dir * (base * q));
+  const double n = k.s * a * (-m * (2.0 + m)), nq = n * q;
+  if (f64::rsqrt_tiny(nq)) z = INV ? ::sqrt(q / n) : ::sqrt(n / q);
+  else z = f64::rsqrt_(nq) * (INV ? q : n);
 }
 
 __device__ __forceinline__ double quad_sum(double v) {
@@ -59,57 +60,64 @@ __device__ __forceinline__ double quad_sum(double v) {
 
 // What the test of a move needs from its proposal, per lane and per pair.
 struct Team64Move {
-  double m, z, U;            // this lane's alpha - 1, hz, half velocity component (momentum units)
-  double deps, ei, ej, r0;   // r0: 1/P on lane 2
-  bool bound;                // both new energies positive
+  double m, z, u;         // this lane's alpha - 1, z, velocity component (momentum units)
+  double deps, E, P, r0;  // energy change, sum and product of the energies before; r0: 1/P on lane 2
+  bool bound;             // both new energies positive
 };
 
 // The proposal of one pair on the four lanes of a quad (whole warps call it).
 // l: the lane's place in the quad; A, B: component l of the two particles'
 // records (px, py, pz, eps); ge: component l of (e, base); Gl: component l of
-// (G - (e.G) e, e.G).  dA, dB: the lane's changes of A and B.
+// (G - (e.G) e, e.G).  A1, B1: the same components after the move.  Where a
+// lane's own part leaves it idle it takes one of the pair's scalars in the
+// same instruction: lane 3 the sum and the product of the energies.
 __device__ __forceinline__ Team64Move team_propose(const Team64Const& k, int l, double A, double B, double ge,
-                                                   double Gl, double base, double& dA, double& dB) {
+                                                   double Gl, double base, double& A1, double& B1) {
   Team64Move v;
-  v.ei = __shfl_sync(0xffffffffu, A, 3, 4);
-  v.ej = __shfl_sync(0xffffffffu, B, 3, 4);
-  const double el = l == 3 ? 0.0 : ge;
-  const double u = A - B;
-  const double E = v.ei + v.ej, P = v.ei * v.ej;
+  const bool e_lane = l == 3;
+  const double el = e_lane ? 0.0 : ge;
+  const double u = A - (e_lane ? -B : B);                    // lane 3: E
+  const double t = (e_lane ? A : ge) * (e_lane ? B : u);     // lane 3: P
+  v.E = __shfl_sync(0xffffffffu, u, 3, 4);
+  v.P = __shfl_sync(0xffffffffu, t, 3, 4);
   // lane 2 takes 1/P (for the entropy term) while the others take 1/E
-  v.r0 = f64::rcp(l == 2 ? P : E);
+  v.r0 = f64::rcp(l == 2 ? v.P : v.E);
   const double iE = __shfl_sync(0xffffffffu, v.r0, 0, 4);
-  team_coeffs<false>(k, l == 3 ? k.x_par : k.x_perp, base, P, iE, v.m, v.z);
-  // u/2 split along and across e: lane 3 holds the component along it
-  const double upar = quad_sum(el * u);
-  v.U = 0.5 * (l == 3 ? upar : __fma_rn(-upar, el, u));
-  const double w = __fma_rn(v.m, v.U, v.z * Gl);
+  team_coeffs<false>(k, e_lane ? k.x_par : k.x_perp, base, v.P, iE, v.m, v.z);
+  // u split along and across e: lane 3 holds the component along it
+  const double upar = quad_sum(e_lane ? 0.0 : t);
+  const double across = __fma_rn(-upar, el, u);
+  v.u = e_lane ? upar : across;
+  const double w = __fma_rn(v.m, v.u, v.z * Gl);
   const double wpar = __shfl_sync(0xffffffffu, w, 3, 4);
-  const double dp = l == 3 ? 0.0 : __fma_rn(wpar, el, w);
+  const double sum = __fma_rn(wpar, el, w);
+  const double dp2 = e_lane ? 0.0 : sum;  // 2 dp
   // kinetic energy change of the pair: dp . (u + dp) / m
-  v.deps = k.de * quad_sum(dp * (u + dp));
-  v.bound = f64::positive(v.ei + v.deps) && f64::positive(v.ej + v.deps);
-  dA = l == 3 ? v.deps : dp;
-  dB = l == 3 ? v.deps : -dp;
+  v.deps = k.de * quad_sum(dp2 * __fma_rn(0.5, dp2, u));
+  const double d = e_lane ? v.deps : dp2;
+  A1 = __fma_rn(e_lane ? 1.0 : 0.5, d, A);
+  B1 = __fma_rn(e_lane ? 1.0 : -0.5, d, B);
+  v.bound = __shfl_sync(0xffffffffu, (int)(f64::positive(A1) && f64::positive(B1)), 3, 4) != 0;
   return v;
 }
 
 // The Metropolis margin a - ln U of Eq. (metropolis-ratio) of a move: the
 // reverse move from v' with the coefficients at the proposed energies, its
-// noise per direction [(1 - alpha' alpha) u/2 - alpha' hz G] / hz'.
+// noise per direction [(1 - alpha' alpha) u - alpha' z G] / z'.
 // c0 = |G|^2 / 2 - ln U.
 __device__ __forceinline__ double team_margin(const Team64Const& k, int l, const Team64Move& v, double Gl, double base,
                                               double c0) {
-  const double fi = v.ei + v.deps, fj = v.ej + v.deps;
+  const double E1 = v.E + v.deps;
+  const double t = v.deps * E1;  // change of the product of the energies
   double mr, iz;
-  team_coeffs<true>(k, l == 3 ? k.x_par : k.x_perp, base, fi * fj, f64::rcp(fi + fj), mr, iz);
+  team_coeffs<true>(k, l == 3 ? k.x_par : k.x_perp, base, v.P + t, f64::rcp(E1 + v.deps), mr, iz);
   const double cr = -__fma_rn(v.m, mr, v.m + mr);
-  const double g = __fma_rn(cr, v.U, -(__fma_rn(mr, v.z, v.z) * Gl)) * iz;
-  // ln|B(v)| - ln|B(v')| = ln(z z') along + 2 ln(z z') across e (lanes 3, 0,
-  // 1); entropy (C_K/kB - 1) ln(eps' products / eps products) (lane 2)
-  const double t = v.deps * ((v.ei + v.ej) + v.deps);
-  const double lg = f64::log1p(l == 2 ? t * v.r0 : __fma_rn(v.z, iz, -1.0));
-  return c0 + quad_sum(__fma_rn(-0.5 * g, g, l == 2 ? k.CKm1 * lg : lg));
+  const double g = __fma_rn(cr, v.u, -(__fma_rn(mr, v.z, v.z) * Gl)) * iz;
+  // ln|B(v)| - ln|B(v')| = ln(z / z') along + 2 ln(z / z') across e (lanes 3,
+  // 0, 1); entropy (C_K/kB - 1) ln(eps' products / eps products) (lane 2)
+  const bool ent = l == 2;
+  const double lg = f64::log1p(__fma_rn(ent ? t : v.z, ent ? v.r0 : iz, ent ? 0.0 : -1.0));
+  return c0 + quad_sum(__fma_rn(-0.5 * g, g, ent ? k.CKm1 * lg : lg));
 }
 
 constexpr int kTeamPairs = 16;    // pairs of a round
@@ -123,8 +131,8 @@ struct Team64Smem {
   D4 s[kLargeBlock];
   FdCells cells;
   uint8_t rsize[kRoundStride];
-  double m[2][kTeamThreads], z[2][kTeamThreads], U[2][kTeamThreads], r0[2][kTeamPairs];
-  double deps[2][kTeamPairs], ei[2][kTeamPairs], ej[2][kTeamPairs];
+  double m[2][kTeamThreads], z[2][kTeamThreads], u[2][kTeamThreads], r0[2][kTeamPairs];
+  double deps[2][kTeamPairs], E[2][kTeamPairs], P[2][kTeamPairs], low[2][kTeamPairs];  // low: the lower new energy
   uint8_t bound[2][kTeamPairs];
   unsigned rejected[2][2];  // quads (their lanes' bits) of the round tested in a step, by its parity and per warp
   unsigned next;
@@ -230,22 +238,23 @@ __global__ void __launch_bounds__(team_threads<EMS>())
       auto propose = [&]() {
         A = rec[4 * ia + l];
         B = rec[4 * ib + l];
-        double dA, dB;
-        v = team_propose(k, l, A, B, cge, cG, cb, dA, dB);
+        double A1, B1;
+        v = team_propose(k, l, A, B, cge, cG, cb, A1, B1);
         moved = live && (v.bound || k.scheme == SDPD_SCHEME_SSA);
         if (moved) {
-          rec[4 * ia + l] = A + dA;
-          rec[4 * ib + l] = B + dB;
+          rec[4 * ia + l] = A1;
+          rec[4 * ib + l] = B1;
         }
+        if (REC && l == 3) sm.low[buf][slot] = fmin(A1, B1);
         if (EMS && act) {
           sm.m[buf][tt] = v.m;
           sm.z[buf][tt] = v.z;
-          sm.U[buf][tt] = v.U;
+          sm.u[buf][tt] = v.u;
           if (l == 2) sm.r0[buf][slot] = v.r0;
           if (l == 0) {
             sm.deps[buf][slot] = v.deps;
-            sm.ei[buf][slot] = v.ei;
-            sm.ej[buf][slot] = v.ej;
+            sm.E[buf][slot] = v.E;
+            sm.P[buf][slot] = v.P;
             sm.bound[buf][slot] = v.bound;
           }
         }
@@ -254,8 +263,9 @@ __global__ void __launch_bounds__(team_threads<EMS>())
       double margin = 0.0;
       if (!tester) {
         if (busy) propose();
+        if (REC && !EMS) __syncwarp();
         if (!EMS && live) {
-          margin = fmin(v.ei + v.deps, v.ej + v.deps);
+          if (REC) margin = sm.low[buf][slot];
           if (k.scheme == SDPD_SCHEME_SSA) negative |= !v.bound;
           else dcs = v.bound ? 0 : 1;
         }
@@ -263,16 +273,16 @@ __global__ void __launch_bounds__(team_threads<EMS>())
         if (busy) {
           v.m = sm.m[buf][tt];
           v.z = sm.z[buf][tt];
-          v.U = sm.U[buf][tt];
+          v.u = sm.u[buf][tt];
           v.r0 = sm.r0[buf][slot];
           v.deps = sm.deps[buf][slot];
-          v.ei = sm.ei[buf][slot];
-          v.ej = sm.ej[buf][slot];
+          v.E = sm.E[buf][slot];
+          v.P = sm.P[buf][slot];
           v.bound = sm.bound[buf][slot];
           const double mg = team_margin(k, l, v, cG, cb, cc);
           if (live) {
             dcs = !v.bound ? 1 : (f64::negative(mg) ? 2 : 0);  // 2: U > exp(a)
-            margin = v.bound ? mg : fmin(v.ei + v.deps, v.ej + v.deps);
+            if (REC) margin = v.bound ? mg : sm.low[buf][slot];
           }
         }
         const unsigned rej = __ballot_sync(0xffffffffu, dcs == 2);
@@ -405,8 +415,8 @@ void launch_colours64(const Consts& c, const Workspace& w, int cur, double dt, u
   k.x_par = -2.0 * c.kpar_m2 * (dt / c.m);
   k.x_perp = -2.0 * c.kperp_m2 * (dt / c.m);
   k.d2 = 2.0 * c.kB / c.C_K;
-  k.s = c.kB * c.m / c.C_K;
-  k.de = -0.5 / c.m;
+  k.s = 4.0 * c.kB * c.m / c.C_K;
+  k.de = -0.25 / c.m;
   k.CKm1 = c.C_K / c.kB - 1.0;
   k.scheme = c.scheme;
   const int64_t nown = (int64_t)(c.nc[0] / 2) * (c.nc[1] / 2) * (c.nc[2] / 2);
