@@ -528,6 +528,7 @@ int sdpd_create(int64_t N, const double box[3], double m, double h, const sdpd_p
   c.fd_variant = fd_default_variant(prm->precision == SDPD_MIXED || prm->sweep_f32 != 0);
   c.pair_threads = 128;
   c.fd_auto = true;
+  c.fd_peers = 0;
   c.scheme = prm->scheme;
   s->prm = *prm;
   s->K = K;
@@ -1403,10 +1404,14 @@ void member_steps(sdpd_handle* h, double dt, int64_t n, uint64_t seed) {
 // joined back into the ensemble stream.
 void ensemble_enqueue(sdpd_ensemble* e, double dt, int64_t nsteps, const uint64_t* seeds) {
   cudaEventRecord(e->fork, e->stream);
+  int64_t blocks = 0;
+  for (const sdpd_handle* h : e->m) blocks += (int64_t)(h->c.nc[0] / 2) * (h->c.nc[1] / 2) * (h->c.nc[2] / 2);
   for (size_t i = 0; i < e->m.size(); ++i) {
     sdpd_handle* h = e->m[i];
     cudaStreamWaitEvent(h->stream, e->fork, 0);
+    h->c.fd_peers = blocks;
     member_steps(h, dt, nsteps, seeds[i]);
+    h->c.fd_peers = 0;
     cudaEventRecord(e->join[i], h->stream);
     cudaStreamWaitEvent(e->stream, e->join[i], 0);
   }
