@@ -315,7 +315,7 @@ typedef struct {
                        4 (1 x 4); with 2 to 4 the Metropolised scheme runs
                        a team of two warps per block instead.  -1 = chosen at
                        launch by the blocks per colour (2 up to 912 of them,
-                       1 up to 4864, else 0; sdpd_get_tuning then reports 0
+                       1 up to 3648, else 0; sdpd_get_tuning then reports 0
                        for float32 and 1 for float64 pair arithmetic); a new
                        handle starts with -1.
                        Float64 pair arithmetic takes 1, 2 and 3 and has one

@@ -877,7 +877,12 @@ static __device__ __noinline__ float fd_uniform_again(uint64_t seed, uint64_t sw
 // state swept with float32 pair arithmetic (P = Fp64) gets its momenta and
 // energies back as their float64 values plus the float32 increments of the
 // visit.  REC: keep a record per pair (every Metropolis margin in float64).
-// Thread blocks of 1 to 4 warps, 128 registers per thread (16 warps per SM).
+// Thread blocks of 1 to 4 warps.  PER_SM thread blocks of 128 threads per SM:
+// 4 (128 registers, 16 warps per SM, some spills) where blocks abound; 3 (168
+// registers, 12 warps, none) up to as many warps, where a round's chain decides.
+// 262,144 particles, 4 sweeps: 4047 us with 4, 3947 with 3; 2 M particles, 2
+// steps: 15.8 ms with 4, 16.5 with 3.  (5 with 96 registers: 4882 us and
+// 16.5 ms; four blocks per warp, 8 lanes each: 17.0 ms.)
 // ---------------------------------------------------------------------------
 // What the lanes of a colour launch count.
 struct FdTally {
@@ -1252,8 +1257,8 @@ __device__ __forceinline__ void fd_finish(const FdRun<P>& f, uint64_t sweep, uns
   }
 }
 
-template <class P, int OPW, bool REC>
-__global__ void __launch_bounds__(128, 4) k_fd_colour(const __grid_constant__ FdRun<P> f) {
+template <class P, int OPW, int PER_SM, bool REC>
+__global__ void __launch_bounds__(128, PER_SM) k_fd_colour(const __grid_constant__ FdRun<P> f) {
   constexpr int GL = 32 / OPW;
   extern __shared__ __align__(32) unsigned char fd_smem_raw[];
   const uint64_t sweep = *f.sweep_ptr;
@@ -1579,7 +1584,7 @@ int fd_resident_blocks() {
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fd_colour<P, kFdOpw[V], REC>, kFdWarps[V] * 32,
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fd_colour<P, kFdOpw[V], V == 0 ? 4 : 3, REC>, kFdWarps[V] * 32,
                                                   fd_smem_bytes<P>(V));
     return std::max(1, sms) * std::max(1, per_sm);
   }();
@@ -1647,7 +1652,7 @@ void launch_colours32(const Consts& c, const Workspace& w, int cur, double dt, u
   f.big_count = w.big_count;
   f.large_list = w.large_list;
   f.large_count = w.large_count;
-  auto kern = opw == 2 ? k_fd_colour<P, 2, REC> : k_fd_colour<P, 1, REC>;
+  auto kern = opw == 1 ? k_fd_colour<P, 1, 3, REC> : (W == 2 ? k_fd_colour<P, 2, 4, REC> : k_fd_colour<P, 2, 3, REC>);
   // a team per block where a warp per block would run it (EMS: only there has
   // the test its own work)
   const bool spec = opw == 1 && c.scheme == SDPD_SCHEME_EMS;

@@ -81,16 +81,18 @@ __host__ __device__ constexpr int fd_default_variant(bool mixed) { return mixed 
 // the autotuner, else by the blocks per colour.  Few blocks: a colour lasts as
 // long as its deepest block, which runs fastest on warps of its own (EMS: two,
 // k_fd_colour_spec); from about six blocks per SM on two blocks per warp use
-// its lanes better.  Microseconds per sweep (EMS, with the random numbers) with
-// schedules 0 / 1 / 2: 216 blocks 621 / 646 / 484, 512 blocks 633 / 653 / 540,
-// 729 blocks 723 / 747 / 645, 1000 blocks 772 / 754 / 867, 1331 blocks 805 /
-// 777 / 962, 2744 blocks 1041 / 966 / 1645; 6859 blocks 1711 / 1734 / 2340.
+// its lanes better, and beyond the 12 warps per SM of schedule 1 the 16 of
+// schedule 0.  Microseconds per sweep (EMS, with the random numbers) with
+// schedules 0 / 1 / 2: 216 blocks 621 / 646 / 484, 512 blocks 718 / 707 / 623,
+// 729 blocks 723 / 747 / 645, 1331 blocks 805 / 753 / 968, 1728 blocks 934 /
+// 850 / 1104, 2744 blocks 1041 / 970 / 1646, 4096 blocks 1091 / 1303 / 2199,
+// 15,625 blocks 3717 / 3856 / 7978.
 // Members of an ensemble share the GPU, so the blocks of all of them count
 // (24 members of 13^3 to 40^3 particles, 4 steps: 9.7 / 9.7 / 12.1 ms).
 inline int fd_launch_variant(const Consts& c) {
   if (!c.fd_auto && c.fd_variant >= 0 && c.fd_variant < kFdVariants) return c.fd_variant;
   const int64_t nown = c.fd_peers > 0 ? c.fd_peers : (int64_t)(c.nc[0] / 2) * (c.nc[1] / 2) * (c.nc[2] / 2);
-  return nown <= 6 * 152 ? 2 : (nown <= 32 * 152 ? 1 : 0);
+  return nown <= 6 * 152 ? 2 : (nown <= 24 * 152 ? 1 : 0);
 }
 __host__ __device__ constexpr bool pair_threads_ok(int t) { return t == 32 || t == 64 || t == 128; }
 // whether a handle takes a block schedule (float64 pair arithmetic: 1 to 3, all
