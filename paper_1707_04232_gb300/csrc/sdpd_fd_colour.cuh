@@ -7,6 +7,7 @@
 #include <type_traits>
 
 #include "sdpd_fd_common.cuh"
+#include "sdpd_rand64.cuh"
 
 namespace sdpd {
 
@@ -122,7 +123,8 @@ __device__ __forceinline__ void pair_randoms_fast(uint64_t seed, uint64_t sweep,
 }
 __device__ __forceinline__ void pair_randoms_fast(uint64_t seed, uint64_t sweep, uint64_t idi, uint64_t idj,
                                                   double G[3], double* U) {
-  pair_randoms(seed, sweep, idi, idj, G, U);
+  double lnU;
+  pair_randoms(seed, sweep, idi, idj, G, U, &lnU);
 }
 
 // alpha = exp(-2 gamma dt / m) and zt = (2/m) zeta of Section 3.2 for both
@@ -667,18 +669,19 @@ __global__ void __launch_bounds__(kStageWarps * 32)
   for (int t = 32 * part + lane; t < np; t += 32 * split) {
     const uint32_t pr = pairs[base + t];
     const int ga = block_gidx(cells, pr & 0xffffu), gb = block_gidx(cells, pr >> 16);  // ga holds the lower id
-    R G[3], U;
+    R G[3], U, lnU;
     // (ids as unsigned 32-bit numbers: the high words of the counter are known to be zero)
-    pair_randoms_fast(seed, sweep, (uint32_t)id[ga], (uint32_t)id[gb], G, &U);
     typename A::V4 v;
     if constexpr (A::mixed) {
+      pair_randoms_fast(seed, sweep, (uint32_t)id[ga], (uint32_t)id[gb], G, &U);
       v = F4{G[0], G[1], G[2], c.scheme == SDPD_SCHEME_EMS ? fm::log(U) : U};
     } else {
+      pair_randoms(seed, sweep, (uint32_t)id[ga], (uint32_t)id[gb], G, &U, &lnU);
       const D4 e = ld4(&geom[base + t]);
       const double gp = e.x * G[0] + e.y * G[1] + e.z * G[2];
       v = D4{G[0] - gp * e.x, G[1] - gp * e.y, G[2] - gp * e.z, gp};
       aux[base + t] = c.scheme == SDPD_SCHEME_EMS
-                          ? 0.5 * (G[0] * G[0] + G[1] * G[1] + G[2] * G[2]) - fm::log(U) : 0.0;
+                          ? 0.5 * (G[0] * G[0] + G[1] * G[1] + G[2] * G[2]) - lnU : 0.0;
     }
     st4(&rnd[base + t], v);
   }

@@ -190,30 +190,6 @@ __device__ __forceinline__ void philox4x64_10(uint64_t c0, uint64_t c1, uint64_t
   out[0] = c0; out[1] = c1; out[2] = c2; out[3] = c3;
 }
 
-// Random numbers of one pair at one sweep: G ~ N(0, I3) and U ~ U(0,1).
-// Key (seed, 0), counter (sweep, id_min, id_max, 0).  Words 0 and 1 give G0,
-// G1 by Box-Muller on two uniforms; word 2 gives G2 by Box-Muller on its two
-// 32-bit halves; word 3 gives U.  Uniforms are (x + 1/2) 2^-b for the top
-// b = 53 bits of a word (32 for the halves of word 2).  The float32 path
-// rounds the same uniforms to float32 (pair_randoms_fast).
-__device__ __forceinline__ void pair_randoms(uint64_t seed, uint64_t sweep, uint64_t idi, uint64_t idj,
-                                             double G[3], double* U) {
-  uint64_t w[4];
-  philox4x64_10(sweep, idi, idj, 0ull, seed, 0ull, w);
-  const double two53 = 1.0 / 9007199254740992.0, two32 = 1.0 / 4294967296.0;
-  double u0 = ((double)(w[0] >> 11) + 0.5) * two53;
-  double u1 = ((double)(w[1] >> 11) + 0.5) * two53;
-  double R = sqrt(-2.0 * log(u0));
-  double s, c;
-  sincospi(2.0 * u1, &s, &c);
-  G[0] = R * c;
-  G[1] = R * s;
-  double u2 = ((double)(uint32_t)(w[2] >> 32) + 0.5) * two32;
-  double u3 = ((double)(uint32_t)(w[2] & 0xffffffffull) + 0.5) * two32;
-  G[2] = sqrt(-2.0 * log(u2)) * cospi(2.0 * u3);
-  *U = ((double)(w[3] >> 11) + 0.5) * two53;
-}
-
 // ---------------------------------------------------------------------------
 // Precision policies.
 //   Fp64: positions float64 absolute in [0, L); all arithmetic float64.
