@@ -318,8 +318,8 @@ typedef struct {
                        1 up to 3648, else 0; sdpd_get_tuning then reports 0
                        for float32 and 1 for float64 pair arithmetic); a new
                        handle starts with -1.
-                       Float64 pair arithmetic takes 1, 2 and 3 and has one
-                       schedule, a team of warps per block */
+                       Float64 pair arithmetic has one schedule, a team of
+                       warps per block, whatever the value */
   int pair_threads; /* threads per block of the density and force passes:
                        32, 64 or 128; 0 = 128 */
 } sdpd_tuning;

@@ -844,7 +844,7 @@ int sdpd_set_tuning(sdpd_t* s, const sdpd_tuning* t) {
   if (!s || !t) return SDPD_ERR_INVALID_ARG;
   const int v = t->fd_variant < 0 ? fd_default_variant(sweep_float(s)) : t->fd_variant;
   const int pt = t->pair_threads == 0 ? 128 : t->pair_threads;
-  if (v >= kFdVariants || !fd_variant_fits(sweep_float(s), v) || !pair_threads_ok(pt))
+  if (v >= kFdVariants || !pair_threads_ok(pt))
     return SDPD_ERR_INVALID_ARG;
   s->c.fd_variant = v;
   s->c.fd_auto = t->fd_variant < 0;
@@ -894,7 +894,7 @@ int sdpd_autotune(sdpd_t* s, double dt, int64_t steps, uint64_t seed, sdpd_tunin
   int bv = v0, bt = 128;
   double bms = INFINITY;
   for (int v = 0; v < kFdVariants; ++v) {
-    if (!fd_variant_fits(sweep_float(s), v)) continue;
+    if (!sweep_float(s) && v != fd_default_variant(false)) continue;  // float64 has one schedule
     const double ms = trial(v, 128);
     if (ms < bms) { bms = ms; bv = v; }
   }
@@ -1582,7 +1582,7 @@ int sdpd_ensemble_autotune(sdpd_ens_t* e, double dt, int64_t steps, const uint64
     std::vector<sdpd_tuning> u(n);
     for (size_t i = 0; i < n; ++i) {
       const bool fl = sweep_float(e->m[i]);
-      u[i] = {fd_variant_fits(fl, v) ? v : fd_default_variant(fl), 128};
+      u[i] = {fl ? v : fd_default_variant(fl), 128};
     }
     cand.push_back(u);
   }

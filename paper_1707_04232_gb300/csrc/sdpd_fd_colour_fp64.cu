@@ -19,8 +19,4 @@ int fd_round_width(const Consts& c, bool float_arith, bool large) {
   return float_arith ? (large ? 32 : 32 / kFdOpw[fd_launch_variant(c)]) : kTeamPairs;
 }
 
-bool fd_variant_fits(bool float_arith, int v) {
-  return float_arith ? v >= 0 && v < kFdVariants : v >= 1 && v <= 3;
-}
-
 }  // namespace sdpd

@@ -95,9 +95,6 @@ inline int fd_launch_variant(const Consts& c) {
   return nown <= 6 * 152 ? 2 : (nown <= 24 * 152 ? 1 : 0);
 }
 __host__ __device__ constexpr bool pair_threads_ok(int t) { return t == 32 || t == 64 || t == 128; }
-// whether a handle takes a block schedule (float64 pair arithmetic: 1 to 3, all
-// of them its one team kernel)
-bool fd_variant_fits(bool float_arith, int v);
 
 // Neighbour-list entry: neighbour index << 6 | stencil offset code, the code
 // holding (o + 1) per axis in 2 bits (x lowest) for o in {-1, 0, +1}.

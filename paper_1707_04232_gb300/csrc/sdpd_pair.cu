@@ -173,15 +173,13 @@ template <int KIND, int T, int PPB>
 __global__ void __launch_bounds__(PPB * T)
     k_density64(Consts c, Arrays<Fp64> a, D4* __restrict__ qp4, const int32_t* __restrict__ cell_start,
                 const int32_t* __restrict__ mrank, int update_eos, int32_t* __restrict__ ncount_by_id,
-                uint32_t* __restrict__ nlist, int32_t* __restrict__ nn, int32_t* __restrict__ ovf_list,
-                int32_t* __restrict__ ovf_count, int32_t* __restrict__ ovf_other, const float4* __restrict__ qf4,
+                uint32_t* __restrict__ nlist, int32_t* __restrict__ nn, const float4* __restrict__ qf4,
                 D4* __restrict__ qr4, uint32_t* __restrict__ cend) {
   extern __shared__ uint32_t list_s[];  // [cap / 4][PPB][4]
   __shared__ double acc_s[PPB];
   __shared__ int cnt_s[PPB];
   const int p = threadIdx.x / T, gl = threadIdx.x % T;
   const int64_t i0 = blockIdx.x * (int64_t)PPB, i = i0 + p;
-  if (blockIdx.x == 0 && threadIdx.x == 0) *ovf_other = 0;  // the other slot: its readers have run
   const bool live = i < c.N;
   const D4 qi = ld4(&a.q4[live ? i : 0]);
   const float4 fi = qf4[live ? i : 0];
@@ -228,7 +226,6 @@ __global__ void __launch_bounds__(PPB * T)
     const int cnt = cnt_s[threadIdx.x];
     if (ncount_by_id) ncount_by_id[a.id[g]] = cnt;
     nn[g] = cnt;
-    if (cnt > c.nbr_cap) ovf_list[atomicAdd(ovf_count, 1)] = (int32_t)g;  // forces from the cells
     const double rho_new = c.m * __fma_rn(c.cW, acc_s[threadIdx.x], c.W0);
     double e = a.eps[g];
     if (update_eos) {
@@ -508,8 +505,7 @@ static inline int pair_block(const Consts& c) { return pair_threads_ok(c.pair_th
 
 template <int KIND>
 static void launch_density64(const Consts& c, const Workspace& w, const Arrays<Fp64>& a, int update_eos,
-                             int32_t* ncount_by_id, int32_t* ovf_list, int32_t* ovf_count, int32_t* ovf_other,
-                             cudaStream_t s) {
+                             int32_t* ncount_by_id, cudaStream_t s) {
   const bool wide = pair64_wide(c);
   const int t = wide ? 128 : pair_block(c), ppb = wide ? 4 : t / kLanes64;
   auto kern = wide ? k_density64<KIND, 32, 4>
@@ -517,8 +513,8 @@ static void launch_density64(const Consts& c, const Workspace& w, const Arrays<F
                               : (t == 64 ? k_density64<KIND, kLanes64, 64 / kLanes64>
                                          : k_density64<KIND, kLanes64, 128 / kLanes64>));
   kern<<<blocks_for(c.N, ppb), t, (size_t)c.nbr_cap * ppb * 4, s>>>(
-      c, a, (D4*)w.qp4, w.cell_start, w.mrank, update_eos, ncount_by_id, w.nlist, w.nn, ovf_list, ovf_count, ovf_other,
-      w.qf4, (D4*)w.qr4, w.cend);
+      c, a, (D4*)w.qp4, w.cell_start, w.mrank, update_eos, ncount_by_id, w.nlist, w.nn, w.qf4,
+      (D4*)w.qr4, w.cend);
 }
 
 template <class P>
@@ -526,20 +522,20 @@ void launch_density(const Consts& c, const Workspace& w, int cur, int update_eos
                     cudaStream_t s) {
   if (c.N == 0) return;
   Arrays<P> a = view<P>(w, cur);
-  const int sl = (*w.ovf_slot ^= 1);  // this pass's slot of the overflow list
-  int32_t* ovf_list = w.ovf_list + (size_t)sl * (size_t)c.N;
-  int32_t* ovf_count = w.ovf_count + sl;
-  int32_t* ovf_other = w.ovf_count + (sl ^ 1);
   if constexpr (P::mixed) {
+    const int sl = (*w.ovf_slot ^= 1);  // this pass's slot of the overflow list
+    int32_t* ovf_list = w.ovf_list + (size_t)sl * (size_t)c.N;
+    int32_t* ovf_count = w.ovf_count + sl;
+    int32_t* ovf_other = w.ovf_count + (sl ^ 1);
     const int t = pair_block(c);
     auto kern = c.kernel == SDPD_KERNEL_LUCY ? k_density<P, SDPD_KERNEL_LUCY> : k_density<P, SDPD_KERNEL_CUBIC>;
     kern<<<blocks_for(c.N, t), t, 0, s>>>(c, a, (typename P::V4*)w.qp4, w.cell_start, w.mrank, w.xmin[0], w.xmin[1],
                                           w.xmin[2], update_eos, ncount_by_id, w.nlist, w.nn, ovf_list, ovf_count,
                                           ovf_other, (typename P::V4*)w.qr4, w.cend);
   } else if (c.kernel == SDPD_KERNEL_LUCY) {
-    launch_density64<SDPD_KERNEL_LUCY>(c, w, a, update_eos, ncount_by_id, ovf_list, ovf_count, ovf_other, s);
+    launch_density64<SDPD_KERNEL_LUCY>(c, w, a, update_eos, ncount_by_id, s);
   } else {
-    launch_density64<SDPD_KERNEL_CUBIC>(c, w, a, update_eos, ncount_by_id, ovf_list, ovf_count, ovf_other, s);
+    launch_density64<SDPD_KERNEL_CUBIC>(c, w, a, update_eos, ncount_by_id, s);
   }
 }
 

@@ -46,16 +46,13 @@ def test_sort_density_and_forces(N, side):
 @pytest.mark.parametrize("N", [700, 2433])
 def test_float64_launch_shapes_are_bitwise_alike(N):
     """Block sizes of the passes, set or left alone, on both sides of the line
-    of a warp per particle; float64 handles take schedules 1 to 3 only."""
+    of a warp per particle, under every schedule of the colour launches."""
     q, p, e = random_box_state(N, 1.0, 1.0, 1.0, 30.0, seed=N)
     out = []
-    for pt in (None, 32, 64, 128):
+    for v, pt in ((0, None), (0, 32), (2, 64), (4, 128)):
         s = sdpd.SDPD(N, 13.0, h=2.5, K=20.0, precision=sdpd.FP64)
         if pt is not None:
-            s.set_tuning(1, pt)
-            for v in (0, 4):
-                with pytest.raises(sdpd.SDPDError):
-                    s.set_tuning(v, pt)
+            s.set_tuning(v, pt)
         s.set_state(q * 13.0, p, e)
         s.step(0.002, 3, seed=3)
         out.append(s.get_state())
