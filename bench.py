@@ -249,11 +249,12 @@ def workload_config(args):
 FLOPS_PER_VISIT = {"density_eos": 18.0, "kick1_drift_bin": 24.0, "kick2": 24.0,
                    "adj_pass_A": 23.0, "adj_pass_B": 66.0}
 FP64_NOMINAL_TFLOPS = 1.25  # GB300 float64, nominal
-# DRAM traffic of one colour launch of the mixed-precision sweep, per
-# particle: dram__bytes_read.sum + dram__bytes_write.sum of one launch at
-# N = 96^3 (50.21 MB + 3.26 MB), divided by the particles every colour
-# launch visits once; a launch's traffic scales with N
-FD_COLOUR_DRAM_BYTES_PER_PARTICLE = (50.207488e6 + 3.262720e6) / 96 ** 3
+# DRAM traffic of an average launch of the mixed-precision sweep stage (eight
+# colour launches and the random numbers), per particle:
+# dram__bytes_read.sum + dram__bytes_write.sum of one launch of each at
+# N = 96^3 (188.82 + 11.56 MB; 143.12 + 485.88 MB); a launch's traffic scales
+# with N
+FD_COLOUR_DRAM_BYTES_PER_PARTICLE = (8 * (188.817152e6 + 11.555328e6) + 143.121920e6 + 485.879552e6) / 9 / 96 ** 3
 FLOPS_PER_PAIR_UPDATE = {"ems": 210.0, "ams": 150.0, "ssa": 140.0}
 
 
@@ -318,7 +319,7 @@ def run_ours(args, rank, world, local_rank):
     alu_peak = (SMS * FP32_LANES_PER_SM * 2 * sm_max * 1e6 / 1e12 if args.precision == "mixed"
                 else FP64_NOMINAL_TFLOPS)  # TFLOP/s of the arithmetic the pair passes use
     if top == "fd_colours":
-        units = o1["n_pairs"] / max(1, top_launches)  # pair updates per colour launch
+        units = o1["n_pairs"] / max(1, top_launches)  # pair updates per launch of the stage
         flops = FLOPS_PER_PAIR_UPDATE[args.scheme] * units
     elif top in FLOPS_PER_VISIT:
         nvisits = w.N * 80.0  # neighbour visits per launch (lattice: 80 per particle)
