@@ -272,7 +272,7 @@ __device__ __forceinline__ int walk64(const Consts& c, bool live, const Home64& 
           const int t = b + u * T + gl;
           cell[u] = (t >= off[1]) + (t >= off[2]);
           js[u] = t + (cell[u] == 0 ? beg[0] : (cell[u] == 1 ? beg[1] - off[1] : beg[2] - off[2]));
-          fj[u] = t < off[3] ? __ldg(&qf4[js[u]]) : make_float4(3e18f, 0.0f, 0.0f, 0.0f);  // (too far)
+          fj[u] = t < off[3] ? __ldg(&qf4[js[u]]) : make_float4(INFINITY, 0.0f, 0.0f, 0.0f);  // (beyond any h)
         }
 #pragma unroll
         for (int u = 0; u < kBatch; ++u) {
