@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(PPB * T)
                 const int32_t* __restrict__ mrank, int update_eos, int32_t* __restrict__ ncount_by_id,
                 uint32_t* __restrict__ nlist, int32_t* __restrict__ nn, const float4* __restrict__ qf4,
                 D4* __restrict__ qr4, uint32_t* __restrict__ cend) {
-  extern __shared__ uint32_t list_s[];  // [cap / 4][PPB][4]
+  extern __shared__ __align__(16) uint32_t list_s[];  // [cap / 4][PPB][4], read as uint4
   __shared__ double acc_s[PPB];
   __shared__ int cnt_s[PPB];
   const int p = threadIdx.x / T, gl = threadIdx.x % T;
