@@ -1505,6 +1505,9 @@ int sdpd_ensemble_step(sdpd_ens_t* e, double dt, int64_t nsteps, const uint64_t*
     shape.push_back(h->cur);
     shape.push_back(h->c.fd_auto ? -1 : h->c.fd_variant);
     shape.push_back(h->c.pair_threads);
+    // an FD-only member's graph holds its schedule's launches only if there
+    // was no valid schedule then (a Verlet step always drops the schedule)
+    shape.push_back(h->prm.fd_only && h->sched_valid);
   }
   if (units > 0) {
     if (!e->exec || e->dt != dt || e->seeds != sv || e->phase != phase || e->shape != shape) {
@@ -1517,8 +1520,10 @@ int sdpd_ensemble_step(sdpd_ens_t* e, double dt, int64_t nsteps, const uint64_t*
       // restored after capture
       std::vector<int> cur0;
       std::vector<int64_t> fd0, vv0, l0;
+      std::vector<bool> valid0;
       for (sdpd_handle* h : e->m) {
         cur0.push_back(h->cur); fd0.push_back(h->fd_step); vv0.push_back(h->vv_step); l0.push_back(h->launches);
+        valid0.push_back(h->sched_valid);
       }
       if (cudaStreamBeginCapture(e->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return SDPD_ERR_CUDA;
       ensemble_enqueue(e, dt, U, seeds);
@@ -1528,6 +1533,7 @@ int sdpd_ensemble_step(sdpd_ens_t* e, double dt, int64_t nsteps, const uint64_t*
         sdpd_handle* h = e->m[i];
         e->launches_per_unit += h->launches - l0[i];
         h->cur = cur0[i]; h->fd_step = fd0[i]; h->vv_step = vv0[i]; h->launches = l0[i];
+        h->sched_valid = valid0[i];
       }
       if (ce != cudaSuccess || cudaGraphInstantiate(&e->exec, e->graph, 0) != cudaSuccess) {
         cudaGetLastError();
