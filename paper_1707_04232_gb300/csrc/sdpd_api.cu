@@ -34,7 +34,6 @@ struct sdpd_handle {
   std::vector<uint32_t> xmin_h[3];
   int64_t pair_rec_cap;
   int device;  // device of the bound workspace; selected on entry to every call
-  int ovf_slot = 0;  // slot of the neighbour-list overflow list of the latest density pass
   // stage timing: event pairs recorded on the stream, reduced at sync points
   bool timing;
   std::vector<cudaEvent_t> ev_pool;
@@ -212,7 +211,6 @@ size_t layout(sdpd_handle* s, Workspace* w, char* base) {
   w->large_count = (uint32_t*)at(16 * 4);
   w->ovf_list = (int32_t*)at(2 * N * 4);
   w->ovf_count = (int32_t*)at(2 * 4);
-  w->ovf_slot = &s->ovf_slot;
   w->blk_hist = (uint32_t*)at(8 * 256 * 4);
   w->blk_order = (int32_t*)at(nc * 4);
   w->pair_rec_count = (unsigned long long*)at(8);
@@ -240,11 +238,16 @@ int launch_status() {
   return e == cudaSuccess ? SDPD_OK : SDPD_ERR_CUDA;
 }
 
+// Empties the overflow list of the current buffer, for a density pass that
+// does not follow one on the other buffer (which would have emptied it).
+void clear_overflow(sdpd_handle* s) { cudaMemsetAsync(s->w.ovf_count + s->cur, 0, 4, s->stream); }
+
 template <class P>
 void do_load(sdpd_handle* s) {
   launch_load<P>(s->c, s->w, s->stream);
   launch_sort<P>(s->c, s->w, 0, s->stream);
   s->cur = 1;
+  if (P::mixed) clear_overflow(s);
   launch_density<P>(s->c, s->w, s->cur, 0, nullptr, s->stream);
   s->launches += 2 + sort_launches(s->c);  // load, sort, density
   s->sched_valid = false;
@@ -1319,6 +1322,7 @@ int debug_get(sdpd_handle* s, int what, void* dst, int64_t cap, int64_t* count) 
     }
     case SDPD_DEBUG_NCOUNT: {
       if (cap < N) return SDPD_ERR_INVALID_ARG;
+      if (mixed) clear_overflow(s);
       if (mixed) launch_density<Mixed>(s->c, s->w, cur, 0, (int32_t*)s->w.io_q, st);
       else launch_density<Fp64>(s->c, s->w, cur, 0, (int32_t*)s->w.io_q, st);
       s->launches += 1;

@@ -359,13 +359,11 @@ struct Workspace {
   int32_t* large_list;           // [8][ncell / 8]: each colour's large blocks
   uint32_t* large_count;         // [8] entries of large_list, then of large_cand, then finished thread blocks
   // particles whose neighbour list overflows its row, listed by the density
-  // pass into one of two slots: [2][N] entries and [2] counts.  A density
-  // pass fills slot *ovf_slot (toggled on the host before each launch) and
-  // clears the other one, which no kernel reads any more (the force passes
-  // read the slot of the latest density pass).
+  // pass (mixed path) per state buffer: [2][N] entries and [2] counts.  A
+  // density pass fills its buffer's list and empties the other one's, whose
+  // readers (the force passes on that buffer) have run.
   int32_t* ovf_list;
   int32_t* ovf_count;
-  int* ovf_slot;                 // host: the slot of the latest density pass
   sdpd_pair_rec* pair_recs;   // debug
   unsigned long long* pair_rec_count;
   int64_t pair_rec_cap;

@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(128, 12) k_density(Consts c, Arrays<P> a, type
   using R = typename P::R;
   using V4 = typename P::V4;
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i == 0) *ovf_other = 0;  // the other slot: its readers have run
+  if (i == 0) *ovf_other = 0;  // the other buffer's list: its readers have run
   if (i >= c.N) return;
   const V4 qi = ld4(&a.q4[i]);
   int cx, cy, cz;
@@ -523,10 +523,9 @@ void launch_density(const Consts& c, const Workspace& w, int cur, int update_eos
   if (c.N == 0) return;
   Arrays<P> a = view<P>(w, cur);
   if constexpr (P::mixed) {
-    const int sl = (*w.ovf_slot ^= 1);  // this pass's slot of the overflow list
-    int32_t* ovf_list = w.ovf_list + (size_t)sl * (size_t)c.N;
-    int32_t* ovf_count = w.ovf_count + sl;
-    int32_t* ovf_other = w.ovf_count + (sl ^ 1);
+    int32_t* ovf_list = w.ovf_list + (size_t)cur * (size_t)c.N;  // this buffer's overflow list
+    int32_t* ovf_count = w.ovf_count + cur;
+    int32_t* ovf_other = w.ovf_count + (cur ^ 1);
     const int t = pair_block(c);
     auto kern = c.kernel == SDPD_KERNEL_LUCY ? k_density<P, SDPD_KERNEL_LUCY> : k_density<P, SDPD_KERNEL_CUBIC>;
     kern<<<blocks_for(c.N, t), t, 0, s>>>(c, a, (typename P::V4*)w.qp4, w.cell_start, w.mrank, w.xmin[0], w.xmin[1],
@@ -540,7 +539,7 @@ void launch_density(const Consts& c, const Workspace& w, int cur, int update_eos
 }
 
 template <class P, int KIND>
-static void launch_force_kind(const Consts& c, const Workspace& w, const Arrays<P>& a, double half_dt,
+static void launch_force_kind(const Consts& c, const Workspace& w, int cur, const Arrays<P>& a, double half_dt,
                               double dt_drift, double* force_by_id, cudaStream_t s) {
   auto qp4 = (const typename P::V4*)w.qp4;
   auto qdx = (typename P::Q*)w.qdx;
@@ -550,14 +549,13 @@ static void launch_force_kind(const Consts& c, const Workspace& w, const Arrays<
     const float3 drift3 =
         make_float3((float)(dt_drift / c.m * c.inv_scale[0]), (float)(dt_drift / c.m * c.inv_scale[1]),
                     (float)(dt_drift / c.m * c.inv_scale[2]));
-    const int sl = *w.ovf_slot;  // the overflow list of the latest density pass
     const int t = pair_block(c);
     k_force<P, KIND><<<blocks_for(c.N, t), t, 0, s>>>(
         c, a, qp4, w.cell_start, w.mrank, w.xmin[0], w.xmin[1], w.xmin[2], half_dt, dt_drift, qdx, qdy, qdz, w.key,
         w.slot, w.cell_count, force_by_id, w.nlist, w.nn, drift3);
     k_force_overflow<P, KIND><<<kOverflowBlocks, 128, 0, s>>>(
         c, a, qp4, w.cell_start, w.mrank, w.xmin[0], w.xmin[1], w.xmin[2], half_dt, dt_drift, qdx, qdy, qdz, w.key,
-        w.slot, w.cell_count, force_by_id, drift3, w.ovf_list + (size_t)sl * (size_t)c.N, w.ovf_count + sl);
+        w.slot, w.cell_count, force_by_id, drift3, w.ovf_list + (size_t)cur * (size_t)c.N, w.ovf_count + cur);
   } else {
     const int t = pair_block(c), lanes = pair64_wide(c) ? 32 : kLanes64;
     auto kern = lanes == 32 ? k_force64<KIND, 32> : k_force64<KIND, kLanes64>;
@@ -571,8 +569,8 @@ void launch_force(const Consts& c, const Workspace& w, int cur, double half_dt, 
                   double* force_by_id, cudaStream_t s) {
   if (c.N == 0) return;
   const Arrays<P> a = view<P>(w, cur);
-  if (c.kernel == SDPD_KERNEL_LUCY) launch_force_kind<P, SDPD_KERNEL_LUCY>(c, w, a, half_dt, dt_drift, force_by_id, s);
-  else launch_force_kind<P, SDPD_KERNEL_CUBIC>(c, w, a, half_dt, dt_drift, force_by_id, s);
+  if (c.kernel == SDPD_KERNEL_LUCY) launch_force_kind<P, SDPD_KERNEL_LUCY>(c, w, cur, a, half_dt, dt_drift, force_by_id, s);
+  else launch_force_kind<P, SDPD_KERNEL_CUBIC>(c, w, cur, a, half_dt, dt_drift, force_by_id, s);
 }
 
 template void launch_density<Fp64>(const Consts&, const Workspace&, int, int, int32_t*, cudaStream_t);

@@ -8,7 +8,7 @@ bit, as the other ensemble tests compare.
 import numpy as np
 import pytest
 
-from paper_1707_04232_gb300.inputs import Workload, lattice_state
+from paper_1707_04232_gb300.inputs import Workload, lattice_state, random_box_state
 
 pytestmark = pytest.mark.gpu
 
@@ -43,3 +43,29 @@ def test_fd_only_member_with_a_new_state_gets_a_new_schedule(precision):
         for s, seed in zip(alone, seeds):
             s.step(0.02, 2, seed=seed)
         assert all(same(m, a) for m, a in zip(members, alone))
+
+
+def test_overflowing_neighbour_lists_after_a_new_state():
+    """A fluid with more neighbours than a list row holds (their forces come
+    from the cells): the replay after a new state, and after a debug read-out,
+    finds the particles of the state's own density pass."""
+    N, L = 3000, 10.4
+    states = []
+    for seed in (1, 2):
+        q, p, e = random_box_state(N, 1.0, 1.0, 1.0, 30.0, seed=seed)
+        states.append((q * L, p, e))
+    member, alone = (sdpd.SDPD(N, L, h=2.5, K=20.0, precision=sdpd.MIXED, scheme=sdpd.SCHEME_NONE,
+                               stream=torch.cuda.Stream()) for _ in range(2))
+    member.set_state(*states[0])
+    alone.set_state(*states[0])
+    assert (member.neighbour_counts() > 160).any()
+    ens = sdpd.SDPDEnsemble([member])
+    for state in (None, states[1], None, states[0]):
+        if state is not None:
+            member.set_state(*state)
+            alone.set_state(*state)
+        else:
+            member.neighbour_counts()
+        ens.step(0.002, 4, [5])
+        alone.step(0.002, 4, seed=5)
+        assert same(member, alone)
