@@ -271,15 +271,16 @@ void sdpd_destroy(sdpd_t* s);
  * members are captured once into one CUDA graph (forked from and joined into
  * the ensemble stream; the capture is redone when dt, the seeds, a
  * member's step count modulo its theta, its state buffer (after
- * sdpd_set_state or sdpd_autotune) or its launch shapes change) and the graph is replayed
+ * sdpd_set_state or sdpd_autotune), its workspace, its launch shapes or, for
+ * an FD-only member, the validity of its sweep schedule change) and the graph is replayed
  * nsteps/U times; the nsteps mod U last steps are enqueued directly.  Every
  * member's result is the same as stepping it alone.  The members' own
  * streams wait for the ensemble's work before later calls on them run.
  * Asynchronous.
  * Errors: SDPD_ERR_INVALID_ARG (bad or repeated member, a member on the
  * ensemble's stream, members' workspaces on different devices, timing or
- * debug on, U > 64), SDPD_ERR_NO_WORKSPACE, SDPD_ERR_CUDA,
- * SDPD_ERR_HOST_MEMORY. */
+ * debug on, U > 64), SDPD_ERR_NO_WORKSPACE, SDPD_ERR_NO_STATE (a member whose
+ * workspace was bound anew), SDPD_ERR_CUDA, SDPD_ERR_HOST_MEMORY. */
 typedef struct sdpd_ensemble sdpd_ens_t;
 int sdpd_ensemble_create(sdpd_t* const* members, int n, void* stream, sdpd_ens_t** out);
 int sdpd_ensemble_step(sdpd_ens_t* e, double dt, int64_t nsteps, const uint64_t* seeds);

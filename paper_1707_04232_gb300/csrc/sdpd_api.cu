@@ -1395,6 +1395,7 @@ struct sdpd_ensemble {
   int64_t unit;                  // steps per graph replay: lcm of 2 and the members' theta
   std::vector<int64_t> phase;    // members' vv_step mod theta when the graph was captured
   std::vector<int> shape;        // members' state buffer and launch shapes at capture
+  std::vector<const char*> ws;   // members' workspaces at capture
 };
 
 namespace {
@@ -1495,6 +1496,8 @@ int sdpd_ensemble_create(sdpd_t* const* members, int n, void* stream, sdpd_ens_t
 int sdpd_ensemble_step(sdpd_ens_t* e, double dt, int64_t nsteps, const uint64_t* seeds) {
   if (!e || !seeds || !(dt > 0) || !isfinite(dt) || nsteps < 0) return SDPD_ERR_INVALID_ARG;
   if (use_device(e->m[0]) != SDPD_OK) return SDPD_ERR_CUDA;
+  for (const sdpd_handle* h : e->m)  // (a workspace bound anew holds no state yet)
+    if (!h->has_state) return SDPD_ERR_NO_STATE;
   // the ensemble stream waits for everything already enqueued on the members
   for (sdpd_handle* h : e->m)
     if (order_streams(h->stream, e->stream) != SDPD_OK) return SDPD_ERR_CUDA;
@@ -1503,7 +1506,9 @@ int sdpd_ensemble_step(sdpd_ens_t* e, double dt, int64_t nsteps, const uint64_t*
   const std::vector<uint64_t> sv(seeds, seeds + e->m.size());
   std::vector<int64_t> phase;
   std::vector<int> shape;
+  std::vector<const char*> ws;
   for (sdpd_handle* h : e->m) {
+    ws.push_back(h->ws);
     phase.push_back(h->vv_step % std::max(1, h->prm.theta));
     // the graph holds the buffer pointers and launch shapes of its capture
     shape.push_back(h->cur);
@@ -1514,7 +1519,7 @@ int sdpd_ensemble_step(sdpd_ens_t* e, double dt, int64_t nsteps, const uint64_t*
     shape.push_back(h->prm.fd_only && h->sched_valid);
   }
   if (units > 0) {
-    if (!e->exec || e->dt != dt || e->seeds != sv || e->phase != phase || e->shape != shape) {
+    if (!e->exec || e->dt != dt || e->seeds != sv || e->phase != phase || e->shape != shape || e->ws != ws) {
       if (e->exec) { cudaGraphExecDestroy(e->exec); e->exec = nullptr; }
       if (e->graph) { cudaGraphDestroy(e->graph); e->graph = nullptr; }
       // capture U steps: each step's sort flips the double-buffered state,
@@ -1547,6 +1552,7 @@ int sdpd_ensemble_step(sdpd_ens_t* e, double dt, int64_t nsteps, const uint64_t*
       e->seeds = sv;
       e->phase = phase;
       e->shape = shape;
+      e->ws = ws;
     }
     for (int64_t u = 0; u < units; ++u)
       if (cudaGraphLaunch(e->exec, e->stream) != cudaSuccess) return SDPD_ERR_CUDA;

@@ -69,3 +69,25 @@ def test_overflowing_neighbour_lists_after_a_new_state():
         ens.step(0.002, 4, [5])
         alone.step(0.002, 4, seed=5)
         assert same(member, alone)
+
+
+def test_member_with_a_new_workspace():
+    """A workspace bound anew holds no state (the call is refused); with a
+    state it is the one that is stepped."""
+    w = Workload(n=10, K=50.0, seed=3)
+    state = lattice_state(w)
+    member, alone = (sdpd.SDPD(w.N, w.L, h=w.h, K=w.K, precision=sdpd.MIXED, stream=torch.cuda.Stream())
+                     for _ in range(2))
+    member.set_state(*state)
+    alone.set_state(*state)
+    ens = sdpd.SDPDEnsemble([member])
+    ens.step(0.005, 2, [9])
+    old, member.workspace = member.workspace, torch.empty_like(member.workspace)
+    torch.cuda.synchronize()
+    assert sdpd.sdpd_bind_workspace(member.h, member.workspace.data_ptr(), member.workspace.numel()) == sdpd.OK
+    assert sdpd.sdpd_ensemble_step(ens.e, 0.005, 2, [9]) == sdpd.ERR_NO_STATE
+    member.set_state(*state)
+    ens.step(0.005, 2, [9])
+    alone.step(0.005, 2, seed=9)
+    assert same(member, alone)
+    del old
