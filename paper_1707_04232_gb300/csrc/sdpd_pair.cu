@@ -229,9 +229,11 @@ __global__ void __launch_bounds__(PPB * T)
     const double rho_new = c.m * __fma_rn(c.cW, acc_s[threadIdx.x], c.W0);
     double e = a.eps[g];
     if (update_eos) {
-      // eps' = E(S(eps, rho), rho') = eps (rho' / rho)^(c_rho / C_K)
+      // eps' = E(S(eps, rho), rho') = eps (rho' / rho)^(c_rho / C_K); a
+      // negative energy (SSA) has no entropy: NaN
       const double ro = a.rho[g];
       e *= exp(c.c_rho / c.C_K * log1p((rho_new - ro) / ro));
+      if (f64::negative(e)) e = __longlong_as_double(0x7ff8000000000000ll);
       a.eps[g] = e;
     }
     a.rho[g] = rho_new;

@@ -35,3 +35,22 @@ def test_density_and_forces_at_any_unit_of_length(N, unit):
     assert (s.neighbour_counts() == O.neighbour_counts(P, q)).all()
     assert np.abs(s.density() - rho).max() <= 1e-12 * rho.max()
     assert np.abs(s.forces() - f).max() <= 1e-12 * np.abs(f).max()
+
+
+def test_negative_energy_has_no_entropy():
+    """A negative internal energy (loaded from the device, where only the
+    status tells of it) becomes NaN in a Verlet step, as the oracle's does."""
+    N, L = 1000, 10.0
+    q, p, e = random_box_state(N, 1.0, 1.0, 1.0, 30.0, seed=6)
+    q = q * L
+    e[[3, 500]] = -2.0
+    P = O.Config(N=N, L=(L,) * 3, K=20.0, scheme=O.SCHEME_NONE).params()
+    _, _, _, eo, _, _ = O.run(P, q, p, e, 0.002, 1, seed=1)
+    s = sdpd.SDPD(N, L, h=2.5, K=20.0, precision=sdpd.FP64, scheme=sdpd.SCHEME_NONE)
+    dev = [torch.from_numpy(x).cuda() for x in (q, p, e)]
+    s.set_state(*dev)
+    s.step(0.002, 1, seed=1)
+    out = [torch.empty_like(x) for x in dev]
+    assert sdpd.sdpd_get_state(s.h, *(x.data_ptr() for x in out), 1) == sdpd.ERR_NONPOSITIVE_ENERGY
+    eg = out[2].cpu().numpy()
+    assert (np.isnan(eg) == np.isnan(eo)).all() and np.isnan(eg).sum() == 2
