@@ -10,8 +10,8 @@ said otherwise:
 * expm1 and log1p 0.75 below 1/4 and 1/8 (above, CUDA's functions bit for bit),
 * unit_log 1.0; the uniforms' cosine and sine 1.4e-16 absolute (half a last
   place each for the table value and the sum, the rest below 0.3e-16),
-* pair_r64 1.5e-13 relative: with d the error of H (2 ulp of rsqrtf, the
-  truncation and the product: 3.6e-7) and g that of 1/H (5.4e-7, of the same
+* pair_r64 2.8e-14 relative: with d the error of H (the roundings of y, 9e-8,
+  and of r^2 and the product, 6e-8 each) and g that of 1/H (2.4e-7, of the same
   sign) it is d (g - d / 2); with a second step half an ulp for r and 3e-16
   relative for 1/r.
 """
@@ -102,7 +102,7 @@ def test_pair_distances(lib):
     x = np.concatenate([spread(1e-12, 10.0), spread(1.0, 4.0, seed=1), spread(1e-36, 1e37),
                         spread(1e-30, 1.1e-30, n=1000)])
     r = np.sqrt(x.astype(LD))
-    assert np.abs(evaluate(lib, "pair_r", x) / r - 1).max() <= 1.5e-13
+    assert np.abs(evaluate(lib, "pair_r", x) / r - 1).max() <= 2.8e-14
     assert np.abs(evaluate(lib, "pair_r2", x) / r - 1).max() <= 2.3e-16
     assert np.abs(evaluate(lib, "pair_rinv", x) * r - 1).max() <= 3e-16
 
