@@ -124,7 +124,11 @@ typedef struct {
 int sdpd_create(int64_t N, const double box[3], double m, double h, const sdpd_params* params,
                 double K, void* stream, sdpd_t** out);
 
-/* Bytes of device workspace the handle needs (256-byte aligned start). */
+/* Bytes of device workspace the handle needs (256-byte aligned start): at unit
+ * density, h = 2.5, about 4.1 KB per particle (7.5 KB with float64 pair
+ * arithmetic), most of it the staged pair data of the sweep; from 32,768 cell
+ * blocks per colour on (160^3 particles) 1.6 to 1.7 KB plus a slice of 4.8
+ * (10.2) GB. */
 size_t sdpd_workspace_bytes(const sdpd_t* s);
 
 /* Bind caller-allocated device memory of at least sdpd_workspace_bytes bytes
@@ -182,17 +186,21 @@ int64_t sdpd_get_fd_step(const sdpd_t* s);
 /* Reset the pair counters of sdpd_obs. */
 int sdpd_reset_counters(sdpd_t* s);
 
-/* Number of CUDA kernels the handle has launched so far (a VV step launches
- * 8, a sweep 9 plus 5 when its schedule is rebuilt -- it is reused while the
- * positions do not change, as in FD-only runs -- sdpd_set_state 8,
- * sdpd_observables 2).  The nine of a sweep are the random numbers of all its
- * pairs and the eight colours. */
+/* Number of CUDA kernels the handle has launched so far: per Verlet step 10
+ * (8 float64), sdpd_set_state 8 -- 4 fewer each with at most 2048 particles and
+ * cells, which one launch sorts --, sdpd_observables 2, a sweep 9 (the random
+ * numbers of all its pairs and the eight colours) plus 5 when its schedule is
+ * rebuilt (it is reused while the positions do not change, as in FD-only
+ * runs).  Systems of more than 32,768 cell blocks per colour whose pair data
+ * would take more than two slices of device memory stage them slice by slice: 3
+ * launches per slice of 32,768 blocks of each colour, plus 4 per schedule. */
 int64_t sdpd_kernel_launches(const sdpd_t* s);
 
 /* Per-stage timing with CUDA events recorded on the handle's stream around
  * every stage that sdpd_step launches.  Stages: 0 first kick + drift +
  * binning, 1 sort, 2 density + EOS, 3 second kick, 4 sweep schedule,
- * 5 the sweep's random numbers and colours (9 launches per sweep); and of sdpd_vv_adjoint: 6 loading
+ * 5 the sweep's random numbers and colours (9 launches per sweep; more by
+ * slices); and of sdpd_vv_adjoint: 6 loading
  * a stored position (bin, sort, density), 7 pair pass A, 8 pair pass B,
  * 9 the elementwise steps between them.  sdpd_stage_times synchronises and
  * returns, per stage, the summed milliseconds and the number of kernel

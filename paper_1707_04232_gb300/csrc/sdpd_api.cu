@@ -191,9 +191,14 @@ size_t layout(sdpd_handle* s, Workspace* w, char* base) {
   w->sched_off = (unsigned long long*)at(nc * 8);
   w->sched_total = (unsigned long long*)at(8);
   w->sched_pair = (uint32_t*)at(cap * 4);
-  w->st_geom = at(cap * rec);
-  w->st_rnd = at(cap * rec);
-  w->st_aux = rec == sizeof(D4) ? (double*)at(cap * 8) : nullptr;
+  const size_t staged = sweep * stage_capacity(c);
+  const bool sliced = sweep && fd_sliced(c);
+  w->st_pair = sliced ? (uint32_t*)at(staged * 4) : w->sched_pair;
+  w->blk_pos = sliced ? (uint32_t*)at(nc * 4) : nullptr;
+  w->st_off = sliced ? (unsigned long long*)at(nc * 8) : w->sched_off;
+  w->st_geom = at(staged * rec);
+  w->st_rnd = at(staged * rec);
+  w->st_aux = rec == sizeof(D4) ? (double*)at(staged * 8) : nullptr;
   w->io_q = (double*)at(3 * N * 8);
   w->io_p = (double*)at(3 * N * 8);
   w->io_e = (double*)at(N * 8);
@@ -209,7 +214,7 @@ size_t layout(sdpd_handle* s, Workspace* w, char* base) {
   w->large_cand = (int32_t*)at(nc * 4);
   w->large_list = (int32_t*)at(nc * 4);
   w->large_count = (uint32_t*)at(16 * 4);
-  w->ovf_list = (int32_t*)at(2 * N * 4);
+  w->ovf_list = P::mixed ? (int32_t*)at(2 * N * 4) : nullptr;
   w->ovf_count = (int32_t*)at(2 * 4);
   w->blk_hist = (uint32_t*)at(8 * 256 * 4);
   w->blk_order = (int32_t*)at(nc * 4);
@@ -360,20 +365,20 @@ void fd_sweep_step(sdpd_handle* s, double dt_fd, uint64_t seed) {
   const int rec = s->w.pair_recs != nullptr;
   if (rec) cudaMemsetAsync(s->w.pair_rec_count, 0, 8, s->stream);
   if (!s->sched_valid) {  // positions unchanged since the last sweep: reuse it
-    StageTimer t(s, 4, 5);
+    StageTimer t(s, 4, schedule_launches(c));
     launch_fd_schedule<P>(c, s->w, s->cur, fd_round_width(c, sweep_float(s), false),
                           fd_round_width(c, sweep_float(s), true), s->stream);
     if constexpr (std::is_same<P, Fp64>::value) {
-      if (s->prm.sweep_f32) launch_stage_geometry<Fp64, Mixed>(c, s->w, s->cur, s->stream);
-      else launch_stage_geometry<Fp64, Fp64>(c, s->w, s->cur, s->stream);
+      if (s->prm.sweep_f32) launch_stage_geometry<Fp64, Mixed>(c, s->w, s->stream);
+      else launch_stage_geometry<Fp64, Fp64>(c, s->w, s->stream);
     } else {
-      launch_stage_geometry<P, P>(c, s->w, s->cur, s->stream);
+      launch_stage_geometry<P, P>(c, s->w, s->stream);
     }
-    s->launches += 5;
+    s->launches += schedule_launches(c);
     s->sched_valid = true;
   }
   {
-    StageTimer t(s, 5, 9);
+    StageTimer t(s, 5, sweep_launches(c));
     if constexpr (std::is_same<P, Fp64>::value) {
       if (s->prm.sweep_f32) launch_fd_colours<Fp64, Mixed>(c, s->w, s->cur, dt_fd, seed, rec, s->stream);
       else launch_fd_colours<Fp64, Fp64>(c, s->w, s->cur, dt_fd, seed, rec, s->stream);
@@ -381,7 +386,7 @@ void fd_sweep_step(sdpd_handle* s, double dt_fd, uint64_t seed) {
       launch_fd_colours<P, P>(c, s->w, s->cur, dt_fd, seed, rec, s->stream);
     }
   }
-  s->launches += 9;
+  s->launches += sweep_launches(c);
   s->fd_step++;
 }
 
@@ -1410,7 +1415,7 @@ void member_steps(sdpd_handle* h, double dt, int64_t n, uint64_t seed) {
 void ensemble_enqueue(sdpd_ensemble* e, double dt, int64_t nsteps, const uint64_t* seeds) {
   cudaEventRecord(e->fork, e->stream);
   int64_t blocks = 0;
-  for (const sdpd_handle* h : e->m) blocks += (int64_t)(h->c.nc[0] / 2) * (h->c.nc[1] / 2) * (h->c.nc[2] / 2);
+  for (const sdpd_handle* h : e->m) blocks += colour_blocks(h->c);
   for (size_t i = 0; i < e->m.size(); ++i) {
     sdpd_handle* h = e->m[i];
     cudaStreamWaitEvent(h->stream, e->fork, 0);

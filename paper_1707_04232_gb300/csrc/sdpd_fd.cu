@@ -782,6 +782,7 @@ __global__ void __launch_bounds__(kLargeThreads)
 // order among blocks of equal depth is free.
 __global__ void k_sched_order_scatter(int64_t ncell, int nc0, int nc1, const uint32_t* __restrict__ hdr,
                                       uint32_t* __restrict__ blk_hist, int32_t* __restrict__ blk_order,
+                                      uint32_t* __restrict__ blk_pos, unsigned long long* __restrict__ st_off,
                                       uint32_t* __restrict__ large_count) {
   if (blockIdx.x == 0 && threadIdx.x < 2) large_count[8 + threadIdx.x] = 0u;  // for the next schedule
   const int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -794,6 +795,10 @@ __global__ void k_sched_order_scatter(int64_t ncell, int nc0, int nc1, const uin
   const int nlev = hd == kHdrBig ? kMaxLevels : (int)(hd >> 16 & 255u);
   const uint32_t pos = atomicAdd(&blk_hist[colour * 256 + nlev], 1u);
   blk_order[colour * (ncell >> 3) + pos] = w;
+  if (blk_pos) {  // the pair data staged by slice
+    blk_pos[o] = pos;
+    st_off[o] = (unsigned long long)(pos % kSliceBlocks) * kLargePairs;
+  }
 }
 
 template <class P>
@@ -824,7 +829,8 @@ void launch_fd_schedule(const Consts& c, const Workspace& w, int cur, int width,
       c, out, std::max(width, large_width), a.id, a.q4, w.xmin[0], w.xmin[1], w.xmin[2], w.nn, w.large_cand,
       w.large_count, w.large_list);
   k_sched_order_scatter<<<(unsigned)((c.ncell + 255) / 256), 256, 0, s>>>(c.ncell, c.nc[0], c.nc[1], w.sched_hdr,
-                                                                         w.blk_hist, w.blk_order, w.large_count);
+                                                                         w.blk_hist, w.blk_order, w.blk_pos,
+                                                                         w.st_off, w.large_count);
 }
 
 // Launch attributes of the schedule's kernels (once per device and process;

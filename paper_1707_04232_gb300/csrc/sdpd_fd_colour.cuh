@@ -565,6 +565,31 @@ inline int stage_split(int64_t ncell) {
   return (int)(n < 1 ? 1 : (n > 16 ? 16 : n));
 }
 
+// The blocks whose pairs a staging launch writes: every block, in place, or a
+// slice (see fd_sliced).
+struct StageJob {
+  int64_t n;             // blocks
+  int split;             // warps per block
+  const int32_t* order;  // slice: its blocks in the colour's order (null: every block)
+  int colour;
+  uint32_t* copy;        // slice: its pairs
+};
+inline StageJob stage_job(int64_t n, const int32_t* order, int colour, uint32_t* copy) {
+  return StageJob{n, stage_split(n), order, colour, copy};
+}
+static inline unsigned stage_grid(const StageJob& job) {
+  return (unsigned)((job.n * job.split + kStageWarps - 1) / kStageWarps);
+}
+
+// Owner cell of entry w of a colour's order.
+__device__ __forceinline__ int64_t order_block(const Consts& c, int colour, int64_t w, int& ox, int& oy, int& oz) {
+  const int hx = c.nc[0] >> 1, hy = c.nc[1] >> 1;
+  ox = 2 * (int)(w % hx) + (colour & 1);
+  oy = 2 * (int)((w / hx) % hy) + ((colour >> 1) & 1);
+  oz = 2 * (int)(w / ((int64_t)hx * hy)) + ((colour >> 2) & 1);
+  return ox + (int64_t)c.nc[0] * (oy + (int64_t)c.nc[1] * oz);
+}
+
 // The block's cells into shared memory, by the whole warp.
 __device__ __forceinline__ void stage_cells(const Consts& c, int64_t o, const int32_t* __restrict__ mrank,
                                             const int32_t* __restrict__ cell_start, int lane, FdCells& cells) {
@@ -593,33 +618,42 @@ __device__ __forceinline__ void stage_cells(const Consts& c, int64_t o, const in
   __syncwarp();
 }
 
+// Owner cell of block blk of a staging launch.
+__device__ __forceinline__ int64_t stage_block(const Consts& c, const StageJob& job, int64_t blk, int& ox, int& oy,
+                                               int& oz) {
+  if (job.order) return order_block(c, job.colour, job.order[blk], ox, oy, oz);
+  owner_coords(c, blk, ox, oy, oz);
+  return blk;
+}
+
 template <class P, class A, int KIND>
 __global__ void __launch_bounds__(kStageWarps * 32)
     k_stage_geometry(Consts c, const typename P::V4* __restrict__ qr4, const int32_t* __restrict__ cell_start,
                      const int32_t* __restrict__ mrank, const uint32_t* __restrict__ xmx,
                      const uint32_t* __restrict__ xmy, const uint32_t* __restrict__ xmz,
                      const uint32_t* __restrict__ hdr, const unsigned long long* __restrict__ sched_off,
-                     const uint32_t* __restrict__ pairs, int split, typename A::V4* __restrict__ geom) {
+                     const uint32_t* __restrict__ pairs, const StageJob job, typename A::V4* __restrict__ geom) {
   using R = typename A::R;
   using S = typename P::R;
   __shared__ FdCells cells_s[kStageWarps];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t wg = (int64_t)blockIdx.x * kStageWarps + warp, o = wg / split;
-  if (o >= c.ncell) return;
-  const int part = (int)(wg - o * split);
+  const int64_t wg = (int64_t)blockIdx.x * kStageWarps + warp, blk = wg / job.split;
+  if (blk >= job.n) return;
+  const int split = job.split, part = (int)(wg - blk * split);
+  int ox, oy, oz;
+  const int64_t o = stage_block(c, job, blk, ox, oy, oz);
   const uint32_t hd = hdr[o];
   const int np = hd == kHdrBig ? 0 : (int)(hd & 0xffffu);
   if (32 * part >= np) return;
   FdCells& cells = cells_s[warp];
   stage_cells(c, o, mrank, cell_start, lane, cells);
-  int ox, oy, oz;
-  owner_coords(c, o, ox, oy, oz);
   BlockGeom<P> geo;
   geo.init(c, ox, oy, oz, xmx, xmy, xmz);
   const S inv_h = (S)c.inv_h, cF = (S)c.cF;
-  const unsigned long long base = sched_off[o];
+  const unsigned long long base = sched_off[o], to = job.order ? (unsigned long long)blk * kLargePairs : base;
   for (int t = 32 * part + lane; t < np; t += 32 * split) {
     const uint32_t pr = pairs[base + t];
+    if (job.order) job.copy[to + t] = pr;
     int da, db;
     const int ga = block_gidx(cells, pr & 0xffffu, da), gb = block_gidx(cells, pr >> 16, db);
     S xa, ya, za, xb, yb, zb, rx, ry, rz;
@@ -637,7 +671,7 @@ __global__ void __launch_bounds__(kStageWarps * 32)
     v.w = (R)fm::div(stage_F<KIND>(r2 * inv_r, inv_h, cF), qa.w * qb.w);
     if constexpr (!A::mixed)  // at r = h the pair does nothing: marked by base = 0
       if (!(c.kperp_m2 * v.w > 0.0) || !(c.kpar_m2 * v.w > 0.0)) v.w = 0.0;
-    st4(&geom[base + t], v);
+    st4(&geom[to + t], v);
   }
 }
 
@@ -653,22 +687,24 @@ __global__ void __launch_bounds__(kStageWarps * 32)
     k_stage_random(Consts c, const int32_t* __restrict__ id, const int32_t* __restrict__ cell_start,
                    const int32_t* __restrict__ mrank, const uint32_t* __restrict__ hdr,
                    const unsigned long long* __restrict__ sched_off, const uint32_t* __restrict__ pairs,
-                   int split, uint64_t seed, const unsigned long long* __restrict__ sweep_ptr,
+                   const StageJob job, uint64_t seed, const unsigned long long* __restrict__ sweep_ptr,
                    const typename A::V4* __restrict__ geom, typename A::V4* __restrict__ rnd,
                    double* __restrict__ aux) {
   using R = typename A::R;
   __shared__ FdCells cells_s[kStageWarps];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t wg = (int64_t)blockIdx.x * kStageWarps + warp, o = wg / split;
-  if (o >= c.ncell) return;
-  const int part = (int)(wg - o * split);
+  const int64_t wg = (int64_t)blockIdx.x * kStageWarps + warp, blk = wg / job.split;
+  if (blk >= job.n) return;
+  const int split = job.split, part = (int)(wg - blk * split);
+  int ox, oy, oz;
+  const int64_t o = stage_block(c, job, blk, ox, oy, oz);
   const uint32_t hd = hdr[o];
   const int np = hd == kHdrBig ? 0 : (int)(hd & 0xffffu);
   if (32 * part >= np) return;
   FdCells& cells = cells_s[warp];
   stage_cells(c, o, mrank, cell_start, lane, cells);
   const uint64_t sweep = *sweep_ptr;
-  const unsigned long long base = sched_off[o];
+  const unsigned long long base = sched_off[o], to = job.order ? (unsigned long long)blk * kLargePairs : base;
   for (int t = 32 * part + lane; t < np; t += 32 * split) {
     const uint32_t pr = pairs[base + t];
     const int ga = block_gidx(cells, pr & 0xffffu), gb = block_gidx(cells, pr >> 16);  // ga holds the lower id
@@ -680,13 +716,13 @@ __global__ void __launch_bounds__(kStageWarps * 32)
       v = F4{G[0], G[1], G[2], c.scheme == SDPD_SCHEME_EMS ? fm::log(U) : U};
     } else {
       pair_randoms(seed, sweep, (uint32_t)id[ga], (uint32_t)id[gb], G, &U, &lnU);
-      const D4 e = ld4(&geom[base + t]);
+      const D4 e = ld4(&geom[to + t]);
       const double gp = e.x * G[0] + e.y * G[1] + e.z * G[2];
       v = D4{G[0] - gp * e.x, G[1] - gp * e.y, G[2] - gp * e.z, gp};
-      aux[base + t] = c.scheme == SDPD_SCHEME_EMS
+      aux[to + t] = c.scheme == SDPD_SCHEME_EMS
                           ? 0.5 * (G[0] * G[0] + G[1] * G[1] + G[2] * G[2]) - lnU : 0.0;
     }
-    st4(&rnd[base + t], v);
+    st4(&rnd[to + t], v);
   }
 }
 
@@ -911,6 +947,12 @@ struct FdRun {
   const uint32_t* pairs;
   const F4 *geom, *rnd;
   int colour;
+  // the launch's blocks: n entries of the colour's order from its entry
+  // `first` on (order points there); pos: null, or (sliced) the places of all
+  // blocks in their colours' orders; last: the colour's last launch
+  int64_t first; unsigned n;
+  const uint32_t* pos;
+  bool last;
   uint64_t seed;
   unsigned long long* sweep_ptr;
   unsigned long long* counters;
@@ -1207,12 +1249,14 @@ __device__ __forceinline__ void fd_finish(const FdRun<P>& f, uint64_t sweep, uns
       if (lane == 0) li = atomicAdd(&queue[3], 1u);
       li = __shfl_sync(0xffffffffu, li, 0);
       if (li >= f.large_count[colour]) break;
-      fd_large_block<P, REC>(f, f.large_list[colour * nown + li], sweep, fd_smem_raw, tally);
+      const int32_t o = f.large_list[colour * nown + li];
+      if (f.pos && ((int64_t)f.pos[o] < f.first || (int64_t)f.pos[o] >= f.first + f.n)) continue;  // of another slice
+      fd_large_block<P, REC>(f, o, sweep, fd_smem_raw, tally);
     }
   }
   // the colour's blocks beyond capacity (listed by the schedule), swept pair
   // by pair by whole warps once the queue is empty
-  for (;;) {
+  while (f.last) {
     unsigned bi = 0;
     if (lane == 0) bi = atomicAdd(&queue[2], 1u);
     bi = __shfl_sync(0xffffffffu, bi, 0);
@@ -1240,7 +1284,7 @@ __device__ __forceinline__ void fd_finish(const FdRun<P>& f, uint64_t sweep, uns
       queue[1] = 0u;
       queue[2] = 0u;
       queue[3] = 0u;
-      if (colour == 7) *f.sweep_ptr = sweep + 1ull;  // (every warp has read it) the sweep is done
+      if (colour == 7 && f.last) *f.sweep_ptr = sweep + 1ull;  // (every warp has read it) the sweep is done
     }
   }
   // counters
@@ -1270,9 +1314,8 @@ __global__ void __launch_bounds__(128, PER_SM) k_fd_colour(const __grid_constant
   const uint64_t sweep = *f.sweep_ptr;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, grp = lane / GL;
   const Consts& c = f.c;
-  const int colour = f.colour;
-  const int hx = c.nc[0] >> 1, hy = c.nc[1] >> 1, hz = c.nc[2] >> 1;
-  const int64_t nown = (int64_t)hx * hy * hz;
+  // (as order_block, whose call here, inside the loop, costs 5%: 1010 us per sweep of 262,144 particles, 968 so)
+  const int colour = f.colour, hx = c.nc[0] >> 1, hy = c.nc[1] >> 1;
   FdSmem& sm = reinterpret_cast<FdSmem*>(fd_smem_raw)[warp * OPW + grp];
   unsigned* queue = f.queue;
   FdTally tally;
@@ -1288,15 +1331,15 @@ __global__ void __launch_bounds__(128, PER_SM) k_fd_colour(const __grid_constant
     unsigned w0 = 0;
     if (lane == 0) w0 = atomicAdd(queue, (unsigned)OPW);
     w0 = __shfl_sync(0xffffffffu, w0, 0);
-    if ((int64_t)w0 >= nown) break;
-    const int64_t wi = (int64_t)w0 + grp;
-    const int64_t w = wi < nown ? (int64_t)f.order[colour * nown + wi] : 0;
+    if (w0 >= f.n) break;
+    const unsigned wi = w0 + grp;
+    const int64_t w = wi < f.n ? (int64_t)f.order[wi] : 0;
     const int ox = 2 * (int)(w % hx) + (colour & 1), oy = 2 * (int)((w / hx) % hy) + ((colour >> 1) & 1),
               oz = 2 * (int)(w / ((int64_t)hx * hy)) + ((colour >> 2) & 1);
     const int64_t o = ox + (int64_t)c.nc[0] * (oy + (int64_t)c.nc[1] * oz);
     const uint32_t hd = f.hdr[o];
     // (large blocks and those beyond capacity, which have the flag's bit set too, come below)
-    const bool live = wi < nown && !(hd & kHdrLargeFlag);
+    const bool live = wi < f.n && !(hd & kHdrLargeFlag);
     fd_run_block<P, GL, REC>(f, live, o, ox, oy, oz, hd, sweep, sm.s, sm.ec, sm.cells, tally);
   }
   fd_finish<P, REC>(f, sweep, fd_smem_raw, tally);
@@ -1334,8 +1377,6 @@ __global__ void __launch_bounds__(64) k_fd_colour_spec(const __grid_constant__ F
   const Consts& c = f.c;
   const Arrays<P>& a = f.a;
   const int colour = f.colour;
-  const int hx = c.nc[0] >> 1, hy = c.nc[1] >> 1, hz = c.nc[2] >> 1;
-  const int64_t nown = (int64_t)hx * hy * hz;
   const S pi_coef = kSame ? (S)c.f_pi_coef : (S)c.pi_coef;
   unsigned* queue = f.queue;
   FdTally tally;
@@ -1346,11 +1387,9 @@ __global__ void __launch_bounds__(64) k_fd_colour_spec(const __grid_constant__ F
     if (t == 0) sm.next = atomicAdd(queue, 1u);
     __syncthreads();
     const unsigned wi = sm.next;
-    if ((int64_t)wi >= nown) break;
-    const int64_t w = f.order[colour * nown + wi];
-    const int ox = 2 * (int)(w % hx) + (colour & 1), oy = 2 * (int)((w / hx) % hy) + ((colour >> 1) & 1),
-              oz = 2 * (int)(w / ((int64_t)hx * hy)) + ((colour >> 2) & 1);
-    const int64_t o = ox + (int64_t)c.nc[0] * (oy + (int64_t)c.nc[1] * oz);
+    if (wi >= f.n) break;
+    int ox, oy, oz;
+    const int64_t o = order_block(c, colour, f.order[wi], ox, oy, oz);
     const uint32_t hd = f.hdr[o];
     const int np = hd & kHdrLargeFlag ? 0 : (int)(hd & 0xffffu), nr = (int)(hd >> 16 & 255u);
     if (np == 0) {  // (large blocks and those beyond capacity come below)
@@ -1621,14 +1660,26 @@ int fd_spec_resident() {
   return n;
 }
 
-// The eight colour launches of one sweep with float32 pair arithmetic.  Few
+// Calls launch(colour, first, n, last) for the colour launches of a sweep: one
+// per colour, or one per slice of each colour, its pair data staged before it
+// by stage(job).
+template <class Stage, class Launch>
+void for_colours(const Consts& c, const Workspace& w, Stage stage, Launch launch) {
+  const int64_t nown = colour_blocks(c), step = fd_sliced(c) ? kSliceBlocks : std::max<int64_t>(1, nown);
+  for (int col = 0; col < 8; ++col)
+    for (int64_t b = 0; b < nown; b += step) {
+      const int64_t n = std::min(step, nown - b);
+      if (fd_sliced(c)) stage(stage_job(n, w.blk_order + col * nown + b, col, w.st_pair));
+      launch(col, b, n, b + n == nown);
+    }
+}
+
+// The colour launches of one sweep with float32 pair arithmetic.  Few
 // blocks spread over as many thread blocks (a warp that finds none left ends).
-template <class P, bool REC>
+template <class P, bool REC, class Stage>
 void launch_colours32(const Consts& c, const Workspace& w, int cur, double dt, uint64_t seed, int variant,
-                      cudaStream_t s) {
-  const int64_t nown = (int64_t)(c.nc[0] / 2) * (c.nc[1] / 2) * (c.nc[2] / 2);
+                      Stage stage, cudaStream_t s) {
   const int opw = kFdOpw[variant], W = kFdWarps[variant];
-  const unsigned gf = (unsigned)std::max<int64_t>(1, std::min<int64_t>((nown + opw - 1) / opw, fd_resident<P, REC>(variant)));
   FdRun<P> f;
   f.c = c;
   f.k = fd_const<float>(c, dt);
@@ -1641,8 +1692,8 @@ void launch_colours32(const Consts& c, const Workspace& w, int cur, double dt, u
   f.xmz = w.xmin[2];
   f.hdr = w.sched_hdr;
   f.rsize = w.sched_rsize;
-  f.sched_off = w.sched_off;
-  f.pairs = w.sched_pair;
+  f.sched_off = w.st_off;
+  f.pairs = w.st_pair;
   f.geom = (const F4*)w.st_geom;
   f.rnd = (const F4*)w.st_rnd;
   f.seed = seed;
@@ -1652,7 +1703,7 @@ void launch_colours32(const Consts& c, const Workspace& w, int cur, double dt, u
   f.recs = REC ? w.pair_recs : nullptr;
   f.rec_count = w.pair_rec_count;
   f.rec_cap = w.pair_rec_cap;
-  f.order = w.blk_order;
+  f.pos = w.blk_pos;
   f.big_perm = w.big_perm;
   f.big_list = w.big_list;
   f.big_count = w.big_count;
@@ -1662,19 +1713,29 @@ void launch_colours32(const Consts& c, const Workspace& w, int cur, double dt, u
   // a team per block where a warp per block would run it (EMS: only there has
   // the test its own work)
   const bool spec = opw == 1 && c.scheme == SDPD_SCHEME_EMS;
-  const unsigned gs = (unsigned)std::max<int64_t>(1, std::min<int64_t>(nown, fd_spec_resident<P, REC>()));
-  for (int col = 0; col < 8; ++col) {
+  for_colours(c, w, stage, [&](int col, int64_t first, int64_t n, bool last) {
     f.colour = col;
     f.queue = w.fd_queue + 4 * col;
-    if (spec) k_fd_colour_spec<P, REC><<<gs, 64, fd_spec_bytes<P>(), s>>>(f);
-    else kern<<<gf, W * 32, fd_smem_bytes<P>(variant), s>>>(f);
-  }
+    f.order = w.blk_order + col * colour_blocks(c) + first;
+    f.first = first;
+    f.n = (unsigned)n;
+    f.last = last;
+    if (spec) {
+      k_fd_colour_spec<P, REC>
+          <<<(unsigned)std::min<int64_t>(n, fd_spec_resident<P, REC>()), 64, fd_spec_bytes<P>(), s>>>(f);
+    } else {
+      const unsigned g = (unsigned)std::min<int64_t>((n + opw - 1) / opw, fd_resident<P, REC>(variant));
+      kern<<<g, W * 32, fd_smem_bytes<P>(variant), s>>>(f);
+    }
+  });
 }
 
 // Fills the resident-block counts of every block schedule ahead of time (a
 // host query, kept out of stream captures).
 void team64_prepare();
-void launch_team64(const Consts& c, const Workspace& w, int cur, double dt, uint64_t seed, int record, cudaStream_t s);
+template <class Stage>
+void launch_team64(const Consts& c, const Workspace& w, int cur, double dt, uint64_t seed, int record, Stage stage,
+                   cudaStream_t s);
 
 template <class P, class A>
 void fd_prepare() {
@@ -1690,23 +1751,24 @@ void fd_prepare() {
   }
 }
 
-static inline unsigned stage_blocks(const Consts& c) {
-  return (unsigned)(((int64_t)c.ncell * stage_split(c.ncell) + kStageWarps - 1) / kStageWarps);
+template <class P, class A>
+void stage_geometry(const Consts& c, const Workspace& w, const StageJob& job, cudaStream_t s) {
+  auto kern = c.kernel == SDPD_KERNEL_LUCY ? k_stage_geometry<P, A, SDPD_KERNEL_LUCY>
+                                           : k_stage_geometry<P, A, SDPD_KERNEL_CUBIC>;
+  kern<<<stage_grid(job), kStageWarps * 32, 0, s>>>(c, (const typename P::V4*)w.qr4, w.cell_start, w.mrank, w.xmin[0],
+                                                   w.xmin[1], w.xmin[2], w.sched_hdr, w.sched_off, w.sched_pair, job,
+                                                   (typename A::V4*)w.st_geom);
 }
 
 // The staged geometry of every scheduled pair (the last launch of a schedule).
 template <class P, class A>
-void launch_stage_geometry(const Consts& c, const Workspace& w, int cur, cudaStream_t s) {
-  if (c.N == 0) return;
-  (void)cur;
-  auto kern = c.kernel == SDPD_KERNEL_LUCY ? k_stage_geometry<P, A, SDPD_KERNEL_LUCY>
-                                           : k_stage_geometry<P, A, SDPD_KERNEL_CUBIC>;
-  kern<<<stage_blocks(c), kStageWarps * 32, 0, s>>>(c, (const typename P::V4*)w.qr4, w.cell_start, w.mrank, w.xmin[0],
-                                                   w.xmin[1], w.xmin[2], w.sched_hdr, w.sched_off, w.sched_pair, stage_split(c.ncell),
-                                                   (typename A::V4*)w.st_geom);
+void launch_stage_geometry(const Consts& c, const Workspace& w, cudaStream_t s) {
+  if (c.N == 0 || fd_sliced(c)) return;
+  stage_geometry<P, A>(c, w, stage_job(c.ncell, nullptr, 0, nullptr), s);
 }
 
-// One sweep: the random numbers of every scheduled pair, then the colours;
+// One sweep: the random numbers of every scheduled pair, then the colours
+// (sliced: geometry, random numbers and colour launch of each slice in turn);
 // the last colour launch advances the sweep counter.
 template <class P, class A>
 void launch_fd_colours(const Consts& c, const Workspace& w, int cur, double dt, uint64_t seed, int record,
@@ -1715,16 +1777,21 @@ void launch_fd_colours(const Consts& c, const Workspace& w, int cur, double dt, 
     launch_advance_sweep(w, s);
     return;
   }
-  k_stage_random<A><<<stage_blocks(c), kStageWarps * 32, 0, s>>>(c, w.id[cur], w.cell_start, w.mrank, w.sched_hdr,
-                                                                w.sched_off, w.sched_pair, stage_split(c.ncell), seed,
-                                                                w.sweep,
-                                                                (const typename A::V4*)w.st_geom,
-                                                                (typename A::V4*)w.st_rnd, w.st_aux);
+  auto random = [&](const StageJob& job) {
+    k_stage_random<A><<<stage_grid(job), kStageWarps * 32, 0, s>>>(
+        c, w.id[cur], w.cell_start, w.mrank, w.sched_hdr, w.sched_off, w.sched_pair, job, seed, w.sweep,
+        (const typename A::V4*)w.st_geom, (typename A::V4*)w.st_rnd, w.st_aux);
+  };
+  auto stage = [&](const StageJob& job) {
+    stage_geometry<P, A>(c, w, job, s);
+    random(job);
+  };
+  if (!fd_sliced(c)) random(stage_job(c.ncell, nullptr, 0, nullptr));
   if constexpr (!A::mixed) {
-    launch_team64(c, w, cur, dt, seed, record, s);
+    launch_team64(c, w, cur, dt, seed, record, stage, s);
   } else {
-    if (record) launch_colours32<P, true>(c, w, cur, dt, seed, fd_launch_variant(c), s);
-    else launch_colours32<P, false>(c, w, cur, dt, seed, fd_launch_variant(c), s);
+    if (record) launch_colours32<P, true>(c, w, cur, dt, seed, fd_launch_variant(c), stage, s);
+    else launch_colours32<P, false>(c, w, cur, dt, seed, fd_launch_variant(c), stage, s);
   }
 }
 

@@ -7,8 +7,8 @@ namespace sdpd {
 
 template void fd_prepare<Fp64, Fp64>();
 template void fd_prepare<Fp64, Mixed>();
-template void launch_stage_geometry<Fp64, Fp64>(const Consts&, const Workspace&, int, cudaStream_t);
-template void launch_stage_geometry<Fp64, Mixed>(const Consts&, const Workspace&, int, cudaStream_t);
+template void launch_stage_geometry<Fp64, Fp64>(const Consts&, const Workspace&, cudaStream_t);
+template void launch_stage_geometry<Fp64, Mixed>(const Consts&, const Workspace&, cudaStream_t);
 template void launch_fd_colours<Fp64, Fp64>(const Consts&, const Workspace&, int, double, uint64_t, int,
                                           cudaStream_t);
 // float64 state, float32 pair arithmetic

@@ -6,7 +6,7 @@
 namespace sdpd {
 
 template void fd_prepare<Mixed, Mixed>();
-template void launch_stage_geometry<Mixed, Mixed>(const Consts&, const Workspace&, int, cudaStream_t);
+template void launch_stage_geometry<Mixed, Mixed>(const Consts&, const Workspace&, cudaStream_t);
 template void launch_fd_colours<Mixed, Mixed>(const Consts&, const Workspace&, int, double, uint64_t, int,
                                     cudaStream_t);
 

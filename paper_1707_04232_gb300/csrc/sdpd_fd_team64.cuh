@@ -148,7 +148,8 @@ __global__ void __launch_bounds__(team_threads<EMS>())
                   const uint32_t* __restrict__ hdr, const uint8_t* __restrict__ rsize,
                   const unsigned long long* __restrict__ sched_off, const uint32_t* __restrict__ pairs,
                   const double* __restrict__ geom, const double* __restrict__ rnd, const double* __restrict__ aux,
-                  int colour, uint64_t seed, unsigned long long* __restrict__ sweep_ptr, unsigned long long* counters,
+                  int colour, unsigned nblk, bool last, uint64_t seed,
+                  unsigned long long* __restrict__ sweep_ptr, unsigned long long* counters,
                   int* status, sdpd_pair_rec* recs, unsigned long long* rec_count, int64_t rec_cap,
                   unsigned* __restrict__ queue, const int32_t* __restrict__ order, int32_t* __restrict__ big_perm,
                   const int2* __restrict__ big_list, const uint32_t* __restrict__ big_count) {
@@ -169,7 +170,7 @@ __global__ void __launch_bounds__(team_threads<EMS>())
     if (t == 0) sm.next = atomicAdd(queue, 1u);
     __syncthreads();
     const unsigned wi = sm.next;
-    if ((int64_t)wi >= nown) break;
+    if (wi >= nblk) break;
     const int64_t w = order[colour * nown + wi];
     const int ox = 2 * (int)(w % hx) + (colour & 1), oy = 2 * (int)((w / hx) % hy) + ((colour >> 1) & 1),
               oz = 2 * (int)(w / ((int64_t)hx * hy)) + ((colour >> 2) & 1);
@@ -344,8 +345,8 @@ __global__ void __launch_bounds__(team_threads<EMS>())
     }
     __syncthreads();  // the team's shared memory is refilled by the next block
   }
-  // blocks beyond capacity, pair by pair, one per warp
-  for (;;) {
+  // blocks beyond capacity, pair by pair, one per warp (by the colour's last launch)
+  while (last) {
     unsigned bi = 0;
     if (lane == 0) bi = atomicAdd(&queue[2], 1u);
     bi = __shfl_sync(0xffffffffu, bi, 0);
@@ -372,7 +373,7 @@ __global__ void __launch_bounds__(team_threads<EMS>())
       queue[0] = 0u;
       queue[1] = 0u;
       queue[2] = 0u;
-      if (colour == 7) *sweep_ptr = sweep + 1ull;  // (every warp has read it) the sweep is done
+      if (colour == 7 && last) *sweep_ptr = sweep + 1ull;  // (every warp has read it) the sweep is done
     }
   }
   const unsigned c_tot = __reduce_add_sync(0xffffffffu, n_tot), c_rb = __reduce_add_sync(0xffffffffu, n_rb),
@@ -411,8 +412,9 @@ void team64_prepare() {
   team64_resident<false, false>();
 }
 
-template <bool EMS, bool REC>
-void launch_colours64(const Consts& c, const Workspace& w, int cur, double dt, uint64_t seed, cudaStream_t s) {
+template <bool EMS, bool REC, class Stage>
+void launch_colours64(const Consts& c, const Workspace& w, int cur, double dt, uint64_t seed, Stage stage,
+                      cudaStream_t s) {
   Team64Const k;
   k.x_par = -2.0 * c.kpar_m2 * (dt / c.m);
   k.x_perp = -2.0 * c.kperp_m2 * (dt / c.m);
@@ -421,22 +423,23 @@ void launch_colours64(const Consts& c, const Workspace& w, int cur, double dt, u
   k.de = -0.25 / c.m;
   k.CKm1 = c.C_K / c.kB - 1.0;
   k.scheme = c.scheme;
-  const int64_t nown = (int64_t)(c.nc[0] / 2) * (c.nc[1] / 2) * (c.nc[2] / 2);
-  const unsigned gf = (unsigned)std::max<int64_t>(1, std::min<int64_t>(nown, team64_resident<EMS, REC>()));
-  for (int col = 0; col < 8; ++col)
-    k_fd_colour64<EMS, REC><<<gf, team_threads<EMS>(), 0, s>>>(
+  for_colours(c, w, stage, [&](int col, int64_t first, int64_t n, bool last) {
+    const unsigned g = (unsigned)std::min<int64_t>(n, team64_resident<EMS, REC>());
+    k_fd_colour64<EMS, REC><<<g, team_threads<EMS>(), 0, s>>>(
         c, fd_const<double>(c, dt), k, view<Fp64>(w, cur), (D4*)w.qp4, w.cell_start, w.mrank, w.sched_hdr,
-        w.sched_rsize, w.sched_off, w.sched_pair, (const double*)w.st_geom, (const double*)w.st_rnd, w.st_aux, col,
-        seed, w.sweep, w.counters, w.status, REC ? w.pair_recs : nullptr, w.pair_rec_count, w.pair_rec_cap,
-        w.fd_queue + 4 * col, w.blk_order, w.big_perm, w.big_list, w.big_count);
+        w.sched_rsize, w.st_off, w.st_pair, (const double*)w.st_geom, (const double*)w.st_rnd, w.st_aux, col,
+        (unsigned)n, last, seed, w.sweep, w.counters, w.status, REC ? w.pair_recs : nullptr, w.pair_rec_count,
+        w.pair_rec_cap, w.fd_queue + 4 * col, w.blk_order + first, w.big_perm, w.big_list, w.big_count);
+  });
 }
-void launch_team64(const Consts& c, const Workspace& w, int cur, double dt, uint64_t seed, int record,
+template <class Stage>
+void launch_team64(const Consts& c, const Workspace& w, int cur, double dt, uint64_t seed, int record, Stage stage,
                    cudaStream_t s) {
   const bool ems = c.scheme == SDPD_SCHEME_EMS;
-  if (ems && record) launch_colours64<true, true>(c, w, cur, dt, seed, s);
-  else if (ems) launch_colours64<true, false>(c, w, cur, dt, seed, s);
-  else if (record) launch_colours64<false, true>(c, w, cur, dt, seed, s);
-  else launch_colours64<false, false>(c, w, cur, dt, seed, s);
+  if (ems && record) launch_colours64<true, true>(c, w, cur, dt, seed, stage, s);
+  else if (ems) launch_colours64<true, false>(c, w, cur, dt, seed, stage, s);
+  else if (record) launch_colours64<false, true>(c, w, cur, dt, seed, stage, s);
+  else launch_colours64<false, false>(c, w, cur, dt, seed, stage, s);
 }
 
 }  // namespace sdpd

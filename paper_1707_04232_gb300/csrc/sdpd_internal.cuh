@@ -72,6 +72,36 @@ struct Consts {
   int64_t fd_peers;  // blocks per colour of the ensemble whose members run at the same time; 0: a system alone
 };
 
+// Blocks of one colour.
+__host__ __device__ inline int64_t colour_blocks(const Consts& c) {
+  return (int64_t)(c.nc[0] >> 1) * (c.nc[1] >> 1) * (c.nc[2] >> 1);
+}
+// The staged pair data of all colours at once take 32 (float32 arithmetic) or
+// 72 bytes for each of the 80 pairs per particle that the lists can hold: 6.1
+// of a float64 handle's 7.5 KB per particle.  Beyond kSliceBlocks blocks per
+// colour, where that is more than twice the memory of a slice, they are staged
+// slice by slice instead: kSliceBlocks blocks of one colour, in the colour's
+// order, with room for the largest block in each block's place, so that no
+// distribution of the particles overflows it.  A sweep then has three launches
+// per slice, each colour more tails, and FD-only runs stage the geometry anew.
+// Sliced against all at once, ms per step and per FD-only step, workspace:
+// 168^3 particles mixed 19.1 / 10.0, 12 GB against 18.0 / 7.9, 19 GB; 256^3
+// mixed 66.4 / 34.4, 30 GB against 62.5 / 27.3, 69 GB (float64: 38 GB against
+// 125); slices of half the size 32.8 against 31.5 at 200^3.
+constexpr int kSliceBlocks = 32768;
+constexpr size_t kSlicePairs = (size_t)kSliceBlocks * kLargePairs;
+inline bool fd_sliced(const Consts& c) {
+  return colour_blocks(c) > kSliceBlocks && sched_pair_capacity(c.N, c.nbr_cap, c.ncell) > 2 * kSlicePairs;
+}
+// Entries of the staged arrays, and kernels per schedule and per sweep.
+inline size_t stage_capacity(const Consts& c) {
+  return fd_sliced(c) ? kSlicePairs : sched_pair_capacity(c.N, c.nbr_cap, c.ncell);
+}
+inline int schedule_launches(const Consts& c) { return fd_sliced(c) ? 4 : 5; }
+inline int sweep_launches(const Consts& c) {
+  return fd_sliced(c) ? 8 * 3 * (int)((colour_blocks(c) + kSliceBlocks - 1) / kSliceBlocks) : 9;
+}
+
 // Block schedules of the colour kernel (see launch_fd_colours) and the
 // thread-block sizes the pair passes accept.
 constexpr int kFdVariants = 5;
@@ -91,7 +121,7 @@ __host__ __device__ constexpr int fd_default_variant(bool mixed) { return mixed 
 // (24 members of 13^3 to 40^3 particles, 4 steps: 9.7 / 9.7 / 12.1 ms).
 inline int fd_launch_variant(const Consts& c) {
   if (!c.fd_auto && c.fd_variant >= 0 && c.fd_variant < kFdVariants) return c.fd_variant;
-  const int64_t nown = c.fd_peers > 0 ? c.fd_peers : (int64_t)(c.nc[0] / 2) * (c.nc[1] / 2) * (c.nc[2] / 2);
+  const int64_t nown = c.fd_peers > 0 ? c.fd_peers : colour_blocks(c);
   return nown <= 6 * 152 ? 2 : (nown <= 24 * 152 ? 1 : 0);
 }
 __host__ __device__ constexpr bool pair_threads_ok(int t) { return t == 32 || t == 64 || t == 128; }
@@ -334,6 +364,10 @@ struct Workspace {
   unsigned long long* sched_off;    // [ncell] where the block's pairs start in the arrays below
   unsigned long long* sched_total;  // entries of those arrays in use
   uint32_t* sched_pair;   // pairs round by round, block after block (local min-id | local max-id << 16)
+  // staged pair data, indexed like sched_pair, or (sliced) by place in the slice
+  unsigned long long* st_off;  // [ncell] where the block's data start: sched_off, or (sliced) its place in the slice
+  uint32_t* st_pair;      // the pairs: sched_pair, or (sliced) the slice's copy
+  uint32_t* blk_pos;      // sliced: [ncell] each block's place in its colour's order
   void* st_geom;          // per scheduled pair: unit vector, F / (rho_i rho_j)
   void* st_rnd;           // per scheduled pair: its random numbers (see k_stage_random)
   double* st_aux;         // float64 pair arithmetic: |G|^2 / 2 - ln U per scheduled pair
@@ -404,12 +438,13 @@ template <class P>
 void launch_force(const Consts& c, const Workspace& w, int cur, double half_dt, double dt_drift,
                   double* force_by_id, cudaStream_t s);
 // the sweep schedule: P the state's storage policy, width the most pairs of a
-// round (large_width: of a large block's); the staged geometry (arithmetic policy A) completes it
+// round (large_width: of a large block's); the staged geometry (arithmetic
+// policy A) completes it, unless the pair data are staged slice by slice
 template <class P>
 void launch_fd_schedule(const Consts& c, const Workspace& w, int cur, int width, int large_width, cudaStream_t s);
 int sched_prepare();  // launch attributes of the schedule's kernels (SDPD_OK or SDPD_ERR_CUDA)
 template <class P, class A>
-void launch_stage_geometry(const Consts& c, const Workspace& w, int cur, cudaStream_t s);
+void launch_stage_geometry(const Consts& c, const Workspace& w, cudaStream_t s);
 // one sweep (random numbers, then the colours): P the state's storage policy,
 // A the pair arithmetic (A = Mixed on float64 state: float32 pair updates)
 template <class P, class A = P>
