@@ -349,10 +349,8 @@ static void launch_pairsum(const Consts& c, const Workspace& w, const D4* vs4, d
                                                                  w.status);
 }
 
-void launch_adj_pairsum(const Consts& c, const Workspace& w, int cur, int mode, const D4* vs4, double* A,
-                        cudaStream_t s) {
+void launch_adj_pairsum(const Consts& c, const Workspace& w, int mode, const D4* vs4, double* A, cudaStream_t s) {
   if (c.N == 0) return;
-  (void)cur;
   if (c.kernel == SDPD_KERNEL_LUCY) {
     if (mode == 0) launch_pairsum<SDPD_KERNEL_LUCY, 0>(c, w, vs4, A, s);
     else launch_pairsum<SDPD_KERNEL_LUCY, 1>(c, w, vs4, A, s);

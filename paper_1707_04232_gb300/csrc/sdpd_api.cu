@@ -503,7 +503,6 @@ int sdpd_create(int64_t N, const double box[3], double m, double h, const sdpd_p
   c.pi_coef = c.c_rho / (c.C_K * c.m);
   c.f_h2 = (float)c.h2;
   c.f_inv_h = 1.0f / (float)c.h;
-  c.f_cW = (float)c.cW;
   c.f_cF = (float)c.cF;
   c.f_m = (float)c.m;
   c.f_m2 = (float)(c.m * c.m);
@@ -527,10 +526,7 @@ int sdpd_create(int64_t N, const double box[3], double m, double h, const sdpd_p
     // by the same bounds r >= h implies r_f^2 >= (1 - 8u) (h - 3 sqrt(3) D)^2
     const double ri = h - 3.0 * sqrt(3.0) * D;
     c.h2_inner = ri > 0.0 ? nextafterf((float)((1.0 - 8.0 * u) * ri * ri), -INFINITY) : -1.0f;
-    for (int d = 0; d < 3; ++d) {
-      c.Lf[d] = (float)c.L[d];
-      c.halfLf[d] = 0.5f * c.Lf[d];
-    }
+    for (int d = 0; d < 3; ++d) c.Lf[d] = (float)c.L[d];
   }
   c.kernel = prm->kernel;
   c.fd_variant = fd_default_variant(prm->precision == SDPD_MIXED || prm->sweep_f32 != 0);
@@ -1156,7 +1152,7 @@ int sdpd_vv_adjoint(sdpd_t* s, void* tape, size_t tape_bytes, const double* gq, 
         launch_adj_gather(c, s->w, s->cur, t.pbar, 0.5 * dt, t.vs4, st);
       }
       StageTimer tm(s, 7, 1);
-      launch_adj_pairsum(c, s->w, s->cur, 0, t.vs4, t.A, st);
+      launch_adj_pairsum(c, s->w, 0, t.vs4, t.A, st);
     }
     {
       StageTimer tm(s, 9, 1);
@@ -1207,7 +1203,7 @@ int sdpd_virial(sdpd_t* s, double* value, double* gq, double* gp, double* geps, 
   double* thbar = s->w.io_q;
   double* sums = s->w.obs + 8;  // slots 8..11 of the observables' output block
   const double wt = 1.0 / (3.0 * c.L[0] * c.L[1] * c.L[2]);
-  launch_adj_pairsum(c, s->w, s->cur, 1, vs4, A, st);
+  launch_adj_pairsum(c, s->w, 1, vs4, A, st);
   launch_adj_mid_virial(c, s->w, s->cur, A, wt, vs4, val_id, grad ? gp : nullptr, geps, thbar, st);
   if (grad) launch_adj_back(c, s->w, s->cur, 1, wt, vs4, 0, gq, thbar, st);
   launch_adj_sum(val_id, c.N, 1, (double*)s->w.obs_partial, sums, st);

@@ -133,11 +133,12 @@ __device__ __forceinline__ bool negative(double x) {
 // float64 instructions per warp.  With one thread per particle the kept
 // neighbour's branch ran on nearly every candidate of the 27 cells (one lane
 // in six keeps one): ~500 evaluations instead of ~80.  Here kLanes64 lanes
-// share a particle (a whole warp where particles are few).  The search is float32: r^2 from the float32 positions
-// decides a candidate unless it lies within its rounding bound of h^2 (then
-// the float64 predicate does), and the kept ones are appended in walk order
-// (ballot and prefix count) to a list in shared memory.  Only list entries
-// see float64 arithmetic, with all lanes at work.
+// share a particle (a whole warp where particles are few).  The search is
+// float32: r^2 from the float32 positions decides a candidate unless it lies
+// within its rounding bound of h^2 (then the float64 predicate does), and the
+// kept ones are appended in walk order (ballot and prefix count) to a list in
+// shared memory.  Only list entries see float64 arithmetic, with all lanes at
+// work.
 // ---------------------------------------------------------------------------
 constexpr int kLanes64 = 8;
 
@@ -330,7 +331,9 @@ __device__ __forceinline__ double group_sum(double v) {
 // Lanes per particle of the float64 passes: with few particles a whole warp
 // each, which spreads them over the SM quarters and shortens every particle's
 // chain; else kLanes64, which costs fewer instructions in all.  The line lies
-// at four warps per SM quarter.
+// at four warps per SM quarter, below where they are even (a Verlet step with a
+// warp and with kLanes64 lanes, us: 1000 particles 46 / 66, 2197 76 / 90, 2744
+// 86 / 100, 3375 99 / 90, 8000 161 / 125).
 inline bool pair64_wide(const Consts& c) { return c.N <= 16 * 152; }
 
 }  // namespace sdpd

@@ -1,7 +1,8 @@
 // sdpd_fd_colour.cuh -- one pair update of the fluctuation/dissipation sweep
-// (Sections 3.2-3.3) and the colour kernel that runs a colour's blocks level
-// by level.  Included by one translation unit per precision, each of which
-// instantiates the block-schedule variants of its precision.
+// (Sections 3.2-3.3), the kernels that stage the pairs' data, and the colour
+// kernels that run a colour's blocks round by round.  Included by one
+// translation unit per precision, each of which instantiates the
+// block-schedule variants of its precision.
 #pragma once
 #include <algorithm>
 #include <type_traits>
@@ -16,7 +17,7 @@ namespace sdpd {
 // ---------------------------------------------------------------------------
 template <class R>
 struct FDConst {
-  R m, inv_m, half_m, inv_h, cF;
+  R inv_m, half_m;
   R kpar_m2, kperp_m2;  // (10/3 eta + 4 zeta) m^2, (5/3 eta - zeta) m^2
   R inv_C_K, kB, two_over_CK, dt_over_m;
   R CKm1;               // C_K / kB - 1
@@ -26,8 +27,9 @@ struct FDConst {
   int scheme;
 };
 
-// Elementary functions of the sweep.  float64: the correctly rounded /
-// accurate library versions.  float32 (mixed path): hardware approximations
+// Elementary functions of the sweep.  float64 (the pairs' geometry and the
+// pair-by-pair sweep; the team kernel has its own, sdpd_f64.cuh): the library's
+// functions.  float32 (mixed path): hardware approximations
 // (relative error ~1e-7) for the proposal coefficients and Box-Muller -- the
 // Metropolis step stays exact for any deterministic proposal coefficients
 // because the forward and reverse moves use the same functions -- and the
@@ -1587,11 +1589,8 @@ __global__ void __launch_bounds__(64) k_fd_colour_spec(const __grid_constant__ F
 template <class R>
 static FDConst<R> fd_const(const Consts& c, double dt) {
   FDConst<R> k;
-  k.m = (R)c.m;
   k.inv_m = (R)(1.0 / c.m);
   k.half_m = (R)(0.5 * c.m);
-  k.inv_h = (R)(1.0 / c.h);
-  k.cF = (R)c.cF;
   k.kpar_m2 = (R)c.kpar_m2;
   k.kperp_m2 = (R)c.kperp_m2;
   k.inv_C_K = (R)(1.0 / c.C_K);

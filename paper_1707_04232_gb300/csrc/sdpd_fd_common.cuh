@@ -6,8 +6,6 @@
 
 namespace sdpd {
 
-constexpr int kRowWords = kMaxBlock / 32;  // words of one bitmap row
-
 // Cells of the block of owner (ox, oy, oz): start / count in storage order,
 // and the local offset of each cell in the block's concatenation.
 struct BlockCells {

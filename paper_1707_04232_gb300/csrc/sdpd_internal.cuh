@@ -53,7 +53,7 @@ struct Consts {
   double pi_coef;            // pressure over rho^2: pi = pi_coef eps / rho, c_rho / (C_K m)
   // the same for float32 arithmetic (a conversion or a division of these by
   // every thread would cost float64 issues)
-  float f_h2, f_inv_h, f_cW, f_cF, f_m, f_m2, f_W0, f_scale[3], f_eos, f_pi_coef;
+  float f_h2, f_inv_h, f_cF, f_m, f_m2, f_W0, f_scale[3], f_eos, f_pi_coef;
   double kpar_m2, kperp_m2;  // (10/3 eta + 4 zeta) m^2 and (5/3 eta - zeta) m^2
   double cW, cF, W0;         // kernel constants and W(0)
   int kernel, scheme;
@@ -64,7 +64,7 @@ struct Consts {
   // set on the host), so it is skipped without float64 arithmetic.
   // Below h2_inner it has r^2 < h^2 for certain; only in between does the
   // float64 predicate decide.
-  float Lf[3], halfLf[3], h2_filter, h2_inner;
+  float Lf[3], h2_filter, h2_inner;
   // launch shapes (results do not depend on them): the block schedule of the
   // sweep's colour launches and the threads per block of the pair passes
   int fd_variant, pair_threads;
@@ -465,8 +465,7 @@ void launch_advance_sweep(const Workspace& w, cudaStream_t s);
 // order.  mode: 0 kick pulled back along v, 1 virial, 2 density term only.
 void launch_adj_gather(const Consts& c, const Workspace& w, int cur, const double* pbar_id, double scale, D4* vs4,
                        cudaStream_t s);
-void launch_adj_pairsum(const Consts& c, const Workspace& w, int cur, int mode, const D4* vs4, double* A,
-                        cudaStream_t s);
+void launch_adj_pairsum(const Consts& c, const Workspace& w, int mode, const D4* vs4, double* A, cudaStream_t s);
 void launch_adj_mid_step(const Consts& c, const Workspace& w, int cur, const double* A, bool kick1, bool kick2,
                          const double* deps_prev, double* Sbar_cur, double* Sbar_prev, const double* epsbar_n,
                          double* epsbar0, D4* vs4, double* thbar, cudaStream_t s);
