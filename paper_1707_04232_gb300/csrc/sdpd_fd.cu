@@ -34,6 +34,7 @@
 // vectors and friction factors).  A sweep is then k_stage_random (the pairs'
 // random numbers) and one colour launch per colour (sdpd_fd_colour.cuh,
 // sdpd_fd_team64.cuh): the pair updates round by round in shared memory.
+// (Large systems: geometry, random numbers and colour launch slice by slice.)
 #include <algorithm>
 #include <type_traits>
 

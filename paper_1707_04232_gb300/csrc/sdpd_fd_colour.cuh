@@ -542,7 +542,8 @@ __device__ __forceinline__ int block_gidx(const FdCells& c, int q) {
 // depends on positions and densities only, and the random numbers once per
 // sweep.  Outside the colour launches this work has full warps and the whole
 // GPU, also when a colour has few blocks; inside them it sat on the path of
-// every block's dependency chain.
+// every block's dependency chain.  Large systems stage both slice by slice, each
+// just before its colour launch (fd_sliced).
 // ---------------------------------------------------------------------------
 constexpr int kStageWarps = 4;
 

@@ -11,10 +11,10 @@
 // across e, lane 3 the energies and the direction along e.  The coefficients
 // (exponential, square root), the components of the proposal and of the
 // reverse noise, and the logarithms of the Metropolis ratio are each
-// evaluated once per instruction for the whole pair: about 85 float64
+// evaluated once per instruction for the whole pair: about 90 float64
 // instructions per round.  Rounds hold at most 16 pairs (8 per warp).
-// One pass of 1000 particles (EMS): 47.0 ms with one lane per pair, 8.0 ms
-// now; 32,768 particles, two steps: 40.4 and 6.3 ms.
+// One pass of 1000 particles (EMS): 46.4 ms with one lane per pair, 8.1 ms
+// now; 32,768 particles, two steps: 40.1 and 6.5 ms.
 //
 // EMS: the proposal and the Metropolis test (about half of them each) run on
 // different warps, one round apart.  Two warps propose round r and write its
