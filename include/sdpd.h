@@ -116,7 +116,8 @@ typedef struct {
  * length h; Section 4: ideal gas of particle size K, heat capacity
  * C_K = 3/2 (K-1) kB).  Host only: validates the parameters (K > 4/3 so that
  * d_ij < 1 in Eq. (sdpd-gamma-sigma); every box side gives an even number
- * >= 4 of cells of side >= h), chooses the cell grid and the workspace size.
+ * >= 4 of cells of side >= h; N <= 2^26, the indices that a neighbour-list
+ * entry holds), chooses the cell grid and the workspace size.
  * stream: a cudaStream_t (NULL = the legacy default stream).
  * Errors: SDPD_ERR_INVALID_ARG, SDPD_ERR_BOX_TOO_SMALL, SDPD_ERR_HOST_MEMORY
  * (the per-cell tables, 4 + 4 + 16 bytes per cell, do not fit in host

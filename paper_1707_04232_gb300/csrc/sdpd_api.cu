@@ -442,7 +442,7 @@ int sdpd_create(int64_t N, const double box[3], double m, double h, const sdpd_p
   if (!out) return SDPD_ERR_INVALID_ARG;
   *out = nullptr;
   if (!box || !prm) return SDPD_ERR_INVALID_ARG;
-  if (N < 0 || N >= (int64_t)INT32_MAX) return SDPD_ERR_INVALID_ARG;
+  if (N < 0 || N > kMaxParticles) return SDPD_ERR_INVALID_ARG;
   if (!(m > 0) || !isfinite(m) || !(h > 0) || !isfinite(h)) return SDPD_ERR_INVALID_ARG;
   if (!(K > 4.0 / 3.0) || !isfinite(K)) return SDPD_ERR_INVALID_ARG;
   if (!(prm->kB > 0) || !isfinite(prm->kB)) return SDPD_ERR_INVALID_ARG;

@@ -128,6 +128,7 @@ __host__ __device__ constexpr bool pair_threads_ok(int t) { return t == 32 || t 
 
 // Neighbour-list entry: neighbour index << 6 | stencil offset code, the code
 // holding (o + 1) per axis in 2 bits (x lowest) for o in {-1, 0, +1}.
+constexpr int64_t kMaxParticles = 1ll << 26;  // indices that an entry holds
 __host__ __device__ __forceinline__ uint32_t nbr_entry(int j, int ox, int oy, int oz) {
   return ((uint32_t)j << 6) | (uint32_t)((ox + 1) | ((oy + 1) << 2) | ((oz + 1) << 4));
 }

@@ -30,3 +30,14 @@ def test_large_systems_take_under_1800_bytes_per_particle_and_a_slice(kw):
 
 def test_up_to_there_a_system_stays_below_a_ninth_of_the_device():
     assert 9 * workspace(160, precision=sdpd.FP64) <= 284208 * 2 ** 20
+
+
+def test_particle_numbers_beyond_a_list_entry_are_refused():
+    """A neighbour-list entry keeps 26 bits of the neighbour's index."""
+    p = sdpd.sdpd_params(kB=1.0, eta=1.0, zeta=0.0, c_rho=-1.0, kernel=sdpd.KERNEL_LUCY, scheme=sdpd.SCHEME_EMS,
+                         precision=sdpd.MIXED, theta=1)
+    for N, expect in ((2 ** 26, sdpd.OK), (2 ** 26 + 1, sdpd.ERR_INVALID_ARG)):
+        st, h = sdpd.sdpd_create(N, (100.0,) * 3, 1.0, 2.5, p, 50.0, 0)
+        assert st == expect
+        if h:
+            sdpd.sdpd_destroy(h)
